@@ -63,7 +63,7 @@ struct ddm_ctx {
   // range selection for ddm_write over a sub-range of updates
   DevBuf sel_offs, sel_list;
   // replay records of the count pass
-  DevBuf rec, blk_next, blk_count, blk_pkt, pkt_first, pkt_nblk, pkt_off, blk_list,
+  DevBuf rec, blk_next, blk_count, pkt_nblk, pkt_off, blk_list,
       blk_counter;
   uint64_t replay_budget = 0;   // bytes; 0 = never record
   uint32_t rec_blocks = 0;      // blocks of the current arena
@@ -469,25 +469,28 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
   c->arena = RecordArena{};
   if (record && c->replay_on && m > 0 && c->tree.n > 0 && c->replay_budget > 0) {
     const uint32_t packets = packets_of(c, m);
-    // bytes per block: records (ten bytes each) and header, next/count/packet/list entries
-    const uint64_t per_block = (uint64_t)kRecWords * sizeof(uint32_t) + 4 * sizeof(uint32_t);
+    // bytes per block: records (ten bytes each) and header, next/count/list entries
+    const uint64_t per_block =
+        (uint64_t)kRecWords * sizeof(uint32_t) + 2 * sizeof(uint32_t) + sizeof(uint4);
     // Blocks the arena holds now, and what the latest recorded pass needed.
     uint64_t have = c->rec.cap / ((size_t)kRecWords * sizeof(uint32_t));
-    for (const DevBuf* b : {&c->blk_next, &c->blk_count, &c->blk_pkt, &c->blk_list})
+    for (const DevBuf* b : {&c->blk_next, &c->blk_count})
       have = std::min<uint64_t>(have, b->cap / sizeof(uint32_t));
+    have = std::min<uint64_t>(have, c->blk_list.cap / sizeof(uint4));
     const uint32_t hint_blocks = c->rec_hint[0], hint_packets = c->rec_hint[1],
                    hint_max = c->rec_hint[2];
     uint64_t want = have;
-    if (have == 0 || (hint_packets && hint_blocks > hint_max)) {
-      // No arena yet, or the last pass ran out of it: size from that pass's
-      // blocks per packet (plus 1/8 and some slack), else 2 per packet.  An
+    if (have < (uint64_t)packets * kRecChains || (hint_packets && hint_blocks > hint_max)) {
+      // No arena yet, not a block for each chain, or the last pass ran out of
+      // it: size from that pass's blocks per packet (plus 1/8 and some
+      // slack), else one per chain and as many again per packet.  An
       // arena that sufficed is kept as it is: the blocks per packet depend on
       // how densely the updates cover the space, so extrapolating them from
       // one plan to the next would reallocate for nothing.
       const uint64_t need =
           hint_packets ? (uint64_t)((double)hint_blocks / (double)hint_packets * 1.125 *
                                     (double)packets) + 64
-                       : 2ull * packets;
+                       : (kRecChains + 1ull) * packets;
       want = std::max(have, need);
     }
     const uint64_t cap_blocks = c->replay_budget / per_block;
@@ -496,9 +499,7 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
     if (want > 0 && ensure(c, c->rec, (size_t)want * kRecWords * sizeof(uint32_t)) == DDM_OK &&
         ensure(c, c->blk_next, (size_t)want * sizeof(uint32_t)) == DDM_OK &&
         ensure(c, c->blk_count, (size_t)want * sizeof(uint32_t)) == DDM_OK &&
-        ensure(c, c->blk_pkt, (size_t)want * sizeof(uint32_t)) == DDM_OK &&
-        ensure(c, c->blk_list, (size_t)want * sizeof(uint32_t)) == DDM_OK &&
-        ensure(c, c->pkt_first, (size_t)packets * kRecChains * sizeof(uint32_t)) == DDM_OK &&
+        ensure(c, c->blk_list, (size_t)want * sizeof(uint4)) == DDM_OK &&
         ensure(c, c->pkt_nblk, (size_t)packets * kRecChains * sizeof(uint32_t)) == DDM_OK &&
         ensure(c, c->pkt_off, ((size_t)packets * kRecChains + 1) * sizeof(unsigned long long)) ==
             DDM_OK &&
@@ -506,12 +507,11 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
       c->arena.rec = static_cast<uint32_t*>(c->rec.p);
       c->arena.blk_next = static_cast<uint32_t*>(c->blk_next.p);
       c->arena.blk_count = static_cast<uint32_t*>(c->blk_count.p);
-      c->arena.pkt_first = static_cast<uint32_t*>(c->pkt_first.p);
-      c->arena.blk_pkt = static_cast<uint32_t*>(c->blk_pkt.p);
-      c->arena.blk_list = static_cast<uint32_t*>(c->blk_list.p);
+      c->arena.blk_list = static_cast<uint4*>(c->blk_list.p);
       c->arena.pkt_nblk = static_cast<uint32_t*>(c->pkt_nblk.p);
       c->arena.pkt_off = static_cast<unsigned long long*>(c->pkt_off.p);
       c->arena.blk_counter = static_cast<uint32_t*>(c->blk_counter.p);
+      c->arena.chains = packets * kRecChains;
       c->arena.max_blocks = (uint32_t)want;
       DDM_CUDA(cudaMemsetAsync(c->blk_counter.p, 0, 4 * sizeof(uint32_t), s));
     }
@@ -699,7 +699,7 @@ int ddm_destroy(ddm_ctx* c) {
                     &c->counters, &c->e, &c->sid, &c->nodes, &c->tab, &c->qe, &c->qid, &c->counts,
                     &c->counts_pos, &c->offsets, &c->pos_offsets, &c->sums, &c->work,
                     &c->sel_offs, &c->sel_list, &c->rec, &c->blk_next, &c->blk_count,
-                    &c->blk_pkt, &c->pkt_first, &c->pkt_nblk, &c->pkt_off,
+                    &c->pkt_nblk, &c->pkt_off,
                     &c->blk_list, &c->blk_counter, &c->inst_s, &c->inst_u, &c->bglog2,
                     &c->bngroups, &c->bgbase, &c->cls_hist, &c->cls_off, &c->probe, &c->aos})
     release(*b);

@@ -82,6 +82,7 @@ struct QueryView {
   uint32_t first;                 // without list: run positions first .. first+nq-1
   uint32_t nq;                    // number of queries to run
   uint32_t qpp_log2;              // log2 of the queries per packet (4 or 5: 16 or 32)
+  uint32_t take_log2;             // log2 of the packets a warp takes per ticket
   uint32_t tmin;                  // count pass: swapped leaf loops from this many queries
 };
 
@@ -220,14 +221,22 @@ cudaError_t launch_export_nodes(const TreeView& t, float* node_lo, float* node_h
 // lane, the hit mask over the leaf's 32 subscriptions, and (16 bits) the
 // query's matches before this leaf counted from the start of the record's
 // block.  Records of a packet are kept in walk order (leaf by leaf, query
-// lanes ascending within a leaf), in chains of fixed-size blocks taken from a
-// shared arena; a block stores its packet, and a header with the matches each
-// query of its chain had before the block's first record, so that a record's
-// place in its query's output is the header entry plus its 16-bit count (a
-// block holds at most 512 records of at most 32 hits: the count stays below
-// 2^14).  After counting, the blocks are listed in plan order and the write
-// pass expands any range of them, every record independently, instead of
-// walking the tree again.
+// lanes ascending within a leaf), in chains of fixed-size blocks of a shared
+// arena; a block has a header with the matches each query of its chain had
+// before the block's first record, so that a record's place in its query's
+// output is the header entry plus its 16-bit count (a block holds at most 512
+// records of at most 32 hits: the count stays below 2^14).  After counting,
+// the blocks are listed in plan order and the write pass expands any range of
+// them, every record independently, instead of walking the tree again.
+//
+// The first block of each chain belongs to it from the start (its header is
+// zero); only the blocks after it are taken from a counter, so that the
+// packets of a sparse problem make no atomic.  When neither chain of a packet
+// needs a second block and their records fit one, the two blocks are one
+// entry of the list, and the write pass takes them as one.  With every block
+// from the counter and an entry each, the count pass of 2.5e7 + 2.5e7 extents
+// (d = 1, alpha = 1) took 2.81 ms and the write pass 2.58 ms; now 1.73 and
+// 1.47 ms.
 constexpr uint32_t kRecBlock = 512;  // records per block: x and hit mask 2 KiB each, counts 1 KiB
 constexpr uint32_t kRecHdr = 16;     // header: one running count per query of the chain
 // words per block: x[kRecBlock], hit mask[kRecBlock], 16-bit counts, header
@@ -236,27 +245,31 @@ constexpr uint32_t kRecWords = 2 * kRecBlock + kRecBlock / 2 + kRecHdr;
 // lanes, so that a block holds the records of at most 16 queries (its pairs
 // land in fewer output runs): the write pass took 127 instead of 134 ms on
 // the clustered d = 3 workload, the count pass 5 ms more.  Chain c of packet
-// p is chain index p * kRecChains + c of the arena's per-chain arrays.
+// p is chain index p * kRecChains + c of the arena's per-chain arrays, and its
+// first block has that number.
 constexpr uint32_t kRecChains = 2;
 constexpr uint32_t kNoBlock = 0xffffffffu;
 struct RecordArena {
   uint32_t* rec;           // [max_blocks][kRecWords]: x, hit mask, 16-bit counts, header
   uint32_t* blk_next;      // [max_blocks] next block of the chain, or kNoBlock
   uint32_t* blk_count;     // [max_blocks] records in the block
-  uint32_t* blk_pkt;       // [max_blocks] packet of the block
-  uint32_t* pkt_first;     // [chains] first block of each chain, or kNoBlock
-  uint32_t* pkt_nblk;      // [chains] blocks of each chain
+  uint32_t* pkt_nblk;      // [chains] list entries of each chain
   unsigned long long* pkt_off;  // [chains + 1] exclusive prefix of pkt_nblk
-  uint32_t* blk_list;      // [max_blocks] blocks in plan order (packet, then chain)
-  uint32_t* blk_counter;   // [0] blocks handed out (may exceed max_blocks),
-                           // [1] blocks the whole pass needed, [2] packets,
-                           // [3] max_blocks (the last two for arena sizing)
+  uint4* blk_list;         // [max_blocks] blocks in plan order (packet, then
+                           // chain): block, packet, its records, and those of
+                           // the next block when the two are one entry
+  uint32_t* blk_counter;   // [0] blocks handed out beyond the chains' first (may
+                           // exceed the arena), [1] such blocks the whole pass
+                           // needed, then (k_block_list) all blocks it needed,
+                           // [2] packets, [3] max_blocks (for arena sizing)
+  uint32_t chains;         // chains of the plan's packets
   uint32_t max_blocks;     // 0: no recording
 };
 // The records of the last count pass are complete (the write pass may
 // replay them) iff recording was on and the arena did not run out.
 __device__ __forceinline__ bool records_complete(const RecordArena& ra) {
-  return ra.max_blocks > 0 && ra.blk_counter[0] <= ra.max_blocks;
+  return ra.max_blocks > 0 &&
+         (unsigned long long)ra.chains + ra.blk_counter[0] <= ra.max_blocks;
 }
 
 // counts[update id] (and counts_pos[sorted position], if not null); records

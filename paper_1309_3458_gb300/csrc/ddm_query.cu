@@ -50,6 +50,11 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
+// The first blocks of a packet's two chains are one list entry: neither chain
+// goes on (`more` blocks after them) and their records fit one block.
+__device__ __forceinline__ bool one_entry(uint32_t more, uint32_t n0, uint32_t n1) {
+  return more == 0u && n0 + n1 <= kRecBlock;
+}
 // Without rank tables (d > 3, or no room for them) the swapped leaf test
 // compares the leaf's 32 subscriptions one by one, which pays only from about
 // this many queries on a leaf.
@@ -207,10 +212,18 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
 
   const uint32_t qpp = 1u << q.qpp_log2;  // queries per packet: 16 or 32
   const uint32_t npk = (q.nq + qpp - 1u) >> q.qpp_log2;
-  for (;;) {
-    uint32_t p = 0;
-    if (lane == 0) p = atomicAdd(work, 1u);
-    p = __shfl_sync(0xffffffffu, p, 0);
+  // Summed over the warp's packets and added once at the end (or before the
+  // 32 bits could run out): atomics on one word by every packet would
+  // serialise the pass.
+  uint32_t ntests = 0;
+  uint32_t p = blockIdx.x * kWarps + wib;
+  for (bool first = true;; first = false) {
+    if (!work) {  // a warp for every packet
+      if (!first) break;
+    } else if (first || (++p & ((1u << q.take_log2) - 1u)) == 0u) {  // the next few packets
+      if (lane == 0) p = atomicAdd(work, 1u) << q.take_log2;
+      p = __shfl_sync(0xffffffffu, p, 0);
+    }
     if (p >= npk) break;
 
     // ---- the packet: up to qpp queries, one per lane ----
@@ -254,7 +267,7 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
       if (a < d)
         s_q[wib][lane][k2] = make_float4(ql[a], qh[a], b < d ? ql[b] : 0.f, b < d ? qh[b] : 0.f);
     }
-    uint32_t cnt = 0, ntests = 0;
+    uint32_t cnt = 0;
     unsigned long long out = 0;
     if (WRITE && valid) out = w.start[w.by_pos ? pos : Q] - base0;
     __syncwarp();
@@ -263,9 +276,9 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
     // leaf by leaf with one coalesced store.  After the arena runs out the
     // packet stops writing but keeps counting the blocks it would need.
     const bool recording = !WRITE && ra.max_blocks > 0;
-    bool rec_write = recording;
-    uint32_t cur0 = kNoBlock, cur1 = kNoBlock, fill0 = kRecBlock, fill1 = kRecBlock;
-    uint32_t nblk0 = 0, nblk1 = 0;
+    bool rec_write = recording && ra.chains <= ra.max_blocks;
+    uint32_t cur0 = p * 2u, cur1 = p * 2u + 1u, fill0 = 0, fill1 = 0;
+    uint32_t nblk0 = 0, nblk1 = 0;  // blocks after each chain's first
     uint32_t blk_cnt = 0;  // this query's matches before its chain's current block
     // Test the 32 level-1 nodes (leaves) from g1 on against the packet box,
     // then run the packet's queries over each surviving leaf.
@@ -512,17 +525,13 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
                 uint32_t b = 0;
                 if (lane == 0) b = atomicAdd(&ra.blk_counter[0], 1u);
                 b = __shfl_sync(0xffffffffu, b, 0);
-                if (b >= ra.max_blocks) {
+                if (b >= ra.max_blocks - ra.chains) {
                   rec_write = false;  // arena exhausted: the write pass walks instead
                 } else {
+                  b += ra.chains;
                   if (lane == 0) {
-                    if (cb == kNoBlock) {
-                      ra.pkt_first[(size_t)p * 2u + ch] = b;
-                    } else {
-                      ra.blk_next[cb] = b;
-                      ra.blk_count[cb] = fl;
-                    }
-                    ra.blk_pkt[b] = p;
+                    ra.blk_next[cb] = b;
+                    ra.blk_count[cb] = fl;
                   }
                   // header: the chain's queries' matches before this leaf
                   if ((uint32_t)(lane >> 4) == (uint32_t)ch) {
@@ -617,42 +626,57 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
       counts[Q] = cnt;
       if (counts_pos) counts_pos[pos] = cnt;
     }
-    if (!WRITE && st && lane == 0 && ntests) atomicAdd(&st->tests, (unsigned long long)ntests);
-    if (recording && lane == 0) {
+    if (!WRITE && (ntests >> 30)) {  // a packet adds at most 32 x 2^25
+      if (st && lane == 0) atomicAdd(&st->tests, (unsigned long long)ntests);
+      ntests = 0;
+    }
+    if (recording) {
+      if (lane == 0 && nblk0 + nblk1) atomicAdd(&ra.blk_counter[1], nblk0 + nblk1);
       if (rec_write) {
-        if (cur0 == kNoBlock) {
-          ra.pkt_first[(size_t)p * 2u] = kNoBlock;
-        } else {
-          ra.blk_next[cur0] = kNoBlock;
-          ra.blk_count[cur0] = fill0;
+        // the first blocks' headers: no query had matches before them
+        const uint32_t ch = (uint32_t)lane >> 4;
+        ra.rec[((size_t)p * 2u + ch) * kRecWords + 2u * kRecBlock + kRecBlock / 2u + (lane & 15)] = 0u;
+        const bool one = one_entry(nblk0 + nblk1, fill0, fill1);
+        if (lane < 2) {
+          const uint32_t cb = lane ? cur1 : cur0, fl = lane ? fill1 : fill0;
+          ra.blk_next[cb] = kNoBlock;
+          ra.blk_count[cb] = fl;
+          uint32_t entries = lane ? (one ? 0u : nblk1 + (fill1 ? 1u : 0u))
+                                  : (one ? (fill0 + fill1 ? 1u : 0u) : nblk0 + (fill0 ? 1u : 0u));
+          ra.pkt_nblk[(size_t)p * 2u + lane] = entries;
         }
-        if (cur1 == kNoBlock) {
-          ra.pkt_first[(size_t)p * 2u + 1u] = kNoBlock;
-        } else {
-          ra.blk_next[cur1] = kNoBlock;
-          ra.blk_count[cur1] = fill1;
-        }
+      } else if (lane < 2) {
+        ra.pkt_nblk[(size_t)p * 2u + lane] = 0u;
       }
-      ra.pkt_nblk[(size_t)p * 2u] = rec_write ? nblk0 : 0u;
-      ra.pkt_nblk[(size_t)p * 2u + 1u] = rec_write ? nblk1 : 0u;
-      if (nblk0 + nblk1) atomicAdd(&ra.blk_counter[1], nblk0 + nblk1);
     }
   }
+  if (!WRITE && st && lane == 0 && ntests) atomicAdd(&st->tests, (unsigned long long)ntests);
 }
 
-// Plan-order list of record blocks: one thread per chain copies it (chains of
-// a packet in lane order, packets in plan order).
+// Plan-order list of record blocks: one thread per packet lists its chains
+// (in lane order, packets in plan order).
 __global__ void k_block_list(RecordArena ra, uint32_t packets) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {  // sizing hint for the next arena
+    ra.blk_counter[1] += ra.chains;
     ra.blk_counter[2] = packets;
     ra.blk_counter[3] = ra.max_blocks;
   }
   if (!records_complete(ra)) return;
-  const uint32_t chains = packets * kRecChains;
-  for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < chains;
+  for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < packets;
        p += gridDim.x * blockDim.x) {
-    unsigned long long at = ra.pkt_off[p];
-    for (uint32_t b = ra.pkt_first[p]; b != kNoBlock; b = ra.blk_next[b]) ra.blk_list[at++] = b;
+    unsigned long long at = ra.pkt_off[(size_t)p * kRecChains];
+    const uint32_t b0 = p * kRecChains, n0 = ra.blk_count[b0], n1 = ra.blk_count[b0 + 1];
+    const uint32_t x0 = ra.blk_next[b0], x1 = ra.blk_next[b0 + 1];
+    if (one_entry((x0 != kNoBlock) + (x1 != kNoBlock), n0, n1)) {
+      if (n0 + n1) ra.blk_list[at] = make_uint4(b0, p, n0, n1);
+      continue;
+    }
+    if (n0) ra.blk_list[at++] = make_uint4(b0, p, n0, 0u);
+    for (uint32_t b = x0; b != kNoBlock; b = ra.blk_next[b])
+      ra.blk_list[at++] = make_uint4(b, p, ra.blk_count[b], 0u);
+    if (n1) ra.blk_list[at++] = make_uint4(b0 + 1u, p, n1, 0u);
+    for (uint32_t b = x1; b != kNoBlock; b = ra.blk_next[b])
+      ra.blk_list[at++] = make_uint4(b, p, ra.blk_count[b], 0u);
   }
 }
 
@@ -712,6 +736,8 @@ __device__ __forceinline__ void st_hinted(uint32_t* a, uint32_t v, unsigned long
 // fields exchanged (roles swapped: the tree holds the updates); kOutIds the
 // compressed output, only each pair's subscription id (4 bytes) at the
 // pair's position.
+// Pairs per list entry of the range up to which entries count as short.
+constexpr uint32_t kShortEntry = 256;
 constexpr int kOutPairs = 0, kOutSwapped = 1, kOutIds = 2;
 // Resident CTAs per SM and records expanded per group (their id loads issued
 // before their stores) of the replay kernel, by output form.  Pairs (8-byte
@@ -735,50 +761,87 @@ struct ReplayShape {
   // a round of 32 records is expanded in whole groups
   static_assert(32 % group == 0, "records in flight must divide a round of 32");
 };
-template <bool FILTER_ID, bool WIDE, bool BATCH, int OUT>
-__global__ void __launch_bounds__(kThreads, ReplayShape<OUT>::ctas)
-k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uint32_t p0,
-         uint32_t p1, uint32_t pb, uint32_t pe, uint32_t idb, uint32_t ide,
-         uint32_t* __restrict__ work, Status* __restrict__ st) {
+// Shared memory of the replay kernel.
+template <bool WIDE, int OUT>
+struct ReplaySmem {
   using Cursor = typename std::conditional<WIDE, unsigned long long, uint32_t>::type;
   // Per record: leaf, hit mask, update id, and the output position of its first
   // pair (32-bit positions, not batched: one 128-bit load per record) or else
-  // the subscription id base, the position then in s_at.
-  __shared__ uint4 s_rec[kWarps][32];
-  __shared__ Cursor s_at[kWarps][32];
-  constexpr bool kDense = ReplayShape<OUT>::dense;
-  // dense expansion: each round's pairs as a list of (record, leaf slot)
-  __shared__ uint32_t s_pre[kDense ? kWarps : 1][32];
-  __shared__ uint16_t s_list[kDense ? kWarps : 1][kDense ? 1024 : 2];
+  // the subscription id base, the position then in `at`.
+  uint4 rec[kWarps][32];
+  Cursor at[kWarps][32];
+  uint4 next[kWarps];  // the next list entry
+  // a round's pairs as a list of (record, leaf slot)
+  uint32_t pre[kWarps][32];
+  uint16_t list[kWarps][1024];
+};
+
+// Expands the list entries [i0, i1).  SHORT: entries of few records, where
+// the time goes into waiting for one load after the other: the next entry is
+// copied to shared memory (asynchronously, no register waits for it) and the
+// ticket after it taken before the current one is expanded.  With long
+// entries this would cost 2% (warps holding work at the end of the pass).
+// Their records have few hits each: every lane lists its own record's bits,
+// and the pairs are then written 32 at a time (as the ids form does), where
+// a step per record would leave most lanes idle.
+template <bool FILTER_ID, bool WIDE, bool BATCH, int OUT, bool SHORT>
+__device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, OUT>& sm, const TreeView& t,
+                                               const QueryView& q, const BatchView& bv,
+                                               const RecordArena& ra, const WriteView& w,
+                                               uint32_t i0, uint32_t i1, uint32_t pb, uint32_t pe,
+                                               uint32_t idb, uint32_t ide,
+                                               unsigned long long base0, unsigned long long need,
+                                               uint32_t* __restrict__ work,
+                                               Status* __restrict__ st) {
+  using Cursor = typename ReplaySmem<WIDE, OUT>::Cursor;
+  constexpr bool kDense = SHORT || ReplayShape<OUT>::dense;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const uint32_t below = (1u << lane) - 1u;  // lanes below this one
   const uint32_t lanebit = 1u << lane;
-  if (!records_complete(ra)) return;  // the walking write pass handles this range
-  const unsigned long long base0 = w.start[w.b_idx];
-  const unsigned long long need = w.start[w.e_idx] - base0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    st->K = need;
-    if (need > w.capacity) atomicOr(&st->err, kErrCapacity);
-  }
-  // Pair positions are bounded by construction: a record's pairs go to its
-  // update's offset plus the matches the count pass had found before it, and
-  // the update's count is the sum of its records' popcounts, so all writes
-  // stay below need <= capacity.
-  if (need > w.capacity) return;
-  if (!WIDE && need > 0xffffffffull) return;  // host picks WIDE for such ranges
   ddm_pair* __restrict__ pairs = w.pairs;
   uint32_t* __restrict__ ids = w.ids;
   const uint32_t* __restrict__ sid = t.sid;
   const unsigned long long keep = l2_policy_evict_last(), stream = l2_policy_evict_first();
-  const unsigned long long i0 = ra.pkt_off[(size_t)p0 * kRecChains],
-                           i1 = ra.pkt_off[(size_t)p1 * kRecChains];
+  // A warp's first entry goes by its number, the others by ticket.  A ticket
+  // is taken ahead (lane 0 holds it) only if there are entries for one.
+  const uint32_t warps = gridDim.x * kWarps;
+  const bool tickets = i1 - i0 > warps;
+  uint32_t held = i0 + blockIdx.x * kWarps + wib;
+  auto fetch = [&]() {
+    if (lane == 0) {
+      const uint32_t i = held;
+      if (i < i1)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(&sm.next[wib])),
+                     "l"(ra.blk_list + i)
+                     : "memory");
+      else
+        sm.next[wib].x = kNoBlock;
+      held = tickets ? i0 + warps + atomicAdd(work, 1u) : i1;
+    }
+  };
+  auto take = [&]() {
+    if (lane == 0) held = tickets ? i0 + warps + atomicAdd(work, 1u) : i1;
+    held = __shfl_sync(0xffffffffu, held, 0);
+  };
+  if (SHORT) fetch();
   for (;;) {
-    unsigned long long i = 0;
-    if (lane == 0) i = i0 + atomicAdd(work, 1u);
-    i = __shfl_sync(0xffffffffu, i, 0);
-    if (i >= i1) break;
-    const uint32_t blk = ra.blk_list[i];
-    const uint32_t p = ra.blk_pkt[blk];
+    uint4 entry;
+    if (SHORT) {
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncwarp();
+      entry = sm.next[wib];
+      if (entry.x == kNoBlock) break;
+      __syncwarp();
+      fetch();
+    } else {
+      const uint32_t i = held;
+      if (i >= i1) break;
+      entry = ra.blk_list[i];
+    }
+    // records [0, na) of block blk, then (one entry for two blocks) the rest
+    // from the next block
+    const uint32_t blk = entry.x, p = entry.y, na = entry.z, nrec = entry.z + entry.w;
     const uint32_t pos = (p << q.qpp_log2) + lane;
     bool valid = (uint32_t)lane < (1u << q.qpp_log2) && pos >= pb && pos < pe;
     uint32_t Q = 0;
@@ -794,16 +857,29 @@ k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uin
       sub_base = (uint32_t)bv.sub_off[b];
     }
     const uint32_t vmask = __ballot_sync(0xffffffffu, valid);
-    if (vmask == 0u) continue;
-    const uint32_t nrec = ra.blk_count[blk];
+    if (vmask == 0u) {
+      if (!SHORT) take();
+      continue;
+    }
     const uint32_t* rec = ra.rec + (size_t)blk * kRecWords;
     const uint16_t* rel = reinterpret_cast<const uint16_t*>(rec + 2u * kRecBlock);
     uint32_t nx = 0u, nhb = 0u, nrel = 0u;
-    if (lane < nrec) {
-      nx = ld_hinted(&rec[lane], stream);
-      nhb = ld_hinted(&rec[kRecBlock + lane], stream);
-      nrel = ld_hinted(&rel[lane], stream);
-    }
+    auto load = [&](uint32_t r0) {
+      const uint32_t r = r0 + (uint32_t)lane;
+      if (r < nrec) {
+        if (na != nrec && r >= na) {  // the second of two blocks
+          const uint32_t* r2 = rec + kRecWords;
+          nx = ld_hinted(&r2[r - na], stream);
+          nhb = ld_hinted(&r2[kRecBlock + r - na], stream);
+          nrel = ld_hinted(&reinterpret_cast<const uint16_t*>(r2 + 2u * kRecBlock)[r - na], stream);
+        } else {
+          nx = ld_hinted(&rec[r], stream);
+          nhb = ld_hinted(&rec[kRecBlock + r], stream);
+          nrel = ld_hinted(&rel[r], stream);
+        }
+      }
+    };
+    load(0u);
     // the block header: lane j holds the matches query j of the chain had
     // before the block
     const uint32_t hdr =
@@ -812,11 +888,7 @@ k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uin
       const uint32_t x = nx, xrel = nrel;
       uint32_t hb = nhb;
       nx = nhb = nrel = 0u;  // lanes past the block's last record hold x = hb = 0
-      if (r0 + 32u + lane < nrec) {
-        nx = ld_hinted(&rec[r0 + 32u + lane], stream);
-        nhb = ld_hinted(&rec[kRecBlock + r0 + 32u + lane], stream);
-        nrel = ld_hinted(&rel[r0 + 32u + lane], stream);
-      }
+      load(r0 + 32u);
       const int qq = (int)(x & 31u);
       // the query's matches before this record: header + the record's count
       const uint32_t bef = __shfl_sync(0xffffffffu, hdr, qq & (int)(kRecHdr - 1)) + xrel;
@@ -826,8 +898,8 @@ k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uin
       const uint32_t sb = BATCH ? __shfl_sync(0xffffffffu, sub_base, qq) : 0u;
       __syncwarp();  // the previous round has read s_rec / s_at
       constexpr bool kPacked = !WIDE && !BATCH;  // position fits the record's fourth word
-      s_rec[wib][lane] = make_uint4(x >> 5, hb, Qq, kPacked ? (uint32_t)o : sb);
-      if (!kPacked) s_at[wib][lane] = o;
+      sm.rec[wib][lane] = make_uint4(x >> 5, hb, Qq, kPacked ? (uint32_t)o : sb);
+      if (!kPacked) sm.at[wib][lane] = o;
       if constexpr (kDense) {
         // The round's pairs, numbered record by record: an exclusive scan of
         // the records' hit counts gives each record's first pair; the hit
@@ -842,21 +914,26 @@ k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uin
           if (lane >= dd) incl += v;
         }
         const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-        s_pre[wib][lane] = incl - c;
+        sm.pre[wib][lane] = incl - c;
         __syncwarp();
+        if (SHORT) {
+          uint32_t k = incl - c;
+          for (uint32_t h = hb; h; h &= h - 1u)
+            sm.list[wib][k++] = (uint16_t)(((uint32_t)lane << 5) | (uint32_t)(__ffs(h) - 1));
+        } else
 #pragma unroll 8
         for (int u = 0; u < 32; ++u) {
-          const uint32_t h = s_rec[wib][u].y;
+          const uint32_t h = sm.rec[wib][u].y;
           if (h & lanebit)
-            s_list[wib][s_pre[wib][u] + __popc(h & below)] = (uint16_t)(((uint32_t)u << 5) | (uint32_t)lane);
+            sm.list[wib][sm.pre[wib][u] + __popc(h & below)] = (uint16_t)(((uint32_t)u << 5) | (uint32_t)lane);
         }
         __syncwarp();
 #pragma unroll 2
         for (uint32_t ti = lane; ti < total; ti += 32u) {
-          const uint32_t ent = s_list[wib][ti];
+          const uint32_t ent = sm.list[wib][ti];
           const uint32_t r = ent >> 5, slot = ent & 31u;
-          const uint4 R = s_rec[wib][r];
-          const Cursor at = (kPacked ? (Cursor)R.w : s_at[wib][r]) + (Cursor)(ti - s_pre[wib][r]);
+          const uint4 R = sm.rec[wib][r];
+          const Cursor at = (kPacked ? (Cursor)R.w : sm.at[wib][r]) + (Cursor)(ti - sm.pre[wib][r]);
           if (!DDM_IN_BOUNDS(R.x * 32u + slot < t.n && (unsigned long long)at < need, st)) continue;
           const uint32_t sv = ld_hinted(sid + R.x * 32u + slot, keep);
           const uint32_t sub = sv - (kPacked ? 0u : R.w);
@@ -879,7 +956,7 @@ k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uin
         uint32_t sv[G];
 #pragma unroll
         for (int u = 0; u < G; ++u) {
-          rr[u] = s_rec[wib][g + u];
+          rr[u] = sm.rec[wib][g + u];
           sv[u] = 0u;
           if ((rr[u].y & lanebit) && DDM_IN_BOUNDS(rr[u].x * 32u + (uint32_t)lane < t.n, st))
             sv[u] = ld_hinted(sid + rr[u].x * 32u + (uint32_t)lane, keep);
@@ -887,7 +964,7 @@ k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uin
 #pragma unroll
         for (int u = 0; u < G; ++u) {
           if (rr[u].y & lanebit) {
-            const Cursor at = kPacked ? (Cursor)rr[u].w : s_at[wib][g + u];
+            const Cursor at = kPacked ? (Cursor)rr[u].w : sm.at[wib][g + u];
             const unsigned long long slot = (unsigned long long)(at + (Cursor)__popc(rr[u].y & below));
             if (!DDM_IN_BOUNDS(slot < need, st)) continue;
             const uint32_t sub = sv[u] - (kPacked ? 0u : rr[u].w);
@@ -903,7 +980,38 @@ k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uin
         }
       }
     }
+    if (!SHORT) take();
   }
+}
+
+template <bool FILTER_ID, bool WIDE, bool BATCH, int OUT>
+__global__ void __launch_bounds__(kThreads, ReplayShape<OUT>::ctas)
+k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uint32_t p0,
+         uint32_t p1, uint32_t pb, uint32_t pe, uint32_t idb, uint32_t ide,
+         uint32_t* __restrict__ work, Status* __restrict__ st) {
+  __shared__ ReplaySmem<WIDE, OUT> sm;
+  if (!records_complete(ra)) return;  // the walking write pass handles this range
+  const unsigned long long base0 = w.start[w.b_idx];
+  const unsigned long long need = w.start[w.e_idx] - base0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    st->K = need;
+    if (need > w.capacity) atomicOr(&st->err, kErrCapacity);
+  }
+  // Pair positions are bounded by construction: a record's pairs go to its
+  // update's offset plus the matches the count pass had found before it, and
+  // the update's count is the sum of its records' popcounts, so all writes
+  // stay below need <= capacity.
+  if (need > w.capacity) return;
+  if (!WIDE && need > 0xffffffffull) return;  // host picks WIDE for such ranges
+  // entries of the range; fewer than max_blocks, so 32 bits hold them
+  const uint32_t i0 = (uint32_t)ra.pkt_off[(size_t)p0 * kRecChains],
+                 i1 = (uint32_t)ra.pkt_off[(size_t)p1 * kRecChains];
+  if (need <= (unsigned long long)kShortEntry * (i1 - i0))
+    replay_entries<FILTER_ID, WIDE, BATCH, OUT, true>(sm, t, q, bv, ra, w, i0, i1, pb, pe, idb, ide,
+                                                      base0, need, work, st);
+  else
+    replay_entries<FILTER_ID, WIDE, BATCH, OUT, false>(sm, t, q, bv, ra, w, i0, i1, pb, pe, idb,
+                                                       ide, base0, need, work, st);
 }
 
 template <bool WRITE, bool BATCH>
@@ -929,18 +1037,28 @@ cudaError_t launch_packets(const TreeView& t, const QueryView& q, const BatchVie
                            const RecordArena& ra, const WriteView& w, uint32_t* work, Status* st,
                            int sms, cudaStream_t s) {
   if (q.nq == 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(work, 0, sizeof(uint32_t), s);
-  if (e) return e;
   const bool open = (flags & DDM_OPEN) != 0;
   const uint32_t packets = (q.nq + (1u << q.qpp_log2) - 1u) >> q.qpp_log2;
   uint32_t blocks = (packets + kWarps - 1) / kWarps;
   const uint32_t cap = (uint32_t)sms * 8u;
   if (blocks > cap) blocks = cap;
+  QueryView qv = q;
+  // Four packets per ticket when every warp of the grid gets 32 such tickets
+  // or more: the tickets are atomics on one word.
+  qv.take_log2 = packets / (blocks * kWarps) >= 32u ? 2u : 0u;
+  // With every warp resident at once each takes one packet, without tickets
+  // (and without the counter to clear).
+  if (blocks <= (uint32_t)sms * DDM_PACKET_MIN_BLOCKS && packets <= blocks * kWarps) {
+    work = nullptr;
+  } else {
+    cudaError_t e = cudaMemsetAsync(work, 0, sizeof(uint32_t), s);
+    if (e) return e;
+  }
   if (bv.count)
-    dispatch_packets<WRITE, true>(t.d, open, blocks, s, t, q, bv, counts, counts_pos, ra, w, work,
+    dispatch_packets<WRITE, true>(t.d, open, blocks, s, t, qv, bv, counts, counts_pos, ra, w, work,
                                   st);
   else
-    dispatch_packets<WRITE, false>(t.d, open, blocks, s, t, q, bv, counts, counts_pos, ra, w,
+    dispatch_packets<WRITE, false>(t.d, open, blocks, s, t, qv, bv, counts, counts_pos, ra, w,
                                    work, st);
   note_launches(1);
   return cudaGetLastError();
