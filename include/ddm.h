@@ -403,7 +403,8 @@ int ddm_set_tuning(ddm_ctx *ctx, int str_shift, uint32_t ctas_per_sm, uint32_t r
  * the Python package picks it per workload):
  *  queries_per_packet -- 16 or 32 queries walk the tree together in one warp
  *                        (default 32; the leaves keep 32 subscriptions, one
- *                        per lane);
+ *                        per lane); a plan of few updates takes fewer, so
+ *                        that its packets occupy the GPU;
  *  swap_min           -- 1..33: a leaf met by at least this many of a
  *                        packet's queries is tested with lane = query: for
  *                        d <= 3 from the leaf's rank tables (its bounds

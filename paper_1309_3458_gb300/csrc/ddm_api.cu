@@ -87,6 +87,7 @@ struct ddm_ctx {
   // tiling (ddm_set_tiling): log2 of the queries per packet, and the number of
   // a packet's queries meeting a leaf from which the count pass swaps the loops
   uint32_t qpp_log2 = 5;
+  uint32_t plan_qpp_log2 = 5;   // of the current plan (smaller for few updates)
   uint32_t tmin = 12;
 
   bool built = false;
@@ -428,7 +429,7 @@ int packet_sms(const ddm_ctx* c) {
 
 // Packets of the count pass (and of its records) covering positions [0, m).
 uint32_t packets_of(const ddm_ctx* c, uint32_t m) {
-  return (uint32_t)(((uint64_t)m + (1u << c->qpp_log2) - 1u) >> c->qpp_log2);
+  return (uint32_t)(((uint64_t)m + (1u << c->plan_qpp_log2) - 1u) >> c->plan_qpp_log2);
 }
 
 QueryView query_view(ddm_ctx* c) {
@@ -439,7 +440,7 @@ QueryView query_view(ddm_ctx* c) {
   q.list = nullptr;
   q.first = 0;
   q.nq = c->m;
-  q.qpp_log2 = c->qpp_log2;
+  q.qpp_log2 = c->plan_qpp_log2;
   q.tmin = c->tmin;
   return q;
 }
@@ -450,6 +451,15 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
   Phase phase("ddm plan");
   c->planned = false;
   const int d = c->tree.d;
+  // Few updates: packets of fewer queries (down to four), until there are
+  // sixteen warps' worth per SM (2,432 packets on 152 SMs).  A packet is one
+  // warp's serial walk, and with fewer packets the chip idles: at 33,333
+  // updates (d = 5, 1,042 packets of 32) a match took 5.3 ms, 3.55 with
+  // packets of 8; at 31,627 (d = 2) a served plan and write 152 and 142 us; at
+  // 30,011 374 and 352 us.  From twice as many packets the smaller ones cost
+  // more walks than they save (served 157 us, d = 2 377 us).
+  c->plan_qpp_log2 = c->qpp_log2;
+  while (c->plan_qpp_log2 > 2 && packets_of(c, m) < (uint32_t)c->sms * 16u) --c->plan_qpp_log2;
   DDM_TRY(ensure(c, c->counts, sizeof(uint32_t) * (m ? m : 1)));
   DDM_TRY(ensure(c, c->counts_pos, sizeof(uint32_t) * (m ? m : 1)));
   DDM_TRY(ensure(c, c->offsets, sizeof(unsigned long long) * ((size_t)m + 1)));
@@ -618,7 +628,7 @@ int write_ordered_async(ddm_ctx* c, uint32_t pb, uint32_t pe, ddm_pair* pairs, u
     w.capacity = capacity;
     auto* work = static_cast<uint32_t*>(c->work.p);
     if (c->arena.max_blocks)
-      DDM_CUDA(launch_replay(c->tree, q, c->bv, c->arena, w, pb >> c->qpp_log2, packets_of(c, pe), pb, pe, false, 0, 0,
+      DDM_CUDA(launch_replay(c->tree, q, c->bv, c->arena, w, pb >> c->plan_qpp_log2, packets_of(c, pe), pb, pe, false, 0, 0,
                              work, c->st_dev, c->sms, s));
     DDM_CUDA(launch_write(c->tree, q, c->bv, c->flags, w, c->arena, work, c->st_dev, packet_sms(c), s));
   } else {

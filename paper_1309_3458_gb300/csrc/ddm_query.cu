@@ -210,7 +210,7 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
     if (need > w.capacity) return;
   }
 
-  const uint32_t qpp = 1u << q.qpp_log2;  // queries per packet: 16 or 32
+  const uint32_t qpp = 1u << q.qpp_log2;  // queries per packet: 4 to 32
   const uint32_t npk = (q.nq + qpp - 1u) >> q.qpp_log2;
   // Summed over the warp's packets and added once at the end (or before the
   // 32 bits could run out): atomics on one word by every packet would
