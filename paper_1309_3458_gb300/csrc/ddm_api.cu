@@ -63,8 +63,8 @@ struct ddm_ctx {
   // range selection for ddm_write over a sub-range of updates
   DevBuf sel_offs, sel_list;
   // replay records of the count pass
-  DevBuf rec, blk_next, blk_count, pkt_nblk, pkt_off, blk_list,
-      blk_counter;
+  DevBuf rec, blk_own, blk_count, pkt_nblk, pkt_off, blk_list,
+      plan_state, order_state;
   uint64_t replay_budget = 0;   // bytes; 0 = never record
   uint32_t rec_blocks = 0;      // blocks of the current arena
   // Blocks needed, packets and blocks held by the latest recorded count
@@ -87,6 +87,7 @@ struct ddm_ctx {
   // tiling (ddm_set_tiling): log2 of the queries per packet, and the number of
   // a packet's queries meeting a leaf from which the count pass swaps the loops
   uint32_t qpp_log2 = 5;
+  bool ordered = false;         // the plan holds the plan order's offsets and entries
   uint32_t plan_qpp_log2 = 5;   // of the current plan (smaller for few updates)
   uint32_t tmin = 12;
 
@@ -446,8 +447,11 @@ QueryView query_view(ddm_ctx* c) {
 }
 
 // Validate U, sort it, count per update, scan (no host synchronisation).
+// `ordered`: the plan order's offsets too (the staged calls); the one-shot
+// calls do not write by plan order, and a staged call after one of them has
+// ready_ordered() compute them.
 int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint32_t flags,
-               bool record, cudaStream_t s, const BatchSet* bs = nullptr) {
+               bool record, bool ordered, cudaStream_t s, const BatchSet* bs = nullptr) {
   Phase phase("ddm plan");
   c->planned = false;
   const int d = c->tree.d;
@@ -464,10 +468,8 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
   DDM_TRY(ensure(c, c->counts_pos, sizeof(uint32_t) * (m ? m : 1)));
   DDM_TRY(ensure(c, c->offsets, sizeof(unsigned long long) * ((size_t)m + 1)));
   DDM_TRY(ensure(c, c->pos_offsets, sizeof(unsigned long long) * ((size_t)m + 1)));
-  // tile sums of the three scans below, one region each
-  const size_t upd_tiles = (size_t)m / kScanTile + 1;
-  const size_t blk_tiles = (size_t)packets_of(c, m) * kRecChains / kScanTile + 1;
-  DDM_TRY(ensure(c, c->sums, sizeof(unsigned long long) * (2 * upd_tiles + blk_tiles + 1)));
+  // tile sums of a range selection (write_async)
+  DDM_TRY(ensure(c, c->sums, sizeof(unsigned long long) * ((size_t)m / kScanTile + 2)));
   DDM_TRY(ensure(c, c->work, sizeof(uint32_t)));
   DDM_TRY(ensure(c, c->qe, sizeof(float2) * (size_t)d * (m ? m : 1)));
   DDM_TRY(ensure(c, c->qid, sizeof(uint32_t) * (m ? m : 1)));
@@ -479,13 +481,13 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
   c->arena = RecordArena{};
   if (record && c->replay_on && m > 0 && c->tree.n > 0 && c->replay_budget > 0) {
     const uint32_t packets = packets_of(c, m);
-    // bytes per block: records (ten bytes each) and header, next/count/list entries
-    const uint64_t per_block =
-        (uint64_t)kRecWords * sizeof(uint32_t) + 2 * sizeof(uint32_t) + sizeof(uint4);
+    // bytes per block: records (ten bytes each) and header, count/owner/list entries
+    const uint64_t per_block = (uint64_t)kRecWords * sizeof(uint32_t) + sizeof(uint32_t) +
+                               sizeof(uint2) + sizeof(uint4);
     // Blocks the arena holds now, and what the latest recorded pass needed.
     uint64_t have = c->rec.cap / ((size_t)kRecWords * sizeof(uint32_t));
-    for (const DevBuf* b : {&c->blk_next, &c->blk_count})
-      have = std::min<uint64_t>(have, b->cap / sizeof(uint32_t));
+    have = std::min<uint64_t>(have, c->blk_count.cap / sizeof(uint32_t));
+    have = std::min<uint64_t>(have, c->blk_own.cap / sizeof(uint2));
     have = std::min<uint64_t>(have, c->blk_list.cap / sizeof(uint4));
     const uint32_t hint_blocks = c->rec_hint[0], hint_packets = c->rec_hint[1],
                    hint_max = c->rec_hint[2];
@@ -507,25 +509,39 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
     if (want > cap_blocks) want = cap_blocks;
     if (want > 0xfffffff0ull) want = 0xfffffff0ull;
     if (want > 0 && ensure(c, c->rec, (size_t)want * kRecWords * sizeof(uint32_t)) == DDM_OK &&
-        ensure(c, c->blk_next, (size_t)want * sizeof(uint32_t)) == DDM_OK &&
+        ensure(c, c->blk_own, (size_t)want * sizeof(uint2)) == DDM_OK &&
         ensure(c, c->blk_count, (size_t)want * sizeof(uint32_t)) == DDM_OK &&
         ensure(c, c->blk_list, (size_t)want * sizeof(uint4)) == DDM_OK &&
-        ensure(c, c->pkt_nblk, (size_t)packets * kRecChains * sizeof(uint32_t)) == DDM_OK &&
-        ensure(c, c->pkt_off, ((size_t)packets * kRecChains + 1) * sizeof(unsigned long long)) ==
-            DDM_OK &&
-        ensure(c, c->blk_counter, 4 * sizeof(uint32_t)) == DDM_OK) {
+        ensure(c, c->pkt_nblk, (size_t)packets * sizeof(uint32_t)) == DDM_OK &&
+        ensure(c, c->pkt_off, ((size_t)packets + 1) * sizeof(unsigned long long)) == DDM_OK) {
       c->arena.rec = static_cast<uint32_t*>(c->rec.p);
-      c->arena.blk_next = static_cast<uint32_t*>(c->blk_next.p);
+      c->arena.blk_own = static_cast<uint2*>(c->blk_own.p);
       c->arena.blk_count = static_cast<uint32_t*>(c->blk_count.p);
       c->arena.blk_list = static_cast<uint4*>(c->blk_list.p);
       c->arena.pkt_nblk = static_cast<uint32_t*>(c->pkt_nblk.p);
       c->arena.pkt_off = static_cast<unsigned long long*>(c->pkt_off.p);
-      c->arena.blk_counter = static_cast<uint32_t*>(c->blk_counter.p);
       c->arena.chains = packets * kRecChains;
       c->arena.max_blocks = (uint32_t)want;
-      DDM_CUDA(cudaMemsetAsync(c->blk_counter.p, 0, 4 * sizeof(uint32_t), s));
     }
   }
+  // Offsets by update id and, for a plan whose order will be written or read
+  // out, by plan position and of the record entries in plan order.  The block
+  // counter (two words) and the scans' state are cleared by one memset.
+  const uint32_t packets = packets_of(c, m);
+  const ScanJob jobs[kMaxScanJobs] = {
+      {counts, m, offsets, true},
+      {counts_pos, m, pos_offsets, false},
+      {c->arena.pkt_nblk, packets, c->arena.pkt_off, false}};
+  const int njobs = !ordered ? 1 : c->arena.max_blocks ? 3 : 2;
+  const size_t state_words = 1 + scan_state_words(jobs, njobs);
+  DDM_TRY(ensure(c, c->plan_state, sizeof(unsigned long long) * state_words));
+  if (!ordered)  // what ready_ordered() needs, so that it never allocates
+    DDM_TRY(ensure(c, c->order_state,
+                   sizeof(unsigned long long) *
+                       scan_state_words(jobs + 1, c->arena.max_blocks ? 2 : 1)));
+  auto* state = static_cast<unsigned long long*>(c->plan_state.p);
+  DDM_CUDA(cudaMemsetAsync(state, 0, sizeof(unsigned long long) * state_words, s));
+  if (c->arena.max_blocks) c->arena.blk_counter = reinterpret_cast<uint32_t*>(state);
   if (m > 0) {
     int cur = 0;
     float2* aos = aos_buffer(c, d, m);
@@ -544,24 +560,35 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
       DDM_CUDA(cudaMemsetAsync(counts_pos, 0, sizeof(uint32_t) * m, s));
     }
   }
-  // offsets by plan position and by update id, and the record blocks' plan
-  // order, in one launch sequence
-  auto* sums = static_cast<unsigned long long*>(c->sums.p);
-  ScanJob jobs[kMaxScanJobs] = {{counts_pos, m, pos_offsets, sums, nullptr},
-                                {counts, m, offsets, sums + upd_tiles, c->st_dev}};
-  int njobs = 2;
-  if (c->arena.max_blocks)
-    jobs[njobs++] = ScanJob{c->arena.pkt_nblk, packets_of(c, m) * kRecChains, c->arena.pkt_off,
-                            sums + 2 * upd_tiles, nullptr};
-  DDM_CUDA(launch_scan_multi(jobs, njobs, s));
-  if (c->arena.max_blocks) DDM_CUDA(launch_block_list(c->arena, packets_of(c, m), s));
-  if (c->arena.max_blocks)  // blocks needed, packets, blocks held: the next arena's sizing hint
-    DDM_CUDA(cudaMemcpyAsync((void*)c->rec_hint, static_cast<uint32_t*>(c->blk_counter.p) + 1,
-                             3 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+  const ScanHint hint{c->arena.max_blocks ? c->rec_hint : nullptr, c->arena.blk_counter,
+                      c->arena.chains, packets, c->arena.max_blocks};
+  DDM_CUDA(launch_scan_multi(jobs, njobs, state + 1, hint, c->st_dev, s));
+  if (ordered && c->arena.max_blocks) DDM_CUDA(launch_block_list(c->arena, c->sms, s));
+  c->ordered = ordered;
   c->ulo = ulo;
   c->uhi = uhi;
   c->flags = flags;
   c->planned = true;
+  return DDM_OK;
+}
+
+// The plan order's offsets and record entries, for a staged call after a
+// one-shot call's plan (a plan made for staged calls has them).
+int ready_ordered(ddm_ctx* c, cudaStream_t s) {
+  if (c->ordered) return DDM_OK;
+  const uint32_t packets = packets_of(c, c->m);
+  const ScanJob jobs[2] = {
+      {static_cast<uint32_t*>(c->counts_pos.p), c->m,
+       static_cast<unsigned long long*>(c->pos_offsets.p), false},
+      {c->arena.pkt_nblk, packets, c->arena.pkt_off, false}};
+  const int njobs = c->arena.max_blocks ? 2 : 1;
+  const size_t words = scan_state_words(jobs, njobs);
+  DDM_TRY(ensure(c, c->order_state, sizeof(unsigned long long) * words));  // done by the plan
+  auto* state = static_cast<unsigned long long*>(c->order_state.p);
+  DDM_CUDA(cudaMemsetAsync(state, 0, sizeof(unsigned long long) * words, s));
+  DDM_CUDA(launch_scan_multi(jobs, njobs, state, ScanHint{}, c->st_dev, s));
+  if (c->arena.max_blocks) DDM_CUDA(launch_block_list(c->arena, c->sms, s));
+  c->ordered = !c->capturing;  // recorded only: it runs with the graph
   return DDM_OK;
 }
 
@@ -598,7 +625,9 @@ int write_async(ddm_ctx* c, uint32_t begin, uint32_t end, ddm_pair* pairs, uint6
     auto* work = static_cast<uint32_t*>(c->work.p);
     if (c->arena.max_blocks) {
       const bool full = begin == 0 && end == c->m;
-      DDM_CUDA(launch_replay(c->tree, query_view(c), c->bv, c->arena, w, 0, packets_of(c, c->m), 0, c->m,
+      RecordArena ra = c->arena;
+      ra.blk_list = nullptr;
+      DDM_CUDA(launch_replay(c->tree, query_view(c), c->bv, ra, w, 0, packets_of(c, c->m), 0, c->m,
                              !full, begin, end, work, c->st_dev, c->sms, s));
     }
     DDM_CUDA(launch_write(c->tree, q, c->bv, c->flags, w, c->arena, work, c->st_dev, packet_sms(c), s));
@@ -613,6 +642,7 @@ int write_ordered_async(ddm_ctx* c, uint32_t pb, uint32_t pe, ddm_pair* pairs, u
                         cudaStream_t s, uint32_t* ids = nullptr) {
   Phase phase("ddm write ordered");
   if (!ids && !base_fits(c)) return DDM_ERR_ARG;
+  DDM_TRY(ready_ordered(c, s));
   if (pe > pb && c->tree.n > 0) {
     QueryView q = query_view(c);
     q.first = pb;
@@ -708,9 +738,9 @@ int ddm_destroy(ddm_ctx* c) {
   for (DevBuf* b : {&c->keys[0], &c->keys[1], &c->vals[0], &c->vals[1], &c->hist, &c->lookback,
                     &c->counters, &c->e, &c->sid, &c->nodes, &c->tab, &c->qe, &c->qid, &c->counts,
                     &c->counts_pos, &c->offsets, &c->pos_offsets, &c->sums, &c->work,
-                    &c->sel_offs, &c->sel_list, &c->rec, &c->blk_next, &c->blk_count,
+                    &c->sel_offs, &c->sel_list, &c->rec, &c->blk_own, &c->blk_count,
                     &c->pkt_nblk, &c->pkt_off,
-                    &c->blk_list, &c->blk_counter, &c->inst_s, &c->inst_u, &c->bglog2,
+                    &c->blk_list, &c->plan_state, &c->order_state, &c->inst_s, &c->inst_u, &c->bglog2,
                     &c->bngroups, &c->bgbase, &c->cls_hist, &c->cls_off, &c->probe, &c->aos})
     release(*b);
   cudaDeviceSynchronize();  // the stream-ordered frees above have run
@@ -801,7 +831,7 @@ int ddm_plan(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint32_
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   StreamUse use(c, s);
   DDM_TRY(reset_status(c, s));
-  DDM_TRY(plan_async(c, ulo, uhi, m, flags, true, s));
+  DDM_TRY(plan_async(c, ulo, uhi, m, flags, true, true, s));
   if (offsets)
     DDM_CUDA(cudaMemcpyAsync(offsets, c->offsets.p, sizeof(unsigned long long) * ((size_t)m + 1),
                              cudaMemcpyDeviceToDevice, s));
@@ -855,7 +885,7 @@ int ddm_plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, u
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   StreamUse use(c, s);
   DDM_TRY(reset_status(c, s));
-  DDM_TRY(plan_async(c, ulo, uhi, m, flags, true, s));
+  DDM_TRY(plan_async(c, ulo, uhi, m, flags, true, true, s));
   return DDM_OK;
 }
 
@@ -896,7 +926,7 @@ int ddm_match_moved(ddm_ctx* c, const float* lo, const float* hi, uint32_t k, co
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   StreamUse use(c, s);
   DDM_TRY(reset_status(c, s));
-  DDM_TRY(plan_async(c, lo, hi, k, flags & DDM_OPEN, true, s));
+  DDM_TRY(plan_async(c, lo, hi, k, flags & DDM_OPEN, true, false, s));
   const bool was = c->swapped;
   c->swapped = (flags & DDM_SWAP_ROLES) != 0;
   const int wrc = write_async(c, 0, k, pairs, capacity, s, ids);
@@ -965,6 +995,7 @@ int ddm_chunk_end_ordered(ddm_ctx* c, uint32_t pos_begin, uint64_t capacity, uin
   if (!g.ok()) return DDM_ERR_CUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   StreamUse use(c, s);
+  DDM_TRY(ready_ordered(c, s));
   DDM_CUDA(launch_chunk_end(static_cast<const unsigned long long*>(c->pos_offsets.p), c->m,
                             pos_begin, capacity, c->st_dev, s));
   DDM_TRY(sync_status(c, s));
@@ -982,6 +1013,7 @@ int ddm_plan_order(ddm_ctx* c, uint32_t* order, uint64_t* order_offsets, void* s
   StreamUse use(c, s);
   if (order && c->m)
     DDM_CUDA(cudaMemcpyAsync(order, c->qid.p, sizeof(uint32_t) * c->m, cudaMemcpyDeviceToDevice, s));
+  if (order_offsets) DDM_TRY(ready_ordered(c, s));
   if (order_offsets)
     DDM_CUDA(cudaMemcpyAsync(order_offsets, c->pos_offsets.p,
                              sizeof(unsigned long long) * ((size_t)c->m + 1),
@@ -1013,7 +1045,7 @@ static int match_impl(ddm_ctx* c, int d, const float* ulo, const float* uhi, uin
   DDM_TRY(reset_status(c, s));
   DDM_TRY(build_async(c, d, slo, shi, n, s));
   c->swapped = swap;
-  DDM_TRY(plan_async(c, ulo, uhi, m, flags & DDM_OPEN, write, s));
+  DDM_TRY(plan_async(c, ulo, uhi, m, flags & DDM_OPEN, write, false, s));
   if (write) DDM_TRY(write_async(c, begin, end, pairs, capacity, s));
   DDM_TRY(sync_status(c, s));
   c->last_tests = c->st_host->tests;
@@ -1068,7 +1100,7 @@ static int batch_impl(ddm_ctx* c, int d, uint32_t count, const float* ulo, const
   c->bv.upd_off = uoff;
   c->bv.sub_off = soff;
   c->bv.q_inst = static_cast<const uint32_t*>(c->inst_u.p);
-  DDM_TRY(plan_async(c, ulo, uhi, m, flags, true, s, &bs_u));
+  DDM_TRY(plan_async(c, ulo, uhi, m, flags, true, false, s, &bs_u));
   DDM_TRY(write_async(c, 0, m, pairs, capacity, s));
   if (pair_off && m > 0)
     DDM_CUDA(launch_gather_offsets(static_cast<const unsigned long long*>(c->offsets.p), m, uoff,

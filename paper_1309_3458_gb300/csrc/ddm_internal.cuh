@@ -231,10 +231,12 @@ cudaError_t launch_export_nodes(const TreeView& t, float* node_lo, float* node_h
 //
 // The first block of each chain belongs to it from the start (its header is
 // zero); only the blocks after it are taken from a counter, so that the
-// packets of a sparse problem make no atomic.  When neither chain of a packet
-// needs a second block and their records fit one, the two blocks are one
-// entry of the list, and the write pass takes them as one.  With every block
-// from the counter and an entry each, the count pass of 2.5e7 + 2.5e7 extents
+// packets of a sparse problem make no atomic.  The two first blocks of a
+// packet are one entry of the write pass, every block after them another.
+// A write laid out by update id takes the entries as they are (packets first,
+// then the blocks handed out); only writes of ranges of the plan order need
+// them listed in that order.  With every block
+// from the counter and listed, the count pass of 2.5e7 + 2.5e7 extents
 // (d = 1, alpha = 1) took 2.81 ms and the write pass 2.58 ms; now 1.73 and
 // 1.47 ms.
 constexpr uint32_t kRecBlock = 512;  // records per block: x and hit mask 2 KiB each, counts 1 KiB
@@ -251,17 +253,18 @@ constexpr uint32_t kRecChains = 2;
 constexpr uint32_t kNoBlock = 0xffffffffu;
 struct RecordArena {
   uint32_t* rec;           // [max_blocks][kRecWords]: x, hit mask, 16-bit counts, header
-  uint32_t* blk_next;      // [max_blocks] next block of the chain, or kNoBlock
+  uint2* blk_own;          // [max_blocks] packet of a block handed out, and its
+                           // number among that packet's blocks handed out
   uint32_t* blk_count;     // [max_blocks] records in the block
-  uint32_t* pkt_nblk;      // [chains] list entries of each chain
-  unsigned long long* pkt_off;  // [chains + 1] exclusive prefix of pkt_nblk
-  uint4* blk_list;         // [max_blocks] blocks in plan order (packet, then
-                           // chain): block, packet, its records, and those of
-                           // the next block when the two are one entry
+  uint32_t* pkt_nblk;      // [packets] entries of each packet
+  unsigned long long* pkt_off;  // [packets + 1] exclusive prefix of pkt_nblk
+  uint4* blk_list;         // [max_blocks] entries in plan order: block, packet,
+                           // its records, and those of the next block when the
+                           // entry is a packet's two first blocks; null: not
+                           // listed
   uint32_t* blk_counter;   // [0] blocks handed out beyond the chains' first (may
                            // exceed the arena), [1] such blocks the whole pass
-                           // needed, then (k_block_list) all blocks it needed,
-                           // [2] packets, [3] max_blocks (for arena sizing)
+                           // needed
   uint32_t chains;         // chains of the plan's packets
   uint32_t max_blocks;     // 0: no recording
 };
@@ -286,13 +289,12 @@ cudaError_t launch_count(const TreeView& t, const QueryView& q, const BatchView&
 cudaError_t launch_write(const TreeView& t, const QueryView& q, const BatchView& bv,
                          uint32_t flags, const WriteView& w, const RecordArena& ra,
                          uint32_t* work, Status* st, int sms, cudaStream_t s);
-// After the count pass: blk_list = every chain's blocks, chains in order
-// (packets in plan order, a packet's two chains in lane order); pkt_off must
-// already hold the prefix of pkt_nblk.
-cudaError_t launch_block_list(const RecordArena& ra, uint32_t packets, cudaStream_t s);
-// Write pass from records: packets [p0, p1) of the plan, positions [pb, pe),
-// and (when id_filter) only updates with ids in [idb, ide).  Does nothing
-// unless `ra` holds complete records.
+// After the count pass: blk_list = every packet's entries, packets in plan
+// order; pkt_off must already hold the prefix of pkt_nblk.
+cudaError_t launch_block_list(const RecordArena& ra, int sms, cudaStream_t s);
+// Write pass from records: positions [pb, pe) of the plan, in packets [p0,
+// p1) (without a list: all packets), and (when id_filter) only updates with
+// ids in [idb, ide).  Does nothing unless `ra` holds complete records.
 cudaError_t launch_replay(const TreeView& t, const QueryView& q, const BatchView& bv,
                           const RecordArena& ra, const WriteView& w, uint32_t p0, uint32_t p1,
                           uint32_t pb, uint32_t pe, bool id_filter, uint32_t idb, uint32_t ide,
@@ -307,18 +309,26 @@ constexpr int kScanTile = 4096;
 // offsets[0..m] = exclusive prefix of counts; offsets[m] and st->K = total.
 cudaError_t launch_scan(const uint32_t* counts, uint32_t m, unsigned long long* offsets,
                         unsigned long long* block_sums, Status* st, cudaStream_t s);
-// Up to kMaxScanJobs independent scans of the form above in one launch
-// sequence (three launches, or one when every job has m <= kScanTile).
-// Each job's `sums` needs max(1, ceil(m / kScanTile)) entries of its own.
+// Up to kMaxScanJobs independent scans of the form above in one launch.
+// `state` holds scan_state_words() words, zeroed by the caller on the stream.
+// `hint` (optional) receives the sizing hint of the plan's record arena.
 struct ScanJob {
   const uint32_t* counts;
   uint32_t m;
   unsigned long long* offsets;
-  unsigned long long* sums;
-  Status* st;
+  bool total_to_k;  // the total goes to st->K too
 };
 constexpr int kMaxScanJobs = 3;
-cudaError_t launch_scan_multi(const ScanJob* jobs, int count, cudaStream_t s);
+// What the last recorded count pass needed, written to host memory: blocks in
+// all, packets, blocks held.
+struct ScanHint {
+  volatile uint32_t* to;  // pinned host memory, or null
+  const uint32_t* blk_counter;
+  uint32_t chains, packets, max_blocks;
+};
+size_t scan_state_words(const ScanJob* jobs, int count);
+cudaError_t launch_scan_multi(const ScanJob* jobs, int count, unsigned long long* state,
+                              const ScanHint& hint, Status* st, cudaStream_t s);
 cudaError_t launch_chunk_end(const unsigned long long* offsets, uint32_t m, uint32_t begin,
                              unsigned long long capacity, Status* st, cudaStream_t s);
 // list = sorted positions i (ascending) with begin <= qid[i] < end; uses

@@ -50,11 +50,6 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-// The first blocks of a packet's two chains are one list entry: neither chain
-// goes on (`more` blocks after them) and their records fit one block.
-__device__ __forceinline__ bool one_entry(uint32_t more, uint32_t n0, uint32_t n1) {
-  return more == 0u && n0 + n1 <= kRecBlock;
-}
 // Without rank tables (d > 3, or no room for them) the swapped leaf test
 // compares the leaf's 32 subscriptions one by one, which pays only from about
 // this many queries on a leaf.
@@ -278,7 +273,7 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
     const bool recording = !WRITE && ra.max_blocks > 0;
     bool rec_write = recording && ra.chains <= ra.max_blocks;
     uint32_t cur0 = p * 2u, cur1 = p * 2u + 1u, fill0 = 0, fill1 = 0;
-    uint32_t nblk0 = 0, nblk1 = 0;  // blocks after each chain's first
+    uint32_t nblk = 0;  // blocks after the chains' first
     uint32_t blk_cnt = 0;  // this query's matches before its chain's current block
     // Test the 32 level-1 nodes (leaves) from g1 on against the packet box,
     // then run the packet's queries over each surviving leaf.
@@ -520,7 +515,6 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
               uint32_t& fl = ch ? fill1 : fill0;
               uint32_t& cb = ch ? cur1 : cur0;
               if (kc == 0u || fl + kc <= kRecBlock) continue;  // the leaf's records start a new block
-              if (ch) ++nblk1; else ++nblk0;
               if (rec_write) {
                 uint32_t b = 0;
                 if (lane == 0) b = atomicAdd(&ra.blk_counter[0], 1u);
@@ -530,7 +524,7 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
                 } else {
                   b += ra.chains;
                   if (lane == 0) {
-                    ra.blk_next[cb] = b;
+                    ra.blk_own[b] = make_uint2(p, nblk);
                     ra.blk_count[cb] = fl;
                   }
                   // header: the chain's queries' matches before this leaf
@@ -542,6 +536,7 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
                 }
               }
               fl = 0;
+              ++nblk;
             }
           }
           if (rec_write && my_hb != 0u) {
@@ -631,52 +626,34 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
       ntests = 0;
     }
     if (recording) {
-      if (lane == 0 && nblk0 + nblk1) atomicAdd(&ra.blk_counter[1], nblk0 + nblk1);
+      if (lane == 0 && nblk) atomicAdd(&ra.blk_counter[1], nblk);
       if (rec_write) {
         // the first blocks' headers: no query had matches before them
         const uint32_t ch = (uint32_t)lane >> 4;
         ra.rec[((size_t)p * 2u + ch) * kRecWords + 2u * kRecBlock + kRecBlock / 2u + (lane & 15)] = 0u;
-        const bool one = one_entry(nblk0 + nblk1, fill0, fill1);
-        if (lane < 2) {
-          const uint32_t cb = lane ? cur1 : cur0, fl = lane ? fill1 : fill0;
-          ra.blk_next[cb] = kNoBlock;
-          ra.blk_count[cb] = fl;
-          uint32_t entries = lane ? (one ? 0u : nblk1 + (fill1 ? 1u : 0u))
-                                  : (one ? (fill0 + fill1 ? 1u : 0u) : nblk0 + (fill0 ? 1u : 0u));
-          ra.pkt_nblk[(size_t)p * 2u + lane] = entries;
-        }
-      } else if (lane < 2) {
-        ra.pkt_nblk[(size_t)p * 2u + lane] = 0u;
+        if (lane < 2) ra.blk_count[lane ? cur1 : cur0] = lane ? fill1 : fill0;
       }
+      if (lane == 0) ra.pkt_nblk[p] = rec_write ? 1u + nblk : 0u;
     }
   }
   if (!WRITE && st && lane == 0 && ntests) atomicAdd(&st->tests, (unsigned long long)ntests);
 }
 
-// Plan-order list of record blocks: one thread per packet lists its chains
-// (in lane order, packets in plan order).
-__global__ void k_block_list(RecordArena ra, uint32_t packets) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {  // sizing hint for the next arena
-    ra.blk_counter[1] += ra.chains;
-    ra.blk_counter[2] = packets;
-    ra.blk_counter[3] = ra.max_blocks;
-  }
+// Plan-order list of the record entries, a thread per entry: packet p's two
+// first blocks at pkt_off[p], the blocks handed out to it behind them.
+__global__ void k_block_list(RecordArena ra) {
   if (!records_complete(ra)) return;
-  for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < packets;
-       p += gridDim.x * blockDim.x) {
-    unsigned long long at = ra.pkt_off[(size_t)p * kRecChains];
-    const uint32_t b0 = p * kRecChains, n0 = ra.blk_count[b0], n1 = ra.blk_count[b0 + 1];
-    const uint32_t x0 = ra.blk_next[b0], x1 = ra.blk_next[b0 + 1];
-    if (one_entry((x0 != kNoBlock) + (x1 != kNoBlock), n0, n1)) {
-      if (n0 + n1) ra.blk_list[at] = make_uint4(b0, p, n0, n1);
-      continue;
+  const uint32_t packets = ra.chains / kRecChains, more = ra.blk_counter[0];
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < packets + more;
+       i += gridDim.x * blockDim.x) {
+    if (i < packets) {
+      const uint32_t b = i * kRecChains;
+      ra.blk_list[ra.pkt_off[i]] = make_uint4(b, i, ra.blk_count[b], ra.blk_count[b + 1]);
+    } else {
+      const uint32_t b = ra.chains + (i - packets);
+      const uint2 own = ra.blk_own[b];
+      ra.blk_list[ra.pkt_off[own.x] + 1u + own.y] = make_uint4(b, own.x, ra.blk_count[b], 0u);
     }
-    if (n0) ra.blk_list[at++] = make_uint4(b0, p, n0, 0u);
-    for (uint32_t b = x0; b != kNoBlock; b = ra.blk_next[b])
-      ra.blk_list[at++] = make_uint4(b, p, ra.blk_count[b], 0u);
-    if (n1) ra.blk_list[at++] = make_uint4(b0 + 1u, p, n1, 0u);
-    for (uint32_t b = x1; b != kNoBlock; b = ra.blk_next[b])
-      ra.blk_list[at++] = make_uint4(b, p, ra.blk_count[b], 0u);
   }
 }
 
@@ -714,9 +691,9 @@ __device__ __forceinline__ void st_hinted(uint32_t* a, uint32_t v, unsigned long
   asm volatile("st.global.L2::cache_hint.u32 [%0], %1, %2;" ::"l"(a), "r"(v), "l"(policy) : "memory");
 }
 
-// Write pass from the records of the count pass.  Work unit: one record
-// block (up to 512 records of one packet), taken from the plan-order block
-// list, so uneven packets spread over the whole GPU.  A warp loads the
+// Write pass from the records of the count pass.  Work unit: one entry (a
+// packet's two first record blocks, or a block of up to 512 records handed
+// out to it), so uneven packets spread over the whole GPU.  A warp loads the
 // block's packet queries (their output offsets) and takes the records 32 at
 // a time (the next 32 are loaded while these expand), one per lane: each lane
 // works out where its record's pairs go (its query's offset, plus the block
@@ -761,6 +738,16 @@ struct ReplayShape {
   // a round of 32 records is expanded in whole groups
   static_assert(32 % group == 0, "records in flight must divide a round of 32");
 };
+// Asynchronous copy of N bytes to shared memory (waited for by
+// cp.async.wait_all).
+template <int N>
+__device__ __forceinline__ void cp_async(void* to, const void* from) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(to)),
+               "l"(from), "n"(N)
+               : "memory");
+}
+
 // Shared memory of the replay kernel.
 template <bool WIDE, int OUT>
 struct ReplaySmem {
@@ -804,19 +791,29 @@ __device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, OUT>& sm, const 
   const unsigned long long keep = l2_policy_evict_last(), stream = l2_policy_evict_first();
   // A warp's first entry goes by its number, the others by ticket.  A ticket
   // is taken ahead (lane 0 holds it) only if there are entries for one.
+  const uint32_t packets = ra.chains / kRecChains;
   const uint32_t warps = gridDim.x * kWarps;
   const bool tickets = i1 - i0 > warps;
   uint32_t held = i0 + blockIdx.x * kWarps + wib;
   auto fetch = [&]() {
     if (lane == 0) {
       const uint32_t i = held;
-      if (i < i1)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                         (uint32_t)__cvta_generic_to_shared(&sm.next[wib])),
-                     "l"(ra.blk_list + i)
-                     : "memory");
-      else
-        sm.next[wib].x = kNoBlock;
+      uint4* nx = &sm.next[wib];
+      if (i >= i1) {
+        nx->x = kNoBlock;
+      } else if (ra.blk_list) {
+        cp_async<16>(nx, ra.blk_list + i);
+      } else if (i < packets) {
+        nx->x = i * kRecChains;
+        nx->y = i;
+        cp_async<8>(&nx->z, ra.blk_count + i * kRecChains);
+      } else {
+        const uint32_t b = ra.chains + (i - packets);
+        nx->x = b;
+        cp_async<4>(&nx->y, &ra.blk_own[b].x);
+        cp_async<4>(&nx->z, ra.blk_count + b);
+        nx->w = 0u;
+      }
       held = tickets ? i0 + warps + atomicAdd(work, 1u) : i1;
     }
   };
@@ -837,11 +834,23 @@ __device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, OUT>& sm, const 
     } else {
       const uint32_t i = held;
       if (i >= i1) break;
-      entry = ra.blk_list[i];
+      if (ra.blk_list) {
+        entry = ra.blk_list[i];
+      } else if (i < packets) {
+        const uint32_t b = i * kRecChains;
+        entry = make_uint4(b, i, ra.blk_count[b], ra.blk_count[b + 1u]);
+      } else {
+        const uint32_t b = ra.chains + (i - packets);
+        entry = make_uint4(b, ra.blk_own[b].x, ra.blk_count[b], 0u);
+      }
     }
     // records [0, na) of block blk, then (one entry for two blocks) the rest
     // from the next block
     const uint32_t blk = entry.x, p = entry.y, na = entry.z, nrec = entry.z + entry.w;
+    if (nrec == 0u) {
+      if (!SHORT) take();
+      continue;
+    }
     const uint32_t pos = (p << q.qpp_log2) + lane;
     bool valid = (uint32_t)lane < (1u << q.qpp_log2) && pos >= pb && pos < pe;
     uint32_t Q = 0;
@@ -1004,8 +1013,9 @@ k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uin
   if (need > w.capacity) return;
   if (!WIDE && need > 0xffffffffull) return;  // host picks WIDE for such ranges
   // entries of the range; fewer than max_blocks, so 32 bits hold them
-  const uint32_t i0 = (uint32_t)ra.pkt_off[(size_t)p0 * kRecChains],
-                 i1 = (uint32_t)ra.pkt_off[(size_t)p1 * kRecChains];
+  const uint32_t i0 = ra.blk_list ? (uint32_t)ra.pkt_off[p0] : 0u;
+  const uint32_t i1 = ra.blk_list ? (uint32_t)ra.pkt_off[p1]
+                                  : ra.chains / kRecChains + ra.blk_counter[0];
   if (need <= (unsigned long long)kShortEntry * (i1 - i0))
     replay_entries<FILTER_ID, WIDE, BATCH, OUT, true>(sm, t, q, bv, ra, w, i0, i1, pb, pe, idb, ide,
                                                       base0, need, work, st);
@@ -1113,11 +1123,10 @@ cudaError_t launch_write(const TreeView& t, const QueryView& q, const BatchView&
   return launch_packets<true>(t, q, bv, flags, nullptr, nullptr, ra, w, work, st, sms, s);
 }
 
-cudaError_t launch_block_list(const RecordArena& ra, uint32_t packets, cudaStream_t s) {
-  if (packets == 0 || ra.max_blocks == 0) return cudaSuccess;
-  uint32_t blocks = (packets + 255) / 256;
-  if (blocks > 4096) blocks = 4096;
-  k_block_list<<<blocks, 256, 0, s>>>(ra, packets);
+cudaError_t launch_block_list(const RecordArena& ra, int sms, cudaStream_t s) {
+  if (ra.max_blocks == 0) return cudaSuccess;
+  const uint32_t need = (ra.max_blocks + 255) / 256, cap = (uint32_t)sms * 8u;
+  k_block_list<<<need < cap ? need : cap, 256, 0, s>>>(ra);
   note_launches(1);
   return cudaGetLastError();
 }
