@@ -1,6 +1,7 @@
 // Host side of the C ABI (include/ddm.h): argument checks, device workspace,
 // stream-ordered launches and the single status read-back per call.
 #include <algorithm>
+#include <cmath>
 #include <utility>
 #include <atomic>
 #include <cstdlib>
@@ -276,6 +277,15 @@ int key_bytes(uint64_t v) {
   return b;
 }
 
+// Re-sort of the ids in buffer pair `cur` inside the plan's groups (in place).
+int seg_pass(ddm_ctx* c, uint32_t cnt, const float* lo_k, int g, const SegPlan& plan, int tile_log2,
+             int cur, cudaStream_t s) {
+  DDM_CUDA(launch_segsort(static_cast<uint32_t*>(c->vals[cur].p), lo_k, cnt, g, plan, tile_log2,
+                          static_cast<unsigned long long*>(c->keys[0].p),
+                          static_cast<unsigned long long*>(c->keys[1].p), c->sms, s));
+  return DDM_OK;
+}
+
 // Batched sets: the instance is the major sort key, and each instance's
 // re-sort groups are sized from its own extent count.
 struct BatchSet {
@@ -297,19 +307,32 @@ int order_set_batch(ddm_ctx* c, int d, const float* lo, const float* hi, uint32_
                                  static_cast<unsigned long long*>(c->keys[0].p),
                                  static_cast<uint32_t*>(c->vals[0].p), aos, c->st_dev, c->sms, s));
   DDM_TRY(sort_pass(c, cnt, 3 + key_bytes(bs.count ? bs.count - 1 : 0), cur, s));
+  // The re-sorts stay inside an instance's groups; the sizes are known on the
+  // device only, so the chunks are planned there.
+  auto* gl = static_cast<int*>(c->bglog2.p);
+  auto* nc = static_cast<uint32_t*>(c->bngroups.p);
+  auto* cb = static_cast<unsigned long long*>(c->bgbase.p);
   for (int k = 1; k < d; ++k) {
-    auto* gl = static_cast<int*>(c->bglog2.p);
-    auto* ng = static_cast<uint32_t*>(c->bngroups.p);
-    auto* gb = static_cast<unsigned long long*>(c->bgbase.p);
-    DDM_CUDA(launch_batch_groups(bs.off, bs.count, d, k, c->str_shift, gl, ng, s));
-    DDM_CUDA(launch_scan(ng, bs.count, gb, static_cast<unsigned long long*>(c->sums.p), nullptr, s));
-    DDM_CUDA(launch_rekey_batch(static_cast<const uint32_t*>(c->vals[*cur].p), lo + (size_t)k * cnt,
-                                cnt, bs.inst, bs.off, gl, gb,
-                                static_cast<unsigned long long*>(c->keys[*cur].p), c->sms, s));
-    // groups: at most one per instance without re-sort plus cnt / 64
-    DDM_TRY(sort_pass(c, cnt, 3 + key_bytes((uint64_t)bs.count + cnt / 64), cur, s));
+    DDM_CUDA(launch_seg_plan(bs.off, bs.count, d, k, c->str_shift, kSegTileLog2, gl, nc, s));
+    DDM_CUDA(launch_scan(nc, bs.count, cb, static_cast<unsigned long long*>(c->sums.p), nullptr, s));
+    DDM_TRY(seg_pass(c, cnt, lo + (size_t)k * cnt, 0, SegPlan{bs.off, gl, cb, bs.count},
+                     kSegTileLog2, *cur, s));
   }
   return DDM_OK;
+}
+
+// Tile of the on-chip re-sort of dimension k for a single problem of cnt
+// extents (no class or set of it has larger groups), or 0 if its groups may be
+// larger than a CTA takes: groups of 2^13 positions reach to about 2e6 (d = 2)
+// or 2e5 (d = 3, k = 1) extents, and beyond there are as many CTAs' worth of
+// positions per group that one radix sort over the set is the better form.
+int seg_tile(uint32_t cnt, int d, int k, int shift) {
+  if (cnt < 64u) return kSegTileLog2;
+  const double nb = (double)((cnt + 31u) / 32u);
+  const double e = std::log2(32.0 * std::pow(nb, (double)(d - k) / (double)d)) + shift;
+  if (e < kSegTileLog2 + 0.49) return kSegTileLog2;
+  if (e < kSegTileLog2Max + 0.49) return kSegTileLog2Max;
+  return 0;
 }
 
 // Tree order for d >= 2: sort by (size class, lower bound), then refine
@@ -322,27 +345,40 @@ int order_set_classes(ddm_ctx* c, int d, const float* lo, const float* hi, uint3
   DDM_TRY(ensure_sort(c, cnt));
   DDM_TRY(ensure(c, c->cls_hist, sizeof(uint32_t) * kClasses));
   DDM_TRY(ensure(c, c->cls_off, sizeof(unsigned long long) * (kClasses + 1)));
-  DDM_TRY(ensure(c, c->inst_s, sizeof(uint32_t) * cnt));
-  DDM_TRY(ensure(c, c->bglog2, sizeof(int) * kClasses));
+  DDM_TRY(ensure(c, c->bglog2, sizeof(int) * kClasses * DDM_MAX_DIMS));
   DDM_TRY(ensure(c, c->bngroups, sizeof(uint32_t) * kClasses));
-  DDM_TRY(ensure(c, c->bgbase, sizeof(unsigned long long) * (kClasses + 1)));
+  DDM_TRY(ensure(c, c->bgbase, sizeof(unsigned long long) * (kClasses + 1) * DDM_MAX_DIMS));
   DDM_TRY(ensure(c, c->sums, sizeof(unsigned long long) * 4));
   auto* hist = static_cast<uint32_t*>(c->cls_hist.p);
   auto* off = static_cast<unsigned long long*>(c->cls_off.p);
-  auto* inst = static_cast<uint32_t*>(c->inst_s.p);
   auto* sums = static_cast<unsigned long long*>(c->sums.p);
   DDM_CUDA(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * kClasses, s));
   DDM_CUDA(launch_validate_class(d, lo, hi, cnt, static_cast<unsigned long long*>(c->keys[0].p),
                                  static_cast<uint32_t*>(c->vals[0].p), hist, aos, c->st_dev,
                                  c->sms, s));
   DDM_TRY(sort_pass(c, cnt, 4, cur, s));  // (class, 24-bit lower bound)
-  DDM_CUDA(launch_scan(hist, kClasses, off, sums, nullptr, s));
-  DDM_CUDA(launch_fill_inst(off, kClasses, cnt, inst, c->sms, s));
+  ClassPlan plan{off, static_cast<int*>(c->bglog2.p), static_cast<unsigned long long*>(c->bgbase.p), {}};
+  int tile_log2[DDM_MAX_DIMS] = {};
   for (int k = 1; k < d; ++k) {
-    auto* gl = static_cast<int*>(c->bglog2.p);
+    tile_log2[k] = seg_tile(cnt, d, k, c->str_shift);
+    plan.tile[k] = 1u << (tile_log2[k] ? tile_log2[k] : kSegTileLog2);
+  }
+  DDM_CUDA(launch_class_plan(hist, d, c->str_shift, plan, s));
+  for (int k = 1; k < d; ++k) {
+    const int* gl = plan.glog2 + k * kClasses;
+    if (tile_log2[k]) {
+      DDM_TRY(seg_pass(c, cnt, lo + (size_t)k * cnt, 0,
+                       SegPlan{off, gl, plan.cbase + k * (kClasses + 1), kClasses}, tile_log2[k],
+                       *cur, s));
+      continue;
+    }
+    // Groups beyond a CTA: one radix sort over the whole set.
+    DDM_TRY(ensure(c, c->inst_s, sizeof(uint32_t) * cnt));
+    auto* inst = static_cast<uint32_t*>(c->inst_s.p);
     auto* ng = static_cast<uint32_t*>(c->bngroups.p);
-    auto* gb = static_cast<unsigned long long*>(c->bgbase.p);
-    DDM_CUDA(launch_batch_groups(off, kClasses, d, k, c->str_shift, gl, ng, s));
+    auto* gb = plan.cbase + k * (kClasses + 1);
+    if (k == 1) DDM_CUDA(launch_fill_inst(off, kClasses, cnt, inst, c->sms, s));
+    DDM_CUDA(launch_batch_groups(off, kClasses, gl, ng, s));
     DDM_CUDA(launch_scan(ng, kClasses, gb, sums, nullptr, s));
     DDM_CUDA(launch_rekey_batch(static_cast<const uint32_t*>(c->vals[*cur].p), lo + (size_t)k * cnt,
                                 cnt, inst, off, gl, gb,
@@ -365,6 +401,11 @@ int order_set(ddm_ctx* c, int d, const float* lo, const float* hi, uint32_t cnt,
   str_groups(cnt, d, glog2, c->str_shift);
   for (int k = 1; k < d; ++k) {
     if (!glog2[k]) continue;
+    if (glog2[k] <= kSegTileLog2Max) {
+      DDM_TRY(seg_pass(c, cnt, lo + (size_t)k * cnt, glog2[k], SegPlan{},
+                       std::max(glog2[k], kSegTileLog2), *cur, s));
+      continue;
+    }
     DDM_CUDA(launch_rekey(static_cast<const uint32_t*>(c->vals[*cur].p), lo + (size_t)k * cnt, cnt,
                           glog2[k], static_cast<unsigned long long*>(c->keys[*cur].p), c->sms, s));
     int gbits = 0;
@@ -720,6 +761,7 @@ int ddm_create(ddm_ctx** out, int device) {
       cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming) != cudaSuccess ||
       cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
       cudaMalloc(&c->st_dev, sizeof(Status)) != cudaSuccess ||
+      ready_group_table() != cudaSuccess ||
       cudaMallocHost(&c->st_host, sizeof(Status)) != cudaSuccess ||
       cudaMallocHost((void**)&c->rec_hint, 3 * sizeof(uint32_t)) != cudaSuccess) {
     cudaGetLastError();

@@ -117,7 +117,8 @@ struct BatchView {
 // (1 <= k < d) of a set of n extents: with nb = n/32 leaves each dimension
 // gets about nb^(1/d) slabs, so dimension k is re-sorted inside groups of
 // 32 * nb^((d-k)/d) positions, rounded to a power of two.  0 = no re-sort
-// (groups of fewer than 64 would not change any leaf's box).
+// (groups of fewer than 64 would not change any leaf's box).  Kernels use the
+// same rule by thresholds (ready_group_table).
 __host__ __device__ inline int str_group_log2(uint32_t n, int d, int k, int shift = 0) {
   if (n < 64u) return 0;
   const double nb = (double)((n + 31u) / 32u);
@@ -170,10 +171,10 @@ cudaError_t launch_fill_inst(const unsigned long long* off, uint32_t count, uint
 cudaError_t launch_validate_batch(int d, const float* lo, const float* hi, uint32_t cnt,
                                   const uint32_t* inst, unsigned long long* keys, uint32_t* vals,
                                   float2* aos, Status* st, int sms, cudaStream_t s);
-// Per instance and dimension k >= 1: group exponent (0 = groups of 1) and
-// group count, for the batched re-sorts.  glog2/ngroups: [count] each.
-cudaError_t launch_batch_groups(const unsigned long long* off, uint32_t count, int d, int k,
-                                int shift, int* glog2, uint32_t* ngroups, cudaStream_t s);
+// Groups of each instance (or class) for a re-sort over the whole set, from
+// its group exponent (0: one group).  glog2/ngroups: [count] each.
+cudaError_t launch_batch_groups(const unsigned long long* off, uint32_t count, const int* glog2,
+                                uint32_t* ngroups, cudaStream_t s);
 // Batched re-sort keys: group = gbase[inst] + (local position >> glog2[inst]).
 cudaError_t launch_rekey_batch(const uint32_t* vals, const float* lo_k, uint32_t cnt,
                                const uint32_t* inst, const unsigned long long* off,
@@ -203,6 +204,37 @@ size_t sort_lookback_words(uint32_t n);
 cudaError_t launch_debug_wait(const uint32_t* word, uint32_t limit, Status* st, cudaStream_t s);
 cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf, Status* st,
                           int sms, cudaStream_t s);
+
+// ---- ddm_segsort.cu -------------------------------------------------------
+// Thresholds of the group exponents, before the first plan on a device.
+cudaError_t ready_group_table();
+// Positions a CTA re-sorts at once (log2 12 or 13).
+constexpr int kSegTileLog2 = 12, kSegTileLog2Max = 13;
+// A set's re-sort in one dimension, by instance (off null: one instance).
+struct SegPlan {
+  const unsigned long long* off;    // [count + 1] positions of each instance
+  const int* glog2;                 // [count] group exponents, 0 = left as it is
+  const unsigned long long* cbase;  // [count + 1] first chunk of each instance
+  uint32_t count;
+};
+// Size classes: written by launch_class_plan from the class histogram.
+struct ClassPlan {
+  unsigned long long* off;    // [257]
+  int* glog2;                 // [d][256], by dimension
+  unsigned long long* cbase;  // [d][257]
+  uint32_t tile[DDM_MAX_DIMS];  // positions per chunk, by dimension
+};
+cudaError_t launch_class_plan(const uint32_t* hist, int d, int shift, const ClassPlan& plan,
+                              cudaStream_t s);
+// Batched sets: glog2 and nchunks (to be scanned into cbase), [count] each.
+cudaError_t launch_seg_plan(const unsigned long long* off, uint32_t count, int d, int k, int shift,
+                            int tile_log2, int* glog2, uint32_t* nchunks, cudaStream_t s);
+// Stable re-sort of the ids in `vals` by the locality key of lo_k inside each
+// group, in place; with one instance g is its group exponent.  tmp0 and tmp1
+// (`total` words each) are used only by groups larger than a chunk's tile.
+cudaError_t launch_segsort(uint32_t* vals, const float* lo_k, uint32_t total, int g,
+                           const SegPlan& plan, int tile_log2, unsigned long long* tmp0,
+                           unsigned long long* tmp1, int sms, cudaStream_t s);
 
 // ---- ddm_tree.cu ----------------------------------------------------------
 void tree_shape(uint32_t n, int* L, uint32_t* cnt, uint32_t* off, uint32_t* total);

@@ -155,18 +155,11 @@ k_validate_batch(int d, const float* __restrict__ lo, const float* __restrict__ 
   if (__ballot_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&st->err, kErrExtent);
 }
 
-__global__ void k_batch_groups(const unsigned long long* __restrict__ off, uint32_t count, int d,
-                               int k, int shift, int* __restrict__ glog2,
-                               uint32_t* __restrict__ ngroups) {
+__global__ void k_batch_groups(const unsigned long long* __restrict__ off, uint32_t count,
+                               const int* __restrict__ glog2, uint32_t* __restrict__ ngroups) {
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
     const uint32_t n = (uint32_t)(off[i + 1] - off[i]);
-    // strictly smaller than the previous dimension's groups, as in str_groups
-    int g = str_group_log2(n, d, k, shift);
-    for (int j = 1; j < k && g > 0; ++j) {
-      const int gp = str_group_log2(n, d, j, shift);
-      if (gp > 0 && g >= gp) g = 0;
-    }
-    glog2[i] = g;
+    const int g = glog2[i];
     // g == 0 (no re-sort): the whole instance is one group whose keys are
     // all equal, so the stable sort keeps it in place.  With g >= 6 every
     // instance has at most n / 64 + 1 groups.
@@ -246,11 +239,11 @@ cudaError_t launch_validate_batch(int d, const float* lo, const float* hi, uint3
   return cudaGetLastError();
 }
 
-cudaError_t launch_batch_groups(const unsigned long long* off, uint32_t count, int d, int k,
-                                int shift, int* glog2, uint32_t* ngroups, cudaStream_t s) {
+cudaError_t launch_batch_groups(const unsigned long long* off, uint32_t count, const int* glog2,
+                                uint32_t* ngroups, cudaStream_t s) {
   if (count == 0) return cudaSuccess;
   const uint32_t blocks = (count + 255) / 256 < 1024 ? (count + 255) / 256 : 1024;
-  k_batch_groups<<<blocks, 256, 0, s>>>(off, count, d, k, shift, glog2, ngroups);
+  k_batch_groups<<<blocks, 256, 0, s>>>(off, count, glog2, ngroups);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -1,0 +1,446 @@
+// Re-sorts inside groups: the sort-tile-recursive refinement of an order.
+//
+// Dimension k >= 1 of a set is re-sorted by lower bound (the 24-bit locality
+// key, stably) inside aligned groups of 2^g consecutive positions of each
+// instance (a batched problem, a size class of the d >= 2 tree, or the whole
+// update set).  A group is a contiguous range, and at the sizes that matter
+// it fits one CTA's shared memory, so the re-sort needs no pass over the whole
+// set: each CTA takes a chunk of whole groups (kSegTile positions, or 2^g if
+// that is more), sorts it on chip and writes its ids back in place.
+//
+// This replaces a radix sort of (group, key) keys over the whole set -- two or
+// three more digits for the group, and per digit either two grid barriers or a
+// full read and write of keys and ids.  Bound by the ranking (instruction
+// issue and shared-memory latency), not by memory: ids are read and written
+// once and one coordinate per element is gathered.  Measured, whole calls: one
+// match of 5e5 + 5e5 extents (d = 2) 425 -> 332 us, 4,096 batched instances
+// (5.8e7 extents) 16.4 -> 13.8 ms, 256 of them in a CUDA graph 443 -> 299 us.
+#include <algorithm>
+#include <mutex>
+
+#include "ddm_internal.cuh"
+
+namespace ddm {
+namespace {
+
+constexpr int kRadix = 256;
+constexpr int kSegThreads = 1024;
+constexpr int kSegWarps = kSegThreads / 32;
+constexpr int kParts = kSegThreads / kRadix;       // threads per digit
+constexpr int kPartWarps = kSegWarps / kParts;     // warps summed by each
+constexpr int kKeyBits = 24;                       // locality key, see ddm_layout.cu
+
+template <int ITEMS>
+struct SegSmem {
+  uint32_t whist[kSegWarps][kRadix];  // per-warp digit counts, then first slots within the digit
+  uint32_t part[kParts][kRadix];
+  uint32_t total[kRadix];             // the tile's keys with each digit
+  uint32_t first[kRadix];             // the digit's first slot in the tile
+  uint32_t wtot[kRadix / 32];
+  uint32_t base[kRadix];              // groups larger than a tile: running positions
+  unsigned long long word[kSegThreads * ITEMS];
+};
+
+// Lanes of the warp holding the same 8-bit digit.
+__device__ __forceinline__ uint32_t same_digit(uint32_t dig) {
+  uint32_t peers = 0xffffffffu;
+#pragma unroll
+  for (int b = 0; b < 8; ++b) {
+    const uint32_t bit = (dig >> b) & 1u;
+    const uint32_t votes = __ballot_sync(0xffffffffu, bit);
+    peers &= bit ? votes : ~votes;
+  }
+  return peers;
+}
+
+// Stable ranking of one tile by one digit: item i of lane l in warp w is
+// element w*32*ITEMS + i*32 + l.  Elements past `valid` hold the largest key,
+// so they rank last; warps without a valid element skip the ranking.  The
+// ballots of all items come first: only a read and a write of the warp's
+// counters per item are left in the serial chain.
+template <int ITEMS>
+__device__ __forceinline__ void rank_digit(SegSmem<ITEMS>& sm,
+                                           const unsigned long long (&word)[ITEMS],
+                                           uint32_t (&rank)[ITEMS], uint32_t valid, int shift) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t below = (1u << lane) - 1u;
+  for (int t = lane; t < kRadix; t += 32) sm.whist[warp][t] = 0u;
+  __syncwarp();
+  if ((uint32_t)warp * (ITEMS * 32) < valid) {
+    uint32_t peers[ITEMS];
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) peers[i] = same_digit((uint32_t)(word[i] >> shift) & 255u);
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+      uint32_t* h = &sm.whist[warp][(uint32_t)(word[i] >> shift) & 255u];
+      const uint32_t before = *h;
+      rank[i] = before + __popc(peers[i] & below);
+      __syncwarp();
+      if ((peers[i] & below) == 0u) *h = before + __popc(peers[i]);
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  // Thread (part, digit): the digit's counts of a quarter of the warps ...
+  const int dig = tid & (kRadix - 1), part = tid / kRadix;
+  uint32_t c[kPartWarps], sum = 0;
+#pragma unroll
+  for (int j = 0; j < kPartWarps; ++j) {
+    c[j] = sm.whist[part * kPartWarps + j][dig];
+    sum += c[j];
+  }
+  sm.part[part][dig] = sum;
+  __syncthreads();
+  // ... become each warp's first slot within the digit, and the digits' totals
+  // their first slots in the tile.
+  uint32_t run = 0, all = 0;
+#pragma unroll
+  for (int q = 0; q < kParts; ++q) {
+    const uint32_t v = sm.part[q][dig];
+    run += q < part ? v : 0u;
+    all += v;
+  }
+#pragma unroll
+  for (int j = 0; j < kPartWarps; ++j) {
+    sm.whist[part * kPartWarps + j][dig] = run;
+    run += c[j];
+  }
+  uint32_t x = all;
+  if (part == 0) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) sm.wtot[warp] = x;
+    sm.total[dig] = all;
+  }
+  __syncthreads();
+  if (part == 0) {
+    uint32_t pre = 0;
+    for (int q = 0; q < warp; ++q) pre += sm.wtot[q];
+    sm.first[dig] = pre + x - all;
+  }
+  __syncthreads();
+}
+
+// (local group, key) of position `at` of a chunk, above its id.
+__device__ __forceinline__ unsigned long long seg_word(uint32_t id, const float* lo_k, uint32_t at,
+                                                       int g) {
+  const uint32_t key = float_key(__ldg(lo_k + id)) >> (32 - kKeyBits);
+  return ((unsigned long long)(((at >> g) << kKeyBits) | key) << 32) | id;
+}
+
+// One chunk of at most a tile.
+template <int ITEMS>
+__device__ __forceinline__ void sort_chunk(SegSmem<ITEMS>& sm, uint32_t* vals, const float* lo_k,
+                                           uint32_t len, int g) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  unsigned long long word[ITEMS];
+  uint32_t rank[ITEMS];
+#pragma unroll
+  for (int i = 0; i < ITEMS; ++i) {
+    const uint32_t at = warp * (ITEMS * 32) + i * 32 + lane;
+    word[i] = at < len ? seg_word(vals[at], lo_k, at, g) : ~0ull;
+  }
+  const int passes = ((len - 1u) >> g) ? 4 : 3;
+  for (int p = 0; p < passes; ++p) {
+    const int shift = 32 + 8 * p;
+    rank_digit<ITEMS>(sm, word, rank, len, shift);
+    if ((uint32_t)warp * (ITEMS * 32) < len) {
+#pragma unroll
+      for (int i = 0; i < ITEMS; ++i) {
+        const uint32_t d = (uint32_t)(word[i] >> shift) & 255u;
+        sm.word[sm.first[d] + sm.whist[warp][d] + rank[i]] = word[i];
+      }
+    }
+    __syncthreads();
+    if (p + 1 < passes && (uint32_t)warp * (ITEMS * 32) < len) {
+#pragma unroll
+      for (int i = 0; i < ITEMS; ++i) word[i] = sm.word[warp * (ITEMS * 32) + i * 32 + lane];
+    }
+  }
+  for (uint32_t q = tid; q < len; q += kSegThreads) vals[q] = (uint32_t)sm.word[q];
+  __syncthreads();  // before the next chunk's words
+}
+
+// One group larger than a tile (an instance of millions of extents): the same
+// digits, tile by tile through two scratch ranges in global memory.
+template <int ITEMS>
+__device__ void sort_large_group(SegSmem<ITEMS>& sm, uint32_t* vals, const float* lo_k,
+                                 uint32_t len, unsigned long long* a, unsigned long long* b) {
+  constexpr uint32_t kTile = kSegThreads * ITEMS;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (uint32_t q = tid; q < len; q += kSegThreads) a[q] = seg_word(vals[q], lo_k, 0u, 0);
+  __syncthreads();
+  for (int p = 0; p < kKeyBits / 8; ++p) {
+    const int shift = 32 + 8 * p;
+    for (int t = tid; t < kRadix; t += kSegThreads) sm.base[t] = 0u;
+    __syncthreads();
+    for (uint32_t q = tid; q < len; q += kSegThreads)
+      atomicAdd(&sm.base[(uint32_t)(__ldcg(a + q) >> shift) & 255u], 1u);
+    __syncthreads();
+    if (warp == 0) {  // exclusive scan of the 256 counts, eight per lane
+      uint32_t c[8], sum = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        c[j] = sm.base[lane * 8 + j];
+        sum += c[j];
+      }
+      uint32_t x = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      uint32_t run = x - sum;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        sm.base[lane * 8 + j] = run;
+        run += c[j];
+      }
+    }
+    __syncthreads();
+    for (uint32_t t0 = 0; t0 < len; t0 += kTile) {
+      const uint32_t valid = min(kTile, len - t0);
+      unsigned long long word[ITEMS];
+      uint32_t rank[ITEMS];
+#pragma unroll
+      for (int i = 0; i < ITEMS; ++i) {
+        const uint32_t at = warp * (ITEMS * 32) + i * 32 + lane;
+        word[i] = at < valid ? __ldcg(a + t0 + at) : ~0ull;
+      }
+      rank_digit<ITEMS>(sm, word, rank, valid, shift);
+#pragma unroll
+      for (int i = 0; i < ITEMS; ++i) {
+        const uint32_t at = warp * (ITEMS * 32) + i * 32 + lane;
+        const uint32_t d = (uint32_t)(word[i] >> shift) & 255u;
+        if (at < valid) b[sm.base[d] + sm.whist[warp][d] + rank[i]] = word[i];
+      }
+      __syncthreads();
+      // padding words have digit 255 and come last: they do not count
+      if (tid < kRadix) sm.base[tid] += sm.total[tid];
+      __syncthreads();
+    }
+    unsigned long long* t = a;
+    a = b;
+    b = t;
+  }
+  for (uint32_t q = tid; q < len; q += kSegThreads) vals[q] = (uint32_t)__ldcg(a + q);
+  __syncthreads();
+}
+
+// Re-sort of one set.  With `off` null: one instance of `total` positions and
+// group exponent g_one; else instance i owns positions [off[i], off[i+1]) with
+// exponent glog2[i] (0: left as it is) and chunks [cbase[i], cbase[i+1]).
+template <int ITEMS>
+__global__ void __launch_bounds__(kSegThreads, 1)
+k_segsort(uint32_t* __restrict__ vals, const float* __restrict__ lo_k, uint32_t total, int g_one,
+          const unsigned long long* __restrict__ off, const int* __restrict__ glog2,
+          const unsigned long long* __restrict__ cbase, uint32_t count,
+          unsigned long long* __restrict__ tmp0, unsigned long long* __restrict__ tmp1) {
+  constexpr uint32_t kTile = kSegThreads * ITEMS;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SegSmem<ITEMS>& sm = *reinterpret_cast<SegSmem<ITEMS>*>(smem_raw);
+  const uint32_t lane = threadIdx.x & 31u;
+  const unsigned long long chunks = off ? cbase[count] : ((unsigned long long)total + kTile - 1) / kTile;
+  for (unsigned long long c = blockIdx.x; c < chunks; c += gridDim.x) {
+    unsigned long long begin = c * kTile, end = min(begin + kTile, (unsigned long long)total);
+    int g = g_one;
+    if (off) {
+      // The instance whose chunks include c: each warp searches the prefix,
+      // 32 places a step (cbase[lo] <= c < cbase[hi]).
+      uint32_t lo = 0, hi = count;
+      while (hi - lo > 1) {
+        const uint32_t step = (hi - lo + 31u) / 32u, at = lo + lane * step;
+        const uint32_t m = __ballot_sync(0xffffffffu, at < hi && cbase[at] <= c);
+        const uint32_t l = 31u - __clz(m);  // lane 0 always holds
+        lo += l * step;
+        hi = min(hi, lo + step);
+      }
+      g = glog2[lo];
+      const unsigned long long size = max((unsigned long long)kTile, 1ull << g);
+      begin = off[lo] + (c - cbase[lo]) * size;
+      end = min(begin + size, off[lo + 1]);
+    }
+    const uint32_t len = (uint32_t)(end - begin);
+    if (len > kTile)
+      sort_large_group<ITEMS>(sm, vals + begin, lo_k, len, tmp0 + begin, tmp1 + begin);
+    else if (len > 1)
+      sort_chunk<ITEMS>(sm, vals + begin, lo_k, len, g);
+  }
+}
+
+// Thresholds of the group exponents: entry (d * 8 + k) * 32 + g = the least
+// leaf count nb at which str_group_log2's G = 32 * nb^((d-k)/d) rounds to 2^g
+// or more (unclamped, without shift).  The double-precision pow and log2 of
+// the rule cost a launch of one small kernel 7 us per dimension; comparing
+// with thresholds gives the same exponents (G grows by far more than a
+// rounding error from one nb to the next).
+__device__ __forceinline__ int group_exponent(double nb, int d, int k) {
+  return (int)floor(log2(32.0 * pow(nb, (double)(d - k) / (double)d)) + 0.5);
+}
+static __device__ uint32_t g_group_table[(DDM_MAX_DIMS + 1) * 8 * 32];
+
+__global__ void k_group_table() {
+  const int d = blockIdx.x / 8, k = blockIdx.x % 8, g = threadIdx.x;
+  if (d < 2 || k < 1 || k >= d) return;
+  uint32_t lo = 1, hi = 1u << 26;  // more than 2^30 / 32 leaves
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi) / 2;
+    if (group_exponent((double)mid, d, k) >= g) hi = mid; else lo = mid + 1;
+  }
+  g_group_table[(d * 8 + k) * 32 + g] = lo;
+}
+
+// str_group_log2 by the table.
+__device__ __forceinline__ int table_group(uint32_t n, int d, int k, int shift) {
+  if (n < 64u) return 0;
+  const uint32_t nb = (n + 31u) / 32u;
+  const uint32_t* t = g_group_table + (d * 8 + k) * 32;
+  int lo = 0, hi = 32;  // t[lo] <= nb (G >= 32 for every nb), t[hi] > nb
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) / 2;
+    if (t[mid] <= nb) lo = mid; else hi = mid;
+  }
+  const int g = lo + shift;
+  if (g < 6 || (1ull << g) >= (unsigned long long)n) return 0;
+  return g;
+}
+// The exponent used for dimension k: strictly smaller than those before it.
+__device__ __forceinline__ int used_group(uint32_t n, int d, int k, int shift) {
+  int g = table_group(n, d, k, shift);
+  for (int j = 1; j < k && g > 0; ++j) {
+    const int gp = table_group(n, d, j, shift);
+    if (gp > 0 && g >= gp) g = 0;
+  }
+  return g;
+}
+__device__ __forceinline__ uint32_t chunks_of(uint32_t n, int g, uint32_t tile) {
+  if (g == 0) return 0u;
+  const unsigned long long size = max((unsigned long long)tile, 1ull << g);
+  return (uint32_t)((n + size - 1) / size);
+}
+
+// Batched sets: each instance's group exponent and chunk count for dimension k.
+__global__ void k_seg_plan(const unsigned long long* __restrict__ off, uint32_t count, int d, int k,
+                           int shift, uint32_t tile, int* __restrict__ glog2,
+                           uint32_t* __restrict__ nchunks) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
+    const uint32_t n = (uint32_t)(off[i + 1] - off[i]);
+    const int g = used_group(n, d, k, shift);
+    glog2[i] = g;
+    nchunks[i] = chunks_of(n, g, tile);
+  }
+}
+
+// Exclusive scan of 256 values over the CTA's 256 threads; *total = their sum.
+__device__ __forceinline__ uint32_t scan256(uint32_t v, uint32_t* s_w, uint32_t* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_w[warp] = x;
+  __syncthreads();
+  uint32_t pre = 0, all = 0;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    pre += q < warp ? s_w[q] : 0u;
+    all += s_w[q];
+  }
+  __syncthreads();
+  *total = all;
+  return pre + x - v;
+}
+
+// Size classes (one CTA): offsets of the 256 classes from their histogram, and
+// for every dimension k >= 1 their group exponents and chunk prefixes.
+__global__ void __launch_bounds__(256)
+k_class_plan(const uint32_t* __restrict__ hist, int d,
+             int shift, ClassPlan plan) {
+  __shared__ uint32_t s_w[8];
+  const int i = threadIdx.x;
+  const uint32_t n = hist[i];
+  uint32_t total;
+  const uint32_t at = scan256(n, s_w, &total);
+  plan.off[i] = at;
+  if (i == 255) plan.off[256] = total;
+  for (int k = 1; k < d; ++k) {
+    const int g = used_group(n, d, k, shift);
+    const uint32_t c = chunks_of(n, g, plan.tile[k]);
+    const uint32_t first = scan256(c, s_w, &total);
+    plan.glog2[k * 256 + i] = g;
+    plan.cbase[k * 257 + i] = first;
+    if (i == 255) plan.cbase[k * 257 + 256] = total;
+  }
+}
+
+template <int ITEMS>
+cudaError_t launch_segsort_items(uint32_t* vals, const float* lo_k, uint32_t total, int g,
+                                 const SegPlan& plan, unsigned long long* tmp0,
+                                 unsigned long long* tmp1, int sms, cudaStream_t s) {
+  const size_t smem = sizeof(SegSmem<ITEMS>);
+  cudaError_t e = cudaFuncSetAttribute(k_segsort<ITEMS>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e) return e;
+  // at most one chunk per instance beyond the whole tiles
+  const uint64_t most = (uint64_t)total / (kSegThreads * ITEMS) + (plan.off ? plan.count : 0u) + 1u;
+  const uint32_t blocks = (uint32_t)std::min<uint64_t>(most, (uint64_t)sms * 2u);
+  k_segsort<ITEMS><<<blocks, kSegThreads, smem, s>>>(vals, lo_k, total, g, plan.off, plan.glog2,
+                                                     plan.cbase, plan.count, tmp0, tmp1);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+// Fills the current device's table, once per process: on a stream of its own,
+// so that no other stream's work is waited for.
+cudaError_t ready_group_table() {
+  static std::mutex lock;
+  static bool done[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e) return e;
+  std::lock_guard<std::mutex> hold(lock);
+  if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
+  cudaStream_t s = nullptr;
+  if ((e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking))) return e;
+  k_group_table<<<(DDM_MAX_DIMS + 1) * 8, 32, 0, s>>>();
+  note_launches(1);
+  e = cudaGetLastError();
+  if (!e) e = cudaStreamSynchronize(s);
+  cudaStreamDestroy(s);
+  if (!e && dev >= 0 && dev < 64) done[dev] = true;
+  return e;
+}
+
+cudaError_t launch_seg_plan(const unsigned long long* off, uint32_t count, int d, int k, int shift,
+                            int tile_log2, int* glog2, uint32_t* nchunks, cudaStream_t s) {
+  if (count == 0) return cudaSuccess;
+  const uint32_t blocks = (count + 255) / 256 < 1024 ? (count + 255) / 256 : 1024;
+  k_seg_plan<<<blocks, 256, 0, s>>>(off, count, d, k, shift, 1u << tile_log2, glog2, nchunks);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_class_plan(const uint32_t* hist, int d, int shift, const ClassPlan& plan,
+                              cudaStream_t s) {
+  k_class_plan<<<1, 256, 0, s>>>(hist, d, shift, plan);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_segsort(uint32_t* vals, const float* lo_k, uint32_t total, int g,
+                           const SegPlan& plan, int tile_log2, unsigned long long* tmp0,
+                           unsigned long long* tmp1, int sms, cudaStream_t s) {
+  if (total <= 1) return cudaSuccess;
+  return tile_log2 == 12
+             ? launch_segsort_items<4>(vals, lo_k, total, g, plan, tmp0, tmp1, sms, s)
+             : launch_segsort_items<8>(vals, lo_k, total, g, plan, tmp0, tmp1, sms, s);
+}
+
+}  // namespace ddm
