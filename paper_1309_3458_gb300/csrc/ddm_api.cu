@@ -27,6 +27,15 @@ struct DevBuf {
   size_t cap = 0;
 };
 
+// Workspace of one set's ordering.
+struct OrderBufs {
+  DevBuf keys[2], vals[2], hist, lookback, counters;  // radix sort
+  DevBuf aos;                                         // interleaved coordinates
+  DevBuf bglog2, bngroups, bgbase, sums;              // re-sort groups of instances
+  DevBuf* all[11] = {&keys[0], &keys[1], &vals[0], &vals[1], &hist, &lookback, &counters, &aos,
+                     &bglog2, &bngroups, &bgbase};
+};
+
 }  // namespace
 
 struct ddm_ctx {
@@ -54,8 +63,11 @@ struct ddm_ctx {
   Status* st_dev = nullptr;
   Status* st_host = nullptr;  // pinned mirror
 
-  // sort scratch (shared by the subscription and the update sorts)
-  DevBuf keys[2], vals[2], hist, lookback, counters;
+  // Ordering workspace: [0] serves both sets in turn; [1] the updates of a
+  // one-shot call, ordered on `side` while the tree is built.
+  OrderBufs ob[2];
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, joined = nullptr;
   // tree
   DevBuf e, sid, nodes, tab;
   bool tables_on = true;        // rank tables of the leaves (ddm_set_tiling)
@@ -74,11 +86,10 @@ struct ddm_ctx {
   volatile uint32_t* rec_hint = nullptr;
   RecordArena arena{};          // arena of the current plan (max_blocks 0 = none)
   // batched instances
-  DevBuf inst_s, inst_u, bglog2, bngroups, bgbase;
+  DevBuf inst_s, inst_u;
   // size classes of the tree order (d >= 2)
   DevBuf cls_hist, cls_off;
   DevBuf probe;                 // word polled by ddm_debug_wait_timeout
-  DevBuf aos;                   // interleaved coordinates of the set being ordered
   BatchView bv{};               // count 0 = single problem
   // tuning knobs (ddm_set_tuning)
   int str_shift = 0;            // added to the re-sort group exponents
@@ -190,9 +201,9 @@ int ensure(ddm_ctx* c, DevBuf& b, size_t bytes) {
 
 // Interleaved copy of a set's coordinates for the gathers by id; NULL (the
 // gathers then read the caller's rows) if it cannot be allocated.
-float2* aos_buffer(ddm_ctx* c, int d, uint32_t cnt) {
-  if (cnt == 0 || ensure(c, c->aos, sizeof(float2) * (size_t)d * cnt) != DDM_OK) return nullptr;
-  return static_cast<float2*>(c->aos.p);
+float2* aos_buffer(ddm_ctx* c, OrderBufs& o, int d, uint32_t cnt) {
+  if (cnt == 0 || ensure(c, o.aos, sizeof(float2) * (size_t)d * cnt) != DDM_OK) return nullptr;
+  return static_cast<float2*>(o.aos.p);
 }
 
 void release(DevBuf& b) {
@@ -235,28 +246,28 @@ int status_code(const Status& st) {
   return DDM_OK;
 }
 
-int ensure_sort(ddm_ctx* c, uint32_t cnt) {
-  DDM_TRY(ensure(c, c->keys[0], sizeof(unsigned long long) * cnt));
-  DDM_TRY(ensure(c, c->keys[1], sizeof(unsigned long long) * cnt));
-  DDM_TRY(ensure(c, c->vals[0], sizeof(uint32_t) * cnt));
-  DDM_TRY(ensure(c, c->vals[1], sizeof(uint32_t) * cnt));
-  DDM_TRY(ensure(c, c->hist, sizeof(uint32_t) * 8 * 256));
-  DDM_TRY(ensure(c, c->counters, sizeof(uint32_t) * 8));
-  DDM_TRY(ensure(c, c->lookback, sizeof(uint32_t) * sort_lookback_words(cnt)));
+int ensure_sort(ddm_ctx* c, OrderBufs& o, uint32_t cnt) {
+  DDM_TRY(ensure(c, o.keys[0], sizeof(unsigned long long) * cnt));
+  DDM_TRY(ensure(c, o.keys[1], sizeof(unsigned long long) * cnt));
+  DDM_TRY(ensure(c, o.vals[0], sizeof(uint32_t) * cnt));
+  DDM_TRY(ensure(c, o.vals[1], sizeof(uint32_t) * cnt));
+  DDM_TRY(ensure(c, o.hist, sizeof(uint32_t) * 8 * 256));
+  DDM_TRY(ensure(c, o.counters, sizeof(uint32_t) * 8));
+  DDM_TRY(ensure(c, o.lookback, sizeof(uint32_t) * sort_lookback_words(cnt)));
   return DDM_OK;
 }
 
 // Radix sort of the keys/ids in buffer pair `cur` over `passes` 8-bit
 // digits; `cur` is updated to the buffer pair holding the result.
-int sort_pass(ddm_ctx* c, uint32_t cnt, int passes, int* cur, cudaStream_t s) {
+int sort_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, int passes, int* cur, cudaStream_t s) {
   SortScratch sc;
-  sc.keys[0] = static_cast<unsigned long long*>(c->keys[*cur].p);
-  sc.keys[1] = static_cast<unsigned long long*>(c->keys[*cur ^ 1].p);
-  sc.vals[0] = static_cast<uint32_t*>(c->vals[*cur].p);
-  sc.vals[1] = static_cast<uint32_t*>(c->vals[*cur ^ 1].p);
-  sc.hist = static_cast<uint32_t*>(c->hist.p);
-  sc.lookback = static_cast<uint32_t*>(c->lookback.p);
-  sc.counters = static_cast<uint32_t*>(c->counters.p);
+  sc.keys[0] = static_cast<unsigned long long*>(o.keys[*cur].p);
+  sc.keys[1] = static_cast<unsigned long long*>(o.keys[*cur ^ 1].p);
+  sc.vals[0] = static_cast<uint32_t*>(o.vals[*cur].p);
+  sc.vals[1] = static_cast<uint32_t*>(o.vals[*cur ^ 1].p);
+  sc.hist = static_cast<uint32_t*>(o.hist.p);
+  sc.lookback = static_cast<uint32_t*>(o.lookback.p);
+  sc.counters = static_cast<uint32_t*>(o.counters.p);
   int out = 0;
   DDM_CUDA(launch_sort64(sc, cnt, passes, &out, c->st_dev, c->sms, s));
   *cur ^= out;
@@ -278,11 +289,11 @@ int key_bytes(uint64_t v) {
 }
 
 // Re-sort of the ids in buffer pair `cur` inside the plan's groups (in place).
-int seg_pass(ddm_ctx* c, uint32_t cnt, const float* lo_k, int g, const SegPlan& plan, int tile_log2,
+int seg_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, const float* lo_k, int g, const SegPlan& plan, int tile_log2,
              int cur, cudaStream_t s) {
-  DDM_CUDA(launch_segsort(static_cast<uint32_t*>(c->vals[cur].p), lo_k, cnt, g, plan, tile_log2,
-                          static_cast<unsigned long long*>(c->keys[0].p),
-                          static_cast<unsigned long long*>(c->keys[1].p), c->sms, s));
+  DDM_CUDA(launch_segsort(static_cast<uint32_t*>(o.vals[cur].p), lo_k, cnt, g, plan, tile_log2,
+                          static_cast<unsigned long long*>(o.keys[0].p),
+                          static_cast<unsigned long long*>(o.keys[1].p), c->sms, s));
   return DDM_OK;
 }
 
@@ -294,28 +305,33 @@ struct BatchSet {
   uint32_t* inst;                 // [cnt] instance of each position (filled here)
 };
 
-int order_set_batch(ddm_ctx* c, int d, const float* lo, const float* hi, uint32_t cnt,
+// Workspace of order_set_batch.
+int ensure_batch(ddm_ctx* c, OrderBufs& o, uint32_t cnt, uint32_t count) {
+  DDM_TRY(ensure_sort(c, o, cnt));
+  DDM_TRY(ensure(c, o.bglog2, sizeof(int) * (count ? count : 1)));
+  DDM_TRY(ensure(c, o.bngroups, sizeof(uint32_t) * (count ? count : 1)));
+  DDM_TRY(ensure(c, o.bgbase, sizeof(unsigned long long) * ((size_t)count + 1)));
+  return ensure(c, o.sums, sizeof(unsigned long long) * ((size_t)cnt / kScanTile + (size_t)count / kScanTile + 2));
+}
+
+int order_set_batch(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const float* hi, uint32_t cnt,
                     const BatchSet& bs, float2* aos, int* cur, cudaStream_t s) {
   *cur = 0;
-  DDM_TRY(ensure_sort(c, cnt));
-  DDM_TRY(ensure(c, c->bglog2, sizeof(int) * (bs.count ? bs.count : 1)));
-  DDM_TRY(ensure(c, c->bngroups, sizeof(uint32_t) * (bs.count ? bs.count : 1)));
-  DDM_TRY(ensure(c, c->bgbase, sizeof(unsigned long long) * ((size_t)bs.count + 1)));
-  DDM_TRY(ensure(c, c->sums, sizeof(unsigned long long) * ((size_t)cnt / kScanTile + (size_t)bs.count / kScanTile + 2)));
+  DDM_TRY(ensure_batch(c, o, cnt, bs.count));
   DDM_CUDA(launch_fill_inst(bs.off, bs.count, cnt, bs.inst, c->sms, s));
   DDM_CUDA(launch_validate_batch(d, lo, hi, cnt, bs.inst,
-                                 static_cast<unsigned long long*>(c->keys[0].p),
-                                 static_cast<uint32_t*>(c->vals[0].p), aos, c->st_dev, c->sms, s));
-  DDM_TRY(sort_pass(c, cnt, 3 + key_bytes(bs.count ? bs.count - 1 : 0), cur, s));
+                                 static_cast<unsigned long long*>(o.keys[0].p),
+                                 static_cast<uint32_t*>(o.vals[0].p), aos, c->st_dev, c->sms, s));
+  DDM_TRY(sort_pass(c, o, cnt, 3 + key_bytes(bs.count ? bs.count - 1 : 0), cur, s));
   // The re-sorts stay inside an instance's groups; the sizes are known on the
   // device only, so the chunks are planned there.
-  auto* gl = static_cast<int*>(c->bglog2.p);
-  auto* nc = static_cast<uint32_t*>(c->bngroups.p);
-  auto* cb = static_cast<unsigned long long*>(c->bgbase.p);
+  auto* gl = static_cast<int*>(o.bglog2.p);
+  auto* nc = static_cast<uint32_t*>(o.bngroups.p);
+  auto* cb = static_cast<unsigned long long*>(o.bgbase.p);
   for (int k = 1; k < d; ++k) {
     DDM_CUDA(launch_seg_plan(bs.off, bs.count, d, k, c->str_shift, kSegTileLog2, gl, nc, s));
-    DDM_CUDA(launch_scan(nc, bs.count, cb, static_cast<unsigned long long*>(c->sums.p), nullptr, s));
-    DDM_TRY(seg_pass(c, cnt, lo + (size_t)k * cnt, 0, SegPlan{bs.off, gl, cb, bs.count},
+    DDM_CUDA(launch_scan(nc, bs.count, cb, static_cast<unsigned long long*>(o.sums.p), nullptr, s));
+    DDM_TRY(seg_pass(c, o, cnt, lo + (size_t)k * cnt, 0, SegPlan{bs.off, gl, cb, bs.count},
                      kSegTileLog2, *cur, s));
   }
   return DDM_OK;
@@ -338,26 +354,26 @@ int seg_tile(uint32_t cnt, int d, int k, int shift) {
 // Tree order for d >= 2: sort by (size class, lower bound), then refine
 // each class by the sort-tile-recursive re-sorts of its own size (the
 // per-instance machinery of batched sets, with the classes as instances).
-int order_set_classes(ddm_ctx* c, int d, const float* lo, const float* hi, uint32_t cnt,
+int order_set_classes(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const float* hi, uint32_t cnt,
                       float2* aos, int* cur, cudaStream_t s) {
   constexpr uint32_t kClasses = 256;
   *cur = 0;
-  DDM_TRY(ensure_sort(c, cnt));
+  DDM_TRY(ensure_sort(c, o, cnt));
   DDM_TRY(ensure(c, c->cls_hist, sizeof(uint32_t) * kClasses));
   DDM_TRY(ensure(c, c->cls_off, sizeof(unsigned long long) * (kClasses + 1)));
-  DDM_TRY(ensure(c, c->bglog2, sizeof(int) * kClasses * DDM_MAX_DIMS));
-  DDM_TRY(ensure(c, c->bngroups, sizeof(uint32_t) * kClasses));
-  DDM_TRY(ensure(c, c->bgbase, sizeof(unsigned long long) * (kClasses + 1) * DDM_MAX_DIMS));
-  DDM_TRY(ensure(c, c->sums, sizeof(unsigned long long) * 4));
+  DDM_TRY(ensure(c, o.bglog2, sizeof(int) * kClasses * DDM_MAX_DIMS));
+  DDM_TRY(ensure(c, o.bngroups, sizeof(uint32_t) * kClasses));
+  DDM_TRY(ensure(c, o.bgbase, sizeof(unsigned long long) * (kClasses + 1) * DDM_MAX_DIMS));
+  DDM_TRY(ensure(c, o.sums, sizeof(unsigned long long) * 4));
   auto* hist = static_cast<uint32_t*>(c->cls_hist.p);
   auto* off = static_cast<unsigned long long*>(c->cls_off.p);
-  auto* sums = static_cast<unsigned long long*>(c->sums.p);
+  auto* sums = static_cast<unsigned long long*>(o.sums.p);
   DDM_CUDA(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * kClasses, s));
-  DDM_CUDA(launch_validate_class(d, lo, hi, cnt, static_cast<unsigned long long*>(c->keys[0].p),
-                                 static_cast<uint32_t*>(c->vals[0].p), hist, aos, c->st_dev,
+  DDM_CUDA(launch_validate_class(d, lo, hi, cnt, static_cast<unsigned long long*>(o.keys[0].p),
+                                 static_cast<uint32_t*>(o.vals[0].p), hist, aos, c->st_dev,
                                  c->sms, s));
-  DDM_TRY(sort_pass(c, cnt, 4, cur, s));  // (class, 24-bit lower bound)
-  ClassPlan plan{off, static_cast<int*>(c->bglog2.p), static_cast<unsigned long long*>(c->bgbase.p), {}};
+  DDM_TRY(sort_pass(c, o, cnt, 4, cur, s));  // (class, 24-bit lower bound)
+  ClassPlan plan{off, static_cast<int*>(o.bglog2.p), static_cast<unsigned long long*>(o.bgbase.p), {}};
   int tile_log2[DDM_MAX_DIMS] = {};
   for (int k = 1; k < d; ++k) {
     tile_log2[k] = seg_tile(cnt, d, k, c->str_shift);
@@ -367,7 +383,7 @@ int order_set_classes(ddm_ctx* c, int d, const float* lo, const float* hi, uint3
   for (int k = 1; k < d; ++k) {
     const int* gl = plan.glog2 + k * kClasses;
     if (tile_log2[k]) {
-      DDM_TRY(seg_pass(c, cnt, lo + (size_t)k * cnt, 0,
+      DDM_TRY(seg_pass(c, o, cnt, lo + (size_t)k * cnt, 0,
                        SegPlan{off, gl, plan.cbase + k * (kClasses + 1), kClasses}, tile_log2[k],
                        *cur, s));
       continue;
@@ -375,42 +391,42 @@ int order_set_classes(ddm_ctx* c, int d, const float* lo, const float* hi, uint3
     // Groups beyond a CTA: one radix sort over the whole set.
     DDM_TRY(ensure(c, c->inst_s, sizeof(uint32_t) * cnt));
     auto* inst = static_cast<uint32_t*>(c->inst_s.p);
-    auto* ng = static_cast<uint32_t*>(c->bngroups.p);
+    auto* ng = static_cast<uint32_t*>(o.bngroups.p);
     auto* gb = plan.cbase + k * (kClasses + 1);
     if (k == 1) DDM_CUDA(launch_fill_inst(off, kClasses, cnt, inst, c->sms, s));
     DDM_CUDA(launch_batch_groups(off, kClasses, gl, ng, s));
     DDM_CUDA(launch_scan(ng, kClasses, gb, sums, nullptr, s));
-    DDM_CUDA(launch_rekey_batch(static_cast<const uint32_t*>(c->vals[*cur].p), lo + (size_t)k * cnt,
+    DDM_CUDA(launch_rekey_batch(static_cast<const uint32_t*>(o.vals[*cur].p), lo + (size_t)k * cnt,
                                 cnt, inst, off, gl, gb,
-                                static_cast<unsigned long long*>(c->keys[*cur].p), c->sms, s));
+                                static_cast<unsigned long long*>(o.keys[*cur].p), c->sms, s));
     // groups: at most one per class without re-sort plus cnt / 64
-    DDM_TRY(sort_pass(c, cnt, 3 + key_bytes((uint64_t)kClasses + cnt / 64), cur, s));
+    DDM_TRY(sort_pass(c, o, cnt, 3 + key_bytes((uint64_t)kClasses + cnt / 64), cur, s));
   }
   return DDM_OK;
 }
 
-int order_set(ddm_ctx* c, int d, const float* lo, const float* hi, uint32_t cnt, bool tree,
+int order_set(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const float* hi, uint32_t cnt, bool tree,
               float2* aos, int* cur, cudaStream_t s) {
   *cur = 0;
-  DDM_TRY(ensure_sort(c, cnt));
-  DDM_CUDA(launch_validate(d, lo, hi, cnt, static_cast<unsigned long long*>(c->keys[0].p),
-                           static_cast<uint32_t*>(c->vals[0].p), tree ? 1 : 2, aos, c->st_dev,
+  DDM_TRY(ensure_sort(c, o, cnt));
+  DDM_CUDA(launch_validate(d, lo, hi, cnt, static_cast<unsigned long long*>(o.keys[0].p),
+                           static_cast<uint32_t*>(o.vals[0].p), tree ? 1 : 2, aos, c->st_dev,
                            c->sms, s));
-  DDM_TRY(sort_pass(c, cnt, tree ? 8 : 3, cur, s));
+  DDM_TRY(sort_pass(c, o, cnt, tree ? 8 : 3, cur, s));
   int glog2[DDM_MAX_DIMS];
   str_groups(cnt, d, glog2, c->str_shift);
   for (int k = 1; k < d; ++k) {
     if (!glog2[k]) continue;
     if (glog2[k] <= kSegTileLog2Max) {
-      DDM_TRY(seg_pass(c, cnt, lo + (size_t)k * cnt, glog2[k], SegPlan{},
+      DDM_TRY(seg_pass(c, o, cnt, lo + (size_t)k * cnt, glog2[k], SegPlan{},
                        std::max(glog2[k], kSegTileLog2), *cur, s));
       continue;
     }
-    DDM_CUDA(launch_rekey(static_cast<const uint32_t*>(c->vals[*cur].p), lo + (size_t)k * cnt, cnt,
-                          glog2[k], static_cast<unsigned long long*>(c->keys[*cur].p), c->sms, s));
+    DDM_CUDA(launch_rekey(static_cast<const uint32_t*>(o.vals[*cur].p), lo + (size_t)k * cnt, cnt,
+                          glog2[k], static_cast<unsigned long long*>(o.keys[*cur].p), c->sms, s));
     int gbits = 0;
     while (gbits < 32 && (((uint64_t)(cnt - 1) >> glog2[k]) >> gbits) != 0) ++gbits;
-    DDM_TRY(sort_pass(c, cnt, 3 + (gbits + 7) / 8, cur, s));
+    DDM_TRY(sort_pass(c, o, cnt, 3 + (gbits + 7) / 8, cur, s));
   }
   return DDM_OK;
 }
@@ -438,13 +454,14 @@ int build_async(ddm_ctx* c, int d, const float* slo, const float* shi, uint32_t 
   DDM_TRY(ensure(c, c->sid, sizeof(uint32_t) * n));
   DDM_TRY(ensure(c, c->nodes, sizeof(float2) * (size_t)d * t.total));
   int cur = 0;
-  float2* aos = aos_buffer(c, d, n);
+  OrderBufs& o = c->ob[0];
+  float2* aos = aos_buffer(c, o, d, n);
   if (bs)
-    DDM_TRY(order_set_batch(c, d, slo, shi, n, *bs, aos, &cur, s));
+    DDM_TRY(order_set_batch(c, o, d, slo, shi, n, *bs, aos, &cur, s));
   else if (d >= 2)
-    DDM_TRY(order_set_classes(c, d, slo, shi, n, aos, &cur, s));
+    DDM_TRY(order_set_classes(c, o, d, slo, shi, n, aos, &cur, s));
   else
-    DDM_TRY(order_set(c, d, slo, shi, n, true, aos, &cur, s));
+    DDM_TRY(order_set(c, o, d, slo, shi, n, true, aos, &cur, s));
   t.e = static_cast<const float2*>(c->e.p);
   t.sid = static_cast<const uint32_t*>(c->sid.p);
   t.nodes = static_cast<const float2*>(c->nodes.p);
@@ -454,7 +471,7 @@ int build_async(ddm_ctx* c, int d, const float* slo, const float* shi, uint32_t 
   if (d <= 3 && c->tables_on &&
       ensure(c, c->tab, sizeof(uint32_t) * 2u * kRankSlot * (size_t)d * t.cnt[1]) == DDM_OK)
     t.tab = static_cast<const uint32_t*>(c->tab.p);
-  DDM_CUDA(launch_build(t, static_cast<const uint32_t*>(c->vals[cur].p), slo, shi, aos,
+  DDM_CUDA(launch_build(t, static_cast<const uint32_t*>(o.vals[cur].p), slo, shi, aos,
                         static_cast<float2*>(c->e.p), static_cast<uint32_t*>(c->sid.p),
                         static_cast<float2*>(c->nodes.p), const_cast<uint32_t*>(t.tab),
                         c->st_dev, s));
@@ -487,12 +504,32 @@ QueryView query_view(ddm_ctx* c) {
   return q;
 }
 
-// Validate U, sort it, count per update, scan (no host synchronisation).
+int ensure_queries(ddm_ctx* c, int d, uint32_t m) {
+  DDM_TRY(ensure(c, c->qe, sizeof(float2) * (size_t)d * (m ? m : 1)));
+  return ensure(c, c->qid, sizeof(uint32_t) * (m ? m : 1));
+}
+
+// Validate U, sort it and gather the queries in plan order (qe, qid).
+int order_updates(ddm_ctx* c, OrderBufs& o, int d, const float* ulo, const float* uhi, uint32_t m,
+                  const BatchSet* bs, float2* aos, cudaStream_t s) {
+  int cur = 0;
+  if (bs)
+    DDM_TRY(order_set_batch(c, o, d, ulo, uhi, m, *bs, aos, &cur, s));
+  else
+    DDM_TRY(order_set(c, o, d, ulo, uhi, m, false, aos, &cur, s));
+  DDM_CUDA(launch_gather(d, static_cast<const uint32_t*>(o.vals[cur].p), ulo, uhi, aos, m,
+                         static_cast<float2*>(c->qe.p), static_cast<uint32_t*>(c->qid.p), c->sms, s));
+  return DDM_OK;
+}
+
+// Validate U, sort it (unless `sorted`: order_updates has run), count per
+// update, scan (no host synchronisation).
 // `ordered`: the plan order's offsets too (the staged calls); the one-shot
 // calls do not write by plan order, and a staged call after one of them has
 // ready_ordered() compute them.
 int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint32_t flags,
-               bool record, bool ordered, cudaStream_t s, const BatchSet* bs = nullptr) {
+               bool record, bool ordered, cudaStream_t s, const BatchSet* bs = nullptr,
+               bool sorted = false) {
   Phase phase("ddm plan");
   c->planned = false;
   const int d = c->tree.d;
@@ -512,8 +549,7 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
   // tile sums of a range selection (write_async)
   DDM_TRY(ensure(c, c->sums, sizeof(unsigned long long) * ((size_t)m / kScanTile + 2)));
   DDM_TRY(ensure(c, c->work, sizeof(uint32_t)));
-  DDM_TRY(ensure(c, c->qe, sizeof(float2) * (size_t)d * (m ? m : 1)));
-  DDM_TRY(ensure(c, c->qid, sizeof(uint32_t) * (m ? m : 1)));
+  DDM_TRY(ensure_queries(c, d, m));
   auto* counts = static_cast<uint32_t*>(c->counts.p);
   auto* counts_pos = static_cast<uint32_t*>(c->counts_pos.p);
   auto* offsets = static_cast<unsigned long long*>(c->offsets.p);
@@ -584,15 +620,7 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
   DDM_CUDA(cudaMemsetAsync(state, 0, sizeof(unsigned long long) * state_words, s));
   if (c->arena.max_blocks) c->arena.blk_counter = reinterpret_cast<uint32_t*>(state);
   if (m > 0) {
-    int cur = 0;
-    float2* aos = aos_buffer(c, d, m);
-    if (bs)
-      DDM_TRY(order_set_batch(c, d, ulo, uhi, m, *bs, aos, &cur, s));
-    else
-      DDM_TRY(order_set(c, d, ulo, uhi, m, false, aos, &cur, s));
-    DDM_CUDA(launch_gather(d, static_cast<const uint32_t*>(c->vals[cur].p), ulo, uhi, aos, m,
-                           static_cast<float2*>(c->qe.p), static_cast<uint32_t*>(c->qid.p), c->sms,
-                           s));
+    if (!sorted) DDM_TRY(order_updates(c, c->ob[0], d, ulo, uhi, m, bs, aos_buffer(c, c->ob[0], d, m), s));
     if (c->tree.n > 0) {
       DDM_CUDA(launch_count(c->tree, query_view(c), c->bv, flags, counts, counts_pos, c->arena,
                             static_cast<uint32_t*>(c->work.p), c->st_dev, packet_sms(c), s));
@@ -708,6 +736,58 @@ int write_ordered_async(ddm_ctx* c, uint32_t pb, uint32_t pe, ddm_pair* pairs, u
   return DDM_OK;
 }
 
+int release_now(ddm_ctx* c, DevBuf& b) {
+  if (b.p) {
+    cudaFreeAsync(b.p, c->cur);
+    c->allocated -= b.cap;
+  }
+  b.p = nullptr;
+  b.cap = 0;
+  return DDM_OK;
+}
+
+// Build and plan of a one-shot call: the updates are ordered on the context's
+// side stream while the tree is built -- both are chains of short launches
+// that leave most of the chip idle.  The side stream starts after the work
+// enqueued so far and the caller's stream goes on after it, so nothing of the
+// call is left on it.  Its workspace is allocated before, on the caller's
+// stream; without room for it the two run one after the other.  Measured, one
+// match: 64 + 64 extents (d = 1) 99 -> 89 us, 5,000 + 5,000 124 -> 109 us, 5e5
+// + 5e5 388 -> 356 us (d = 1) and 328 -> 272 us (d = 2), 2.5e7 + 2.5e7 8.15 ->
+// 7.94 ms; 256 batched instances in a graph 289 -> 198 us.
+int build_and_plan(ddm_ctx* c, int d, const float* slo, const float* shi, uint32_t n,
+                   const float* ulo, const float* uhi, uint32_t m, uint32_t flags, bool record,
+                   bool swap, cudaStream_t s, const BatchSet* bs_s = nullptr,
+                   const BatchSet* bs_u = nullptr, const BatchView* bv = nullptr) {
+  OrderBufs& o = c->ob[1];
+  auto sequel = [&](bool sorted) {
+    c->swapped = swap;
+    if (bv) c->bv = *bv;
+    return plan_async(c, ulo, uhi, m, flags, record, false, s, bs_u, sorted);
+  };
+  if (m > 0 && n > 0) {
+    int rc = bs_u ? ensure_batch(c, o, m, bs_u->count) : ensure_sort(c, o, m);
+    if (rc == DDM_OK) rc = ensure_queries(c, d, m);
+    if (rc == DDM_OK) {
+      float2* aos = aos_buffer(c, o, d, m);
+      DDM_CUDA(cudaEventRecord(c->fork, s));
+      rc = build_async(c, d, slo, shi, n, s, bs_s);
+      if (rc == DDM_OK) {
+        DDM_CUDA(cudaStreamWaitEvent(c->side, c->fork, 0));
+        rc = order_updates(c, o, d, ulo, uhi, m, bs_u, aos, c->side);
+        DDM_CUDA(cudaEventRecord(c->joined, c->side));  // also after an error: joined before returning
+        DDM_CUDA(cudaStreamWaitEvent(s, c->joined, 0));
+        if (rc == DDM_OK) rc = sequel(true);
+      }
+    }
+    if (rc != DDM_ERR_NOMEM) return rc;
+    for (DevBuf* b : o.all) release_now(c, *b);
+    release_now(c, o.sums);
+  }
+  DDM_TRY(build_async(c, d, slo, shi, n, s, bs_s));
+  return sequel(false);
+}
+
 int reset_status(ddm_ctx* c, cudaStream_t s) {
   DDM_CUDA(cudaMemsetAsync(c->st_dev, 0, sizeof(Status), s));
   return DDM_OK;
@@ -759,6 +839,9 @@ int ddm_create(ddm_ctx** out, int device) {
       cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, (void*)&keep_all) !=
           cudaSuccess ||
       cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->joined, cudaEventDisableTiming) != cudaSuccess ||
       cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
       cudaMalloc(&c->st_dev, sizeof(Status)) != cudaSuccess ||
       ready_group_table() != cudaSuccess ||
@@ -777,17 +860,23 @@ int ddm_destroy(ddm_ctx* c) {
   if (!c) return DDM_OK;
   DeviceGuard g(c->device);
   cudaDeviceSynchronize();
-  for (DevBuf* b : {&c->keys[0], &c->keys[1], &c->vals[0], &c->vals[1], &c->hist, &c->lookback,
-                    &c->counters, &c->e, &c->sid, &c->nodes, &c->tab, &c->qe, &c->qid, &c->counts,
+  for (OrderBufs& o : c->ob) {
+    for (DevBuf* b : o.all) release(*b);
+    release(o.sums);
+  }
+  for (DevBuf* b : {&c->e, &c->sid, &c->nodes, &c->tab, &c->qe, &c->qid, &c->counts,
                     &c->counts_pos, &c->offsets, &c->pos_offsets, &c->sums, &c->work,
                     &c->sel_offs, &c->sel_list, &c->rec, &c->blk_own, &c->blk_count,
                     &c->pkt_nblk, &c->pkt_off,
-                    &c->blk_list, &c->plan_state, &c->order_state, &c->inst_s, &c->inst_u, &c->bglog2,
-                    &c->bngroups, &c->bgbase, &c->cls_hist, &c->cls_off, &c->probe, &c->aos})
+                    &c->blk_list, &c->plan_state, &c->order_state, &c->inst_s, &c->inst_u,
+                    &c->cls_hist, &c->cls_off, &c->probe})
     release(*b);
   cudaDeviceSynchronize();  // the stream-ordered frees above have run
   if (c->pool) cudaMemPoolDestroy(c->pool);
   if (c->done) cudaEventDestroy(c->done);
+  if (c->fork) cudaEventDestroy(c->fork);
+  if (c->joined) cudaEventDestroy(c->joined);
+  if (c->side) cudaStreamDestroy(c->side);
   if (c->st_dev) cudaFree(c->st_dev);
   if (c->st_host) cudaFreeHost(c->st_host);
   if (c->rec_hint) cudaFreeHost((void*)c->rec_hint);
@@ -1085,9 +1174,7 @@ static int match_impl(ddm_ctx* c, int d, const float* ulo, const float* uhi, uin
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   StreamUse use(c, s);
   DDM_TRY(reset_status(c, s));
-  DDM_TRY(build_async(c, d, slo, shi, n, s));
-  c->swapped = swap;
-  DDM_TRY(plan_async(c, ulo, uhi, m, flags & DDM_OPEN, write, false, s));
+  DDM_TRY(build_and_plan(c, d, slo, shi, n, ulo, uhi, m, flags & DDM_OPEN, write, swap, s));
   if (write) DDM_TRY(write_async(c, begin, end, pairs, capacity, s));
   DDM_TRY(sync_status(c, s));
   c->last_tests = c->st_host->tests;
@@ -1137,12 +1224,8 @@ static int batch_impl(ddm_ctx* c, int d, uint32_t count, const float* ulo, const
   const auto* soff = reinterpret_cast<const unsigned long long*>(sub_off);
   BatchSet bs_s{soff, count, static_cast<uint32_t*>(c->inst_s.p)};
   BatchSet bs_u{uoff, count, static_cast<uint32_t*>(c->inst_u.p)};
-  DDM_TRY(build_async(c, d, slo, shi, n, s, &bs_s));
-  c->bv.count = count;
-  c->bv.upd_off = uoff;
-  c->bv.sub_off = soff;
-  c->bv.q_inst = static_cast<const uint32_t*>(c->inst_u.p);
-  DDM_TRY(plan_async(c, ulo, uhi, m, flags, true, false, s, &bs_u));
+  const BatchView bv{count, uoff, soff, static_cast<const uint32_t*>(c->inst_u.p)};
+  DDM_TRY(build_and_plan(c, d, slo, shi, n, ulo, uhi, m, flags, true, false, s, &bs_s, &bs_u, &bv));
   DDM_TRY(write_async(c, 0, m, pairs, capacity, s));
   if (pair_off && m > 0)
     DDM_CUDA(launch_gather_offsets(static_cast<const unsigned long long*>(c->offsets.p), m, uoff,
@@ -1193,7 +1276,7 @@ int ddm_refit(ddm_ctx* c, const float* sub_lo, const float* sub_hi, void* stream
   c->planned = false;
   Phase phase("ddm refit");
   if (c->tree.n > 0) {
-    float2* aos = aos_buffer(c, c->tree.d, c->tree.n);
+    float2* aos = aos_buffer(c, c->ob[0], c->tree.d, c->tree.n);
     DDM_CUDA(launch_validate(c->tree.d, sub_lo, sub_hi, c->tree.n, nullptr, nullptr, 0, aos,
                              c->st_dev, c->sms, s));
     // Same order, new coordinates: gather through the tree's own id column and

@@ -451,8 +451,10 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target, Sta
   return *s_abort == 0;
 }
 
+// Two CTAs per SM up to 4,096-key tiles (64 registers, no spill): a one-shot
+// call sorts both of its sets at the same time.
 template <int ITEMS>
-__global__ void __launch_bounds__(kSmallThreads, 1)
+__global__ void __launch_bounds__(kSmallThreads, ITEMS <= 8 ? 2 : 1)
 k_sort_grid(unsigned long long* __restrict__ keys0, uint32_t* __restrict__ vals0,
             unsigned long long* __restrict__ keys1, uint32_t* __restrict__ vals1, uint32_t n,
             int passes, uint32_t* __restrict__ table, uint32_t* __restrict__ bar,
