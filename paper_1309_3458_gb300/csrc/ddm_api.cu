@@ -297,6 +297,15 @@ int seg_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, const float* lo_k, int g, c
   return DDM_OK;
 }
 
+// Sets up to this size are ordered by counting.  Quadratic against the cluster
+// sort's passes, of which a d = 1 tree needs eight, the others three or four.
+// Measured, one match of n + n extents, by radix sort and by counting: d = 1,
+// n = 64: 90 / 65 us, 4,096: 105 / 78, 8,192: 112 / 92, 10,000: 116 / 111 (and
+// 117 / 122 at 12,000); d = 2, n = 64: 91 / 81, 4,096: 123 / 115, 6,000: 126 /
+// 122, 8,192: 126 / 134; d = 3, n = 4,096: 155 / 150, 6,000: 155 / 152, 8,192:
+// 159 / 163.
+uint32_t rank_sort_max(int d) { return d == 1 ? 8192u : 6144u; }
+
 // Batched sets: the instance is the major sort key, and each instance's
 // re-sort groups are sized from its own extent count.
 struct BatchSet {
@@ -369,10 +378,15 @@ int order_set_classes(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const fl
   auto* off = static_cast<unsigned long long*>(c->cls_off.p);
   auto* sums = static_cast<unsigned long long*>(o.sums.p);
   DDM_CUDA(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * kClasses, s));
-  DDM_CUDA(launch_validate_class(d, lo, hi, cnt, static_cast<unsigned long long*>(o.keys[0].p),
-                                 static_cast<uint32_t*>(o.vals[0].p), hist, aos, c->st_dev,
-                                 c->sms, s));
-  DDM_TRY(sort_pass(c, o, cnt, 4, cur, s));  // (class, 24-bit lower bound)
+  if (cnt <= rank_sort_max(d)) {
+    DDM_CUDA(launch_rank_sort(kRankClass, d, lo, hi, cnt, static_cast<uint32_t*>(o.vals[0].p), hist,
+                              aos, nullptr, nullptr, c->st_dev, s));
+  } else {
+    DDM_CUDA(launch_validate_class(d, lo, hi, cnt, static_cast<unsigned long long*>(o.keys[0].p),
+                                   static_cast<uint32_t*>(o.vals[0].p), hist, aos, c->st_dev,
+                                   c->sms, s));
+    DDM_TRY(sort_pass(c, o, cnt, 4, cur, s));  // (class, 24-bit lower bound)
+  }
   ClassPlan plan{off, static_cast<int*>(o.bglog2.p), static_cast<unsigned long long*>(o.bgbase.p), {}};
   int tile_log2[DDM_MAX_DIMS] = {};
   for (int k = 1; k < d; ++k) {
@@ -405,14 +419,25 @@ int order_set_classes(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const fl
   return DDM_OK;
 }
 
+// `tree`: the d = 1 tree's order, else the updates'.  *gathered (updates): qe
+// and qid are written too.
 int order_set(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const float* hi, uint32_t cnt, bool tree,
-              float2* aos, int* cur, cudaStream_t s) {
+              float2* aos, int* cur, bool* gathered, cudaStream_t s) {
   *cur = 0;
+  *gathered = false;
   DDM_TRY(ensure_sort(c, o, cnt));
-  DDM_CUDA(launch_validate(d, lo, hi, cnt, static_cast<unsigned long long*>(o.keys[0].p),
-                           static_cast<uint32_t*>(o.vals[0].p), tree ? 1 : 2, aos, c->st_dev,
-                           c->sms, s));
-  DDM_TRY(sort_pass(c, o, cnt, tree ? 8 : 3, cur, s));
+  if (cnt <= rank_sort_max(d)) {
+    *gathered = !tree && d == 1;  // no re-sorts follow
+    DDM_CUDA(launch_rank_sort(tree ? kRankTree : kRankLocal, d, lo, hi, cnt,
+                              static_cast<uint32_t*>(o.vals[0].p), nullptr, aos,
+                              *gathered ? static_cast<float2*>(c->qe.p) : nullptr,
+                              *gathered ? static_cast<uint32_t*>(c->qid.p) : nullptr, c->st_dev, s));
+  } else {
+    DDM_CUDA(launch_validate(d, lo, hi, cnt, static_cast<unsigned long long*>(o.keys[0].p),
+                             static_cast<uint32_t*>(o.vals[0].p), tree ? 1 : 2, aos, c->st_dev,
+                             c->sms, s));
+    DDM_TRY(sort_pass(c, o, cnt, tree ? 8 : 3, cur, s));
+  }
   int glog2[DDM_MAX_DIMS];
   str_groups(cnt, d, glog2, c->str_shift);
   for (int k = 1; k < d; ++k) {
@@ -454,6 +479,7 @@ int build_async(ddm_ctx* c, int d, const float* slo, const float* shi, uint32_t 
   DDM_TRY(ensure(c, c->sid, sizeof(uint32_t) * n));
   DDM_TRY(ensure(c, c->nodes, sizeof(float2) * (size_t)d * t.total));
   int cur = 0;
+  bool gathered = false;
   OrderBufs& o = c->ob[0];
   float2* aos = aos_buffer(c, o, d, n);
   if (bs)
@@ -461,7 +487,7 @@ int build_async(ddm_ctx* c, int d, const float* slo, const float* shi, uint32_t 
   else if (d >= 2)
     DDM_TRY(order_set_classes(c, o, d, slo, shi, n, aos, &cur, s));
   else
-    DDM_TRY(order_set(c, o, d, slo, shi, n, true, aos, &cur, s));
+    DDM_TRY(order_set(c, o, d, slo, shi, n, true, aos, &cur, &gathered, s));
   t.e = static_cast<const float2*>(c->e.p);
   t.sid = static_cast<const uint32_t*>(c->sid.p);
   t.nodes = static_cast<const float2*>(c->nodes.p);
@@ -513,10 +539,12 @@ int ensure_queries(ddm_ctx* c, int d, uint32_t m) {
 int order_updates(ddm_ctx* c, OrderBufs& o, int d, const float* ulo, const float* uhi, uint32_t m,
                   const BatchSet* bs, float2* aos, cudaStream_t s) {
   int cur = 0;
+  bool gathered = false;
   if (bs)
     DDM_TRY(order_set_batch(c, o, d, ulo, uhi, m, *bs, aos, &cur, s));
   else
-    DDM_TRY(order_set(c, o, d, ulo, uhi, m, false, aos, &cur, s));
+    DDM_TRY(order_set(c, o, d, ulo, uhi, m, false, aos, &cur, &gathered, s));
+  if (gathered) return DDM_OK;
   DDM_CUDA(launch_gather(d, static_cast<const uint32_t*>(o.vals[cur].p), ulo, uhi, aos, m,
                          static_cast<float2*>(c->qe.p), static_cast<uint32_t*>(c->qid.p), c->sms, s));
   return DDM_OK;
@@ -572,14 +600,14 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
     if (have < (uint64_t)packets * kRecChains || (hint_packets && hint_blocks > hint_max)) {
       // No arena yet, not a block for each chain, or the last pass ran out of
       // it: size from that pass's blocks per packet (plus 1/8 and some
-      // slack), else one per chain and as many again per packet.  An
+      // slack), else one per chain and an eighth of a block per packet.  An
       // arena that sufficed is kept as it is: the blocks per packet depend on
       // how densely the updates cover the space, so extrapolating them from
       // one plan to the next would reallocate for nothing.
       const uint64_t need =
           hint_packets ? (uint64_t)((double)hint_blocks / (double)hint_packets * 1.125 *
                                     (double)packets) + 64
-                       : (kRecChains + 1ull) * packets;
+                       : (uint64_t)kRecChains * packets + packets / 8 + 64;
       want = std::max(have, need);
     }
     const uint64_t cap_blocks = c->replay_budget / per_block;

@@ -205,6 +205,15 @@ cudaError_t launch_debug_wait(const uint32_t* word, uint32_t limit, Status* st, 
 cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf, Status* st,
                           int sms, cudaStream_t s);
 
+// ---- ddm_ranksort.cu ------------------------------------------------------
+// Validation, first order (vals) and optional interleaved copy of a small set
+// in one launch, the order of launch_validate's or launch_validate_class's
+// keys (hist as there); qe and qid (optional) receive the set in that order.
+enum { kRankTree = 1, kRankLocal = 2, kRankClass = 3 };
+cudaError_t launch_rank_sort(int mode, int d, const float* lo, const float* hi, uint32_t n,
+                             uint32_t* vals, uint32_t* hist, float2* aos, float2* qe, uint32_t* qid,
+                             Status* st, cudaStream_t s);
+
 // ---- ddm_segsort.cu -------------------------------------------------------
 // Thresholds of the group exponents, before the first plan on a device.
 cudaError_t ready_group_table();

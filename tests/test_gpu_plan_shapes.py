@@ -103,3 +103,36 @@ def test_entry_limit(ctx, records):
     _, ou, os_ = oracle.itm_pairs(*arrays)
     assert K == len(ou)
     assert np.array_equal(np.sort(keys(pu, ps)), np.sort(keys(ou, os_)))
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 31, 63, 64, 65, 2047, 2049, 2051, 6144, 6145, 8191, 8192, 8193])
+def test_order_by_counting(ctx, n):
+    """Tree and plan order of small sets, around the staged chunk of keys, the
+    extents of a CTA and the switch to the radix sort, with ties and signed
+    zeros, against numpy's stable sorts (d = 1) and the oracle (d = 2)."""
+    import torch
+    from tests.test_gpu_parity import order_key
+    rng = np.random.default_rng(n)
+    lo = rng.integers(-9, 9, size=(1, n)).astype(np.float32) * np.float32(0.5)
+    hi = lo + rng.integers(0, 3, size=(1, n)).astype(np.float32)
+    lo[0, : n // 7] = -0.0
+    hi = np.maximum(lo, hi)
+    S = to_dev((lo, hi))
+    ddm.ddm_build(ctx, S[0], S[1])
+    order = torch.empty(n, dtype=torch.int32, device="cuda")
+    ddm.ddm_tree_export(ctx, order)
+    want = np.lexsort((np.arange(n), order_key(hi[0]), order_key(lo[0])))
+    assert np.array_equal(order.cpu().numpy(), want)
+    ddm.ddm_plan(ctx, S[0], S[1])
+    ddm.ddm_plan_order(ctx, order)
+    want = np.argsort(order_key(lo[0]) >> np.uint32(8), kind="stable")
+    assert np.array_equal(order.cpu().numpy(), want)
+    bad = S[1].clone()
+    bad[0, n - 1] = float("nan")
+    with pytest.raises(ddm.DDMError) as e:
+        ddm.ddm_build(ctx, S[0], bad)
+    assert e.value.code == ddm.DDM_ERR_EXTENT
+    arrays = sparse_with_wide(n, n, 2, wide=1, seed=n)
+    K, pu, ps = gpu_match(ctx, arrays)
+    _, ou, os_ = oracle.itm_pairs(*arrays)
+    assert np.array_equal(np.sort(keys(pu, ps)), np.sort(keys(ou, os_)))
