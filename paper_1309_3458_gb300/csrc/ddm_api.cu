@@ -72,7 +72,7 @@ struct ddm_ctx {
   DevBuf e, sid, nodes, tab;
   bool tables_on = true;        // rank tables of the leaves (ddm_set_tiling)
   // plan: sorted updates, per-update counts and offsets
-  DevBuf qe, qid, counts, counts_pos, offsets, pos_offsets, sums, work;
+  DevBuf qe, qid, counts, counts_pos, offsets, pos_offsets, sums;
   // range selection for ddm_write over a sub-range of updates
   DevBuf sel_offs, sel_list;
   // replay records of the count pass
@@ -102,6 +102,15 @@ struct ddm_ctx {
   bool ordered = false;         // the plan holds the plan order's offsets and entries
   uint32_t plan_qpp_log2 = 5;   // of the current plan (smaller for few updates)
   uint32_t tmin = 12;
+
+  // Within one call: the status block (with the ticket words) is zero from
+  // reset_status() to the words' first use.
+  bool work_zeroed[2] = {false, false};
+  // Within one synchronising call: a walking write pass held back, to be run
+  // only if the replay reports incomplete records.
+  bool walk_pending = false;
+  QueryView walk_q{};
+  WriteView walk_w{};
 
   bool built = false;
   bool attached = false;        // tree borrowed from another context (ddm_attach)
@@ -161,6 +170,8 @@ class StreamUse {
     c->capturing = capturing_;
   }
   ~StreamUse() {
+    c_->work_zeroed[0] = c_->work_zeroed[1] = false;
+    c_->walk_pending = false;
     if (!capturing_ && cudaEventRecord(c_->done, s_) == cudaSuccess) {
       c_->done_pending = true;
       c_->last = s_;
@@ -174,6 +185,13 @@ class StreamUse {
   cudaStream_t s_;
   bool capturing_ = false;
 };
+
+// Whether ticket word i is still zero from this call's reset_status().
+bool zeroed_work(ddm_ctx* c, int i) {
+  const bool z = c->work_zeroed[i];
+  c->work_zeroed[i] = false;
+  return z;
+}
 
 int ensure(ddm_ctx* c, DevBuf& b, size_t bytes) {
   if (bytes <= b.cap) return DDM_OK;
@@ -232,7 +250,17 @@ bool set_ok(int d, const float* lo, const float* hi, uint32_t cnt) {
   return true;
 }
 
+int walk_write(ddm_ctx* c, const QueryView& q, const WriteView& w, cudaStream_t s);
+
+// Reads the status block back (and runs the walking write pass held back by
+// this call if the replay asked for it).
 int sync_status(ddm_ctx* c, cudaStream_t s) {
+  DDM_CUDA(cudaMemcpyAsync(c->st_host, c->st_dev, sizeof(Status), cudaMemcpyDeviceToHost, s));
+  DDM_CUDA(cudaStreamSynchronize(s));
+  if (!c->walk_pending) return DDM_OK;
+  c->walk_pending = false;
+  if (!c->st_host->walk) return DDM_OK;
+  DDM_TRY(walk_write(c, c->walk_q, c->walk_w, s));
   DDM_CUDA(cudaMemcpyAsync(c->st_host, c->st_dev, sizeof(Status), cudaMemcpyDeviceToHost, s));
   DDM_CUDA(cudaStreamSynchronize(s));
   return DDM_OK;
@@ -576,7 +604,6 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
   DDM_TRY(ensure(c, c->pos_offsets, sizeof(unsigned long long) * ((size_t)m + 1)));
   // tile sums of a range selection (write_async)
   DDM_TRY(ensure(c, c->sums, sizeof(unsigned long long) * ((size_t)m / kScanTile + 2)));
-  DDM_TRY(ensure(c, c->work, sizeof(uint32_t)));
   DDM_TRY(ensure_queries(c, d, m));
   auto* counts = static_cast<uint32_t*>(c->counts.p);
   auto* counts_pos = static_cast<uint32_t*>(c->counts_pos.p);
@@ -651,7 +678,7 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
     if (!sorted) DDM_TRY(order_updates(c, c->ob[0], d, ulo, uhi, m, bs, aos_buffer(c, c->ob[0], d, m), s));
     if (c->tree.n > 0) {
       DDM_CUDA(launch_count(c->tree, query_view(c), c->bv, flags, counts, counts_pos, c->arena,
-                            static_cast<uint32_t*>(c->work.p), c->st_dev, packet_sms(c), s));
+                            c->st_dev->work, zeroed_work(c, 0), c->st_dev, packet_sms(c), s));
     } else {
       DDM_CUDA(cudaMemsetAsync(counts, 0, sizeof(uint32_t) * m, s));
       DDM_CUDA(cudaMemsetAsync(counts_pos, 0, sizeof(uint32_t) * m, s));
@@ -666,6 +693,23 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
   c->uhi = uhi;
   c->flags = flags;
   c->planned = true;
+  return DDM_OK;
+}
+
+int walk_write(ddm_ctx* c, const QueryView& q, const WriteView& w, cudaStream_t s) {
+  DDM_CUDA(launch_write(c->tree, q, c->bv, c->flags, w, c->arena, c->st_dev->work, c->st_dev,
+                        packet_sms(c), s));
+  return DDM_OK;
+}
+
+// The walking write pass behind a replay: it does nothing when the records
+// are complete, which is the rule, so a call that synchronises holds it back
+// until it has read the status; the others launch it.
+int walk_or_hold(ddm_ctx* c, const QueryView& q, const WriteView& w, bool synced, cudaStream_t s) {
+  if (!synced || !c->arena.max_blocks) return walk_write(c, q, w, s);
+  c->walk_pending = true;
+  c->walk_q = q;
+  c->walk_w = w;
   return DDM_OK;
 }
 
@@ -694,7 +738,7 @@ int ready_ordered(ddm_ctx* c, cudaStream_t s) {
 bool base_fits(const ddm_ctx* c) { return (uint64_t)c->upd_base + c->m <= (1ull << 32); }
 
 int write_async(ddm_ctx* c, uint32_t begin, uint32_t end, ddm_pair* pairs, uint64_t capacity,
-                cudaStream_t s, const uint32_t* qids = nullptr) {
+                bool synced, cudaStream_t s, const uint32_t* qids = nullptr) {
   Phase phase("ddm write");
   if (!qids && !c->swapped && !c->bv.count && !base_fits(c)) return DDM_ERR_ARG;
   if (end > begin && c->tree.n > 0) {
@@ -719,15 +763,15 @@ int write_async(ddm_ctx* c, uint32_t begin, uint32_t end, ddm_pair* pairs, uint6
     w.e_idx = end;
     w.pairs = pairs;
     w.capacity = capacity;
-    auto* work = static_cast<uint32_t*>(c->work.p);
     if (c->arena.max_blocks) {
       const bool full = begin == 0 && end == c->m;
       RecordArena ra = c->arena;
       ra.blk_list = nullptr;
       DDM_CUDA(launch_replay(c->tree, query_view(c), c->bv, ra, w, 0, packets_of(c, c->m), 0, c->m,
-                             !full, begin, end, work, c->st_dev, c->sms, s));
+                             !full, begin, end, c->st_dev->work + 1, zeroed_work(c, 1), c->st_dev,
+                             c->sms, s));
     }
-    DDM_CUDA(launch_write(c->tree, q, c->bv, c->flags, w, c->arena, work, c->st_dev, packet_sms(c), s));
+    DDM_TRY(walk_or_hold(c, q, w, synced, s));
   } else {
     DDM_CUDA(cudaMemsetAsync(&c->st_dev->K, 0, sizeof(unsigned long long), s));
   }
@@ -753,11 +797,10 @@ int write_ordered_async(ddm_ctx* c, uint32_t pb, uint32_t pe, ddm_pair* pairs, u
     w.pairs = pairs;
     w.ids = ids;
     w.capacity = capacity;
-    auto* work = static_cast<uint32_t*>(c->work.p);
     if (c->arena.max_blocks)
       DDM_CUDA(launch_replay(c->tree, q, c->bv, c->arena, w, pb >> c->plan_qpp_log2, packets_of(c, pe), pb, pe, false, 0, 0,
-                             work, c->st_dev, c->sms, s));
-    DDM_CUDA(launch_write(c->tree, q, c->bv, c->flags, w, c->arena, work, c->st_dev, packet_sms(c), s));
+                             c->st_dev->work + 1, zeroed_work(c, 1), c->st_dev, c->sms, s));
+    DDM_TRY(walk_or_hold(c, q, w, true, s));
   } else {
     DDM_CUDA(cudaMemsetAsync(&c->st_dev->K, 0, sizeof(unsigned long long), s));
   }
@@ -818,6 +861,7 @@ int build_and_plan(ddm_ctx* c, int d, const float* slo, const float* shi, uint32
 
 int reset_status(ddm_ctx* c, cudaStream_t s) {
   DDM_CUDA(cudaMemsetAsync(c->st_dev, 0, sizeof(Status), s));
+  c->work_zeroed[0] = c->work_zeroed[1] = true;
   return DDM_OK;
 }
 
@@ -893,7 +937,7 @@ int ddm_destroy(ddm_ctx* c) {
     release(o.sums);
   }
   for (DevBuf* b : {&c->e, &c->sid, &c->nodes, &c->tab, &c->qe, &c->qid, &c->counts,
-                    &c->counts_pos, &c->offsets, &c->pos_offsets, &c->sums, &c->work,
+                    &c->counts_pos, &c->offsets, &c->pos_offsets, &c->sums,
                     &c->sel_offs, &c->sel_list, &c->rec, &c->blk_own, &c->blk_count,
                     &c->pkt_nblk, &c->pkt_off,
                     &c->blk_list, &c->plan_state, &c->order_state, &c->inst_s, &c->inst_u,
@@ -1012,7 +1056,7 @@ int ddm_write(ddm_ctx* c, uint32_t begin, uint32_t end, ddm_pair* pairs, uint64_
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   StreamUse use(c, s);
   DDM_TRY(reset_status(c, s));
-  DDM_TRY(write_async(c, begin, end, pairs, capacity, s));
+  DDM_TRY(write_async(c, begin, end, pairs, capacity, true, s));
   DDM_TRY(sync_status(c, s));
   if (k_out) *k_out = c->st_host->K;
   return status_code(*c->st_host);
@@ -1058,7 +1102,7 @@ int ddm_write_async(ddm_ctx* c, uint32_t begin, uint32_t end, ddm_pair* pairs, u
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   StreamUse use(c, s);
   // keep the plan's error bits; the write sets K (and the capacity bit)
-  DDM_TRY(write_async(c, begin, end, pairs, capacity, s));
+  DDM_TRY(write_async(c, begin, end, pairs, capacity, false, s));
   if (k_dev)
     DDM_CUDA(cudaMemcpyAsync(k_dev, &c->st_dev->K, sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
   if (err_dev)
@@ -1088,7 +1132,7 @@ int ddm_match_moved(ddm_ctx* c, const float* lo, const float* hi, uint32_t k, co
   DDM_TRY(plan_async(c, lo, hi, k, flags & DDM_OPEN, true, false, s));
   const bool was = c->swapped;
   c->swapped = (flags & DDM_SWAP_ROLES) != 0;
-  const int wrc = write_async(c, 0, k, pairs, capacity, s, ids);
+  const int wrc = write_async(c, 0, k, pairs, capacity, true, s, ids);
   c->swapped = was;
   DDM_TRY(wrc);
   DDM_TRY(sync_status(c, s));
@@ -1203,7 +1247,7 @@ static int match_impl(ddm_ctx* c, int d, const float* ulo, const float* uhi, uin
   StreamUse use(c, s);
   DDM_TRY(reset_status(c, s));
   DDM_TRY(build_and_plan(c, d, slo, shi, n, ulo, uhi, m, flags & DDM_OPEN, write, swap, s));
-  if (write) DDM_TRY(write_async(c, begin, end, pairs, capacity, s));
+  if (write) DDM_TRY(write_async(c, begin, end, pairs, capacity, true, s));
   DDM_TRY(sync_status(c, s));
   c->last_tests = c->st_host->tests;
   if (k_out) *k_out = c->st_host->K;
@@ -1254,7 +1298,9 @@ static int batch_impl(ddm_ctx* c, int d, uint32_t count, const float* ulo, const
   BatchSet bs_u{uoff, count, static_cast<uint32_t*>(c->inst_u.p)};
   const BatchView bv{count, uoff, soff, static_cast<const uint32_t*>(c->inst_u.p)};
   DDM_TRY(build_and_plan(c, d, slo, shi, n, ulo, uhi, m, flags, true, false, s, &bs_s, &bs_u, &bv));
-  DDM_TRY(write_async(c, 0, m, pairs, capacity, s));
+  // a k_dev or pair_off copy is enqueued behind the write: only a plain
+  // synchronising call can hold the walking pass back
+  DDM_TRY(write_async(c, 0, m, pairs, capacity, sync && !k_dev && !err_dev, s));
   if (pair_off && m > 0)
     DDM_CUDA(launch_gather_offsets(static_cast<const unsigned long long*>(c->offsets.p), m, uoff,
                                    count, reinterpret_cast<unsigned long long*>(pair_off), s));

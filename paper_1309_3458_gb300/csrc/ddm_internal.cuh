@@ -26,9 +26,10 @@ constexpr unsigned kErrChecked = 8u;  // checked build: an index failed its boun
 struct Status {
   unsigned long long K;    // pairs counted (plan) or written (write)
   unsigned int err;        // kErr* bits
-  unsigned int pad;
+  unsigned int walk;       // the replay found the records incomplete
   unsigned long long aux;  // call-specific (chunk end, ...)
   unsigned long long tests;  // count pass: (query, leaf) tests, 32 subscriptions each
+  unsigned int work[2];    // tickets of the packet kernels and of the replay
 };
 
 __device__ inline void note_out_of_bounds(Status* st) {
@@ -320,10 +321,11 @@ __device__ __forceinline__ bool records_complete(const RecordArena& ra) {
 // into `ra` when ra.max_blocks > 0.  With bv.count > 0 every query only
 // matches its own instance's subscriptions and pairs carry instance-local ids.
 // `sms` sizes the persistent grids: pass SMs x CTAs-per-SM / 8 to change the
-// default of 8 CTAs of 256 threads per SM (tuning knob).
+// default of 8 CTAs of 256 threads per SM (tuning knob).  `zeroed`: *work is
+// zero already.
 cudaError_t launch_count(const TreeView& t, const QueryView& q, const BatchView& bv,
                          uint32_t flags, uint32_t* counts, uint32_t* counts_pos,
-                         const RecordArena& ra, uint32_t* work, Status* st, int sms,
+                         const RecordArena& ra, uint32_t* work, bool zeroed, Status* st, int sms,
                          cudaStream_t s);
 // Walking write pass; it does nothing when `ra` holds complete records (the
 // replay kernel, launched next to it, writes the pairs then).
@@ -335,11 +337,11 @@ cudaError_t launch_write(const TreeView& t, const QueryView& q, const BatchView&
 cudaError_t launch_block_list(const RecordArena& ra, int sms, cudaStream_t s);
 // Write pass from records: positions [pb, pe) of the plan, in packets [p0,
 // p1) (without a list: all packets), and (when id_filter) only updates with
-// ids in [idb, ide).  Does nothing unless `ra` holds complete records.
+// ids in [idb, ide).  Only sets st->walk unless `ra` holds complete records.
 cudaError_t launch_replay(const TreeView& t, const QueryView& q, const BatchView& bv,
                           const RecordArena& ra, const WriteView& w, uint32_t p0, uint32_t p1,
                           uint32_t pb, uint32_t pe, bool id_filter, uint32_t idb, uint32_t ide,
-                          uint32_t* work, Status* st, int sms, cudaStream_t s);
+                          uint32_t* work, bool zeroed, Status* st, int sms, cudaStream_t s);
 // pair_off[i] = offsets[min(upd_off[i], m)] for i <= count.
 cudaError_t launch_gather_offsets(const unsigned long long* offsets, uint32_t m,
                                   const unsigned long long* upd_off, uint32_t count,

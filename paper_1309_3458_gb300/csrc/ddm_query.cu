@@ -999,7 +999,10 @@ k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uin
          uint32_t p1, uint32_t pb, uint32_t pe, uint32_t idb, uint32_t ide,
          uint32_t* __restrict__ work, Status* __restrict__ st) {
   __shared__ ReplaySmem<WIDE, OUT> sm;
-  if (!records_complete(ra)) return;  // the walking write pass handles this range
+  if (!records_complete(ra)) {  // the walking write pass handles this range
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->walk = 1u;
+    return;
+  }
   const unsigned long long base0 = w.start[w.b_idx];
   const unsigned long long need = w.start[w.e_idx] - base0;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1044,8 +1047,8 @@ void dispatch_packets(int d, bool open, uint32_t blocks, cudaStream_t s, const T
 template <bool WRITE>
 cudaError_t launch_packets(const TreeView& t, const QueryView& q, const BatchView& bv,
                            uint32_t flags, uint32_t* counts, uint32_t* counts_pos,
-                           const RecordArena& ra, const WriteView& w, uint32_t* work, Status* st,
-                           int sms, cudaStream_t s) {
+                           const RecordArena& ra, const WriteView& w, uint32_t* work, bool zeroed,
+                           Status* st, int sms, cudaStream_t s) {
   if (q.nq == 0) return cudaSuccess;
   const bool open = (flags & DDM_OPEN) != 0;
   const uint32_t packets = (q.nq + (1u << q.qpp_log2) - 1u) >> q.qpp_log2;
@@ -1060,7 +1063,7 @@ cudaError_t launch_packets(const TreeView& t, const QueryView& q, const BatchVie
   // (and without the counter to clear).
   if (blocks <= (uint32_t)sms * DDM_PACKET_MIN_BLOCKS && packets <= blocks * kWarps) {
     work = nullptr;
-  } else {
+  } else if (!zeroed) {
     cudaError_t e = cudaMemsetAsync(work, 0, sizeof(uint32_t), s);
     if (e) return e;
   }
@@ -1111,16 +1114,16 @@ __global__ void k_gather_offsets(const unsigned long long* __restrict__ offsets,
 
 cudaError_t launch_count(const TreeView& t, const QueryView& q, const BatchView& bv,
                          uint32_t flags, uint32_t* counts, uint32_t* counts_pos,
-                         const RecordArena& ra, uint32_t* work, Status* st, int sms,
+                         const RecordArena& ra, uint32_t* work, bool zeroed, Status* st, int sms,
                          cudaStream_t s) {
   WriteView w{};
-  return launch_packets<false>(t, q, bv, flags, counts, counts_pos, ra, w, work, st, sms, s);
+  return launch_packets<false>(t, q, bv, flags, counts, counts_pos, ra, w, work, zeroed, st, sms, s);
 }
 
 cudaError_t launch_write(const TreeView& t, const QueryView& q, const BatchView& bv,
                          uint32_t flags, const WriteView& w, const RecordArena& ra,
                          uint32_t* work, Status* st, int sms, cudaStream_t s) {
-  return launch_packets<true>(t, q, bv, flags, nullptr, nullptr, ra, w, work, st, sms, s);
+  return launch_packets<true>(t, q, bv, flags, nullptr, nullptr, ra, w, work, false, st, sms, s);
 }
 
 cudaError_t launch_block_list(const RecordArena& ra, int sms, cudaStream_t s) {
@@ -1134,11 +1137,13 @@ cudaError_t launch_block_list(const RecordArena& ra, int sms, cudaStream_t s) {
 cudaError_t launch_replay(const TreeView& t, const QueryView& q, const BatchView& bv,
                           const RecordArena& ra, const WriteView& w, uint32_t p0, uint32_t p1,
                           uint32_t pb, uint32_t pe, bool id_filter, uint32_t idb, uint32_t ide,
-                          uint32_t* work, Status* st, int sms, cudaStream_t s) {
+                          uint32_t* work, bool zeroed, Status* st, int sms, cudaStream_t s) {
   if (p1 <= p0) return cudaSuccess;
   if ((w.ids || w.swap) && (id_filter || bv.count)) return cudaErrorInvalidValue;  // see dispatch_replay
-  cudaError_t e = cudaMemsetAsync(work, 0, sizeof(uint32_t), s);
-  if (e) return e;
+  if (!zeroed) {
+    cudaError_t e = cudaMemsetAsync(work, 0, sizeof(uint32_t), s);
+    if (e) return e;
+  }
   // Cursors fit 32 bits when the range's pairs do; the capacity bounds them.
   const bool wide = w.capacity > 0xffffffffull;
   if (id_filter) {
