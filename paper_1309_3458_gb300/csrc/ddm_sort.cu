@@ -9,7 +9,7 @@
 //   * up to one resident tile per SM: one cooperative launch runs every pass,
 //     the tiles exchanging digit counts across bounded grid barriers
 //     (k_sort_grid);
-//   * beyond (and under stream capture): onesweep, after Adinets & Merrill
+//   * beyond: onesweep, after Adinets & Merrill
 //     ("Onesweep", 2022): one histogram pass over the keys computes all eight
 //     8-bit digit histograms at once, a tiny kernel scans them into digit
 //     bases, and each digit pass is ONE kernel: a CTA takes the next tile
@@ -18,8 +18,7 @@
 //     digit bit) and per-warp counters, publishes its per-digit counts,
 //     resolves its global per-digit offsets by decoupled look-back over
 //     earlier tiles, and scatters through shared memory so that global
-//     stores come out as runs of equal digits.  Under stream capture, sets of
-//     up to 8,192 keys take one CTA instead (k_sort_small).
+//     stores come out as runs of equal digits.
 // Every wait is bounded: after kSpinLimit polls a CTA records kErrTimeout and
 // carries on (look-back) or returns (grid barrier), so the kernels always
 // terminate.
@@ -273,7 +272,6 @@ k_onesweep(const unsigned long long* __restrict__ in_keys, const uint32_t* __res
 // count (threads < 256, digit = thread) the tile's keys with that digit.
 constexpr int kSmallThreads = 512;
 constexpr int kSmallWarps = kSmallThreads / 32;
-constexpr uint32_t kSmallTile = kSmallThreads * kItems;  // 8192
 
 struct RankSmem {
   uint32_t whist[kSmallWarps][kRadix];
@@ -329,64 +327,9 @@ __device__ __forceinline__ uint32_t rank_tile(RankSmem& sm, const unsigned long 
   return count;
 }
 
-// Small arrays (n <= kSmallTile): one CTA of 512 threads runs every digit
-// pass in shared memory, with the tile's own digit offsets in place of the
-// look-back, so the whole sort is one launch.
-struct SmallSortSmem {
-  RankSmem r;
-  unsigned long long keys[kSmallTile];
-  uint32_t vals[kSmallTile];
-};
-
-__global__ void __launch_bounds__(kSmallThreads, 1)
-k_sort_small(const unsigned long long* __restrict__ in_keys, const uint32_t* __restrict__ in_vals,
-             unsigned long long* __restrict__ out_keys, uint32_t* __restrict__ out_vals,
-             uint32_t n, int passes) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  SmallSortSmem& sm = *reinterpret_cast<SmallSortSmem*>(smem_raw);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  unsigned long long key[kItems];
-  uint32_t val[kItems], dig[kItems], rank[kItems];
-#pragma unroll
-  for (int i = 0; i < kItems; ++i) {
-    const uint32_t local = warp * (kItems * 32) + i * 32 + lane;
-    key[i] = local < n ? in_keys[local] : 0ull;
-    val[i] = local < n ? in_vals[local] : 0u;
-  }
-  for (int p = 0; p < passes; ++p) {
-    rank_tile<kItems>(sm.r, key, dig, rank, n, p * kRadixBits);
-#pragma unroll
-    for (int i = 0; i < kItems; ++i) {
-      if (dig[i] < kRadix) {
-        const uint32_t slot = sm.r.lstart[dig[i]] + sm.r.whist[warp][dig[i]] + rank[i];
-        sm.keys[slot] = key[i];
-        sm.vals[slot] = val[i];
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < kItems; ++i) {
-      const uint32_t local = warp * (kItems * 32) + i * 32 + lane;
-      if (local < n) {
-        key[i] = sm.keys[local];
-        val[i] = sm.vals[local];
-      }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < kItems; ++i) {
-    const uint32_t local = warp * (kItems * 32) + i * 32 + lane;
-    if (local < n) {
-      out_keys[local] = key[i];
-      out_vals[local] = val[i];
-    }
-  }
-}
-
 // Mid-size arrays (up to kGridMaxTiles tiles of 512 * ITEMS keys, all CTAs
 // resident): one cooperative launch runs every pass.  CTA g holds tile g in
-// registers and ranks it as k_sort_small does; the tiles then exchange their
+// registers and ranks it (rank_tile); the tiles then exchange their
 // digit counts through global memory across a grid barrier, each CTA takes
 // its digit offsets from the counts (no look-back chain), scatters, and a
 // second barrier ends the pass.  Tiles come in groups of kGridGroup: a tile
@@ -829,45 +772,30 @@ cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf, 
   if (n <= 1 || passes <= 0) return cudaSuccess;
   if (passes > kPasses) passes = kPasses;
   cudaError_t e;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if ((e = cudaStreamIsCapturing(s, &cap))) return e;
   // Up to 16 tiles of 2,048 keys: one cluster, keys kept on chip; else one
   // cooperative launch when every tile can be resident at once, with the
   // smallest tile that allows it.  Measured (8 passes, one GB300): 5,000
   // keys 33 us in a cluster, 53 cooperative, 51 in one CTA; 25,000 keys 41,
   // 57 (2,048-key tiles) and 100 (8,192-key tiles); 250,000 keys 76
-  // cooperative.  Not under stream capture: the single-CTA or multi-launch
-  // form is recorded instead.
-  if (cap == cudaStreamCaptureStatusNone) {
-    bool done = false;
-    if ((e = try_sort_cluster<4>(sc, n, passes, s, &done)) || done) {
-      *out_buf = passes & 1;
-      return e;
-    }
-    if ((e = try_sort_grid<4>(sc, n, passes, st, sms, s, &done)) || done) {
-      *out_buf = passes & 1;
-      return e;
-    }
-    if ((e = try_sort_grid<8>(sc, n, passes, st, sms, s, &done)) || done) {
-      *out_buf = passes & 1;
-      return e;
-    }
-    if ((e = try_sort_grid<16>(sc, n, passes, st, sms, s, &done)) || done) {
-      *out_buf = passes & 1;
-      return e;
-    }
+  // cooperative.  Under stream capture too (the launches become graph nodes
+  // with the same attributes): 256 batched instances in a graph took 187 us
+  // with the multi-launch form recorded instead, 149 with these.
+  bool done = false;
+  if ((e = try_sort_cluster<4>(sc, n, passes, s, &done)) || done) {
+    *out_buf = passes & 1;
+    return e;
   }
-  if (n <= kSmallTile) {  // one CTA, every pass in shared memory
-    const size_t smem = sizeof(SmallSortSmem);
-    if ((e = cudaFuncSetAttribute(k_sort_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem)))
-      return e;
-    const int out = passes & 1;
-    k_sort_small<<<1, kSmallThreads, smem, s>>>(sc.keys[0], sc.vals[0], sc.keys[out], sc.vals[out],
-                                                n, passes);
-    note_launches(1);
-    *out_buf = out;
-    return cudaGetLastError();
+  if ((e = try_sort_grid<4>(sc, n, passes, st, sms, s, &done)) || done) {
+    *out_buf = passes & 1;
+    return e;
+  }
+  if ((e = try_sort_grid<8>(sc, n, passes, st, sms, s, &done)) || done) {
+    *out_buf = passes & 1;
+    return e;
+  }
+  if ((e = try_sort_grid<16>(sc, n, passes, st, sms, s, &done)) || done) {
+    *out_buf = passes & 1;
+    return e;
   }
   const uint32_t tiles = (n + kSortTile - 1) / kSortTile;
   if ((e = cudaMemsetAsync(sc.hist, 0, sizeof(uint32_t) * kPasses * kRadix, s))) return e;
