@@ -302,18 +302,55 @@ int sort_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, int passes, int* cur, cuda
   return DDM_OK;
 }
 
-// Sort a set into the spatial order used by the tree: dimension-0 key first,
-// then, for each further dimension with a group size, a stable re-sort by
-// that dimension's lower bound inside aligned groups.  Validates the set on
-// the way.  Returns the buffer pair whose vals hold the order.
-// Bytes needed to hold values 0..v.
-int key_bytes(uint64_t v) {
+// A set is sorted into the spatial order used by the tree: dimension-0 key
+// first, then, for each further dimension with a group size, a stable re-sort
+// by that dimension's lower bound inside aligned groups.  The order_set
+// functions validate the set on the way and return the buffer pair whose vals
+// hold the order.
+
+// Bits needed to hold values 0..v.
+int bits_of(uint64_t v) {
   int b = 0;
   while (v) {
     ++b;
-    v >>= 8;
+    v >>= 1;
   }
   return b;
+}
+// Bits of a set's ids in packed words.
+int id_bits_of(uint32_t cnt) { return std::max(bits_of(cnt - 1u), 1); }
+
+// Packed sort of a set (launch_sort_packed): the ids end up in vals[0], so
+// *cur becomes 0.  A source's k32 lies in vals[1].
+int packed_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, const uint32_t* hi, bool source, int key_bits,
+                int id_bits, int* cur, cudaStream_t s) {
+  SortScratch sc;
+  for (int b = 0; b < 2; ++b) {
+    sc.keys[b] = static_cast<unsigned long long*>(o.keys[b].p);
+    sc.vals[b] = static_cast<uint32_t*>(o.vals[b].p);
+  }
+  sc.hist = static_cast<uint32_t*>(o.hist.p);
+  sc.lookback = static_cast<uint32_t*>(o.lookback.p);
+  sc.counters = static_cast<uint32_t*>(o.counters.p);
+  const SortSource src{source ? sc.vals[1] : nullptr, hi, 24, id_bits};
+  DDM_CUDA(launch_sort_packed(sc, src, cnt, key_bits, c->st_dev, c->sms, s));
+  *cur = 0;
+  return DDM_OK;
+}
+
+// Re-sort of the ids in vals[*cur] by (group, locality key) over the whole
+// set, `groups` numbered groups: the keys are written by `rekey`(keys[0],
+// id_bits), packed with the ids if they fit one word.
+template <typename Rekey>
+int resort_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, uint64_t groups, int* cur, Rekey rekey,
+                cudaStream_t s) {
+  const int key_bits = 24 + bits_of(groups - 1u), id_bits = id_bits_of(cnt);
+  if (key_bits + id_bits <= 64) {
+    DDM_CUDA(rekey(static_cast<unsigned long long*>(o.keys[0].p), id_bits));
+    return packed_pass(c, o, cnt, nullptr, false, key_bits, id_bits, cur, s);
+  }
+  DDM_CUDA(rekey(static_cast<unsigned long long*>(o.keys[*cur].p), 0));
+  return sort_pass(c, o, cnt, (key_bits + 7) / 8, cur, s);
 }
 
 // Re-sort of the ids in buffer pair `cur` inside the plan's groups (in place).
@@ -356,10 +393,17 @@ int order_set_batch(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const floa
   *cur = 0;
   DDM_TRY(ensure_batch(c, o, cnt, bs.count));
   DDM_CUDA(launch_fill_inst(bs.off, bs.count, cnt, bs.inst, c->sms, s));
+  const int inst_bits = bits_of(bs.count ? bs.count - 1u : 0u), id_bits = id_bits_of(cnt);
+  const bool packed = inst_bits + 24 + id_bits <= 64;
   DDM_CUDA(launch_validate_batch(d, lo, hi, cnt, bs.inst,
                                  static_cast<unsigned long long*>(o.keys[0].p),
-                                 static_cast<uint32_t*>(o.vals[0].p), aos, c->st_dev, c->sms, s));
-  DDM_TRY(sort_pass(c, o, cnt, 3 + key_bytes(bs.count ? bs.count - 1 : 0), cur, s));
+                                 static_cast<uint32_t*>(o.vals[0].p),
+                                 packed ? static_cast<uint32_t*>(o.vals[1].p) : nullptr, aos,
+                                 c->st_dev, c->sms, s));
+  if (packed)
+    DDM_TRY(packed_pass(c, o, cnt, inst_bits ? bs.inst : nullptr, true, 24 + inst_bits, id_bits, cur, s));
+  else
+    DDM_TRY(sort_pass(c, o, cnt, (24 + inst_bits + 7) / 8, cur, s));
   // The re-sorts stay inside an instance's groups; the sizes are known on the
   // device only, so the chunks are planned there.
   auto* gl = static_cast<int*>(o.bglog2.p);
@@ -410,10 +454,10 @@ int order_set_classes(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const fl
     DDM_CUDA(launch_rank_sort(kRankClass, d, lo, hi, cnt, static_cast<uint32_t*>(o.vals[0].p), hist,
                               aos, nullptr, nullptr, c->st_dev, s));
   } else {
-    DDM_CUDA(launch_validate_class(d, lo, hi, cnt, static_cast<unsigned long long*>(o.keys[0].p),
-                                   static_cast<uint32_t*>(o.vals[0].p), hist, aos, c->st_dev,
-                                   c->sms, s));
-    DDM_TRY(sort_pass(c, o, cnt, 4, cur, s));  // (class, 24-bit lower bound)
+    DDM_CUDA(launch_validate_class(d, lo, hi, cnt, static_cast<uint32_t*>(o.vals[1].p), hist, aos,
+                                   c->st_dev, c->sms, s));
+    // (class, 24-bit lower bound)
+    DDM_TRY(packed_pass(c, o, cnt, nullptr, true, 32, id_bits_of(cnt), cur, s));
   }
   ClassPlan plan{off, static_cast<int*>(o.bglog2.p), static_cast<unsigned long long*>(o.bgbase.p), {}};
   int tile_log2[DDM_MAX_DIMS] = {};
@@ -438,11 +482,14 @@ int order_set_classes(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const fl
     if (k == 1) DDM_CUDA(launch_fill_inst(off, kClasses, cnt, inst, c->sms, s));
     DDM_CUDA(launch_batch_groups(off, kClasses, gl, ng, s));
     DDM_CUDA(launch_scan(ng, kClasses, gb, sums, nullptr, s));
-    DDM_CUDA(launch_rekey_batch(static_cast<const uint32_t*>(o.vals[*cur].p), lo + (size_t)k * cnt,
-                                cnt, inst, off, gl, gb,
-                                static_cast<unsigned long long*>(o.keys[*cur].p), c->sms, s));
     // groups: at most one per class without re-sort plus cnt / 64
-    DDM_TRY(sort_pass(c, o, cnt, 3 + key_bytes((uint64_t)kClasses + cnt / 64), cur, s));
+    DDM_TRY(resort_pass(
+        c, o, cnt, (uint64_t)kClasses + cnt / 64 + 1, cur,
+        [&](unsigned long long* keys, int id_bits) {
+          return launch_rekey_batch(static_cast<const uint32_t*>(o.vals[*cur].p), lo + (size_t)k * cnt,
+                                    cnt, inst, off, gl, gb, keys, id_bits, c->sms, s);
+        },
+        s));
   }
   return DDM_OK;
 }
@@ -461,10 +508,15 @@ int order_set(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const float* hi,
                               *gathered ? static_cast<float2*>(c->qe.p) : nullptr,
                               *gathered ? static_cast<uint32_t*>(c->qid.p) : nullptr, c->st_dev, s));
   } else {
-    DDM_CUDA(launch_validate(d, lo, hi, cnt, static_cast<unsigned long long*>(o.keys[0].p),
-                             static_cast<uint32_t*>(o.vals[0].p), tree ? 1 : 2, aos, c->st_dev,
+    DDM_CUDA(launch_validate(d, lo, hi, cnt,
+                             tree ? static_cast<unsigned long long*>(o.keys[0].p) : nullptr,
+                             static_cast<uint32_t*>(o.vals[0].p),
+                             tree ? nullptr : static_cast<uint32_t*>(o.vals[1].p), aos, c->st_dev,
                              c->sms, s));
-    DDM_TRY(sort_pass(c, o, cnt, tree ? 8 : 3, cur, s));
+    if (tree)
+      DDM_TRY(sort_pass(c, o, cnt, 8, cur, s));
+    else
+      DDM_TRY(packed_pass(c, o, cnt, nullptr, true, 24, id_bits_of(cnt), cur, s));
   }
   int glog2[DDM_MAX_DIMS];
   str_groups(cnt, d, glog2, c->str_shift);
@@ -475,11 +527,13 @@ int order_set(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const float* hi,
                        std::max(glog2[k], kSegTileLog2), *cur, s));
       continue;
     }
-    DDM_CUDA(launch_rekey(static_cast<const uint32_t*>(o.vals[*cur].p), lo + (size_t)k * cnt, cnt,
-                          glog2[k], static_cast<unsigned long long*>(o.keys[*cur].p), c->sms, s));
-    int gbits = 0;
-    while (gbits < 32 && (((uint64_t)(cnt - 1) >> glog2[k]) >> gbits) != 0) ++gbits;
-    DDM_TRY(sort_pass(c, o, cnt, 3 + (gbits + 7) / 8, cur, s));
+    DDM_TRY(resort_pass(
+        c, o, cnt, ((uint64_t)(cnt - 1u) >> glog2[k]) + 1u, cur,
+        [&](unsigned long long* keys, int id_bits) {
+          return launch_rekey(static_cast<const uint32_t*>(o.vals[*cur].p), lo + (size_t)k * cnt, cnt,
+                              glog2[k], keys, id_bits, c->sms, s);
+        },
+        s));
   }
   return DDM_OK;
 }
@@ -1351,7 +1405,7 @@ int ddm_refit(ddm_ctx* c, const float* sub_lo, const float* sub_hi, void* stream
   Phase phase("ddm refit");
   if (c->tree.n > 0) {
     float2* aos = aos_buffer(c, c->ob[0], c->tree.d, c->tree.n);
-    DDM_CUDA(launch_validate(c->tree.d, sub_lo, sub_hi, c->tree.n, nullptr, nullptr, 0, aos,
+    DDM_CUDA(launch_validate(c->tree.d, sub_lo, sub_hi, c->tree.n, nullptr, nullptr, nullptr, aos,
                              c->st_dev, c->sms, s));
     // Same order, new coordinates: gather through the tree's own id column and
     // recompute every node's per-dimension (minlower, maxupper).

@@ -146,32 +146,34 @@ __host__ __device__ inline uint32_t float_key(float f) {
 void note_launches(unsigned count);
 
 // ---- ddm_layout.cu --------------------------------------------------------
-// Validate a set (lo <= hi, no NaN in every dimension) and, when keys is
-// not null, emit the sort key with the identity payload: key_mode 1 gives
-// (key(lo0) << 32 | key(hi0)) (tree order), key_mode 2 gives key(lo0).
+// Validate a set (lo <= hi, no NaN in every dimension) and emit the sort key,
+// if asked for: keys and vals (id) for the d = 1 tree's order, (key(lo0) <<
+// 32 | key(hi0)); k32 for a locality order, the top 24 bits of key(lo0).
 // aos (optional, cnt * d float2): an interleaved copy of the coordinates,
 // aos[i*d + k] = (lo_k, hi_k) of extent i, written while validating, so that
 // the gathers by id read one contiguous record per extent instead of 2d
 // scattered words.
 cudaError_t launch_validate(int d, const float* lo, const float* hi, uint32_t cnt,
-                            unsigned long long* keys, uint32_t* vals, int key_mode, float2* aos,
+                            unsigned long long* keys, uint32_t* vals, uint32_t* k32, float2* aos,
                             Status* st, int sms, cudaStream_t s);
-// keys[i] = (i >> glog2) << 32 | key(lo_k[vals[i]]): re-sort inside groups.
+// keys[i] = (i >> glog2) << 24 | the top 24 bits of key(lo_k[vals[i]]): re-sort
+// inside groups; with id_bits > 0 the packed word, above the id vals[i].
 cudaError_t launch_rekey(const uint32_t* vals, const float* lo_k, uint32_t cnt, int glog2,
-                         unsigned long long* keys, int sms, cudaStream_t s);
+                         unsigned long long* keys, int id_bits, int sms, cudaStream_t s);
 // Batched sets: inst[i] = instance owning position i (off has count+1 entries).
 // Validation and class-major tree keys for d >= 2; hist[256] (zeroed by the
 // caller) receives the number of extents of each size class.
 cudaError_t launch_validate_class(int d, const float* lo, const float* hi, uint32_t cnt,
-                                  unsigned long long* keys, uint32_t* vals, uint32_t* hist,
-                                  float2* aos, Status* st, int sms, cudaStream_t s);
+                                  uint32_t* k32, uint32_t* hist, float2* aos, Status* st, int sms,
+                                  cudaStream_t s);
 // inst[i] = the b with off[b] <= i < off[b+1], for 0 <= i < total.
 cudaError_t launch_fill_inst(const unsigned long long* off, uint32_t count, uint32_t total,
                              uint32_t* inst, int sms, cudaStream_t s);
-// Batched validation + keys: keys[i] = inst[i] << 32 | key(lo0[i]).
+// Batched validation + keys: the top 24 bits of key(lo0[i]) in k32 or, below
+// inst[i], in keys (with vals = ids).
 cudaError_t launch_validate_batch(int d, const float* lo, const float* hi, uint32_t cnt,
                                   const uint32_t* inst, unsigned long long* keys, uint32_t* vals,
-                                  float2* aos, Status* st, int sms, cudaStream_t s);
+                                  uint32_t* k32, float2* aos, Status* st, int sms, cudaStream_t s);
 // Groups of each instance (or class) for a re-sort over the whole set, from
 // its group exponent (0: one group).  glog2/ngroups: [count] each.
 cudaError_t launch_batch_groups(const unsigned long long* off, uint32_t count, const int* glog2,
@@ -180,7 +182,7 @@ cudaError_t launch_batch_groups(const unsigned long long* off, uint32_t count, c
 cudaError_t launch_rekey_batch(const uint32_t* vals, const float* lo_k, uint32_t cnt,
                                const uint32_t* inst, const unsigned long long* off,
                                const int* glog2, const unsigned long long* gbase,
-                               unsigned long long* keys, int sms, cudaStream_t s);
+                               unsigned long long* keys, int id_bits, int sms, cudaStream_t s);
 // qe[k][i] = (lo_k, hi_k)[vals[i]], qid[i] = vals[i].
 cudaError_t launch_gather(int d, const uint32_t* vals, const float* lo, const float* hi,
                           const float2* aos, uint32_t cnt, float2* qe, uint32_t* qid, int sms,
@@ -205,6 +207,18 @@ size_t sort_lookback_words(uint32_t n);
 cudaError_t launch_debug_wait(const uint32_t* word, uint32_t limit, Status* st, cudaStream_t s);
 cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf, Status* st,
                           int sms, cudaStream_t s);
+// The same for keys that fit one 64-bit word together with the id: words key
+// << id_bits | id, sorted by key_bits bits above id_bits; the ids come out in
+// vals[0].  With a source the words are built from it (its arrays may not
+// overlap keys[] or vals[0]), else they are in keys[0].
+struct SortSource {
+  const uint32_t* k32;  // [n] low part of the key, or null
+  const uint32_t* hi;   // optional [n]: the part above k32_bits
+  int k32_bits;
+  int id_bits;
+};
+cudaError_t launch_sort_packed(SortScratch sc, const SortSource& src, uint32_t n, int key_bits,
+                               Status* st, int sms, cudaStream_t s);
 
 // ---- ddm_ranksort.cu ------------------------------------------------------
 // Validation, first order (vals) and optional interleaved copy of a small set

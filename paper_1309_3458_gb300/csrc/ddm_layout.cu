@@ -35,8 +35,8 @@ constexpr int kLocalityDrop = 32 - kLocalityBits;
 
 __global__ void __launch_bounds__(kThreads)
 k_validate(int d, const float* __restrict__ lo, const float* __restrict__ hi, uint32_t cnt,
-           unsigned long long* __restrict__ keys, uint32_t* __restrict__ vals, int key_mode,
-           float2* __restrict__ aos, Status* __restrict__ st) {
+           unsigned long long* __restrict__ keys, uint32_t* __restrict__ vals,
+           uint32_t* __restrict__ k32, float2* __restrict__ aos, Status* __restrict__ st) {
   bool bad = false;
   const uint32_t stride = gridDim.x * blockDim.x;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += stride) {
@@ -49,21 +49,24 @@ k_validate(int d, const float* __restrict__ lo, const float* __restrict__ hi, ui
     }
     if (keys) {
       const float a = __ldg(lo + i), b = __ldg(hi + i);
-      keys[i] = key_mode == 1 ? ((unsigned long long)float_key(a) << 32) | float_key(b)
-                              : (unsigned long long)(float_key(a) >> kLocalityDrop);
+      keys[i] = ((unsigned long long)float_key(a) << 32) | float_key(b);
       vals[i] = i;
     }
+    if (k32) k32[i] = float_key(__ldg(lo + i)) >> kLocalityDrop;
   }
   if (__ballot_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&st->err, kErrExtent);
 }
 
 __global__ void __launch_bounds__(kThreads)
 k_rekey(const uint32_t* __restrict__ vals, const float* __restrict__ lo_k, uint32_t cnt, int glog2,
-        unsigned long long* __restrict__ keys) {
+        unsigned long long* __restrict__ keys, int id_bits) {
   const uint32_t stride = gridDim.x * blockDim.x;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += stride)
-    keys[i] = ((unsigned long long)(i >> glog2) << kLocalityBits) |
-              (float_key(__ldg(lo_k + vals[i])) >> kLocalityDrop);
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += stride) {
+    const uint32_t id = vals[i];
+    const unsigned long long k = ((unsigned long long)(i >> glog2) << kLocalityBits) |
+                                 (float_key(__ldg(lo_k + id)) >> kLocalityDrop);
+    keys[i] = id_bits ? (k << id_bits) | id : k;
+  }
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -90,8 +93,8 @@ k_gather(int d, const uint32_t* __restrict__ vals, const float* __restrict__ lo,
 // the coordinates whatever the order).  hist[class] counts the extents.
 __global__ void __launch_bounds__(kThreads)
 k_validate_class(int d, const float* __restrict__ lo, const float* __restrict__ hi, uint32_t cnt,
-                 unsigned long long* __restrict__ keys, uint32_t* __restrict__ vals,
-                 uint32_t* __restrict__ hist, float2* __restrict__ aos, Status* __restrict__ st) {
+                 uint32_t* __restrict__ k32, uint32_t* __restrict__ hist, float2* __restrict__ aos,
+                 Status* __restrict__ st) {
   __shared__ uint32_t s_h[256];
   for (int i = threadIdx.x; i < 256; i += blockDim.x) s_h[i] = 0u;
   __syncthreads();
@@ -107,9 +110,7 @@ k_validate_class(int d, const float* __restrict__ lo, const float* __restrict__ 
       if (aos) aos[(size_t)i * d + k] = make_float2(a, b);
     }
     const uint32_t cls = (__float_as_uint(side) >> 23) & 0xffu;
-    keys[i] = ((unsigned long long)cls << kLocalityBits) |
-              (float_key(__ldg(lo + i)) >> kLocalityDrop);
-    vals[i] = i;
+    k32[i] = (cls << kLocalityBits) | (float_key(__ldg(lo + i)) >> kLocalityDrop);
     atomicAdd(&s_h[cls], 1u);
   }
   if (__ballot_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&st->err, kErrExtent);
@@ -138,7 +139,8 @@ k_fill_inst(const unsigned long long* __restrict__ off, uint32_t count, uint32_t
 __global__ void __launch_bounds__(kThreads)
 k_validate_batch(int d, const float* __restrict__ lo, const float* __restrict__ hi, uint32_t cnt,
                  const uint32_t* __restrict__ inst, unsigned long long* __restrict__ keys,
-                 uint32_t* __restrict__ vals, float2* __restrict__ aos, Status* __restrict__ st) {
+                 uint32_t* __restrict__ vals, uint32_t* __restrict__ k32, float2* __restrict__ aos,
+                 Status* __restrict__ st) {
   bool bad = false;
   const uint32_t stride = gridDim.x * blockDim.x;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += stride) {
@@ -148,9 +150,13 @@ k_validate_batch(int d, const float* __restrict__ lo, const float* __restrict__ 
       bad |= !(a <= b);
       if (aos) aos[(size_t)i * d + k] = make_float2(a, b);
     }
-    keys[i] = ((unsigned long long)inst[i] << kLocalityBits) |
-              (float_key(__ldg(lo + i)) >> kLocalityDrop);
-    vals[i] = i;
+    const uint32_t key = float_key(__ldg(lo + i)) >> kLocalityDrop;
+    if (k32) {
+      k32[i] = key;
+    } else {
+      keys[i] = ((unsigned long long)inst[i] << kLocalityBits) | key;
+      vals[i] = i;
+    }
   }
   if (__ballot_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&st->err, kErrExtent);
 }
@@ -171,18 +177,21 @@ __global__ void __launch_bounds__(kThreads)
 k_rekey_batch(const uint32_t* __restrict__ vals, const float* __restrict__ lo_k, uint32_t cnt,
               const uint32_t* __restrict__ inst, const unsigned long long* __restrict__ off,
               const int* __restrict__ glog2, const unsigned long long* __restrict__ gbase,
-              unsigned long long* __restrict__ keys) {
+              unsigned long long* __restrict__ keys, int id_bits) {
   const uint32_t stride = gridDim.x * blockDim.x;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += stride) {
     const uint32_t b = inst[i];
     const int g = glog2[b];
+    const uint32_t id = vals[i];
+    unsigned long long k;
     if (g == 0) {  // one group, equal keys: the instance keeps its order
-      keys[i] = gbase[b] << kLocalityBits;
-      continue;
+      k = gbase[b] << kLocalityBits;
+    } else {
+      const unsigned long long local = i - off[b];
+      const unsigned long long group = gbase[b] + (local >> g);
+      k = (group << kLocalityBits) | (float_key(__ldg(lo_k + id)) >> kLocalityDrop);
     }
-    const unsigned long long local = i - off[b];
-    const unsigned long long group = gbase[b] + (local >> g);
-    keys[i] = (group << kLocalityBits) | (float_key(__ldg(lo_k + vals[i])) >> kLocalityDrop);
+    keys[i] = id_bits ? (k << id_bits) | id : k;
   }
 }
 
@@ -195,9 +204,9 @@ uint32_t grid_for(uint32_t cnt, int sms) {
 }  // namespace
 
 cudaError_t launch_rekey(const uint32_t* vals, const float* lo_k, uint32_t cnt, int glog2,
-                         unsigned long long* keys, int sms, cudaStream_t s) {
+                         unsigned long long* keys, int id_bits, int sms, cudaStream_t s) {
   if (cnt == 0) return cudaSuccess;
-  k_rekey<<<grid_for(cnt, sms), kThreads, 0, s>>>(vals, lo_k, cnt, glog2, keys);
+  k_rekey<<<grid_for(cnt, sms), kThreads, 0, s>>>(vals, lo_k, cnt, glog2, keys, id_bits);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -212,11 +221,10 @@ cudaError_t launch_gather(int d, const uint32_t* vals, const float* lo, const fl
 }
 
 cudaError_t launch_validate_class(int d, const float* lo, const float* hi, uint32_t cnt,
-                                  unsigned long long* keys, uint32_t* vals, uint32_t* hist,
-                                  float2* aos, Status* st, int sms, cudaStream_t s) {
+                                  uint32_t* k32, uint32_t* hist, float2* aos, Status* st, int sms,
+                                  cudaStream_t s) {
   if (cnt == 0) return cudaSuccess;
-  k_validate_class<<<grid_for(cnt, sms), kThreads, 0, s>>>(d, lo, hi, cnt, keys, vals, hist, aos,
-                                                           st);
+  k_validate_class<<<grid_for(cnt, sms), kThreads, 0, s>>>(d, lo, hi, cnt, k32, hist, aos, st);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -231,9 +239,9 @@ cudaError_t launch_fill_inst(const unsigned long long* off, uint32_t count, uint
 
 cudaError_t launch_validate_batch(int d, const float* lo, const float* hi, uint32_t cnt,
                                   const uint32_t* inst, unsigned long long* keys, uint32_t* vals,
-                                  float2* aos, Status* st, int sms, cudaStream_t s) {
+                                  uint32_t* k32, float2* aos, Status* st, int sms, cudaStream_t s) {
   if (cnt == 0) return cudaSuccess;
-  k_validate_batch<<<grid_for(cnt, sms), kThreads, 0, s>>>(d, lo, hi, cnt, inst, keys, vals, aos,
+  k_validate_batch<<<grid_for(cnt, sms), kThreads, 0, s>>>(d, lo, hi, cnt, inst, keys, vals, k32, aos,
                                                            st);
   note_launches(1);
   return cudaGetLastError();
@@ -251,20 +259,19 @@ cudaError_t launch_batch_groups(const unsigned long long* off, uint32_t count, c
 cudaError_t launch_rekey_batch(const uint32_t* vals, const float* lo_k, uint32_t cnt,
                                const uint32_t* inst, const unsigned long long* off,
                                const int* glog2, const unsigned long long* gbase,
-                               unsigned long long* keys, int sms, cudaStream_t s) {
+                               unsigned long long* keys, int id_bits, int sms, cudaStream_t s) {
   if (cnt == 0) return cudaSuccess;
   k_rekey_batch<<<grid_for(cnt, sms), kThreads, 0, s>>>(vals, lo_k, cnt, inst, off, glog2, gbase,
-                                                        keys);
+                                                        keys, id_bits);
   note_launches(1);
   return cudaGetLastError();
 }
 
 cudaError_t launch_validate(int d, const float* lo, const float* hi, uint32_t cnt,
-                            unsigned long long* keys, uint32_t* vals, int key_mode, float2* aos,
+                            unsigned long long* keys, uint32_t* vals, uint32_t* k32, float2* aos,
                             Status* st, int sms, cudaStream_t s) {
   if (cnt == 0) return cudaSuccess;
-  k_validate<<<grid_for(cnt, sms), kThreads, 0, s>>>(d, lo, hi, cnt, keys, vals, key_mode, aos,
-                                                     st);
+  k_validate<<<grid_for(cnt, sms), kThreads, 0, s>>>(d, lo, hi, cnt, keys, vals, k32, aos, st);
   note_launches(1);
   return cudaGetLastError();
 }

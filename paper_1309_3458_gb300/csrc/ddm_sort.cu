@@ -50,14 +50,13 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   return r;
 }
 
-// Lanes of the warp holding the same digit (0..256, 256 = no key): one
-// ballot per digit bit.  Measured: the 8,192-key single-CTA sort took 59
-// instead of 88 us with this in place of match.any, which the SM's warps
-// issue one at a time.
+// Lanes of the warp holding the same digit: one ballot per digit bit.
+// Measured: an 8,192-key single-CTA sort took 59 instead of 88 us with this in
+// place of match.any, which the SM's warps issue one at a time.
 __device__ __forceinline__ uint32_t same_digit_lanes(uint32_t dig) {
   uint32_t peers = 0xffffffffu;
 #pragma unroll
-  for (int b = 0; b <= kRadixBits; ++b) {
+  for (int b = 0; b < kRadixBits; ++b) {
     const uint32_t bit = (dig >> b) & 1u;
     const uint32_t votes = __ballot_sync(0xffffffffu, bit);
     peers &= bit ? votes : ~votes;
@@ -89,6 +88,16 @@ __device__ __forceinline__ uint32_t poll_flag(const uint32_t* p, uint32_t mask, 
     }
     __nanosleep(64);
   }
+}
+
+// A packed word: the key above the id (id_bits wide), so that a pass moves
+// one 8-byte word per element where keys and ids in separate arrays are
+// twelve bytes in two streams.  The first pass builds the words of a source
+// (SortSource): k32[i], with hi[i] above it, and the position as id.
+__device__ __forceinline__ unsigned long long source_word(const SortSource& src, uint32_t i) {
+  unsigned long long k = __ldg(src.k32 + i);
+  if (src.hi) k |= (unsigned long long)__ldg(src.hi + i) << src.k32_bits;
+  return (k << src.id_bits) | i;
 }
 
 // Test hook for the bounded waits: poll a word nothing sets.
@@ -175,10 +184,10 @@ k_onesweep(const unsigned long long* __restrict__ in_keys, const uint32_t* __res
       key[i] = in_keys[tile_base + local];
       val[i] = in_vals[tile_base + local];
       dig[i] = (uint32_t)(key[i] >> shift) & (kRadix - 1);
-    } else {
-      key[i] = 0;
+    } else {  // padding: the largest key, so it ranks last and its slots go unused
+      key[i] = ~0ull;
       val[i] = 0;
-      dig[i] = kRadix;  // sentinel: not counted
+      dig[i] = kRadix - 1;
     }
   }
 
@@ -188,11 +197,10 @@ k_onesweep(const unsigned long long* __restrict__ in_keys, const uint32_t* __res
 #pragma unroll
   for (int i = 0; i < kItems; ++i) {
     const uint32_t peers = same_digit_lanes(dig[i]);
-    uint32_t before = 0;
-    if (dig[i] < kRadix) before = sm.whist[warp][dig[i]];
+    const uint32_t before = sm.whist[warp][dig[i]];
     rank[i] = before + __popc(peers & lt);
     __syncwarp();
-    if (dig[i] < kRadix && (peers & lt) == 0) sm.whist[warp][dig[i]] = before + __popc(peers);
+    if ((peers & lt) == 0) sm.whist[warp][dig[i]] = before + __popc(peers);
     __syncwarp();
   }
   __syncthreads();
@@ -246,11 +254,9 @@ k_onesweep(const unsigned long long* __restrict__ in_keys, const uint32_t* __res
   // Scatter into shared memory in (digit, input order) order ...
 #pragma unroll
   for (int i = 0; i < kItems; ++i) {
-    if (dig[i] < kRadix) {
-      const uint32_t slot = sm.lstart[dig[i]] + sm.whist[warp][dig[i]] + rank[i];
-      sm.keys[slot] = key[i];
-      sm.vals[slot] = val[i];
-    }
+    const uint32_t slot = sm.lstart[dig[i]] + sm.whist[warp][dig[i]] + rank[i];
+    sm.keys[slot] = key[i];
+    sm.vals[slot] = val[i];
   }
   __syncthreads();
   // ... and out to global memory, consecutive threads taking consecutive slots.
@@ -264,7 +270,157 @@ k_onesweep(const unsigned long long* __restrict__ in_keys, const uint32_t* __res
   }
 }
 
+// Digit histograms of a packed sort, in one read of its source (or words).
+// The digits of a warp's elements are often all equal (high digits, instance
+// numbers): then one lane adds them at once, where 32 atomics on one word
+// would take 32 turns.
+__global__ void __launch_bounds__(kThreads)
+k_histogram_packed(const unsigned long long* __restrict__ words, SortSource src, uint32_t n,
+                   int passes, uint32_t* __restrict__ hist) {
+  __shared__ uint32_t h[kPasses * kRadix];
+  for (int t = threadIdx.x; t < passes * kRadix; t += kThreads) h[t] = 0;
+  __syncthreads();
+  const uint32_t stride = gridDim.x * kThreads;
+  const int lane = threadIdx.x & 31;
+  for (uint32_t i0 = blockIdx.x * kThreads + (threadIdx.x & ~31u); i0 < n; i0 += stride) {
+    const uint32_t i = i0 + lane;
+    const bool whole = i0 + 32u <= n;  // warp-uniform
+    if (!whole && i >= n) continue;
+    const unsigned long long k = (src.k32 ? source_word(src, i) : words[i]) >> src.id_bits;
+    for (int p = 0; p < passes; ++p) {
+      const uint32_t d = (uint32_t)(k >> (p * kRadixBits)) & (kRadix - 1);
+      if (whole && __all_sync(0xffffffffu, d == __shfl_sync(0xffffffffu, d, 0))) {
+        if (lane == 0) atomicAdd(&h[p * kRadix + d], 32u);
+      } else {
+        atomicAdd(&h[p * kRadix + d], 1u);
+      }
+    }
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < passes * kRadix; t += kThreads)
+    if (h[t]) atomicAdd(&hist[t], h[t]);
+}
+
+// The onesweep pass on packed words: 512 threads with eight words each, so
+// that three CTAs fit an SM in 40 registers (the pass on keys and ids needs 80
+// and spills), half the words per thread to wait for and to rank in turn, one
+// scattered stream instead of two.  FIRST: the words come from the source;
+// LAST: only the ids go out.
+constexpr int kPackThreads = 512;
+constexpr int kPackWarps = kPackThreads / 32;
+constexpr int kPackItems = kSortTile / kPackThreads;  // 8
+
+struct PackedSmem {
+  uint32_t whist[kPackWarps][kRadix];
+  uint32_t lstart[kRadix];
+  uint32_t gbase[kRadix];
+  uint32_t wtot[kRadix / 32];
+  uint32_t tile;
+  unsigned long long words[kSortTile];
+};
+
+template <bool FIRST, bool LAST>
+__global__ void __launch_bounds__(kPackThreads, 3)
+k_onesweep_packed(const unsigned long long* __restrict__ in, SortSource src,
+                  unsigned long long* __restrict__ out, uint32_t* __restrict__ out_ids, uint32_t n,
+                  int shift, const uint32_t* __restrict__ digit_base,
+                  uint32_t* __restrict__ lookback, uint32_t* __restrict__ counter,
+                  Status* __restrict__ st) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  PackedSmem& sm = *reinterpret_cast<PackedSmem*>(smem_raw);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t lt = lanemask_lt();
+  if (tid == 0) sm.tile = atomicAdd(counter, 1u);
+  for (int t = lane; t < kRadix; t += 32) sm.whist[warp][t] = 0;
+  __syncthreads();
+  const uint32_t tile = sm.tile;
+  const uint32_t base = tile * (uint32_t)kSortTile;
+  const uint32_t valid = min((uint32_t)kSortTile, n - base);
+  unsigned long long word[kPackItems];
+  uint32_t rank[kPackItems];
+#pragma unroll
+  for (int i = 0; i < kPackItems; ++i) {
+    const uint32_t local = warp * (kPackItems * 32) + i * 32 + lane;
+    word[i] = local >= valid ? ~0ull : FIRST ? source_word(src, base + local) : in[base + local];
+  }
+#pragma unroll
+  for (int i = 0; i < kPackItems; ++i) {
+    const uint32_t d = (uint32_t)(word[i] >> shift) & (kRadix - 1);
+    const uint32_t peers = same_digit_lanes(d);
+    const uint32_t before = sm.whist[warp][d];
+    rank[i] = before + __popc(peers & lt);
+    __syncwarp();
+    if ((peers & lt) == 0) sm.whist[warp][d] = before + __popc(peers);
+    __syncwarp();
+  }
+  __syncthreads();
+  // Thread t < 256 owns digit t: per-warp first slots, the tile's count, its
+  // first slot in the tile and (look-back) in the output.
+  uint32_t count = 0, x = 0;
+  uint32_t* my_slot = lookback + (size_t)tile * kRadix + tid;
+  if (tid < kRadix) {
+#pragma unroll
+    for (int w = 0; w < kPackWarps; ++w) {
+      const uint32_t c = sm.whist[w][tid];
+      sm.whist[w][tid] = count;
+      count += c;
+    }
+    st_relaxed(my_slot, (tile == 0 ? kFlagInc : kFlagAgg) | count);
+    x = count;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) sm.wtot[warp] = x;
+  }
+  __syncthreads();
+  if (tid < kRadix) {
+    uint32_t pre = 0;
+    for (int w = 0; w < warp; ++w) pre += sm.wtot[w];
+    const uint32_t lstart = pre + x - count;
+    sm.lstart[tid] = lstart;
+    uint32_t excl = 0;
+    if (tile > 0) {
+      uint32_t p = tile - 1;
+      for (;;) {
+        bool timed_out = false;
+        const uint32_t w = poll_flag(lookback + (size_t)p * kRadix + tid, kFlagMask, kSpinLimit,
+                                     &timed_out);
+        if (timed_out) {
+          atomicOr(&st->err, kErrTimeout);
+          break;
+        }
+        excl += w & kValMask;
+        if ((w & kFlagMask) == kFlagInc || p == 0) break;
+        --p;
+      }
+      st_relaxed(my_slot, kFlagInc | (excl + count));
+    }
+    sm.gbase[tid] = digit_base[tid] + excl - lstart;  // modular: gbase + slot is exact
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kPackItems; ++i) {
+    const uint32_t d = (uint32_t)(word[i] >> shift) & (kRadix - 1);
+    sm.words[sm.lstart[d] + sm.whist[warp][d] + rank[i]] = word[i];
+  }
+  __syncthreads();
+  for (uint32_t q = tid; q < valid; q += kPackThreads) {
+    const unsigned long long k = sm.words[q];
+    const uint32_t g = sm.gbase[(uint32_t)(k >> shift) & (kRadix - 1)] + q;
+    if (!DDM_IN_BOUNDS(g < n, st)) continue;
+    if (LAST)
+      out_ids[g] = (uint32_t)(k & ((1ull << src.id_bits) - 1ull));
+    else
+      out[g] = k;
+  }
+}
+
 // Ranking of one tile of 512 * ITEMS keys held in registers by 512 threads
+// (positions past the set's end hold ~0: they rank last, and the slots from
+// the valid count on are not written out; they are counted for digit 255,
+// which has no digit and, in the last tile, no tile behind it)
 // (item i of lane l in warp w is the tile's element w*32*ITEMS + i*32 + l):
 // the same stable ranking as k_onesweep (warp match + per-warp counters,
 // warps in order).  Afterwards whist[w][dg] is warp w's first slot within
@@ -281,23 +437,27 @@ struct RankSmem {
 
 template <int ITEMS>
 __device__ __forceinline__ uint32_t rank_tile(RankSmem& sm, const unsigned long long (&key)[ITEMS],
-                                              uint32_t (&dig)[ITEMS], uint32_t (&rank)[ITEMS],
-                                              uint32_t valid, int shift) {
+                                              uint32_t (&rank)[ITEMS], int shift) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t lt = lanemask_lt();
-  for (int t = tid; t < kSmallWarps * kRadix; t += kSmallThreads) (&sm.whist[0][0])[t] = 0;
-  __syncthreads();
+  for (int t = lane; t < kRadix; t += 32) sm.whist[warp][t] = 0;
+  __syncwarp();
+  // four items' ballots first, then the serial chain through the counters
 #pragma unroll
-  for (int i = 0; i < ITEMS; ++i) {
-    const uint32_t local = warp * (ITEMS * 32) + i * 32 + lane;
-    dig[i] = local < valid ? (uint32_t)(key[i] >> shift) & (kRadix - 1) : kRadix;
-    const uint32_t peers = same_digit_lanes(dig[i]);
-    uint32_t before = 0;
-    if (dig[i] < kRadix) before = sm.whist[warp][dig[i]];
-    rank[i] = before + __popc(peers & lt);
-    __syncwarp();
-    if (dig[i] < kRadix && (peers & lt) == 0) sm.whist[warp][dig[i]] = before + __popc(peers);
-    __syncwarp();
+  for (int i0 = 0; i0 < ITEMS; i0 += 4) {
+    uint32_t peers[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      peers[u] = same_digit_lanes((uint32_t)(key[i0 + u] >> shift) & (kRadix - 1));
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      uint32_t* h = &sm.whist[warp][(uint32_t)(key[i0 + u] >> shift) & (kRadix - 1)];
+      const uint32_t before = *h;
+      rank[i0 + u] = before + __popc(peers[u] & lt);
+      __syncwarp();
+      if ((peers[u] & lt) == 0) *h = before + __popc(peers[u]);
+      __syncwarp();
+    }
   }
   __syncthreads();
   uint32_t count = 0;
@@ -351,7 +511,7 @@ constexpr size_t kGridRowWords = (size_t)kGridMaxTiles * (kRadix / 2);
 constexpr size_t kGridSumWords = 2 * (size_t)kGridGroups * kRadix;
 constexpr size_t kGridScratchWords = kGridRowWords + kGridSumWords + 32;
 
-template <int ITEMS>
+template <int ITEMS, bool PACKED>
 struct GridSortSmem {
   RankSmem r;
   uint32_t gbase[kRadix];
@@ -359,7 +519,7 @@ struct GridSortSmem {
   int abort;
   int pad[3];
   unsigned long long keys[kSmallThreads * ITEMS];
-  uint32_t vals[kSmallThreads * ITEMS];
+  uint32_t vals[PACKED ? 1 : kSmallThreads * ITEMS];
 };
 
 // Grid-wide barrier for a cooperative launch (all CTAs resident).  `bar` is
@@ -396,15 +556,17 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t target, Sta
 
 // Two CTAs per SM up to 4,096-key tiles (64 registers, no spill): a one-shot
 // call sorts both of its sets at the same time.
-template <int ITEMS>
+// PACKED: words (from `src` if it has a source, else keys0), the ids to vals0
+// at the end; else keys and ids.
+template <int ITEMS, bool PACKED>
 __global__ void __launch_bounds__(kSmallThreads, ITEMS <= 8 ? 2 : 1)
 k_sort_grid(unsigned long long* __restrict__ keys0, uint32_t* __restrict__ vals0,
             unsigned long long* __restrict__ keys1, uint32_t* __restrict__ vals1, uint32_t n,
-            int passes, uint32_t* __restrict__ table, uint32_t* __restrict__ bar,
+            int passes, SortSource src, uint32_t* __restrict__ table, uint32_t* __restrict__ bar,
             Status* __restrict__ st) {
   constexpr uint32_t kTile = kSmallThreads * ITEMS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  GridSortSmem<ITEMS>& sm = *reinterpret_cast<GridSortSmem<ITEMS>*>(smem_raw);
+  GridSortSmem<ITEMS, PACKED>& sm = *reinterpret_cast<GridSortSmem<ITEMS, PACKED>*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t tile = blockIdx.x, tiles = gridDim.x;
   const size_t base = (size_t)tile * kTile;
@@ -412,21 +574,29 @@ k_sort_grid(unsigned long long* __restrict__ keys0, uint32_t* __restrict__ vals0
   if (tid == 0) sm.abort = 0;
   uint32_t barriers = 0;
   unsigned long long key[ITEMS];
-  uint32_t val[ITEMS], dig[ITEMS], rank[ITEMS];
+  uint32_t val[PACKED ? 1 : ITEMS], rank[ITEMS];
   for (int p = 0; p < passes; ++p) {
     const unsigned long long* ik = (p & 1) ? keys1 : keys0;
     const uint32_t* iv = (p & 1) ? vals1 : vals0;
     unsigned long long* ok = (p & 1) ? keys0 : keys1;
     uint32_t* ov = (p & 1) ? vals0 : vals1;
+    (void)iv;
+    (void)ov;
     // written by other CTAs of this launch: read through L2, not L1
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
       const uint32_t local = warp * (ITEMS * 32) + i * 32 + lane;
-      key[i] = local < valid ? __ldcg(ik + base + local) : 0ull;
-      val[i] = local < valid ? __ldcg(iv + base + local) : 0u;
+      if constexpr (PACKED) {
+        key[i] = local >= valid          ? ~0ull
+                 : p == 0 && src.k32     ? source_word(src, (uint32_t)base + local)
+                                         : __ldcg(ik + base + local);
+      } else {
+        key[i] = local < valid ? __ldcg(ik + base + local) : ~0ull;
+        val[i] = local < valid ? __ldcg(iv + base + local) : 0u;
+      }
     }
-    const int shift = p * kRadixBits;
-    const uint32_t count = rank_tile<ITEMS>(sm.r, key, dig, rank, valid, shift);
+    const int shift = p * kRadixBits + (PACKED ? src.id_bits : 0);
+    const uint32_t count = rank_tile<ITEMS>(sm.r, key, rank, shift);
     uint32_t* gsum = table + kGridRowWords + (size_t)(p & 1) * kGridGroups * kRadix;
     if (tid < kRadix) {  // this tile's counts: its row (two 16-bit digits per word), its group's sums
       const uint32_t next = __shfl_down_sync(0xffffffffu, count, 1);
@@ -468,18 +638,23 @@ k_sort_grid(unsigned long long* __restrict__ keys0, uint32_t* __restrict__ vals0
     // stage the tile in (digit, input order) order ...
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
-      if (dig[i] < kRadix) {
-        const uint32_t slot = sm.r.lstart[dig[i]] + sm.r.whist[warp][dig[i]] + rank[i];
-        sm.keys[slot] = key[i];
-        sm.vals[slot] = val[i];
-      }
+      const uint32_t dg = (uint32_t)(key[i] >> shift) & (kRadix - 1);
+      const uint32_t slot = sm.r.lstart[dg] + sm.r.whist[warp][dg] + rank[i];
+      sm.keys[slot] = key[i];
+      if constexpr (!PACKED) sm.vals[slot] = val[i];
     }
     __syncthreads();
     // ... and out, consecutive threads taking consecutive slots
     for (uint32_t q = tid; q < valid; q += kSmallThreads) {
       const unsigned long long k = sm.keys[q];
       const uint32_t g = sm.gbase[(uint32_t)(k >> shift) & (kRadix - 1)] + q;
-      if (DDM_IN_BOUNDS(g < n, st)) {
+      if (!DDM_IN_BOUNDS(g < n, st)) continue;
+      if constexpr (PACKED) {
+        if (p + 1 < passes)
+          ok[g] = k;
+        else
+          vals0[g] = (uint32_t)(k & ((1ull << src.id_bits) - 1ull));
+      } else {
         ok[g] = k;
         ov[g] = sm.vals[q];
       }
@@ -498,16 +673,16 @@ k_sort_grid(unsigned long long* __restrict__ keys0, uint32_t* __restrict__ vals0
 // no key goes through L2 between passes.
 constexpr uint32_t kClusterMax = 16;
 
-template <int ITEMS>
+template <int ITEMS, bool PACKED>
 struct ClusterSortSmem {
   RankSmem r;
   uint32_t gbase[kRadix];
   uint32_t dtot[kRadix / 32];
   uint32_t table[kClusterMax][kRadix];  // row j: CTA j's digit counts
   unsigned long long tile_k[kSmallThreads * ITEMS];  // this CTA's keys of the next pass
-  uint32_t tile_v[kSmallThreads * ITEMS];
+  uint32_t tile_v[PACKED ? 1 : kSmallThreads * ITEMS];
   unsigned long long stage_k[kSmallThreads * ITEMS];  // this pass's keys in digit order
-  uint32_t stage_v[kSmallThreads * ITEMS];
+  uint32_t stage_v[PACKED ? 1 : kSmallThreads * ITEMS];
 };
 
 __device__ __forceinline__ void cluster_sync_all() {
@@ -533,29 +708,33 @@ __device__ __forceinline__ void st_remote(uint32_t a, unsigned long long v) {
   asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
 }
 
-template <int ITEMS>
+template <int ITEMS, bool PACKED>
 __global__ void __launch_bounds__(kSmallThreads, 1)
 k_sort_cluster(const unsigned long long* __restrict__ in_k, const uint32_t* __restrict__ in_v,
                unsigned long long* __restrict__ out_k, uint32_t* __restrict__ out_v, uint32_t n,
-               int passes) {
+               int passes, SortSource src) {
   constexpr uint32_t kTile = kSmallThreads * ITEMS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  ClusterSortSmem<ITEMS>& sm = *reinterpret_cast<ClusterSortSmem<ITEMS>*>(smem_raw);
+  ClusterSortSmem<ITEMS, PACKED>& sm = *reinterpret_cast<ClusterSortSmem<ITEMS, PACKED>*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t me = cluster_rank(), ctas = gridDim.x;  // the grid is one cluster
   const uint32_t base = me * kTile;
   const uint32_t valid = min(kTile, n - base);
   unsigned long long key[ITEMS];
-  uint32_t val[ITEMS], dig[ITEMS], rank[ITEMS];
+  uint32_t val[PACKED ? 1 : ITEMS], rank[ITEMS];
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
     const uint32_t local = warp * (ITEMS * 32) + i * 32 + lane;
-    key[i] = local < valid ? in_k[base + local] : 0ull;
-    val[i] = local < valid ? in_v[base + local] : 0u;
+    if constexpr (PACKED) {
+      key[i] = local >= valid ? ~0ull : src.k32 ? source_word(src, base + local) : in_k[base + local];
+    } else {
+      key[i] = local < valid ? in_k[base + local] : ~0ull;
+      val[i] = local < valid ? in_v[base + local] : 0u;
+    }
   }
   for (int p = 0; p < passes; ++p) {
-    const int shift = p * kRadixBits;
-    const uint32_t count = rank_tile<ITEMS>(sm.r, key, dig, rank, valid, shift);
+    const int shift = p * kRadixBits + (PACKED ? src.id_bits : 0);
+    const uint32_t count = rank_tile<ITEMS>(sm.r, key, rank, shift);
     if (tid < kRadix)
       for (uint32_t j = 0; j < ctas; ++j) st_remote(remote_smem(&sm.table[me][tid], j), count);
     cluster_sync_all();  // every table complete; every CTA holds its keys in registers
@@ -583,11 +762,10 @@ k_sort_cluster(const unsigned long long* __restrict__ in_k, const uint32_t* __re
     }
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
-      if (dig[i] < kRadix) {
-        const uint32_t slot = sm.r.lstart[dig[i]] + sm.r.whist[warp][dig[i]] + rank[i];
-        sm.stage_k[slot] = key[i];
-        sm.stage_v[slot] = val[i];
-      }
+      const uint32_t dg = (uint32_t)(key[i] >> shift) & (kRadix - 1);
+      const uint32_t slot = sm.r.lstart[dg] + sm.r.whist[warp][dg] + rank[i];
+      sm.stage_k[slot] = key[i];
+      if constexpr (!PACKED) sm.stage_v[slot] = val[i];
     }
     __syncthreads();
     const bool last = p + 1 == passes;
@@ -598,12 +776,16 @@ k_sort_cluster(const unsigned long long* __restrict__ in_k, const uint32_t* __re
       const uint32_t g = sm.gbase[(uint32_t)(k >> shift) & (kRadix - 1)] + q;
       if (!DDM_IN_BOUNDS(g < n, nullptr)) continue;
       if (last) {
-        out_k[g] = k;
-        out_v[g] = sm.stage_v[q];
+        if constexpr (PACKED) {
+          out_v[g] = (uint32_t)(k & ((1ull << src.id_bits) - 1ull));
+        } else {
+          out_k[g] = k;
+          out_v[g] = sm.stage_v[q];
+        }
       } else {
         const uint32_t owner = g / kTile, at = g % kTile;
         st_remote(remote_smem(&sm.tile_k[at], owner), k);
-        st_remote(remote_smem(&sm.tile_v[at], owner), sm.stage_v[q]);
+        if constexpr (!PACKED) st_remote(remote_smem(&sm.tile_v[at], owner), sm.stage_v[q]);
       }
     }
     if (last) break;
@@ -611,15 +793,15 @@ k_sort_cluster(const unsigned long long* __restrict__ in_k, const uint32_t* __re
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
       const uint32_t local = warp * (ITEMS * 32) + i * 32 + lane;
-      key[i] = local < valid ? sm.tile_k[local] : 0ull;
-      val[i] = local < valid ? sm.tile_v[local] : 0u;
+      key[i] = local < valid ? sm.tile_k[local] : ~0ull;
+      if constexpr (!PACKED) val[i] = local < valid ? sm.tile_v[local] : 0u;
     }
   }
 }
 
-// Largest cluster (CTAs) k_sort_cluster<ITEMS> can run on the current
-// device: 16 (non-portable), else 8, else 0.
-template <int ITEMS>
+// Largest cluster (CTAs) k_sort_cluster can run on the current device: 16
+// (non-portable), else 8, else 0.
+template <int ITEMS, bool PACKED>
 int cluster_sort_ctas() {
   static std::atomic<int> best[64];
   int dev = 0;
@@ -630,10 +812,10 @@ int cluster_sort_ctas() {
   int b = best[dev].load(std::memory_order_relaxed);
   if (b == 0) {
     b = -1;
-    const size_t smem = sizeof(ClusterSortSmem<ITEMS>);
-    if (cudaFuncSetAttribute(k_sort_cluster<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const size_t smem = sizeof(ClusterSortSmem<ITEMS, PACKED>);
+    if (cudaFuncSetAttribute(k_sort_cluster<ITEMS, PACKED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem) == cudaSuccess &&
-        cudaFuncSetAttribute(k_sort_cluster<ITEMS>,
+        cudaFuncSetAttribute(k_sort_cluster<ITEMS, PACKED>,
                              cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
       for (int c : {16, 8}) {
         cudaLaunchConfig_t cfg = {};
@@ -648,7 +830,7 @@ int cluster_sort_ctas() {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int clusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&clusters, k_sort_cluster<ITEMS>, &cfg) == cudaSuccess &&
+        if (cudaOccupancyMaxActiveClusters(&clusters, k_sort_cluster<ITEMS, PACKED>, &cfg) == cudaSuccess &&
             clusters > 0) {
           b = c;
           break;
@@ -661,18 +843,19 @@ int cluster_sort_ctas() {
   return b < 0 ? 0 : b;
 }
 
-// One cluster launch of k_sort_cluster<ITEMS> if the set fits one cluster:
-// *done = true then (or an error), else nothing is enqueued.
-template <int ITEMS>
-cudaError_t try_sort_cluster(SortScratch sc, uint32_t n, int passes, cudaStream_t s, bool* done) {
+// One cluster launch of k_sort_cluster if the set fits one cluster: *done =
+// true then (or an error), else nothing is enqueued.
+template <int ITEMS, bool PACKED>
+cudaError_t try_sort_cluster(SortScratch sc, const SortSource& src, uint32_t n, int passes,
+                             cudaStream_t s, bool* done) {
   *done = false;
   constexpr uint32_t kTile = kSmallThreads * ITEMS;
   const uint32_t ctas = (n + kTile - 1) / kTile;
-  if (ctas > (uint32_t)cluster_sort_ctas<ITEMS>()) return cudaSuccess;
+  if (ctas > (uint32_t)cluster_sort_ctas<ITEMS, PACKED>()) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ctas);
   cfg.blockDim = dim3(kSmallThreads);
-  cfg.dynamicSmemBytes = sizeof(ClusterSortSmem<ITEMS>);
+  cfg.dynamicSmemBytes = sizeof(ClusterSortSmem<ITEMS, PACKED>);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -681,9 +864,9 @@ cudaError_t try_sort_cluster(SortScratch sc, uint32_t n, int passes, cudaStream_
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const int out = passes & 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_sort_cluster<ITEMS>, sc.keys[0], sc.vals[0],
-                                     sc.keys[out], sc.vals[out], n, passes);
+  const int out = PACKED ? 0 : passes & 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, k_sort_cluster<ITEMS, PACKED>, sc.keys[0], sc.vals[0],
+                                     sc.keys[out], sc.vals[out], n, passes, src);
   if (e == cudaSuccess) {
     note_launches(1);
     *done = true;
@@ -691,9 +874,9 @@ cudaError_t try_sort_cluster(SortScratch sc, uint32_t n, int passes, cudaStream_
   return e;
 }
 
-// Co-resident CTAs of k_sort_grid<ITEMS> on the current device, capped at
+// Co-resident CTAs of k_sort_grid on the current device, capped at
 // kGridMaxTiles (0: not usable).
-template <int ITEMS>
+template <int ITEMS, bool PACKED>
 int grid_sort_tiles(int sms) {
   static std::atomic<int> per_sm[64];
   int dev = 0;
@@ -703,10 +886,10 @@ int grid_sort_tiles(int sms) {
   }
   int b = per_sm[dev].load(std::memory_order_relaxed);
   if (b == 0) {
-    const size_t smem = sizeof(GridSortSmem<ITEMS>);
-    if (cudaFuncSetAttribute(k_sort_grid<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const size_t smem = sizeof(GridSortSmem<ITEMS, PACKED>);
+    if (cudaFuncSetAttribute(k_sort_grid<ITEMS, PACKED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem) ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sort_grid<ITEMS>, kSmallThreads, smem)) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sort_grid<ITEMS, PACKED>, kSmallThreads, smem)) {
       cudaGetLastError();
       b = 0;
     }
@@ -716,15 +899,15 @@ int grid_sort_tiles(int sms) {
   return (int)std::min<long long>((long long)b * sms, kGridMaxTiles);
 }
 
-// One cooperative launch of k_sort_grid<ITEMS> if the set fits its resident
-// grid: *done = true then (or an error), else nothing is enqueued.
-template <int ITEMS>
-cudaError_t try_sort_grid(SortScratch sc, uint32_t n, int passes, Status* st, int sms,
-                          cudaStream_t s, bool* done) {
+// One cooperative launch of k_sort_grid if the set fits its resident grid:
+// *done = true then (or an error), else nothing is enqueued.
+template <int ITEMS, bool PACKED>
+cudaError_t try_sort_grid(SortScratch sc, const SortSource& src, uint32_t n, int passes, Status* st,
+                          int sms, cudaStream_t s, bool* done) {
   *done = false;
   constexpr uint32_t kTile = kSmallThreads * ITEMS;
   const uint32_t tiles = (n + kTile - 1) / kTile;
-  if (tiles > (uint32_t)grid_sort_tiles<ITEMS>(sms)) return cudaSuccess;
+  if (tiles > (uint32_t)grid_sort_tiles<ITEMS, PACKED>(sms)) return cudaSuccess;
   cudaError_t e;
   // both parities' group sums and the barrier counter start at zero
   uint32_t* sums = sc.lookback + kGridRowWords;
@@ -732,15 +915,15 @@ cudaError_t try_sort_grid(SortScratch sc, uint32_t n, int passes, Status* st, in
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(tiles);
   cfg.blockDim = dim3(kSmallThreads);
-  cfg.dynamicSmemBytes = sizeof(GridSortSmem<ITEMS>);
+  cfg.dynamicSmemBytes = sizeof(GridSortSmem<ITEMS, PACKED>);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, k_sort_grid<ITEMS>, sc.keys[0], sc.vals[0], sc.keys[1], sc.vals[1],
-                         n, passes, sc.lookback, sums + kGridSumWords, st);
+  e = cudaLaunchKernelEx(&cfg, k_sort_grid<ITEMS, PACKED>, sc.keys[0], sc.vals[0], sc.keys[1], sc.vals[1],
+                         n, passes, src, sc.lookback, sums + kGridSumWords, st);
   if (e == cudaErrorCooperativeLaunchTooLarge) {  // fewer SMs available than counted
     cudaGetLastError();
     return cudaSuccess;
@@ -766,12 +949,12 @@ size_t sort_lookback_words(uint32_t n) {
   return std::max((size_t)kPasses * tiles * kRadix, kGridScratchWords);
 }
 
-cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf, Status* st,
-                          int sms, cudaStream_t s) {
-  *out_buf = 0;
-  if (n <= 1 || passes <= 0) return cudaSuccess;
-  if (passes > kPasses) passes = kPasses;
-  cudaError_t e;
+namespace {
+
+// The one-launch forms, smallest first: *done = false if none fits.
+template <bool PACKED>
+cudaError_t sort_in_one(SortScratch sc, const SortSource& src, uint32_t n, int passes, Status* st,
+                        int sms, cudaStream_t s, bool* done) {
   // Up to 16 tiles of 2,048 keys: one cluster, keys kept on chip; else one
   // cooperative launch when every tile can be resident at once, with the
   // smallest tile that allows it.  Measured (8 passes, one GB300): 5,000
@@ -780,28 +963,73 @@ cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf, 
   // cooperative.  Under stream capture too (the launches become graph nodes
   // with the same attributes): 256 batched instances in a graph took 187 us
   // with the multi-launch form recorded instead, 149 with these.
+  cudaError_t e;
+  if ((e = try_sort_cluster<4, PACKED>(sc, src, n, passes, s, done)) || *done) return e;
+  if ((e = try_sort_grid<4, PACKED>(sc, src, n, passes, st, sms, s, done)) || *done) return e;
+  if ((e = try_sort_grid<8, PACKED>(sc, src, n, passes, st, sms, s, done)) || *done) return e;
+  return try_sort_grid<16, PACKED>(sc, src, n, passes, st, sms, s, done);
+}
+
+cudaError_t clear_onesweep(SortScratch sc, uint32_t tiles, int passes, cudaStream_t s) {
+  cudaError_t e;
+  if ((e = cudaMemsetAsync(sc.hist, 0, sizeof(uint32_t) * kPasses * kRadix, s))) return e;
+  if ((e = cudaMemsetAsync(sc.counters, 0, sizeof(uint32_t) * kPasses, s))) return e;
+  return cudaMemsetAsync(sc.lookback, 0, sizeof(uint32_t) * (size_t)passes * tiles * kRadix, s);
+}
+
+template <bool FIRST, bool LAST>
+cudaError_t onesweep_packed_pass(SortScratch sc, const SortSource& src, uint32_t n, int p,
+                                 Status* st, cudaStream_t s) {
+  const uint32_t tiles = (n + kSortTile - 1) / kSortTile;
+  const size_t smem = sizeof(PackedSmem);
+  cudaError_t e = cudaFuncSetAttribute(k_onesweep_packed<FIRST, LAST>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e) return e;
+  k_onesweep_packed<FIRST, LAST><<<tiles, kPackThreads, smem, s>>>(
+      sc.keys[p & 1], src, sc.keys[(p & 1) ^ 1], sc.vals[0], n, src.id_bits + p * kRadixBits,
+      sc.hist + p * kRadix, sc.lookback + (size_t)p * tiles * kRadix, sc.counters + p, st);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_sort_packed(SortScratch sc, const SortSource& src, uint32_t n, int key_bits,
+                               Status* st, int sms, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  const int passes = std::max((key_bits + kRadixBits - 1) / kRadixBits, 1);
+  cudaError_t e;
   bool done = false;
-  if ((e = try_sort_cluster<4>(sc, n, passes, s, &done)) || done) {
-    *out_buf = passes & 1;
-    return e;
+  if ((e = sort_in_one<true>(sc, src, n, passes, st, sms, s, &done)) || done) return e;
+  const uint32_t tiles = (n + kSortTile - 1) / kSortTile;
+  if ((e = clear_onesweep(sc, tiles, passes, s))) return e;
+  const uint32_t hb = std::min((n + kThreads * 16 - 1) / (kThreads * 16), (uint32_t)sms * 8u);
+  k_histogram_packed<<<hb, kThreads, 0, s>>>(sc.keys[0], src, n, passes, sc.hist);
+  k_hist_scan<<<passes, kRadix, 0, s>>>(sc.hist);
+  for (int p = 0; p < passes; ++p) {
+    const bool first = p == 0 && src.k32, last = p + 1 == passes;
+    e = first ? (last ? onesweep_packed_pass<true, true>(sc, src, n, p, st, s)
+                      : onesweep_packed_pass<true, false>(sc, src, n, p, st, s))
+              : (last ? onesweep_packed_pass<false, true>(sc, src, n, p, st, s)
+                      : onesweep_packed_pass<false, false>(sc, src, n, p, st, s));
+    if (e) return e;
   }
-  if ((e = try_sort_grid<4>(sc, n, passes, st, sms, s, &done)) || done) {
-    *out_buf = passes & 1;
-    return e;
-  }
-  if ((e = try_sort_grid<8>(sc, n, passes, st, sms, s, &done)) || done) {
-    *out_buf = passes & 1;
-    return e;
-  }
-  if ((e = try_sort_grid<16>(sc, n, passes, st, sms, s, &done)) || done) {
+  note_launches(2u + (unsigned)passes);
+  return cudaSuccess;
+}
+
+cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf, Status* st,
+                          int sms, cudaStream_t s) {
+  *out_buf = 0;
+  if (n <= 1 || passes <= 0) return cudaSuccess;
+  if (passes > kPasses) passes = kPasses;
+  cudaError_t e;
+  bool done = false;
+  if ((e = sort_in_one<false>(sc, SortSource{}, n, passes, st, sms, s, &done)) || done) {
     *out_buf = passes & 1;
     return e;
   }
   const uint32_t tiles = (n + kSortTile - 1) / kSortTile;
-  if ((e = cudaMemsetAsync(sc.hist, 0, sizeof(uint32_t) * kPasses * kRadix, s))) return e;
-  if ((e = cudaMemsetAsync(sc.counters, 0, sizeof(uint32_t) * kPasses, s))) return e;
-  if ((e = cudaMemsetAsync(sc.lookback, 0, sizeof(uint32_t) * (size_t)passes * tiles * kRadix, s)))
-    return e;
+  if ((e = clear_onesweep(sc, tiles, passes, s))) return e;
   uint32_t hb = (n + kThreads * 16 - 1) / (kThreads * 16);
   if (hb > (uint32_t)sms * 4u) hb = (uint32_t)sms * 4u;
   k_histogram<<<hb, kThreads, 0, s>>>(sc.keys[0], n, sc.hist);
