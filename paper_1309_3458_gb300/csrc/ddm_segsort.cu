@@ -24,21 +24,22 @@ namespace ddm {
 namespace {
 
 constexpr int kRadix = 256;
-constexpr int kSegThreads = 1024;
-constexpr int kSegWarps = kSegThreads / 32;
-constexpr int kParts = kSegThreads / kRadix;       // threads per digit
-constexpr int kPartWarps = kSegWarps / kParts;     // warps summed by each
+constexpr int kPartWarps = 8;                      // warps whose counts a thread sums
 constexpr int kKeyBits = 24;                       // locality key, see ddm_layout.cu
 
-template <int ITEMS>
+template <int THREADS, int ITEMS>
 struct SegSmem {
-  uint32_t whist[kSegWarps][kRadix];  // per-warp digit counts, then first slots within the digit
-  uint32_t part[kParts][kRadix];
+  static constexpr int warps = THREADS / 32;
+  static constexpr int parts = THREADS / kRadix;  // threads per digit
+  static_assert(parts * kPartWarps == warps, "a thread per digit and eight warps");
+  uint32_t whist[warps][kRadix];      // per-warp digit counts, then first slots within the digit
+  uint32_t part[parts][kRadix];
   uint32_t total[kRadix];             // the tile's keys with each digit
   uint32_t first[kRadix];             // the digit's first slot in the tile
   uint32_t wtot[kRadix / 32];
   uint32_t base[kRadix];              // groups larger than a tile: running positions
-  unsigned long long word[kSegThreads * ITEMS];
+  uint32_t range[2];                  // least and largest key of a chunk
+  unsigned long long word[THREADS * ITEMS];
 };
 
 // Lanes of the warp holding the same 8-bit digit.
@@ -58,8 +59,8 @@ __device__ __forceinline__ uint32_t same_digit(uint32_t dig) {
 // so they rank last; warps without a valid element skip the ranking.  The
 // ballots of all items come first: only a read and a write of the warp's
 // counters per item are left in the serial chain.
-template <int ITEMS>
-__device__ __forceinline__ void rank_digit(SegSmem<ITEMS>& sm,
+template <int THREADS, int ITEMS>
+__device__ __forceinline__ void rank_digit(SegSmem<THREADS, ITEMS>& sm,
                                            const unsigned long long (&word)[ITEMS],
                                            uint32_t (&rank)[ITEMS], uint32_t valid, int shift) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -95,7 +96,7 @@ __device__ __forceinline__ void rank_digit(SegSmem<ITEMS>& sm,
   // their first slots in the tile.
   uint32_t run = 0, all = 0;
 #pragma unroll
-  for (int q = 0; q < kParts; ++q) {
+  for (int q = 0; q < THREADS / kRadix; ++q) {
     const uint32_t v = sm.part[q][dig];
     run += q < part ? v : 0u;
     all += v;
@@ -124,30 +125,56 @@ __device__ __forceinline__ void rank_digit(SegSmem<ITEMS>& sm,
   __syncthreads();
 }
 
-// (local group, key) of position `at` of a chunk, above its id.
-__device__ __forceinline__ unsigned long long seg_word(uint32_t id, const float* lo_k, uint32_t at,
-                                                       int g) {
-  const uint32_t key = float_key(__ldg(lo_k + id)) >> (32 - kKeyBits);
-  return ((unsigned long long)(((at >> g) << kKeyBits) | key) << 32) | id;
-}
-
-// One chunk of at most a tile.
-template <int ITEMS>
-__device__ __forceinline__ void sort_chunk(SegSmem<ITEMS>& sm, uint32_t* vals, const float* lo_k,
-                                           uint32_t len, int g) {
+// One chunk of at most a tile.  Its words hold the key above the least key of
+// the chunk, in as many bits as the range needs, with the group above that:
+// coordinates of one scale range over some 20 of the 24 bits, so that a
+// chunk of several groups usually takes three digits instead of four.
+template <int THREADS, int ITEMS>
+__device__ __forceinline__ void sort_chunk(SegSmem<THREADS, ITEMS>& sm, uint32_t* vals,
+                                           const float* lo_k, uint32_t len, int g) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool any = (uint32_t)warp * (ITEMS * 32) < len;  // warps past the chunk idle
   unsigned long long word[ITEMS];
   uint32_t rank[ITEMS];
+  if (tid < 2) sm.range[tid] = tid ? 0u : 0xffffffffu;
+  uint32_t id[ITEMS], key[ITEMS], least = 0xffffffffu, most = 0u;
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
     const uint32_t at = warp * (ITEMS * 32) + i * 32 + lane;
-    word[i] = at < len ? seg_word(vals[at], lo_k, at, g) : ~0ull;
+    id[i] = at < len ? vals[at] : 0u;
   }
-  const int passes = ((len - 1u) >> g) ? 4 : 3;
+#pragma unroll
+  for (int i = 0; i < ITEMS; ++i) {
+    const uint32_t at = warp * (ITEMS * 32) + i * 32 + lane;
+    if (at < len) {
+      key[i] = float_key(__ldg(lo_k + id[i])) >> (32 - kKeyBits);
+      least = min(least, key[i]);
+      most = max(most, key[i]);
+    }
+  }
+  __syncthreads();
+  if (any) {
+    least = __reduce_min_sync(0xffffffffu, least);
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 0) {
+      atomicMin(&sm.range[0], least);
+      atomicMax(&sm.range[1], most);
+    }
+  }
+  __syncthreads();
+  least = sm.range[0];
+  const int bits = 32 - __clz(sm.range[1] - least), groups = (int)((len - 1u) >> g);
+  const int passes = max((bits + 32 - __clz(groups) + 7) / 8, 1);
+#pragma unroll
+  for (int i = 0; i < ITEMS; ++i) {
+    const uint32_t at = warp * (ITEMS * 32) + i * 32 + lane;
+    word[i] = at < len ? ((unsigned long long)(((at >> g) << bits) | (key[i] - least)) << 32) | id[i]
+                       : ~0ull;
+  }
   for (int p = 0; p < passes; ++p) {
     const int shift = 32 + 8 * p;
-    rank_digit<ITEMS>(sm, word, rank, len, shift);
-    if ((uint32_t)warp * (ITEMS * 32) < len) {
+    rank_digit<THREADS, ITEMS>(sm, word, rank, len, shift);
+    if (any) {
 #pragma unroll
       for (int i = 0; i < ITEMS; ++i) {
         const uint32_t d = (uint32_t)(word[i] >> shift) & 255u;
@@ -155,29 +182,32 @@ __device__ __forceinline__ void sort_chunk(SegSmem<ITEMS>& sm, uint32_t* vals, c
       }
     }
     __syncthreads();
-    if (p + 1 < passes && (uint32_t)warp * (ITEMS * 32) < len) {
+    if (p + 1 < passes && any) {
 #pragma unroll
       for (int i = 0; i < ITEMS; ++i) word[i] = sm.word[warp * (ITEMS * 32) + i * 32 + lane];
     }
   }
-  for (uint32_t q = tid; q < len; q += kSegThreads) vals[q] = (uint32_t)sm.word[q];
+  for (uint32_t q = tid; q < len; q += THREADS) vals[q] = (uint32_t)sm.word[q];
   __syncthreads();  // before the next chunk's words
 }
 
 // One group larger than a tile (an instance of millions of extents): the same
 // digits, tile by tile through two scratch ranges in global memory.
-template <int ITEMS>
-__device__ void sort_large_group(SegSmem<ITEMS>& sm, uint32_t* vals, const float* lo_k,
+template <int THREADS, int ITEMS>
+__device__ void sort_large_group(SegSmem<THREADS, ITEMS>& sm, uint32_t* vals, const float* lo_k,
                                  uint32_t len, unsigned long long* a, unsigned long long* b) {
-  constexpr uint32_t kTile = kSegThreads * ITEMS;
+  constexpr uint32_t kTile = THREADS * ITEMS;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (uint32_t q = tid; q < len; q += kSegThreads) a[q] = seg_word(vals[q], lo_k, 0u, 0);
+  for (uint32_t q = tid; q < len; q += THREADS) {
+    const uint32_t id = vals[q];
+    a[q] = ((unsigned long long)(float_key(__ldg(lo_k + id)) >> (32 - kKeyBits)) << 32) | id;
+  }
   __syncthreads();
   for (int p = 0; p < kKeyBits / 8; ++p) {
     const int shift = 32 + 8 * p;
-    for (int t = tid; t < kRadix; t += kSegThreads) sm.base[t] = 0u;
+    for (int t = tid; t < kRadix; t += THREADS) sm.base[t] = 0u;
     __syncthreads();
-    for (uint32_t q = tid; q < len; q += kSegThreads)
+    for (uint32_t q = tid; q < len; q += THREADS)
       atomicAdd(&sm.base[(uint32_t)(__ldcg(a + q) >> shift) & 255u], 1u);
     __syncthreads();
     if (warp == 0) {  // exclusive scan of the 256 counts, eight per lane
@@ -210,7 +240,7 @@ __device__ void sort_large_group(SegSmem<ITEMS>& sm, uint32_t* vals, const float
         const uint32_t at = warp * (ITEMS * 32) + i * 32 + lane;
         word[i] = at < valid ? __ldcg(a + t0 + at) : ~0ull;
       }
-      rank_digit<ITEMS>(sm, word, rank, valid, shift);
+      rank_digit<THREADS, ITEMS>(sm, word, rank, valid, shift);
 #pragma unroll
       for (int i = 0; i < ITEMS; ++i) {
         const uint32_t at = warp * (ITEMS * 32) + i * 32 + lane;
@@ -226,22 +256,22 @@ __device__ void sort_large_group(SegSmem<ITEMS>& sm, uint32_t* vals, const float
     a = b;
     b = t;
   }
-  for (uint32_t q = tid; q < len; q += kSegThreads) vals[q] = (uint32_t)__ldcg(a + q);
+  for (uint32_t q = tid; q < len; q += THREADS) vals[q] = (uint32_t)__ldcg(a + q);
   __syncthreads();
 }
 
 // Re-sort of one set.  With `off` null: one instance of `total` positions and
 // group exponent g_one; else instance i owns positions [off[i], off[i+1]) with
 // exponent glog2[i] (0: left as it is) and chunks [cbase[i], cbase[i+1]).
-template <int ITEMS>
-__global__ void __launch_bounds__(kSegThreads, 1)
+template <int THREADS, int ITEMS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS)
 k_segsort(uint32_t* __restrict__ vals, const float* __restrict__ lo_k, uint32_t total, int g_one,
           const unsigned long long* __restrict__ off, const int* __restrict__ glog2,
           const unsigned long long* __restrict__ cbase, uint32_t count,
           unsigned long long* __restrict__ tmp0, unsigned long long* __restrict__ tmp1) {
-  constexpr uint32_t kTile = kSegThreads * ITEMS;
+  constexpr uint32_t kTile = THREADS * ITEMS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  SegSmem<ITEMS>& sm = *reinterpret_cast<SegSmem<ITEMS>*>(smem_raw);
+  SegSmem<THREADS, ITEMS>& sm = *reinterpret_cast<SegSmem<THREADS, ITEMS>*>(smem_raw);
   const uint32_t lane = threadIdx.x & 31u;
   const unsigned long long chunks = off ? cbase[count] : ((unsigned long long)total + kTile - 1) / kTile;
   for (unsigned long long c = blockIdx.x; c < chunks; c += gridDim.x) {
@@ -265,9 +295,9 @@ k_segsort(uint32_t* __restrict__ vals, const float* __restrict__ lo_k, uint32_t 
     }
     const uint32_t len = (uint32_t)(end - begin);
     if (len > kTile)
-      sort_large_group<ITEMS>(sm, vals + begin, lo_k, len, tmp0 + begin, tmp1 + begin);
+      sort_large_group<THREADS, ITEMS>(sm, vals + begin, lo_k, len, tmp0 + begin, tmp1 + begin);
     else if (len > 1)
-      sort_chunk<ITEMS>(sm, vals + begin, lo_k, len, g);
+      sort_chunk<THREADS, ITEMS>(sm, vals + begin, lo_k, len, g);
   }
 }
 
@@ -378,18 +408,18 @@ k_class_plan(const uint32_t* __restrict__ hist, int d,
   }
 }
 
-template <int ITEMS>
+template <int THREADS, int ITEMS>
 cudaError_t launch_segsort_items(uint32_t* vals, const float* lo_k, uint32_t total, int g,
                                  const SegPlan& plan, unsigned long long* tmp0,
                                  unsigned long long* tmp1, int sms, cudaStream_t s) {
-  const size_t smem = sizeof(SegSmem<ITEMS>);
-  cudaError_t e = cudaFuncSetAttribute(k_segsort<ITEMS>,
+  const size_t smem = sizeof(SegSmem<THREADS, ITEMS>);
+  cudaError_t e = cudaFuncSetAttribute(k_segsort<THREADS, ITEMS>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e) return e;
   // at most one chunk per instance beyond the whole tiles
-  const uint64_t most = (uint64_t)total / (kSegThreads * ITEMS) + (plan.off ? plan.count : 0u) + 1u;
-  const uint32_t blocks = (uint32_t)std::min<uint64_t>(most, (uint64_t)sms * 2u);
-  k_segsort<ITEMS><<<blocks, kSegThreads, smem, s>>>(vals, lo_k, total, g, plan.off, plan.glog2,
+  const uint64_t most = (uint64_t)total / (THREADS * ITEMS) + (plan.off ? plan.count : 0u) + 1u;
+  const uint32_t blocks = (uint32_t)std::min<uint64_t>(most, (uint64_t)sms * (2048 / THREADS));
+  k_segsort<THREADS, ITEMS><<<blocks, THREADS, smem, s>>>(vals, lo_k, total, g, plan.off, plan.glog2,
                                                      plan.cbase, plan.count, tmp0, tmp1);
   note_launches(1);
   return cudaGetLastError();
@@ -438,9 +468,15 @@ cudaError_t launch_segsort(uint32_t* vals, const float* lo_k, uint32_t total, in
                            const SegPlan& plan, int tile_log2, unsigned long long* tmp0,
                            unsigned long long* tmp1, int sms, cudaStream_t s) {
   if (total <= 1) return cudaSuccess;
-  return tile_log2 == 12
-             ? launch_segsort_items<4>(vals, lo_k, total, g, plan, tmp0, tmp1, sms, s)
-             : launch_segsort_items<8>(vals, lo_k, total, g, plan, tmp0, tmp1, sms, s);
+  if (tile_log2 != kSegTileLog2)
+    return launch_segsort_items<1024, 8>(vals, lo_k, total, g, plan, tmp0, tmp1, sms, s);
+  // More chunks than SMs: CTAs of half the threads, two to an SM, so that one
+  // ranks while the other waits (2 x 2.9e7 positions of 4,096 instances: 2.00
+  // ms with CTAs of 1,024 threads and all 24 key bits, 1.34 now).  Else a
+  // chunk's latency counts: more threads.
+  if ((total >> kSegTileLog2) > (uint32_t)sms)
+    return launch_segsort_items<512, 8>(vals, lo_k, total, g, plan, tmp0, tmp1, sms, s);
+  return launch_segsort_items<1024, 4>(vals, lo_k, total, g, plan, tmp0, tmp1, sms, s);
 }
 
 }  // namespace ddm
