@@ -87,6 +87,7 @@ struct ddm_ctx {
   RecordArena arena{};          // arena of the current plan (max_blocks 0 = none)
   // batched instances
   DevBuf inst_s, inst_u;
+  DevBuf leaf_off;              // padded tree of a batch
   // size classes of the tree order (d >= 2)
   DevBuf cls_hist, cls_off;
   DevBuf probe;                 // word polled by ddm_debug_wait_timeout
@@ -377,21 +378,27 @@ struct BatchSet {
   const unsigned long long* off;  // [count + 1] positions of each instance
   uint32_t count;
   uint32_t* inst;                 // [cnt] instance of each position (filled here)
+  uint32_t padded;                // positions of the padded tree (BatchView), 0: not padded
+  unsigned long long* leaf_off;   // [count + 1] of the padded tree (filled here), or null
 };
 
 // Workspace of order_set_batch.
-int ensure_batch(ddm_ctx* c, OrderBufs& o, uint32_t cnt, uint32_t count) {
+int ensure_batch(ddm_ctx* c, OrderBufs& o, int d, uint32_t cnt, uint32_t count) {
   DDM_TRY(ensure_sort(c, o, cnt));
-  DDM_TRY(ensure(c, o.bglog2, sizeof(int) * (count ? count : 1)));
-  DDM_TRY(ensure(c, o.bngroups, sizeof(uint32_t) * (count ? count : 1)));
-  DDM_TRY(ensure(c, o.bgbase, sizeof(unsigned long long) * ((size_t)count + 1)));
-  return ensure(c, o.sums, sizeof(unsigned long long) * ((size_t)cnt / kScanTile + (size_t)count / kScanTile + 2));
+  DDM_TRY(ensure(c, o.bglog2, sizeof(int) * (size_t)d * count));
+  return ensure(c, o.bgbase, sizeof(unsigned long long) * (size_t)d * ((size_t)count + 1));
 }
 
 int order_set_batch(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const float* hi, uint32_t cnt,
                     const BatchSet& bs, float2* aos, int* cur, cudaStream_t s) {
   *cur = 0;
-  DDM_TRY(ensure_batch(c, o, cnt, bs.count));
+  DDM_TRY(ensure_batch(c, o, d, cnt, bs.count));
+  // Sizes are known on the device only, so the chunks of the re-sorts and the
+  // leaves are planned there.
+  auto* gl = static_cast<int*>(o.bglog2.p);
+  auto* cb = static_cast<unsigned long long*>(o.bgbase.p);
+  if (d > 1 || bs.leaf_off)
+    DDM_CUDA(launch_batch_plan(bs.off, bs.count, d, c->str_shift, kSegTileLog2, gl, cb, bs.leaf_off, s));
   DDM_CUDA(launch_fill_inst(bs.off, bs.count, cnt, bs.inst, c->sms, s));
   const int inst_bits = bits_of(bs.count ? bs.count - 1u : 0u), id_bits = id_bits_of(cnt);
   const bool packed = inst_bits + 24 + id_bits <= 64;
@@ -404,17 +411,11 @@ int order_set_batch(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const floa
     DDM_TRY(packed_pass(c, o, cnt, inst_bits ? bs.inst : nullptr, true, 24 + inst_bits, id_bits, cur, s));
   else
     DDM_TRY(sort_pass(c, o, cnt, (24 + inst_bits + 7) / 8, cur, s));
-  // The re-sorts stay inside an instance's groups; the sizes are known on the
-  // device only, so the chunks are planned there.
-  auto* gl = static_cast<int*>(o.bglog2.p);
-  auto* nc = static_cast<uint32_t*>(o.bngroups.p);
-  auto* cb = static_cast<unsigned long long*>(o.bgbase.p);
-  for (int k = 1; k < d; ++k) {
-    DDM_CUDA(launch_seg_plan(bs.off, bs.count, d, k, c->str_shift, kSegTileLog2, gl, nc, s));
-    DDM_CUDA(launch_scan(nc, bs.count, cb, static_cast<unsigned long long*>(o.sums.p), nullptr, s));
-    DDM_TRY(seg_pass(c, o, cnt, lo + (size_t)k * cnt, 0, SegPlan{bs.off, gl, cb, bs.count},
+  // The re-sorts stay inside an instance's groups.
+  for (int k = 1; k < d; ++k)
+    DDM_TRY(seg_pass(c, o, cnt, lo + (size_t)k * cnt, 0,
+                     SegPlan{bs.off, gl + (size_t)k * bs.count, cb + (size_t)k * (bs.count + 1u), bs.count},
                      kSegTileLog2, *cur, s));
-  }
   return DDM_OK;
 }
 
@@ -549,6 +550,8 @@ int build_async(ddm_ctx* c, int d, const float* slo, const float* shi, uint32_t 
   if (!bs) c->bv = BatchView{};
   c->planned = false;
   TreeView t{};
+  const uint32_t set_n = n;
+  if (bs && bs->padded) n = bs->padded;  // positions of the tree; set_n of them hold extents
   t.d = d;
   t.n = n;
   if (n == 0) {
@@ -563,9 +566,11 @@ int build_async(ddm_ctx* c, int d, const float* slo, const float* shi, uint32_t 
   int cur = 0;
   bool gathered = false;
   OrderBufs& o = c->ob[0];
-  float2* aos = aos_buffer(c, o, d, n);
+  float2* aos = aos_buffer(c, o, d, set_n);
+  LeafMap map{};
+  if (bs && bs->padded) map = LeafMap{bs->off, bs->leaf_off, bs->count};
   if (bs)
-    DDM_TRY(order_set_batch(c, o, d, slo, shi, n, *bs, aos, &cur, s));
+    DDM_TRY(order_set_batch(c, o, d, slo, shi, set_n, *bs, aos, &cur, s));
   else if (d >= 2)
     DDM_TRY(order_set_classes(c, o, d, slo, shi, n, aos, &cur, s));
   else
@@ -579,7 +584,7 @@ int build_async(ddm_ctx* c, int d, const float* slo, const float* shi, uint32_t 
   if (d <= 3 && c->tables_on &&
       ensure(c, c->tab, sizeof(uint32_t) * 2u * kRankSlot * (size_t)d * t.cnt[1]) == DDM_OK)
     t.tab = static_cast<const uint32_t*>(c->tab.p);
-  DDM_CUDA(launch_build(t, static_cast<const uint32_t*>(o.vals[cur].p), slo, shi, aos,
+  DDM_CUDA(launch_build(t, set_n, map, static_cast<const uint32_t*>(o.vals[cur].p), slo, shi, aos,
                         static_cast<float2*>(c->e.p), static_cast<uint32_t*>(c->sid.p),
                         static_cast<float2*>(c->nodes.p), const_cast<uint32_t*>(t.tab),
                         c->st_dev, s));
@@ -891,7 +896,7 @@ int build_and_plan(ddm_ctx* c, int d, const float* slo, const float* shi, uint32
     return plan_async(c, ulo, uhi, m, flags, record, false, s, bs_u, sorted);
   };
   if (m > 0 && n > 0) {
-    int rc = bs_u ? ensure_batch(c, o, m, bs_u->count) : ensure_sort(c, o, m);
+    int rc = bs_u ? ensure_batch(c, o, d, m, bs_u->count) : ensure_sort(c, o, m);
     if (rc == DDM_OK) rc = ensure_queries(c, d, m);
     if (rc == DDM_OK) {
       float2* aos = aos_buffer(c, o, d, m);
@@ -995,6 +1000,7 @@ int ddm_destroy(ddm_ctx* c) {
                     &c->sel_offs, &c->sel_list, &c->rec, &c->blk_own, &c->blk_count,
                     &c->pkt_nblk, &c->pkt_off,
                     &c->blk_list, &c->plan_state, &c->order_state, &c->inst_s, &c->inst_u,
+                    &c->leaf_off,
                     &c->cls_hist, &c->cls_off, &c->probe})
     release(*b);
   cudaDeviceSynchronize();  // the stream-ordered frees above have run
@@ -1348,9 +1354,14 @@ static int batch_impl(ddm_ctx* c, int d, uint32_t count, const float* ulo, const
   DDM_TRY(reset_status(c, s));
   const auto* uoff = reinterpret_cast<const unsigned long long*>(upd_off);
   const auto* soff = reinterpret_cast<const unsigned long long*>(sub_off);
-  BatchSet bs_s{soff, count, static_cast<uint32_t*>(c->inst_s.p)};
-  BatchSet bs_u{uoff, count, static_cast<uint32_t*>(c->inst_u.p)};
-  const BatchView bv{count, uoff, soff, static_cast<const uint32_t*>(c->inst_u.p)};
+  // Whole leaves per instance when that adds at most a quarter of positions.
+  const uint64_t positions = ((uint64_t)n + 31ull * count + 31u) / 32u * 32u;
+  const uint32_t padded = n >= 128ull * count && positions <= DDM_MAX_EXTENTS ? (uint32_t)positions : 0u;
+  DDM_TRY(ensure(c, c->leaf_off, sizeof(unsigned long long) * ((size_t)count + 1)));
+  auto* leaf_off = padded ? static_cast<unsigned long long*>(c->leaf_off.p) : nullptr;
+  BatchSet bs_s{soff, count, static_cast<uint32_t*>(c->inst_s.p), padded, leaf_off};
+  BatchSet bs_u{uoff, count, static_cast<uint32_t*>(c->inst_u.p), 0u, nullptr};
+  const BatchView bv{count, uoff, soff, static_cast<const uint32_t*>(c->inst_u.p), leaf_off};
   DDM_TRY(build_and_plan(c, d, slo, shi, n, ulo, uhi, m, flags, true, false, s, &bs_s, &bs_u, &bv));
   // a k_dev or pair_off copy is enqueued behind the write: only a plain
   // synchronising call can hold the walking pass back
@@ -1409,7 +1420,7 @@ int ddm_refit(ddm_ctx* c, const float* sub_lo, const float* sub_hi, void* stream
                              c->st_dev, c->sms, s));
     // Same order, new coordinates: gather through the tree's own id column and
     // recompute every node's per-dimension (minlower, maxupper).
-    DDM_CUDA(launch_build(c->tree, c->tree.sid, sub_lo, sub_hi, aos, static_cast<float2*>(c->e.p),
+    DDM_CUDA(launch_build(c->tree, c->tree.n, LeafMap{}, c->tree.sid, sub_lo, sub_hi, aos, static_cast<float2*>(c->e.p),
                           static_cast<uint32_t*>(c->sid.p), static_cast<float2*>(c->nodes.p),
                           const_cast<uint32_t*>(c->tree.tab), c->st_dev, s));
   }

@@ -69,7 +69,8 @@ struct TreeView {
   // dimension k) / 2k + 1 (upper bounds), kRankSlot words at
   // (g * 2d + slot) * kRankSlot: the leaf's 32 bounds sorted ascending (float
   // bits, padding positions +inf), then at word 35 + c the mask of the leaf
-  // positions holding the c smallest (c = 0..32).
+  // positions holding the c smallest (c = 0..32); word 32 of slot 0 is the
+  // mask of the leaf's positions that hold an extent.
   const uint32_t* tab;
 };
 constexpr uint32_t kRankSlot = 68;  // words per rank-table slot (16-byte multiple)
@@ -107,11 +108,27 @@ struct WriteView {
 // concatenated sets; sorting keeps these ranges (the instance is the major
 // key), so they hold in sorted order too.  q_inst[p] = instance of the update
 // at sorted position p.  count == 0: a single problem.
+//
+// Whole leaves (leaf_off set): the tree's positions are padded so that every
+// instance starts a leaf: instance i owns leaves [leaf_off[i], leaf_off[i+1]),
+// subscriptions in the same order, the rest of its last leaf empty.  Without
+// that, leaves straddle the re-sort groups of an instance (and instances), and
+// the box of such a leaf spans a whole slab, so that every query of the slab
+// tests it: 5.2 leaf tests per query on the 4,096-instance workload.
 struct BatchView {
   uint32_t count;
   const unsigned long long* upd_off;  // [count + 1]
   const unsigned long long* sub_off;  // [count + 1]
   const uint32_t* q_inst;             // [m]
+  const unsigned long long* leaf_off; // [count + 1], or null: positions are not padded
+};
+// How a padded tree's leaves are filled: leaf l holds the sorted positions
+// from off[b] + 32 * (l - leaf_off[b]) on, b the instance owning it; leaves
+// past the last are empty.
+struct LeafMap {
+  const unsigned long long* off;
+  const unsigned long long* leaf_off;  // [count + 1], null: the tree is not padded
+  uint32_t count;
 };
 
 // Exponent of the sort-tile-recursive group size for re-sorting dimension k
@@ -250,9 +267,12 @@ struct ClassPlan {
 };
 cudaError_t launch_class_plan(const uint32_t* hist, int d, int shift, const ClassPlan& plan,
                               cudaStream_t s);
-// Batched sets: glog2 and nchunks (to be scanned into cbase), [count] each.
-cudaError_t launch_seg_plan(const unsigned long long* off, uint32_t count, int d, int k, int shift,
-                            int tile_log2, int* glog2, uint32_t* nchunks, cudaStream_t s);
+// Batched sets: group exponents glog2 [d][count] and first chunks cbase
+// [d][count + 1] of every dimension, and (optional) first leaves leaf_off
+// [count + 1] of a padded tree.
+cudaError_t launch_batch_plan(const unsigned long long* off, uint32_t count, int d, int shift,
+                              int tile_log2, int* glog2, unsigned long long* cbase,
+                              unsigned long long* leaf_off, cudaStream_t s);
 // Stable re-sort of the ids in `vals` by the locality key of lo_k inside each
 // group, in place; with one instance g is its group exponent.  tmp0 and tmp1
 // (`total` words each) are used only by groups larger than a chunk's tile.
@@ -266,9 +286,11 @@ void tree_shape(uint32_t n, int* L, uint32_t* cnt, uint32_t* off, uint32_t* tota
 // re-sorted by lower bound inside aligned groups of 2^glog2[k] positions;
 // `shift` is added to every exponent (tuning knob, 0 = the STR sizes).
 void str_groups(uint32_t n, int d, int* glog2, int shift = 0);
-cudaError_t launch_build(const TreeView& t, const uint32_t* sorted_ids, const float* lo,
-                         const float* hi, const float2* aos, float2* e, uint32_t* sid,
-                         float2* nodes, uint32_t* tab, Status* st, cudaStream_t s);
+// `set_n` extents in lo / hi (t.n unless the tree is padded by `map`).
+cudaError_t launch_build(const TreeView& t, uint32_t set_n, const LeafMap& map,
+                         const uint32_t* sorted_ids, const float* lo, const float* hi,
+                         const float2* aos, float2* e, uint32_t* sid, float2* nodes, uint32_t* tab,
+                         Status* st, cudaStream_t s);
 cudaError_t launch_export_nodes(const TreeView& t, float* node_lo, float* node_hi, cudaStream_t s);
 
 // ---- ddm_query.cu ---------------------------------------------------------

@@ -205,6 +205,9 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
     if (need > w.capacity) return;
   }
 
+  // Batched, leaves of one instance each: a query meeting a leaf's range may
+  // match all of it.
+  const bool whole = !BATCH || bv.leaf_off;
   const uint32_t qpp = 1u << q.qpp_log2;  // queries per packet: 4 to 32
   const uint32_t npk = (q.nq + qpp - 1u) >> q.qpp_log2;
   // Summed over the warp's packets and added once at the end (or before the
@@ -231,12 +234,18 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
     }
     // Position range of the subscriptions this query may match, and the
     // update id written into pairs (instance-local when batched).
-    uint32_t r_lo = 0, r_hi = (uint32_t)n, Qout = WRITE ? Q + w.qbase : Q;
+    uint32_t r_lo = 0, r_hi = (uint32_t)n, Qout = WRITE ? Q + w.qbase : Q, s_base = 0;
     if (WRITE && w.qids && valid) Qout = w.qids[Q];
     if (BATCH && valid) {
       const uint32_t b = bv.q_inst[pos];
-      r_lo = (uint32_t)bv.sub_off[b];
-      r_hi = (uint32_t)bv.sub_off[b + 1];
+      if (whole) {
+        r_lo = (uint32_t)bv.leaf_off[b] * 32u;
+        r_hi = (uint32_t)bv.leaf_off[b + 1] * 32u;
+      } else {
+        r_lo = (uint32_t)bv.sub_off[b];
+        r_hi = (uint32_t)bv.sub_off[b + 1];
+      }
+      if (WRITE) s_base = (uint32_t)bv.sub_off[b];
       Qout = Q - (uint32_t)bv.upd_off[b];
     }
     uint32_t g_lo = 0, g_hi = (uint32_t)n;  // union of the packet's ranges
@@ -330,7 +339,7 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
 #pragma unroll
           for (int j = lane; j < NV; j += 32) dst[j] = __ldg(src + j);
           __syncwarp();
-          uint32_t hbm = __ballot_sync(0xffffffffu, iv);  // padding positions of the last leaf
+          uint32_t hbm = s_tab[wib][32];  // positions that hold an extent
 #pragma unroll
           for (int k = 0; k < D; ++k) {
             const uint32_t* sl = &s_tab[wib][2 * k * kRankSlot];
@@ -347,7 +356,7 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
             hbm &= sl[35 + c] & ~sh[35 + c2];
           }
           __syncwarp();
-          if (BATCH) {  // only this query's instance: positions [r_lo, r_hi)
+          if (!whole) {  // only this query's instance: positions [r_lo, r_hi)
             const uint32_t base = (g1 + cl) * 32u;
             const uint32_t a = r_lo > base ? min(r_lo - base, 32u) : 0u;
             const uint32_t b = r_hi > base ? min(r_hi - base, 32u) : 0u;
@@ -402,8 +411,7 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
               }
             }
             __syncwarp();
-            hbm &= __ballot_sync(0xffffffffu, iv);  // padding lanes of the last leaf
-            if (BATCH) {  // only this query's instance: positions [r_lo, r_hi)
+            if (!whole) {  // only this query's instance: positions [r_lo, r_hi)
               const uint32_t base = (g1 + cl) * 32u;
               const uint32_t a = r_lo > base ? min(r_lo - base, 32u) : 0u;
               const uint32_t b = r_hi > base ? min(r_hi - base, 32u) : 0u;
@@ -426,13 +434,15 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
             const float4* rows = &s_q[wib][0][0];
             uint32_t* hbw = reinterpret_cast<uint32_t*>(&s_q[wib][0][0]);
             auto test = [&](uint32_t r) {
-              if constexpr (D >= 1 && D <= 3 && !BATCH) {
-                const float4 b0 = rows[r], b1 = D == 3 ? rows[r + 1] : b0;
-                hbw[4 * r + HB] = OPEN ? seg_ballot_lt<D>(ev, b0, b1) : seg_ballot_le<D>(ev, b0, b1);
-                return;
+              if constexpr (D >= 1 && D <= 3) {
+                if (whole) {
+                  const float4 b0 = rows[r], b1 = D == 3 ? rows[r + 1] : b0;
+                  hbw[4 * r + HB] = OPEN ? seg_ballot_lt<D>(ev, b0, b1) : seg_ballot_le<D>(ev, b0, b1);
+                  return;
+                }
               }
               bool hit = iv;
-              if (BATCH) {
+              if (!whole) {
                 const uint2 rg = s_rng[wib][r / RW];
                 hit = hit & (i >= rg.x) & (i < rg.y);
               }
@@ -463,11 +473,11 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
             qm &= qm - 1u;
             bool hit = iv;
             uint32_t sub_base = 0;
-            if (BATCH) {
+            if (!whole) {
               const uint2 rg = s_rng[wib][qq];
               hit = hit & (i >= rg.x) & (i < rg.y);
-              sub_base = rg.x;
             }
+            if (BATCH && WRITE) sub_base = __shfl_sync(0xffffffffu, s_base, qq);
   #pragma unroll
             for (int k2 = 0; k2 < DP; ++k2) {
               if (2 * k2 < d) {

@@ -352,15 +352,75 @@ __device__ __forceinline__ uint32_t chunks_of(uint32_t n, int g, uint32_t tile) 
   return (uint32_t)((n + size - 1) / size);
 }
 
-// Batched sets: each instance's group exponent and chunk count for dimension k.
-__global__ void k_seg_plan(const unsigned long long* __restrict__ off, uint32_t count, int d, int k,
-                           int shift, uint32_t tile, int* __restrict__ glog2,
-                           uint32_t* __restrict__ nchunks) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-    const uint32_t n = (uint32_t)(off[i + 1] - off[i]);
-    const int g = used_group(n, d, k, shift);
-    glog2[i] = g;
-    nchunks[i] = chunks_of(n, g, tile);
+// Exclusive scan of one value per thread over 1,024 threads; *total = the sum.
+__device__ __forceinline__ uint32_t scan1024(uint32_t v, uint32_t* s_w, uint32_t* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_w[warp] = x;
+  __syncthreads();
+  uint32_t w = s_w[lane];  // every warp scans the 32 warp totals
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
+    if (lane >= o) w += y;
+  }
+  *total = __shfl_sync(0xffffffffu, w, 31);
+  const uint32_t pre = __shfl_sync(0xffffffffu, w, (warp + 31) & 31);
+  __syncthreads();
+  return (warp ? pre : 0u) + x - v;
+}
+
+// Batched sets (one CTA, 4,096 instances a round): the prefix of leaves of a
+// padded tree and, for every dimension k >= 1, each instance's group exponent
+// and the prefix of chunks.  One launch, where a launch per step (counts,
+// scan) put seven on the way of a small batch.
+__global__ void __launch_bounds__(1024)
+k_batch_plan(const unsigned long long* __restrict__ off, uint32_t count, int d, int shift,
+             uint32_t tile, int* __restrict__ glog2, unsigned long long* __restrict__ cbase,
+             unsigned long long* __restrict__ leaf_off) {
+  constexpr int kEach = 4;
+  __shared__ uint32_t s_w[32];
+  unsigned long long carry[DDM_MAX_DIMS] = {};  // [0]: leaves
+  for (uint32_t c0 = 0; c0 < count; c0 += 1024u * kEach) {
+    uint32_t n[kEach];
+    const uint32_t i0 = c0 + threadIdx.x * kEach;
+#pragma unroll
+    for (int u = 0; u < kEach; ++u) n[u] = i0 + u < count ? (uint32_t)(off[i0 + u + 1] - off[i0 + u]) : 0u;
+#pragma unroll
+    for (int k = 0; k < DDM_MAX_DIMS; ++k) {
+      if (k >= d || (k == 0 && !leaf_off)) continue;
+      uint32_t v[kEach], sum = 0, total;
+#pragma unroll
+      for (int u = 0; u < kEach; ++u) {
+        if (k == 0) {
+          v[u] = (n[u] + 31u) / 32u;
+        } else {
+          const int g = used_group(n[u], d, k, shift);
+          if (i0 + u < count) glog2[(size_t)k * count + i0 + u] = g;
+          v[u] = chunks_of(n[u], g, tile);
+        }
+        sum += v[u];
+      }
+      unsigned long long at = carry[k] + scan1024(sum, s_w, &total);
+      unsigned long long* out = k == 0 ? leaf_off : cbase + (size_t)k * (count + 1u);
+#pragma unroll
+      for (int u = 0; u < kEach; ++u) {
+        if (i0 + u < count) out[i0 + u] = at;
+        at += v[u];
+      }
+      carry[k] += total;
+    }
+  }
+  if (threadIdx.x == 0) {
+    if (leaf_off) leaf_off[count] = carry[0];
+#pragma unroll
+    for (int k = 1; k < DDM_MAX_DIMS; ++k)
+      if (k < d) cbase[(size_t)k * (count + 1u) + count] = carry[k];
   }
 }
 
@@ -448,11 +508,10 @@ cudaError_t ready_group_table() {
   return e;
 }
 
-cudaError_t launch_seg_plan(const unsigned long long* off, uint32_t count, int d, int k, int shift,
-                            int tile_log2, int* glog2, uint32_t* nchunks, cudaStream_t s) {
-  if (count == 0) return cudaSuccess;
-  const uint32_t blocks = (count + 255) / 256 < 1024 ? (count + 255) / 256 : 1024;
-  k_seg_plan<<<blocks, 256, 0, s>>>(off, count, d, k, shift, 1u << tile_log2, glog2, nchunks);
+cudaError_t launch_batch_plan(const unsigned long long* off, uint32_t count, int d, int shift,
+                              int tile_log2, int* glog2, unsigned long long* cbase,
+                              unsigned long long* leaf_off, cudaStream_t s) {
+  k_batch_plan<<<1, 1024, 0, s>>>(off, count, d, shift, 1u << tile_log2, glog2, cbase, leaf_off);
   note_launches(1);
   return cudaGetLastError();
 }

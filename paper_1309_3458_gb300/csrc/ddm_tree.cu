@@ -40,8 +40,10 @@ __device__ __forceinline__ float warp_min(float v) {
 // Sorts the warp's 32 keys ascending (bitonic network over shuffles; ties by
 // lane) and writes them and their prefix masks into one rank-table slot of
 // kRankSlot words: slot[j] = the j-th smallest key, slot[35 + c] = the bits
-// of the lanes holding the c smallest keys (c = 0..32; words 32..35 are 0).
-__device__ __forceinline__ void rank_slot(float key, int lane, uint32_t* __restrict__ slot) {
+// of the lanes holding the c smallest keys (c = 0..32; words 33..35 are 0,
+// word 32 is `w32`).
+__device__ __forceinline__ void rank_slot(float key, int lane, uint32_t w32,
+                                          uint32_t* __restrict__ slot) {
   uint32_t idx = (uint32_t)lane;
 #pragma unroll
   for (int k = 2; k <= 32; k <<= 1) {
@@ -65,35 +67,52 @@ __device__ __forceinline__ void rank_slot(float key, int lane, uint32_t* __restr
   }
   slot[lane] = __float_as_uint(key);
   slot[36 + lane] = m;
-  if (lane < 4) slot[32 + lane] = 0u;
+  if (lane < 4) slot[32 + lane] = lane ? 0u : w32;
 }
 
 // Gather the sorted SoA layout and build levels 1 and 2.  One CTA of 1024
 // threads covers 1024 sorted positions: one warp per level-1 node, and the
-// CTA's 32 level-1 nodes form level-2 node blockIdx.x.  With `tab` (d <= 3)
+// CTA's 32 level-1 nodes form level-2 node blockIdx.x.  In a padded tree (map)
+// a leaf's extents come from its instance, and empty positions hold NaN bounds,
+// which fail every comparison.  With `tab` (d <= 3)
 // it also writes every leaf's rank tables: per dimension k, its 32 lower
 // bounds (slot 2k) and 32 upper bounds (slot 2k + 1) sorted, with prefix
 // masks, padding positions holding +inf.
 __global__ void __launch_bounds__(1024)
-k_gather_build(TreeView t, const uint32_t* __restrict__ sorted_ids, const float* __restrict__ lo,
-               const float* __restrict__ hi, const float2* __restrict__ aos,
-               float2* __restrict__ e, uint32_t* __restrict__ sid, float2* __restrict__ nodes,
-               uint32_t* __restrict__ tab, Status* __restrict__ st) {
+k_gather_build(TreeView t, uint32_t set_n, LeafMap map, const uint32_t* __restrict__ sorted_ids,
+               const float* __restrict__ lo, const float* __restrict__ hi,
+               const float2* __restrict__ aos, float2* __restrict__ e, uint32_t* __restrict__ sid,
+               float2* __restrict__ nodes, uint32_t* __restrict__ tab, Status* __restrict__ st) {
   __shared__ float s_min[DDM_MAX_DIMS][32], s_max[DDM_MAX_DIMS][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t n = t.n;
   const uint32_t i = blockIdx.x * 1024u + threadIdx.x;
-  const bool valid = i < n;
-  uint32_t id = 0;
-  bool valid_id = valid;
-  if (valid) {
-    id = sorted_ids[i];
-    valid_id = DDM_IN_BOUNDS(id < n, st);
-    if (!valid_id) id = 0;
-    sid[i] = id;
-  }
   const uint32_t g = blockIdx.x * 32u + w;
   const bool gvalid = g < t.cnt[1];
+  bool valid = i < n;
+  uint32_t id = 0, from = i;
+  if (map.leaf_off && gvalid) {  // warp-uniform
+    valid = false;
+    if (g < map.leaf_off[map.count]) {
+      // the instance owning leaf g: 32 places a step
+      uint32_t b = 0, hi = map.count;  // leaf_off[b] <= g < leaf_off[hi]
+      while (hi - b > 1) {
+        const uint32_t step = (hi - b + 31u) / 32u, at = b + (uint32_t)lane * step;
+        const uint32_t m = __ballot_sync(0xffffffffu, at < hi && map.leaf_off[at] <= g);
+        b += (31u - __clz(m)) * step;
+        hi = min(hi, b + step);
+      }
+      const unsigned long long j = map.off[b] + (g - map.leaf_off[b]) * 32u + lane;
+      valid = j < map.off[b + 1];
+      from = (uint32_t)j;
+    }
+  }
+  if (valid) {
+    id = sorted_ids[from];
+    if (!DDM_IN_BOUNDS(id < set_n && i < n, st)) id = 0;
+    sid[i] = id;
+  }
+  const uint32_t held = __ballot_sync(0xffffffffu, valid);
   for (int k = 0; k < t.d; ++k) {
     float a = FLT_MAX, b = -FLT_MAX;
     if (valid) {
@@ -102,17 +121,19 @@ k_gather_build(TreeView t, const uint32_t* __restrict__ sorted_ids, const float*
         a = v.x;
         b = v.y;
       } else {
-        a = lo[(size_t)k * n + id];
-        b = hi[(size_t)k * n + id];
+        a = lo[(size_t)k * set_n + id];
+        b = hi[(size_t)k * set_n + id];
       }
       e[(size_t)k * n + i] = make_float2(a, b);
+    } else if (map.leaf_off && i < n) {
+      e[(size_t)k * n + i] = make_float2(NAN, NAN);
     }
     const float mn = warp_min(valid ? a : INFINITY);
     const float mx = warp_max(valid ? b : -INFINITY);
     if (tab && gvalid) {  // warp-uniform
       uint32_t* slot = tab + ((size_t)g * 2u * (uint32_t)t.d + 2u * (uint32_t)k) * kRankSlot;
-      rank_slot(valid ? a : INFINITY, lane, slot);
-      rank_slot(valid ? b : INFINITY, lane, slot + kRankSlot);
+      rank_slot(valid ? a : INFINITY, lane, held, slot);
+      rank_slot(valid ? b : INFINITY, lane, held, slot + kRankSlot);
     }
     if (lane == 0) {
       if (gvalid) nodes[(size_t)k * t.total + t.off[1] + g] = make_float2(mn, mx);
@@ -191,12 +212,14 @@ void str_groups(uint32_t n, int d, int* glog2, int shift) {
   }
 }
 
-cudaError_t launch_build(const TreeView& t, const uint32_t* sorted_ids, const float* lo,
-                         const float* hi, const float2* aos, float2* e, uint32_t* sid,
-                         float2* nodes, uint32_t* tab, Status* st, cudaStream_t s) {
+cudaError_t launch_build(const TreeView& t, uint32_t set_n, const LeafMap& map,
+                         const uint32_t* sorted_ids, const float* lo, const float* hi,
+                         const float2* aos, float2* e, uint32_t* sid, float2* nodes, uint32_t* tab,
+                         Status* st, cudaStream_t s) {
   if (t.n == 0) return cudaSuccess;
   const uint32_t blocks = (t.n + 1023) / 1024;
-  k_gather_build<<<blocks, 1024, 0, s>>>(t, sorted_ids, lo, hi, aos, e, sid, nodes, tab, st);
+  k_gather_build<<<blocks, 1024, 0, s>>>(t, set_n, map, sorted_ids, lo, hi, aos, e, sid, nodes, tab,
+                                         st);
   if (t.L >= 3) k_build_upper<<<1, 1024, 0, s>>>(t, nodes);
   note_launches(t.L >= 3 ? 2u : 1u);
   return cudaGetLastError();
