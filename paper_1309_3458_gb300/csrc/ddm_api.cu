@@ -288,7 +288,8 @@ int ensure_sort(ddm_ctx* c, OrderBufs& o, uint32_t cnt) {
 
 // Radix sort of the keys/ids in buffer pair `cur` over `passes` 8-bit
 // digits; `cur` is updated to the buffer pair holding the result.
-int sort_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, int passes, int* cur, cudaStream_t s) {
+int sort_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, int passes, int* cur, cudaStream_t s,
+              const uint32_t* run_if = nullptr) {
   SortScratch sc;
   sc.keys[0] = static_cast<unsigned long long*>(o.keys[*cur].p);
   sc.keys[1] = static_cast<unsigned long long*>(o.keys[*cur ^ 1].p);
@@ -298,7 +299,7 @@ int sort_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, int passes, int* cur, cuda
   sc.lookback = static_cast<uint32_t*>(o.lookback.p);
   sc.counters = static_cast<uint32_t*>(o.counters.p);
   int out = 0;
-  DDM_CUDA(launch_sort64(sc, cnt, passes, &out, c->st_dev, c->sms, s));
+  DDM_CUDA(launch_sort64(sc, cnt, passes, &out, run_if, c->st_dev, c->sms, s));
   *cur ^= out;
   return DDM_OK;
 }
@@ -324,7 +325,7 @@ int id_bits_of(uint32_t cnt) { return std::max(bits_of(cnt - 1u), 1); }
 // Packed sort of a set (launch_sort_packed): the ids end up in vals[0], so
 // *cur becomes 0.  A source's k32 lies in vals[1].
 int packed_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, const uint32_t* hi, bool source, int key_bits,
-                int id_bits, int* cur, cudaStream_t s) {
+                int id_bits, int* cur, cudaStream_t s, bool words_out = false) {
   SortScratch sc;
   for (int b = 0; b < 2; ++b) {
     sc.keys[b] = static_cast<unsigned long long*>(o.keys[b].p);
@@ -333,7 +334,7 @@ int packed_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, const uint32_t* hi, bool
   sc.hist = static_cast<uint32_t*>(o.hist.p);
   sc.lookback = static_cast<uint32_t*>(o.lookback.p);
   sc.counters = static_cast<uint32_t*>(o.counters.p);
-  const SortSource src{source ? sc.vals[1] : nullptr, hi, 24, id_bits};
+  const SortSource src{source ? sc.vals[1] : nullptr, hi, 24, id_bits, words_out};
   DDM_CUDA(launch_sort_packed(sc, src, cnt, key_bits, c->st_dev, c->sms, s));
   *cur = 0;
   return DDM_OK;
@@ -509,15 +510,17 @@ int order_set(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const float* hi,
                               *gathered ? static_cast<float2*>(c->qe.p) : nullptr,
                               *gathered ? static_cast<uint32_t*>(c->qid.p) : nullptr, c->st_dev, s));
   } else {
-    DDM_CUDA(launch_validate(d, lo, hi, cnt,
-                             tree ? static_cast<unsigned long long*>(o.keys[0].p) : nullptr,
-                             static_cast<uint32_t*>(o.vals[0].p),
-                             tree ? nullptr : static_cast<uint32_t*>(o.vals[1].p), aos, c->st_dev,
-                             c->sms, s));
-    if (tree)
-      DDM_TRY(sort_pass(c, o, cnt, 8, cur, s));
-    else
-      DDM_TRY(packed_pass(c, o, cnt, nullptr, true, 24, id_bits_of(cnt), cur, s));
+    DDM_CUDA(launch_validate(d, lo, hi, cnt, static_cast<uint32_t*>(o.vals[1].p), tree, aos,
+                             c->st_dev, c->sms, s));
+    const int id_bits = id_bits_of(cnt);
+    DDM_TRY(packed_pass(c, o, cnt, nullptr, true, tree ? 32 : 24, id_bits, cur, s, tree));
+    if (tree) {  // ties by upper bound; with long runs of ties the sort by both bounds
+      auto* keys = static_cast<unsigned long long*>(o.keys[0].p);
+      auto* vals = static_cast<uint32_t*>(o.vals[0].p);
+      DDM_CUDA(launch_tie_order(keys, cnt, id_bits, hi, vals, &c->st_dev->redo, c->sms, s));
+      DDM_CUDA(launch_tree_keys(lo, hi, cnt, keys, vals, &c->st_dev->redo, c->sms, s));
+      DDM_TRY(sort_pass(c, o, cnt, 8, cur, s, &c->st_dev->redo));  // an even number: vals[0] either way
+    }
   }
   int glog2[DDM_MAX_DIMS];
   str_groups(cnt, d, glog2, c->str_shift);
@@ -1416,8 +1419,7 @@ int ddm_refit(ddm_ctx* c, const float* sub_lo, const float* sub_hi, void* stream
   Phase phase("ddm refit");
   if (c->tree.n > 0) {
     float2* aos = aos_buffer(c, c->ob[0], c->tree.d, c->tree.n);
-    DDM_CUDA(launch_validate(c->tree.d, sub_lo, sub_hi, c->tree.n, nullptr, nullptr, nullptr, aos,
-                             c->st_dev, c->sms, s));
+    DDM_CUDA(launch_validate(c->tree.d, sub_lo, sub_hi, c->tree.n, nullptr, false, aos, c->st_dev, c->sms, s));
     // Same order, new coordinates: gather through the tree's own id column and
     // recompute every node's per-dimension (minlower, maxupper).
     DDM_CUDA(launch_build(c->tree, c->tree.n, LeafMap{}, c->tree.sid, sub_lo, sub_hi, aos, static_cast<float2*>(c->e.p),

@@ -30,6 +30,8 @@ struct Status {
   unsigned long long aux;  // call-specific (chunk end, ...)
   unsigned long long tests;  // count pass: (query, leaf) tests, 32 subscriptions each
   unsigned int work[2];    // tickets of the packet kernels and of the replay
+  unsigned int redo;       // d = 1 tree: ties too long for the short way
+  unsigned int pad;
 };
 
 __device__ inline void note_out_of_bounds(Status* st) {
@@ -163,16 +165,20 @@ __host__ __device__ inline uint32_t float_key(float f) {
 void note_launches(unsigned count);
 
 // ---- ddm_layout.cu --------------------------------------------------------
-// Validate a set (lo <= hi, no NaN in every dimension) and emit the sort key,
-// if asked for: keys and vals (id) for the d = 1 tree's order, (key(lo0) <<
-// 32 | key(hi0)); k32 for a locality order, the top 24 bits of key(lo0).
+// Validate a set (lo <= hi, no NaN in every dimension) and (k32 set) emit its
+// sort key: key(lo0), whole or its top 24 bits (a locality order).
 // aos (optional, cnt * d float2): an interleaved copy of the coordinates,
 // aos[i*d + k] = (lo_k, hi_k) of extent i, written while validating, so that
 // the gathers by id read one contiguous record per extent instead of 2d
 // scattered words.
 cudaError_t launch_validate(int d, const float* lo, const float* hi, uint32_t cnt,
-                            unsigned long long* keys, uint32_t* vals, uint32_t* k32, float2* aos,
-                            Status* st, int sms, cudaStream_t s);
+                            uint32_t* k32, bool whole_key, float2* aos, Status* st, int sms,
+                            cudaStream_t s);
+// Sort keys of the d = 1 tree's order, (key(lo) << 32 | key(hi)), and ids;
+// nothing when *run_if is 0.
+cudaError_t launch_tree_keys(const float* lo, const float* hi, uint32_t cnt,
+                             unsigned long long* keys, uint32_t* vals, const uint32_t* run_if,
+                             int sms, cudaStream_t s);
 // keys[i] = (i >> glog2) << 24 | the top 24 bits of key(lo_k[vals[i]]): re-sort
 // inside groups; with id_bits > 0 the packed word, above the id vals[i].
 cudaError_t launch_rekey(const uint32_t* vals, const float* lo_k, uint32_t cnt, int glog2,
@@ -222,8 +228,9 @@ size_t sort_lookback_words(uint32_t n);
 // Test hook: one warp polls `word` (which nothing sets) with the sort's
 // bounded wait, at most `limit` polls, and records kErrTimeout.
 cudaError_t launch_debug_wait(const uint32_t* word, uint32_t limit, Status* st, cudaStream_t s);
-cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf, Status* st,
-                          int sms, cudaStream_t s);
+// With `run_if` the kernels do nothing when *run_if is 0.
+cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf,
+                          const uint32_t* run_if, Status* st, int sms, cudaStream_t s);
 // The same for keys that fit one 64-bit word together with the id: words key
 // << id_bits | id, sorted by key_bits bits above id_bits; the ids come out in
 // vals[0].  With a source the words are built from it (its arrays may not
@@ -233,7 +240,14 @@ struct SortSource {
   const uint32_t* hi;   // optional [n]: the part above k32_bits
   int k32_bits;
   int id_bits;
+  bool words_out;       // the sorted words go to keys[0] instead (an even number of passes)
 };
+// Order of a d = 1 tree from the words sorted by lower bound: ties put in the
+// order of their upper bound, ids to vals; *redo (zero before) is set if a
+// run of ties is too long for that.
+cudaError_t launch_tie_order(const unsigned long long* words, uint32_t n, int id_bits,
+                             const float* hi, uint32_t* vals, uint32_t* redo, int sms,
+                             cudaStream_t s);
 cudaError_t launch_sort_packed(SortScratch sc, const SortSource& src, uint32_t n, int key_bits,
                                Status* st, int sms, cudaStream_t s);
 

@@ -3,10 +3,10 @@
 // Every extent must have lo <= hi with no NaN in every dimension (the
 // paper's segments [low, high], Section III-A); a violation raises
 // kErrExtent.  For the subscription set of a d = 1 tree the same pass emits
-// the 64-bit sort key of the interval tree order of Section IV -- lower
-// bound, ties broken by upper bound -- as (key(lo0) << 32 | key(hi0)), and
-// the identity id payload, so a stable radix sort leaves remaining ties in id
-// order.  Every other order (d > 1 trees, the updates) is a locality order:
+// the lower bound's key; ties are put in the order of their upper bounds
+// after the sort (ddm_sort.cu), or, with long runs of them, the set is sorted
+// by (key(lo0) << 32 | key(hi0)): the interval tree order of Section IV, with
+// remaining ties in id order.  Every other order (d > 1 trees, the updates) is a locality order:
 // its keys hold the top 24 bits of key(lo) below a class, group or instance.
 //
 // For d > 1 the order is then refined one dimension at a time: inside
@@ -35,8 +35,8 @@ constexpr int kLocalityDrop = 32 - kLocalityBits;
 
 __global__ void __launch_bounds__(kThreads)
 k_validate(int d, const float* __restrict__ lo, const float* __restrict__ hi, uint32_t cnt,
-           unsigned long long* __restrict__ keys, uint32_t* __restrict__ vals,
-           uint32_t* __restrict__ k32, float2* __restrict__ aos, Status* __restrict__ st) {
+           uint32_t* __restrict__ k32, bool whole_key, float2* __restrict__ aos,
+           Status* __restrict__ st) {
   bool bad = false;
   const uint32_t stride = gridDim.x * blockDim.x;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += stride) {
@@ -47,14 +47,21 @@ k_validate(int d, const float* __restrict__ lo, const float* __restrict__ hi, ui
       bad |= !(a <= b);  // false for NaN as well as for lo > hi
       if (aos) aos[(size_t)i * d + k] = make_float2(a, b);
     }
-    if (keys) {
-      const float a = __ldg(lo + i), b = __ldg(hi + i);
-      keys[i] = ((unsigned long long)float_key(a) << 32) | float_key(b);
-      vals[i] = i;
-    }
-    if (k32) k32[i] = float_key(__ldg(lo + i)) >> kLocalityDrop;
+    if (k32) k32[i] = float_key(__ldg(lo + i)) >> (whole_key ? 0 : kLocalityDrop);
   }
   if (__ballot_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&st->err, kErrExtent);
+}
+
+__global__ void __launch_bounds__(kThreads)
+k_tree_keys(const float* __restrict__ lo, const float* __restrict__ hi, uint32_t cnt,
+            unsigned long long* __restrict__ keys, uint32_t* __restrict__ vals,
+            const uint32_t* __restrict__ run_if) {
+  if (*run_if == 0u) return;
+  const uint32_t stride = gridDim.x * blockDim.x;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += stride) {
+    keys[i] = ((unsigned long long)float_key(__ldg(lo + i)) << 32) | float_key(__ldg(hi + i));
+    vals[i] = i;
+  }
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -280,11 +287,20 @@ cudaError_t launch_rekey_batch(const uint32_t* vals, const float* lo_k, uint32_t
   return cudaGetLastError();
 }
 
-cudaError_t launch_validate(int d, const float* lo, const float* hi, uint32_t cnt,
-                            unsigned long long* keys, uint32_t* vals, uint32_t* k32, float2* aos,
-                            Status* st, int sms, cudaStream_t s) {
+cudaError_t launch_tree_keys(const float* lo, const float* hi, uint32_t cnt,
+                             unsigned long long* keys, uint32_t* vals, const uint32_t* run_if,
+                             int sms, cudaStream_t s) {
   if (cnt == 0) return cudaSuccess;
-  k_validate<<<grid_for(cnt, sms), kThreads, 0, s>>>(d, lo, hi, cnt, keys, vals, k32, aos, st);
+  k_tree_keys<<<grid_for(cnt, sms), kThreads, 0, s>>>(lo, hi, cnt, keys, vals, run_if);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_validate(int d, const float* lo, const float* hi, uint32_t cnt,
+                            uint32_t* k32, bool whole_key, float2* aos, Status* st, int sms,
+                            cudaStream_t s) {
+  if (cnt == 0) return cudaSuccess;
+  k_validate<<<grid_for(cnt, sms), kThreads, 0, s>>>(d, lo, hi, cnt, k32, whole_key, aos, st);
   note_launches(1);
   return cudaGetLastError();
 }

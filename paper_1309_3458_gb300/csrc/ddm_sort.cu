@@ -110,7 +110,9 @@ __global__ void k_debug_wait(const uint32_t* __restrict__ word, uint32_t limit,
 
 // All eight digit histograms in one read of the keys.
 __global__ void __launch_bounds__(kThreads)
-k_histogram(const unsigned long long* __restrict__ keys, uint32_t n, uint32_t* __restrict__ hist) {
+k_histogram(const unsigned long long* __restrict__ keys, uint32_t n, uint32_t* __restrict__ hist,
+            const uint32_t* __restrict__ run_if) {
+  if (run_if && *run_if == 0u) return;
   __shared__ uint32_t h[kPasses * kRadix];
   for (int t = threadIdx.x; t < kPasses * kRadix; t += kThreads) h[t] = 0;
   __syncthreads();
@@ -161,7 +163,9 @@ __global__ void __launch_bounds__(kThreads, 3)
 k_onesweep(const unsigned long long* __restrict__ in_keys, const uint32_t* __restrict__ in_vals,
            unsigned long long* __restrict__ out_keys, uint32_t* __restrict__ out_vals, uint32_t n,
            int shift, const uint32_t* __restrict__ digit_base, uint32_t* __restrict__ lookback,
-           uint32_t* __restrict__ counter, Status* __restrict__ st) {
+           uint32_t* __restrict__ counter, const uint32_t* __restrict__ run_if,
+           Status* __restrict__ st) {
+  if (run_if && *run_if == 0u) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   OnesweepSmem& sm = *reinterpret_cast<OnesweepSmem*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -571,8 +575,9 @@ template <int ITEMS, bool PACKED>
 __global__ void __launch_bounds__(kSmallThreads, ITEMS <= 8 ? 2 : 1)
 k_sort_grid(unsigned long long* __restrict__ keys0, uint32_t* __restrict__ vals0,
             unsigned long long* __restrict__ keys1, uint32_t* __restrict__ vals1, uint32_t n,
-            int passes, SortSource src, uint32_t* __restrict__ table, uint32_t* __restrict__ bar,
-            Status* __restrict__ st) {
+            int passes, SortSource src, const uint32_t* __restrict__ run_if,
+            uint32_t* __restrict__ table, uint32_t* __restrict__ bar, Status* __restrict__ st) {
+  if (run_if && *run_if == 0u) return;  // every CTA alike, before any barrier
   constexpr uint32_t kTile = kSmallThreads * ITEMS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   GridSortSmem<ITEMS, PACKED>& sm = *reinterpret_cast<GridSortSmem<ITEMS, PACKED>*>(smem_raw);
@@ -659,7 +664,7 @@ k_sort_grid(unsigned long long* __restrict__ keys0, uint32_t* __restrict__ vals0
       const uint32_t g = sm.gbase[(uint32_t)(k >> shift) & (kRadix - 1)] + q;
       if (!DDM_IN_BOUNDS(g < n, st)) continue;
       if constexpr (PACKED) {
-        if (p + 1 < passes)
+        if (p + 1 < passes || src.words_out)
           ok[g] = k;
         else
           vals0[g] = (uint32_t)(k & ((1ull << src.id_bits) - 1ull));
@@ -721,7 +726,8 @@ template <int ITEMS, bool PACKED>
 __global__ void __launch_bounds__(kSmallThreads, 1)
 k_sort_cluster(const unsigned long long* __restrict__ in_k, const uint32_t* __restrict__ in_v,
                unsigned long long* __restrict__ out_k, uint32_t* __restrict__ out_v, uint32_t n,
-               int passes, SortSource src) {
+               int passes, SortSource src, const uint32_t* __restrict__ run_if) {
+  if (run_if && *run_if == 0u) return;  // every CTA of the cluster alike
   constexpr uint32_t kTile = kSmallThreads * ITEMS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ClusterSortSmem<ITEMS, PACKED>& sm = *reinterpret_cast<ClusterSortSmem<ITEMS, PACKED>*>(smem_raw);
@@ -786,7 +792,10 @@ k_sort_cluster(const unsigned long long* __restrict__ in_k, const uint32_t* __re
       if (!DDM_IN_BOUNDS(g < n, nullptr)) continue;
       if (last) {
         if constexpr (PACKED) {
-          out_v[g] = (uint32_t)(k & ((1ull << src.id_bits) - 1ull));
+          if (src.words_out)
+            out_k[g] = k;
+          else
+            out_v[g] = (uint32_t)(k & ((1ull << src.id_bits) - 1ull));
         } else {
           out_k[g] = k;
           out_v[g] = sm.stage_v[q];
@@ -805,6 +814,53 @@ k_sort_cluster(const unsigned long long* __restrict__ in_k, const uint32_t* __re
       key[i] = local < valid ? sm.tile_k[local] : ~0ull;
       if constexpr (!PACKED) val[i] = local < valid ? sm.tile_v[local] : 0u;
     }
+  }
+}
+
+// The d = 1 tree's order is by lower bound, upper bound, id.  The upper bound
+// matters only among equal lower bounds, so the set is sorted by the lower
+// bound alone (four digits instead of eight), and the thread at the start of
+// each run of equal keys puts the run in the order of the upper bounds
+// (stably: ids ascend already).  Runs longer than kMaxRun ask for the full
+// sort (*redo), which waits behind this in launches that do nothing otherwise.
+constexpr uint32_t kMaxRun = 32;
+__global__ void __launch_bounds__(256)
+k_tie_order(const unsigned long long* __restrict__ words, uint32_t n, int id_bits,
+            const float* __restrict__ hi, uint32_t* __restrict__ vals, uint32_t* __restrict__ redo) {
+  const unsigned long long idm = (1ull << id_bits) - 1ull;
+  for (uint32_t i = blockIdx.x * 256u + threadIdx.x; i < n; i += gridDim.x * 256u) {
+    const unsigned long long w = words[i], k = w >> id_bits;
+    if (i > 0 && (words[i - 1] >> id_bits) == k) continue;  // inside a run
+    if (i + 1 == n || (words[i + 1] >> id_bits) != k) {
+      vals[i] = (uint32_t)(w & idm);
+      continue;
+    }
+    uint32_t len = 1, last = float_key(__ldg(hi + (uint32_t)(w & idm)));
+    bool ordered = true;
+    for (; i + len < n; ++len) {
+      const unsigned long long v = words[i + len];
+      if ((v >> id_bits) != k) break;
+      if (len == kMaxRun) {
+        *redo = 1u;
+        return;  // the full sort overwrites vals
+      }
+      const uint32_t u = float_key(__ldg(hi + (uint32_t)(v & idm)));
+      ordered = ordered && last <= u;
+      last = u;
+    }
+    if (ordered) {
+      for (uint32_t j = 0; j < len; ++j) vals[i + j] = (uint32_t)(words[i + j] & idm);
+      continue;
+    }
+    unsigned long long run[kMaxRun];  // (upper bound, id), insertion sort
+    for (uint32_t j = 0; j < len; ++j) {
+      const uint32_t id = (uint32_t)(words[i + j] & idm);
+      const unsigned long long x = ((unsigned long long)float_key(__ldg(hi + id)) << 32) | id;
+      uint32_t at = j;
+      for (; at > 0 && run[at - 1] > x; --at) run[at] = run[at - 1];
+      run[at] = x;
+    }
+    for (uint32_t j = 0; j < len; ++j) vals[i + j] = (uint32_t)run[j];
   }
 }
 
@@ -856,7 +912,7 @@ int cluster_sort_ctas() {
 // true then (or an error), else nothing is enqueued.
 template <int ITEMS, bool PACKED>
 cudaError_t try_sort_cluster(SortScratch sc, const SortSource& src, uint32_t n, int passes,
-                             cudaStream_t s, bool* done) {
+                             const uint32_t* run_if, cudaStream_t s, bool* done) {
   *done = false;
   constexpr uint32_t kTile = kSmallThreads * ITEMS;
   const uint32_t ctas = (n + kTile - 1) / kTile;
@@ -875,7 +931,7 @@ cudaError_t try_sort_cluster(SortScratch sc, const SortSource& src, uint32_t n, 
   cfg.numAttrs = 1;
   const int out = PACKED ? 0 : passes & 1;
   cudaError_t e = cudaLaunchKernelEx(&cfg, k_sort_cluster<ITEMS, PACKED>, sc.keys[0], sc.vals[0],
-                                     sc.keys[out], sc.vals[out], n, passes, src);
+                                     sc.keys[out], sc.vals[out], n, passes, src, run_if);
   if (e == cudaSuccess) {
     note_launches(1);
     *done = true;
@@ -911,8 +967,8 @@ int grid_sort_tiles(int sms) {
 // One cooperative launch of k_sort_grid if the set fits its resident grid:
 // *done = true then (or an error), else nothing is enqueued.
 template <int ITEMS, bool PACKED>
-cudaError_t try_sort_grid(SortScratch sc, const SortSource& src, uint32_t n, int passes, Status* st,
-                          int sms, cudaStream_t s, bool* done) {
+cudaError_t try_sort_grid(SortScratch sc, const SortSource& src, uint32_t n, int passes,
+                          const uint32_t* run_if, Status* st, int sms, cudaStream_t s, bool* done) {
   *done = false;
   constexpr uint32_t kTile = kSmallThreads * ITEMS;
   const uint32_t tiles = (n + kTile - 1) / kTile;
@@ -932,7 +988,7 @@ cudaError_t try_sort_grid(SortScratch sc, const SortSource& src, uint32_t n, int
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   e = cudaLaunchKernelEx(&cfg, k_sort_grid<ITEMS, PACKED>, sc.keys[0], sc.vals[0], sc.keys[1], sc.vals[1],
-                         n, passes, src, sc.lookback, sums + kGridSumWords, st);
+                         n, passes, src, run_if, sc.lookback, sums + kGridSumWords, st);
   if (e == cudaErrorCooperativeLaunchTooLarge) {  // fewer SMs available than counted
     cudaGetLastError();
     return cudaSuccess;
@@ -962,8 +1018,8 @@ namespace {
 
 // The one-launch forms, smallest first: *done = false if none fits.
 template <bool PACKED>
-cudaError_t sort_in_one(SortScratch sc, const SortSource& src, uint32_t n, int passes, Status* st,
-                        int sms, cudaStream_t s, bool* done) {
+cudaError_t sort_in_one(SortScratch sc, const SortSource& src, uint32_t n, int passes,
+                        const uint32_t* run_if, Status* st, int sms, cudaStream_t s, bool* done) {
   // Up to 16 tiles of 2,048 keys: one cluster, keys kept on chip; else one
   // cooperative launch when every tile can be resident at once, with the
   // smallest tile that allows it.  Measured (8 passes, one GB300): 5,000
@@ -973,10 +1029,10 @@ cudaError_t sort_in_one(SortScratch sc, const SortSource& src, uint32_t n, int p
   // with the same attributes): 256 batched instances in a graph took 187 us
   // with the multi-launch form recorded instead, 149 with these.
   cudaError_t e;
-  if ((e = try_sort_cluster<4, PACKED>(sc, src, n, passes, s, done)) || *done) return e;
-  if ((e = try_sort_grid<4, PACKED>(sc, src, n, passes, st, sms, s, done)) || *done) return e;
-  if ((e = try_sort_grid<8, PACKED>(sc, src, n, passes, st, sms, s, done)) || *done) return e;
-  return try_sort_grid<16, PACKED>(sc, src, n, passes, st, sms, s, done);
+  if ((e = try_sort_cluster<4, PACKED>(sc, src, n, passes, run_if, s, done)) || *done) return e;
+  if ((e = try_sort_grid<4, PACKED>(sc, src, n, passes, run_if, st, sms, s, done)) || *done) return e;
+  if ((e = try_sort_grid<8, PACKED>(sc, src, n, passes, run_if, st, sms, s, done)) || *done) return e;
+  return try_sort_grid<16, PACKED>(sc, src, n, passes, run_if, st, sms, s, done);
 }
 
 cudaError_t clear_onesweep(SortScratch sc, uint32_t tiles, int passes, cudaStream_t s) {
@@ -1002,20 +1058,30 @@ cudaError_t onesweep_packed_pass(SortScratch sc, const SortSource& src, uint32_t
 
 }  // namespace
 
+cudaError_t launch_tie_order(const unsigned long long* words, uint32_t n, int id_bits,
+                             const float* hi, uint32_t* vals, uint32_t* redo, int sms,
+                             cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  const uint32_t need = (n + 255) / 256, cap = (uint32_t)sms * 64u;
+  k_tie_order<<<need < cap ? need : cap, 256, 0, s>>>(words, n, id_bits, hi, vals, redo);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_sort_packed(SortScratch sc, const SortSource& src, uint32_t n, int key_bits,
                                Status* st, int sms, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   const int passes = std::max((key_bits + kRadixBits - 1) / kRadixBits, 1);
   cudaError_t e;
   bool done = false;
-  if ((e = sort_in_one<true>(sc, src, n, passes, st, sms, s, &done)) || done) return e;
+  if ((e = sort_in_one<true>(sc, src, n, passes, nullptr, st, sms, s, &done)) || done) return e;
   const uint32_t tiles = (n + kSortTile - 1) / kSortTile;
   if ((e = clear_onesweep(sc, tiles, passes, s))) return e;
   const uint32_t hb = std::min((n + kThreads * 16 - 1) / (kThreads * 16), (uint32_t)sms * 8u);
   k_histogram_packed<<<hb, kThreads, 0, s>>>(sc.keys[0], src, n, passes, sc.hist);
   k_hist_scan<<<passes, kRadix, 0, s>>>(sc.hist);
   for (int p = 0; p < passes; ++p) {
-    const bool first = p == 0 && src.k32, last = p + 1 == passes;
+    const bool first = p == 0 && src.k32, last = p + 1 == passes && !src.words_out;
     e = first ? (last ? onesweep_packed_pass<true, true>(sc, src, n, p, st, s)
                       : onesweep_packed_pass<true, false>(sc, src, n, p, st, s))
               : (last ? onesweep_packed_pass<false, true>(sc, src, n, p, st, s)
@@ -1026,14 +1092,14 @@ cudaError_t launch_sort_packed(SortScratch sc, const SortSource& src, uint32_t n
   return cudaSuccess;
 }
 
-cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf, Status* st,
-                          int sms, cudaStream_t s) {
+cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf,
+                          const uint32_t* run_if, Status* st, int sms, cudaStream_t s) {
   *out_buf = 0;
   if (n <= 1 || passes <= 0) return cudaSuccess;
   if (passes > kPasses) passes = kPasses;
   cudaError_t e;
   bool done = false;
-  if ((e = sort_in_one<false>(sc, SortSource{}, n, passes, st, sms, s, &done)) || done) {
+  if ((e = sort_in_one<false>(sc, SortSource{}, n, passes, run_if, st, sms, s, &done)) || done) {
     *out_buf = passes & 1;
     return e;
   }
@@ -1041,7 +1107,7 @@ cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf, 
   if ((e = clear_onesweep(sc, tiles, passes, s))) return e;
   uint32_t hb = (n + kThreads * 16 - 1) / (kThreads * 16);
   if (hb > (uint32_t)sms * 4u) hb = (uint32_t)sms * 4u;
-  k_histogram<<<hb, kThreads, 0, s>>>(sc.keys[0], n, sc.hist);
+  k_histogram<<<hb, kThreads, 0, s>>>(sc.keys[0], n, sc.hist, run_if);
   k_hist_scan<<<kPasses, kRadix, 0, s>>>(sc.hist);
   const size_t smem = sizeof(OnesweepSmem);
   if ((e = cudaFuncSetAttribute(k_onesweep, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1053,7 +1119,7 @@ cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf, 
                                              sc.vals[src ^ 1], n, p * kRadixBits,
                                              sc.hist + p * kRadix,
                                              sc.lookback + (size_t)p * tiles * kRadix,
-                                             sc.counters + p, st);
+                                             sc.counters + p, run_if, st);
   }
   note_launches(2u + (unsigned)passes);
   *out_buf = passes & 1;
