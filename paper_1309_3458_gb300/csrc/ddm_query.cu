@@ -59,6 +59,13 @@ constexpr uint32_t kCompareSwapMin = 24;
 #define DDM_PACKET_MIN_BLOCKS 4
 #endif
 
+// The d = 1 count pass fits six in 40 registers and, waiting for memory most of
+// the time, gains by them: 1.71 ms with four at 2.5e7 + 2.5e7 extents, 1.52
+// with five, 1.46 with six.
+template <int D, bool WRITE>
+constexpr int packet_ctas() {
+  return D == 1 && !WRITE ? 6 : DDM_PACKET_MIN_BLOCKS;
+}
 template <bool OPEN>
 __device__ __forceinline__ bool le(float a, float b) {
   return OPEN ? (a < b) : (a <= b);
@@ -70,16 +77,17 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   return r;
 }
 
+// Largest / smallest value of the warp (sm_100 has the float reduction; five
+// shuffles and five selects otherwise).
 __device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
 }
-
 __device__ __forceinline__ float warp_min(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
+  float r;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
 }
 
 // Ballot of the d-dimensional segment test (Alg. 1 in every dimension,
@@ -170,7 +178,7 @@ DDM_SEG_OR(lt)
 // BATCH: every query matches only its instance's subscription positions, and
 // pairs carry instance-local ids.
 template <int D, bool OPEN, bool WRITE, bool BATCH>
-__global__ void __launch_bounds__(kThreads, DDM_PACKET_MIN_BLOCKS)
+__global__ void __launch_bounds__(kThreads, packet_ctas<D, WRITE>())
 k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
           uint32_t* __restrict__ counts_pos, RecordArena ra, WriteView w,
           uint32_t* __restrict__ work, Status* __restrict__ st) {
@@ -567,36 +575,50 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
       }
     };
 
-    if (t.L == 1) {
-      leaves(0);
+    // The up to 32 level-l nodes from b on that meet the packet's box (and,
+    // batched, its instances' positions).
+    auto meeting = [&](int l, uint32_t b) {
+      const uint32_t ch = b + lane;
+      const bool cv = ch < t.cnt[l];
+      bool ok = cv;
+      if (BATCH) {  // a node that exists spans no more positions than the tree
+        const int sh = kLog2Fan * l;
+        ok = ok && (ch << sh) < g_hi && ((ch + 1u) << sh) > g_lo;
+      }
+#pragma unroll
+      for (int k = 0; k < DM; ++k) {
+        if (k < d) {
+          const float2 v = cv ? t.nodes[k * total + t.off[l] + ch] : make_float2(INFINITY, -INFINITY);
+          ok = ok & le<OPEN>(v.x, gh[k]) & le<OPEN>(gl[k], v.y);
+        }
+      }
+      return __ballot_sync(0xffffffffu, ok);
+    };
+    // Where the walk starts: at the top level, or, batched, at the lowest level
+    // where 32 nodes span the packet's instances (a small instance's leaves).
+    int top = t.L;
+    uint32_t from = 0;
+    bool walk = true;
+    if (BATCH) {
+      walk = g_hi > g_lo;
+      for (top = 1; top < t.L; ++top)
+        if (((g_hi - 1u) >> (kLog2Fan * top)) - (g_lo >> (kLog2Fan * top)) < 32u) break;
+      from = top < t.L ? g_lo >> (kLog2Fan * top) : 0u;
+    }
+    if (!walk) {
+    } else if (top == 1) {
+      leaves(from);
     } else {
-      // Depth-first walk over levels L..2; mask[l] holds the surviving, not
+      // Depth-first walk over levels top..2; mask[l] holds the surviving, not
       // yet visited nodes among the 32 level-l nodes starting at base[l].
       uint32_t mask[kMaxLevels + 1], base[kMaxLevels + 1];
-      int lvl = t.L;
-      {
-        const bool cv = (uint32_t)lane < t.cnt[lvl];
-        bool ok = cv;
-        if (BATCH) {
-          const unsigned long long span = 1ull << (kLog2Fan * lvl);
-          ok = ok && (unsigned long long)lane * span < g_hi &&
-               ((unsigned long long)lane + 1) * span > g_lo;
-        }
-#pragma unroll
-        for (int k = 0; k < DM; ++k) {
-          if (k < d) {
-            const float2 v = cv ? t.nodes[k * total + t.off[lvl] + lane]
-                                : make_float2(INFINITY, -INFINITY);
-            ok = ok & le<OPEN>(v.x, gh[k]) & le<OPEN>(gl[k], v.y);
-          }
-        }
-        mask[lvl] = __ballot_sync(0xffffffffu, ok);
-        base[lvl] = 0;
-      }
+      int lvl = top;
+      mask[lvl] = meeting(lvl, from);
+      base[lvl] = from;
       for (;;) {
         const uint32_t mk = mask[lvl];
         if (mk == 0u) {
-          if (lvl == t.L) break;
+          if (lvl == top) break;
           ++lvl;
           continue;
         }
@@ -605,24 +627,8 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
         if (lvl == 2) {
           leaves(g * 32u);
         } else {
-          const uint32_t ch = g * 32u + lane;
-          const bool cv = ch < t.cnt[lvl - 1];
-          bool ok = cv;
-          if (BATCH) {
-            const unsigned long long span = 1ull << (kLog2Fan * (lvl - 1));
-            ok = ok && (unsigned long long)ch * span < g_hi &&
-                 ((unsigned long long)ch + 1) * span > g_lo;
-          }
-#pragma unroll
-          for (int k = 0; k < DM; ++k) {
-            if (k < d) {
-              const float2 v = cv ? t.nodes[k * total + t.off[lvl - 1] + ch]
-                                  : make_float2(INFINITY, -INFINITY);
-              ok = ok & le<OPEN>(v.x, gh[k]) & le<OPEN>(gl[k], v.y);
-            }
-          }
           --lvl;
-          mask[lvl] = __ballot_sync(0xffffffffu, ok);
+          mask[lvl] = meeting(lvl, g * 32u);
           base[lvl] = g * 32u;
         }
       }
@@ -968,7 +974,6 @@ __device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, OUT>& sm, const 
         continue;
       }
       __syncwarp();
-#pragma unroll 1
       constexpr int G = ReplayShape<OUT>::group;
       for (int g = 0; g < 32; g += G) {
         uint4 rr[G];
@@ -1071,7 +1076,7 @@ cudaError_t launch_packets(const TreeView& t, const QueryView& q, const BatchVie
   qv.take_log2 = packets / (blocks * kWarps) >= 32u ? 2u : 0u;
   // With every warp resident at once each takes one packet, without tickets
   // (and without the counter to clear).
-  if (blocks <= (uint32_t)sms * DDM_PACKET_MIN_BLOCKS && packets <= blocks * kWarps) {
+  if (blocks <= (uint32_t)sms * packet_ctas<0, WRITE>() && packets <= blocks * kWarps) {
     work = nullptr;
   } else if (!zeroed) {
     cudaError_t e = cudaMemsetAsync(work, 0, sizeof(uint32_t), s);
