@@ -61,10 +61,12 @@ constexpr uint32_t kCompareSwapMin = 24;
 
 // The d = 1 count pass fits six in 40 registers and, waiting for memory most of
 // the time, gains by them: 1.71 ms with four at 2.5e7 + 2.5e7 extents, 1.52
-// with five, 1.46 with six.
+// with five, 1.46 with six.  For d > 3 the bounds of more dimensions want more
+// registers: the pass of 33,333 queries (d = 5) took 1.17 ms with four CTAs,
+// 1.02 with three, 1.09 with two (2.75 with a run-time dimension count).
 template <int D, bool WRITE>
 constexpr int packet_ctas() {
-  return D == 1 && !WRITE ? 6 : DDM_PACKET_MIN_BLOCKS;
+  return WRITE ? DDM_PACKET_MIN_BLOCKS : D == 1 ? 6 : D > 3 ? 3 : DDM_PACKET_MIN_BLOCKS;
 }
 template <bool OPEN>
 __device__ __forceinline__ bool le(float a, float b) {
@@ -174,7 +176,8 @@ DDM_SEG_OR(le)
 DDM_SEG_OR(lt)
 #undef DDM_SEG_OR
 
-// D > 0: compile-time dimension count; D == 0: runtime d (up to 8).
+// D > 0: compile-time dimension count (every count pass; write passes up to
+// 3); D == 0: runtime d (up to 8).
 // BATCH: every query matches only its instance's subscription positions, and
 // pairs carry instance-local ids.
 template <int D, bool OPEN, bool WRITE, bool BATCH>
@@ -887,12 +890,16 @@ __device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, OUT>& sm, const 
       continue;
     }
     const uint32_t* rec = ra.rec + (size_t)blk * kRecWords;
+    // SHORT: the records of both blocks as one sequence; else one block after
+    // the other (a select per load would cost the long entries 3%).
+    uint32_t todo = SHORT ? nrec : na, rest = SHORT ? 0u : nrec - na;
+    for (;;) {
     const uint16_t* rel = reinterpret_cast<const uint16_t*>(rec + 2u * kRecBlock);
     uint32_t nx = 0u, nhb = 0u, nrel = 0u;
     auto load = [&](uint32_t r0) {
       const uint32_t r = r0 + (uint32_t)lane;
-      if (r < nrec) {
-        if (na != nrec && r >= na) {  // the second of two blocks
+      if (r < todo) {
+        if (SHORT && r >= na) {  // the second of two blocks
           const uint32_t* r2 = rec + kRecWords;
           nx = ld_hinted(&r2[r - na], stream);
           nhb = ld_hinted(&r2[kRecBlock + r - na], stream);
@@ -909,7 +916,7 @@ __device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, OUT>& sm, const 
     // before the block
     const uint32_t hdr =
         lane < (int)kRecHdr ? ld_hinted(&rec[2u * kRecBlock + kRecBlock / 2u + lane], stream) : 0u;
-    for (uint32_t r0 = 0; r0 < nrec; r0 += 32u) {
+    for (uint32_t r0 = 0; r0 < todo; r0 += 32u) {
       const uint32_t x = nx, xrel = nrel;
       uint32_t hb = nhb;
       nx = nhb = nrel = 0u;  // lanes past the block's last record hold x = hb = 0
@@ -1004,6 +1011,11 @@ __device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, OUT>& sm, const 
         }
       }
     }
+    if (rest == 0u) break;
+    rec += kRecWords;
+    todo = rest;
+    rest = 0u;
+    }
     if (!SHORT) take();
   }
 }
@@ -1054,7 +1066,21 @@ void dispatch_packets(int d, bool open, uint32_t blocks, cudaStream_t s, const T
     case 1: open ? DDM_LAUNCH(1, true) : DDM_LAUNCH(1, false); break;
     case 2: open ? DDM_LAUNCH(2, true) : DDM_LAUNCH(2, false); break;
     case 3: open ? DDM_LAUNCH(3, true) : DDM_LAUNCH(3, false); break;
-    default: open ? DDM_LAUNCH(0, true) : DDM_LAUNCH(0, false); break;
+#define DDM_COUNT(DD)                                          \
+  if constexpr (!WRITE) {                                       \
+    open ? DDM_LAUNCH(DD, true) : DDM_LAUNCH(DD, false);        \
+    break;                                                      \
+  }                                                             \
+  [[fallthrough]]
+    case 4: DDM_COUNT(4);
+    case 5: DDM_COUNT(5);
+    case 6: DDM_COUNT(6);
+    case 7: DDM_COUNT(7);
+    case 8: DDM_COUNT(8);
+#undef DDM_COUNT
+    default:
+      if constexpr (WRITE) open ? DDM_LAUNCH(0, true) : DDM_LAUNCH(0, false);
+      break;
   }
 #undef DDM_LAUNCH
 }
