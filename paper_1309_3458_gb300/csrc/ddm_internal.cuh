@@ -263,8 +263,8 @@ cudaError_t launch_rank_sort(int mode, int d, const float* lo, const float* hi, 
 // ---- ddm_segsort.cu -------------------------------------------------------
 // Thresholds of the group exponents, before the first plan on a device.
 cudaError_t ready_group_table();
-// Positions a CTA re-sorts at once (log2 12 or 13).
-constexpr int kSegTileLog2 = 12, kSegTileLog2Max = 13;
+// Positions a CTA re-sorts at once (log2 10 to 13).
+constexpr int kSegTileLog2Min = 10, kSegTileLog2 = 12, kSegTileLog2Max = 13;
 // A set's re-sort in one dimension, by instance (off null: one instance).
 struct SegPlan {
   const unsigned long long* off;    // [count + 1] positions of each instance

@@ -59,8 +59,8 @@ __device__ __forceinline__ uint32_t same_digit(uint32_t dig) {
 // so they rank last; warps without a valid element skip the ranking.  The
 // ballots of all items come first: only a read and a write of the warp's
 // counters per item are left in the serial chain.
-template <int THREADS, int ITEMS>
-__device__ __forceinline__ void rank_digit(SegSmem<THREADS, ITEMS>& sm,
+template <int THREADS, int ITEMS, typename Smem>
+__device__ __forceinline__ void rank_digit(Smem& sm,
                                            const unsigned long long (&word)[ITEMS],
                                            uint32_t (&rank)[ITEMS], uint32_t valid, int shift) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -129,9 +129,9 @@ __device__ __forceinline__ void rank_digit(SegSmem<THREADS, ITEMS>& sm,
 // the chunk, in as many bits as the range needs, with the group above that:
 // coordinates of one scale range over some 20 of the 24 bits, so that a
 // chunk of several groups usually takes three digits instead of four.
-template <int THREADS, int ITEMS>
-__device__ __forceinline__ void sort_chunk(SegSmem<THREADS, ITEMS>& sm, uint32_t* vals,
-                                           const float* lo_k, uint32_t len, int g) {
+template <int THREADS, int ITEMS, typename Smem>
+__device__ __forceinline__ void sort_chunk(Smem& sm, uint32_t* vals, const float* lo_k,
+                                           uint32_t len, int g) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool any = (uint32_t)warp * (ITEMS * 32) < len;  // warps past the chunk idle
   unsigned long long word[ITEMS];
@@ -296,8 +296,12 @@ k_segsort(uint32_t* __restrict__ vals, const float* __restrict__ lo_k, uint32_t 
     const uint32_t len = (uint32_t)(end - begin);
     if (len > kTile)
       sort_large_group<THREADS, ITEMS>(sm, vals + begin, lo_k, len, tmp0 + begin, tmp1 + begin);
-    else if (len > 1)
+    else if (len > THREADS * 2 || (ITEMS == 2 && len > THREADS))
       sort_chunk<THREADS, ITEMS>(sm, vals + begin, lo_k, len, g);
+    else if (len > THREADS)
+      sort_chunk<THREADS, 2>(sm, vals + begin, lo_k, len, g);
+    else if (len > 1)
+      sort_chunk<THREADS, 1>(sm, vals + begin, lo_k, len, g);
   }
 }
 
@@ -527,8 +531,12 @@ cudaError_t launch_segsort(uint32_t* vals, const float* lo_k, uint32_t total, in
                            const SegPlan& plan, int tile_log2, unsigned long long* tmp0,
                            unsigned long long* tmp1, int sms, cudaStream_t s) {
   if (total <= 1) return cudaSuccess;
-  if (tile_log2 != kSegTileLog2)
+  if (tile_log2 == kSegTileLog2Max)
     return launch_segsort_items<1024, 8>(vals, lo_k, total, g, plan, tmp0, tmp1, sms, s);
+  if (tile_log2 == 10)
+    return launch_segsort_items<1024, 1>(vals, lo_k, total, g, plan, tmp0, tmp1, sms, s);
+  if (tile_log2 == 11)
+    return launch_segsort_items<1024, 2>(vals, lo_k, total, g, plan, tmp0, tmp1, sms, s);
   // More chunks than SMs: CTAs of half the threads, two to an SM, so that one
   // ranks while the other waits (2 x 2.9e7 positions of 4,096 instances: 2.00
   // ms with CTAs of 1,024 threads and all 24 key bits, 1.34 now).  Else a
