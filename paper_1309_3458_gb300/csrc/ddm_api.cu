@@ -879,14 +879,13 @@ int write_ordered_async(ddm_ctx* c, uint32_t pb, uint32_t pe, ddm_pair* pairs, u
   return DDM_OK;
 }
 
-int release_now(ddm_ctx* c, DevBuf& b) {
+void release_now(ddm_ctx* c, DevBuf& b) {
   if (b.p) {
     cudaFreeAsync(b.p, c->cur);
     c->allocated -= b.cap;
   }
   b.p = nullptr;
   b.cap = 0;
-  return DDM_OK;
 }
 
 // Build and plan of a one-shot call: the updates are ordered on the context's
@@ -924,8 +923,10 @@ int build_and_plan(ddm_ctx* c, int d, const float* slo, const float* shi, uint32
       }
     }
     if (rc != DDM_ERR_NOMEM) return rc;
-    for (DevBuf* b : o.all) release_now(c, *b);
-    release_now(c, o.sums);
+    if (!c->capturing) {  // a recorded call neither allocates nor frees
+      for (DevBuf* b : o.all) release_now(c, *b);
+      release_now(c, o.sums);
+    }
   }
   DDM_TRY(build_async(c, d, slo, shi, n, s, bs_s));
   return sequel(false);

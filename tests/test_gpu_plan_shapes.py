@@ -136,3 +136,60 @@ def test_order_by_counting(ctx, n):
     K, pu, ps = gpu_match(ctx, arrays)
     _, ou, os_ = oracle.itm_pairs(*arrays)
     assert np.array_equal(np.sort(keys(pu, ps)), np.sort(keys(ou, os_)))
+
+
+def test_staged_calls_after_one_shot(ctx):
+    """A one-shot call leaves a plan whose order's offsets and entries are made
+    by the first staged call that needs them: the same as ddm_plan's."""
+    import torch
+    m, n = 5003, 4001
+    U = to_dev(sparse_with_wide(m, n, 2, wide=9, seed=3))
+    order = [torch.empty(m, dtype=torch.int32, device="cuda") for _ in range(3)]
+    offs = [torch.empty(m + 1, dtype=torch.int64, device="cuda") for _ in range(3)]
+    ids = [None] * 3
+    for i in range(3):
+        if i == 0:
+            ddm.ddm_build(ctx, U[2], U[3])
+            K = ddm.ddm_plan(ctx, U[0], U[1])
+        elif i == 1:
+            pairs = torch.empty((K, 2), dtype=torch.int32, device="cuda")
+            assert ddm.ddm_match(ctx, *U, pairs) == K
+        else:
+            assert ddm.ddm_count(ctx, *U) == K
+        ids[i] = torch.empty(K, dtype=torch.int32, device="cuda")
+        e = ddm.ddm_chunk_end_ordered(ctx, 0, K // 2)
+        k = ddm.ddm_write_ordered_ids(ctx, 0, e, ids[i])
+        ddm.ddm_plan_order(ctx, order[i], offs[i])
+        ddm.ddm_write_ordered_ids(ctx, e, m, ids[i][k:])
+    for i in (1, 2):
+        assert torch.equal(order[i], order[0]) and torch.equal(offs[i], offs[0])
+        assert torch.equal(ids[i], ids[0])
+
+
+def test_scratch_limits():
+    """With room for one ordering workspace but not for two, a one-shot call
+    orders its sets one after the other: under every limit it gives the pairs
+    of the unlimited call or DDM_ERR_NOMEM, and the context stays usable."""
+    import torch
+    U = to_dev(sparse_with_wide(20011, 30011, 2, wide=5, seed=8))
+    h = ddm.ddm_create(0)
+    K = ddm.ddm_count(h, *U)
+    want = torch.empty((K, 2), dtype=torch.int32, device="cuda")
+    assert ddm.ddm_match(h, *U, want) == K
+    ddm.ddm_destroy(h)
+    ok = failed = 0
+    for mib in [1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 16, 24, 32, 64]:
+        h = ddm.ddm_create(0)
+        ddm.ddm_debug_set_alloc_limit(h, mib << 20)
+        pairs = torch.empty((K, 2), dtype=torch.int32, device="cuda")
+        try:
+            assert ddm.ddm_match(h, *U, pairs) == K
+            assert torch.equal(pairs, want)
+            ok += 1
+        except ddm.DDMError as e:
+            assert e.code == ddm.DDM_ERR_NOMEM
+            failed += 1
+        ddm.ddm_debug_set_alloc_limit(h, 0)
+        assert ddm.ddm_match(h, *U, pairs) == K and torch.equal(pairs, want)
+        ddm.ddm_destroy(h)
+    assert ok >= 3 and failed >= 1
