@@ -334,7 +334,9 @@ int packed_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, const uint32_t* hi, bool
   sc.hist = static_cast<uint32_t*>(o.hist.p);
   sc.lookback = static_cast<uint32_t*>(o.lookback.p);
   sc.counters = static_cast<uint32_t*>(o.counters.p);
-  const SortSource src{source ? sc.vals[1] : nullptr, hi, 24, id_bits, words_out};
+  // the d = 1 tree's words: sorted by both bounds instead if ties abound
+  const SortSource src{source ? sc.vals[1] : nullptr, hi, 24, id_bits, words_out,
+                       words_out ? &c->st_dev->redo : nullptr};
   DDM_CUDA(launch_sort_packed(sc, src, cnt, key_bits, c->st_dev, c->sms, s));
   *cur = 0;
   return DDM_OK;

@@ -166,7 +166,8 @@ void note_launches(unsigned count);
 
 // ---- ddm_layout.cu --------------------------------------------------------
 // Validate a set (lo <= hi, no NaN in every dimension) and (k32 set) emit its
-// sort key: key(lo0), whole or its top 24 bits (a locality order).
+// sort key: key(lo0), whole (d = 1 tree; st->redo is then set if the lower
+// bounds tie in long runs) or its top 24 bits (a locality order).
 // aos (optional, cnt * d float2): an interleaved copy of the coordinates,
 // aos[i*d + k] = (lo_k, hi_k) of extent i, written while validating, so that
 // the gathers by id read one contiguous record per extent instead of 2d
@@ -241,10 +242,11 @@ struct SortSource {
   int k32_bits;
   int id_bits;
   bool words_out;       // the sorted words go to keys[0] instead (an even number of passes)
+  const uint32_t* skip_if;  // optional: nothing is done when *skip_if is set
 };
 // Order of a d = 1 tree from the words sorted by lower bound: ties put in the
 // order of their upper bound, ids to vals; *redo (zero before) is set if a
-// run of ties is too long for that.
+// run of ties is too long for that (nothing is done if it was set).
 cudaError_t launch_tie_order(const unsigned long long* words, uint32_t n, int id_bits,
                              const float* hi, uint32_t* vals, uint32_t* redo, int sms,
                              cudaStream_t s);

@@ -2,10 +2,10 @@
 //
 // The intersection matrix M of Section III is sparse and is returned in
 // compressed form: update j's matches occupy [offsets[j], offsets[j+1]) of
-// the pair list, and offsets[m] = K (which can exceed 2^32).  Classic
-// reduce-then-scan over tiles of 4096 counts: per-tile sums, one CTA scans
-// the tile sums, then each tile scans its counts from its tile offset.  No
-// kernel waits on another CTA.
+// the pair list, and offsets[m] = K (which can exceed 2^32).  A plan's scans
+// are one launch with decoupled look-back (k_scan_multi); the other users take
+// reduce-then-scan over tiles of 4096 counts: per-tile sums, one CTA scans the
+// tile sums, then each tile scans its counts from its tile offset.
 #include <atomic>
 
 #include "ddm_internal.cuh"

@@ -1,7 +1,8 @@
-// LSD radix sort of 64-bit keys with a 32-bit payload.
+// LSD radix sort of 64-bit words: keys packed above their ids, or keys with a
+// 32-bit payload.
 //
-// Sorts the subscriptions into the interval tree order of Section IV (lower
-// bound, then upper bound; the stable passes keep remaining ties in id
+// Sorts the subscriptions into the interval tree order of Section IV (by lower
+// bound, ties then put in the order of the upper bound, remaining ties in id
 // order), and the updates and the re-sorts into locality orders.  Three
 // forms by size, each a stable sort over 8-bit digits:
 //   * up to 16 tiles of 2,048 keys: one thread-block cluster keeps the keys
@@ -10,8 +11,8 @@
 //     the tiles exchanging digit counts across bounded grid barriers
 //     (k_sort_grid);
 //   * beyond: onesweep, after Adinets & Merrill
-//     ("Onesweep", 2022): one histogram pass over the keys computes all eight
-//     8-bit digit histograms at once, a tiny kernel scans them into digit
+//     ("Onesweep", 2022): one histogram pass over the keys computes all
+//     digit histograms at once, a tiny kernel scans them into digit
 //     bases, and each digit pass is ONE kernel: a CTA takes the next tile
 //     (ticket from an atomic counter, so every earlier tile is already
 //     resident), ranks its keys per digit with a warp match (one ballot per
@@ -282,6 +283,7 @@ k_onesweep(const unsigned long long* __restrict__ in_keys, const uint32_t* __res
 __global__ void __launch_bounds__(kThreads)
 k_histogram_packed(const unsigned long long* __restrict__ words, SortSource src, uint32_t n,
                    int passes, uint32_t* __restrict__ hist) {
+  if (src.skip_if && *src.skip_if) return;
   __shared__ uint32_t h[kPasses * kRadix];
   for (int t = threadIdx.x; t < passes * kRadix; t += kThreads) h[t] = 0;
   __syncthreads();
@@ -339,6 +341,7 @@ k_onesweep_packed(const unsigned long long* __restrict__ in, SortSource src,
                   int shift, const uint32_t* __restrict__ digit_base,
                   uint32_t* __restrict__ lookback, uint32_t* __restrict__ counter,
                   Status* __restrict__ st) {
+  if (src.skip_if && *src.skip_if) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   PackedSmem& sm = *reinterpret_cast<PackedSmem*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -577,7 +580,7 @@ k_sort_grid(unsigned long long* __restrict__ keys0, uint32_t* __restrict__ vals0
             unsigned long long* __restrict__ keys1, uint32_t* __restrict__ vals1, uint32_t n,
             int passes, SortSource src, const uint32_t* __restrict__ run_if,
             uint32_t* __restrict__ table, uint32_t* __restrict__ bar, Status* __restrict__ st) {
-  if (run_if && *run_if == 0u) return;  // every CTA alike, before any barrier
+  if ((run_if && *run_if == 0u) || (src.skip_if && *src.skip_if)) return;  // every CTA alike
   constexpr uint32_t kTile = kSmallThreads * ITEMS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   GridSortSmem<ITEMS, PACKED>& sm = *reinterpret_cast<GridSortSmem<ITEMS, PACKED>*>(smem_raw);
@@ -727,7 +730,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
 k_sort_cluster(const unsigned long long* __restrict__ in_k, const uint32_t* __restrict__ in_v,
                unsigned long long* __restrict__ out_k, uint32_t* __restrict__ out_v, uint32_t n,
                int passes, SortSource src, const uint32_t* __restrict__ run_if) {
-  if (run_if && *run_if == 0u) return;  // every CTA of the cluster alike
+  if ((run_if && *run_if == 0u) || (src.skip_if && *src.skip_if)) return;  // every CTA alike
   constexpr uint32_t kTile = kSmallThreads * ITEMS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ClusterSortSmem<ITEMS, PACKED>& sm = *reinterpret_cast<ClusterSortSmem<ITEMS, PACKED>*>(smem_raw);
@@ -827,6 +830,7 @@ constexpr uint32_t kMaxRun = 32;
 __global__ void __launch_bounds__(256)
 k_tie_order(const unsigned long long* __restrict__ words, uint32_t n, int id_bits,
             const float* __restrict__ hi, uint32_t* __restrict__ vals, uint32_t* __restrict__ redo) {
+  if (*reinterpret_cast<volatile uint32_t*>(redo)) return;
   const unsigned long long idm = (1ull << id_bits) - 1ull;
   for (uint32_t i = blockIdx.x * 256u + threadIdx.x; i < n; i += gridDim.x * 256u) {
     const unsigned long long w = words[i], k = w >> id_bits;

@@ -193,3 +193,23 @@ def test_scratch_limits():
         assert ddm.ddm_match(h, *U, pairs) == K and torch.equal(pairs, want)
         ddm.ddm_destroy(h)
     assert ok >= 3 and failed >= 1
+
+
+@pytest.mark.parametrize("n", [8193, 10000, 40007, 1300001])
+@pytest.mark.parametrize("values", [1, 60, 2000, 100000])
+def test_d1_tree_order_with_ties(ctx, n, values):
+    """Lower bounds that tie in runs of every length around the limit of the
+    short way, sampled as heavily tied or not: the exact (lower, upper, id)
+    order either way."""
+    import torch
+    from tests.test_gpu_parity import order_key
+    rng = np.random.default_rng(n + values)
+    lo = (rng.integers(0, values, size=(1, n)) - values // 2).astype(np.float32)
+    lo[0, :40] = values            # one run of 40 among shorter ones
+    hi = lo + rng.integers(0, 4, size=(1, n)).astype(np.float32)
+    S = to_dev((lo, hi))
+    ddm.ddm_build(ctx, S[0], S[1])
+    order = torch.empty(n, dtype=torch.int32, device="cuda")
+    ddm.ddm_tree_export(ctx, order)
+    want = np.lexsort((np.arange(n), order_key(hi[0]), order_key(lo[0])))
+    assert np.array_equal(order.cpu().numpy(), want)
