@@ -767,19 +767,27 @@ __device__ __forceinline__ void cp_async(void* to, const void* from) {
                : "memory");
 }
 
-// Shared memory of the replay kernel.
-template <bool WIDE, int OUT>
+// Shared memory of the replay kernel.  Kept small in the pairs forms: the
+// subscription ids are read through L1 (58% hits), and what shared memory
+// takes L1 loses (22 KB per CTA, with a list of a whole round's pairs, cost
+// the dense write pass 4%).
+template <bool WIDE, bool BATCH, int OUT>
 struct ReplaySmem {
   using Cursor = typename std::conditional<WIDE, unsigned long long, uint32_t>::type;
+  static constexpr bool packed = !WIDE && !BATCH;  // position fits the record's fourth word
+  static constexpr bool dense = ReplayShape<OUT>::dense;
+  // pairs listed at a time: a whole round's (dense form), else a window
+  static constexpr uint32_t window = dense ? 1024u : 128u;
+  using Pre = typename std::conditional<dense, uint32_t, uint16_t>::type;
   // Per record: leaf, hit mask, update id, and the output position of its first
   // pair (32-bit positions, not batched: one 128-bit load per record) or else
   // the subscription id base, the position then in `at`.
   uint4 rec[kWarps][32];
-  Cursor at[kWarps][32];
+  Cursor at[packed ? 1 : kWarps][32];
   uint4 next[kWarps];  // the next list entry
   // a round's pairs as a list of (record, leaf slot)
-  uint32_t pre[kWarps][32];
-  uint16_t list[kWarps][1024];
+  Pre pre[kWarps][32];
+  uint16_t list[kWarps][window];
 };
 
 // Expands the list entries [i0, i1).  SHORT: entries of few records, where
@@ -791,7 +799,7 @@ struct ReplaySmem {
 // and the pairs are then written 32 at a time (as the ids form does), where
 // a step per record would leave most lanes idle.
 template <bool FILTER_ID, bool WIDE, bool BATCH, int OUT, bool SHORT>
-__device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, OUT>& sm, const TreeView& t,
+__device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, BATCH, OUT>& sm, const TreeView& t,
                                                const QueryView& q, const BatchView& bv,
                                                const RecordArena& ra, const WriteView& w,
                                                uint32_t i0, uint32_t i1, uint32_t pb, uint32_t pe,
@@ -799,7 +807,8 @@ __device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, OUT>& sm, const 
                                                unsigned long long base0, unsigned long long need,
                                                uint32_t* __restrict__ work,
                                                Status* __restrict__ st) {
-  using Cursor = typename ReplaySmem<WIDE, OUT>::Cursor;
+  using Smem = ReplaySmem<WIDE, BATCH, OUT>;
+  using Cursor = typename Smem::Cursor;
   constexpr bool kDense = SHORT || ReplayShape<OUT>::dense;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const uint32_t below = (1u << lane) - 1u;  // lanes below this one
@@ -929,7 +938,7 @@ __device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, OUT>& sm, const 
       const uint32_t Qq = __shfl_sync(0xffffffffu, Qout, qq);
       const uint32_t sb = BATCH ? __shfl_sync(0xffffffffu, sub_base, qq) : 0u;
       __syncwarp();  // the previous round has read s_rec / s_at
-      constexpr bool kPacked = !WIDE && !BATCH;  // position fits the record's fourth word
+      constexpr bool kPacked = Smem::packed;
       sm.rec[wib][lane] = make_uint4(x >> 5, hb, Qq, kPacked ? (uint32_t)o : sb);
       if (!kPacked) sm.at[wib][lane] = o;
       if constexpr (kDense) {
@@ -946,23 +955,27 @@ __device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, OUT>& sm, const 
           if (lane >= dd) incl += v;
         }
         const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-        sm.pre[wib][lane] = incl - c;
+        sm.pre[wib][lane] = (typename Smem::Pre)(incl - c);
         __syncwarp();
-        if (SHORT) {
-          uint32_t k = incl - c;
-          for (uint32_t h = hb; h; h &= h - 1u)
-            sm.list[wib][k++] = (uint16_t)(((uint32_t)lane << 5) | (uint32_t)(__ffs(h) - 1));
-        } else
+        constexpr uint32_t W = Smem::window;
+        for (uint32_t w0 = 0; w0 < total; w0 += W) {  // once, when the window holds a round
+          if (SHORT) {
+            uint32_t k = incl - c - w0;
+            for (uint32_t h = hb; h; h &= h - 1u, ++k)
+              if (k < W) sm.list[wib][k] = (uint16_t)(((uint32_t)lane << 5) | (uint32_t)(__ffs(h) - 1));
+          } else {
 #pragma unroll 8
-        for (int u = 0; u < 32; ++u) {
-          const uint32_t h = sm.rec[wib][u].y;
-          if (h & lanebit)
-            sm.list[wib][sm.pre[wib][u] + __popc(h & below)] = (uint16_t)(((uint32_t)u << 5) | (uint32_t)lane);
-        }
-        __syncwarp();
+            for (int u = 0; u < 32; ++u) {
+              const uint32_t h = sm.rec[wib][u].y;
+              if (h & lanebit)
+                sm.list[wib][sm.pre[wib][u] + __popc(h & below)] = (uint16_t)(((uint32_t)u << 5) | (uint32_t)lane);
+            }
+          }
+          __syncwarp();
+          const uint32_t w1 = min(total, w0 + W);
 #pragma unroll 2
-        for (uint32_t ti = lane; ti < total; ti += 32u) {
-          const uint32_t ent = sm.list[wib][ti];
+        for (uint32_t ti = w0 + lane; ti < w1; ti += 32u) {
+          const uint32_t ent = sm.list[wib][ti - w0];
           const uint32_t r = ent >> 5, slot = ent & 31u;
           const uint4 R = sm.rec[wib][r];
           const Cursor at = (kPacked ? (Cursor)R.w : sm.at[wib][r]) + (Cursor)(ti - sm.pre[wib][r]);
@@ -977,6 +990,8 @@ __device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, OUT>& sm, const 
             pr.sub = OUT == kOutSwapped ? R.z : sub;
             st_hinted(pairs + (unsigned long long)at, pr, stream);
           }
+        }
+          if (W < 1024u) __syncwarp();  // the list is read before the next window
         }
         continue;
       }
@@ -1025,7 +1040,7 @@ __global__ void __launch_bounds__(kThreads, ReplayShape<OUT>::ctas)
 k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uint32_t p0,
          uint32_t p1, uint32_t pb, uint32_t pe, uint32_t idb, uint32_t ide,
          uint32_t* __restrict__ work, Status* __restrict__ st) {
-  __shared__ ReplaySmem<WIDE, OUT> sm;
+  __shared__ ReplaySmem<WIDE, BATCH, OUT> sm;
   if (!records_complete(ra)) {  // the walking write pass handles this range
     if (blockIdx.x == 0 && threadIdx.x == 0) st->walk = 1u;
     return;
