@@ -761,7 +761,8 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
   const ScanHint hint{c->arena.max_blocks ? c->rec_hint : nullptr, c->arena.blk_counter,
                       c->arena.chains, packets, c->arena.max_blocks};
   DDM_CUDA(launch_scan_multi(jobs, njobs, state + 1, hint, c->st_dev, s));
-  if (ordered && c->arena.max_blocks) DDM_CUDA(launch_block_list(c->arena, c->sms, s));
+  if (ordered && c->arena.max_blocks)
+    DDM_CUDA(launch_block_list(c->arena, pos_offsets + m, c->sms, s));
   c->ordered = ordered;
   c->ulo = ulo;
   c->uhi = uhi;
@@ -802,7 +803,8 @@ int ready_ordered(ddm_ctx* c, cudaStream_t s) {
   auto* state = static_cast<unsigned long long*>(c->order_state.p);
   DDM_CUDA(cudaMemsetAsync(state, 0, sizeof(unsigned long long) * words, s));
   DDM_CUDA(launch_scan_multi(jobs, njobs, state, ScanHint{}, c->st_dev, s));
-  if (c->arena.max_blocks) DDM_CUDA(launch_block_list(c->arena, c->sms, s));
+  if (c->arena.max_blocks)
+    DDM_CUDA(launch_block_list(c->arena, jobs[0].offsets + c->m, c->sms, s));
   c->ordered = !c->capturing;  // recorded only: it runs with the graph
   return DDM_OK;
 }

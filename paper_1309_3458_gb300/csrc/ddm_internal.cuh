@@ -325,10 +325,11 @@ cudaError_t launch_export_nodes(const TreeView& t, float* node_lo, float* node_h
 //
 // The first block of each chain belongs to it from the start (its header is
 // zero); only the blocks after it are taken from a counter, so that the
-// packets of a sparse problem make no atomic.  The two first blocks of a
-// packet are one entry of the write pass, every block after them another.
-// A write laid out by update id takes the entries as they are (packets first,
-// then the blocks handed out); only writes of ranges of the plan order need
+// packets of a sparse problem make no atomic.  Every block is an entry of the
+// write pass, but for the two first blocks of a packet, which are one if the
+// plan has few pairs per entry.
+// A write laid out by update id takes the blocks as they are (the chains'
+// first, then those handed out); only writes of ranges of the plan order need
 // them listed in that order.  With every block
 // from the counter and listed, the count pass of 2.5e7 + 2.5e7 extents
 // (d = 1, alpha = 1) took 2.81 ms and the write pass 2.58 ms; now 1.73 and
@@ -350,18 +351,22 @@ struct RecordArena {
   uint2* blk_own;          // [max_blocks] packet of a block handed out, and its
                            // number among that packet's blocks handed out
   uint32_t* blk_count;     // [max_blocks] records in the block
-  uint32_t* pkt_nblk;      // [packets] entries of each packet
+  uint32_t* pkt_nblk;      // [packets] blocks of each packet, the two first as one
   unsigned long long* pkt_off;  // [packets + 1] exclusive prefix of pkt_nblk
   uint4* blk_list;         // [max_blocks] entries in plan order: block, packet,
-                           // its records, and those of the next block when the
-                           // entry is a packet's two first blocks; null: not
-                           // listed
+                           // its records, and those of the next block if the
+                           // entry is a packet's two first blocks (plans with
+                           // short entries); null: not listed
   uint32_t* blk_counter;   // [0] blocks handed out beyond the chains' first (may
                            // exceed the arena), [1] such blocks the whole pass
                            // needed
   uint32_t chains;         // chains of the plan's packets
   uint32_t max_blocks;     // 0: no recording
 };
+// Pairs per entry of a plan up to which its entries count as short: the write
+// pass then takes a packet's two first blocks as one entry and expands by
+// listing pairs instead of record by record.
+constexpr uint32_t kShortEntry = 256;
 // The records of the last count pass are complete (the write pass may
 // replay them) iff recording was on and the arena did not run out.
 __device__ __forceinline__ bool records_complete(const RecordArena& ra) {
@@ -385,8 +390,10 @@ cudaError_t launch_write(const TreeView& t, const QueryView& q, const BatchView&
                          uint32_t flags, const WriteView& w, const RecordArena& ra,
                          uint32_t* work, Status* st, int sms, cudaStream_t s);
 // After the count pass: blk_list = every packet's entries, packets in plan
-// order; pkt_off must already hold the prefix of pkt_nblk.
-cudaError_t launch_block_list(const RecordArena& ra, int sms, cudaStream_t s);
+// order; pkt_off must already hold the prefix of pkt_nblk, and *pairs the
+// plan's pairs.
+cudaError_t launch_block_list(const RecordArena& ra, const unsigned long long* pairs, int sms,
+                              cudaStream_t s);
 // Write pass from records: positions [pb, pe) of the plan, in packets [p0,
 // p1) (without a list: all packets), and (when id_filter) only updates with
 // ids in [idb, ide).  Only sets st->walk unless `ra` holds complete records.

@@ -658,21 +658,24 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
   if (!WRITE && st && lane == 0 && ntests) atomicAdd(&st->tests, (unsigned long long)ntests);
 }
 
-// Plan-order list of the record entries, a thread per entry: packet p's two
-// first blocks at pkt_off[p], the blocks handed out to it behind them.
-__global__ void k_block_list(RecordArena ra) {
+__device__ __forceinline__ bool short_entries(const RecordArena& ra, unsigned long long pairs) {
+  return pairs <= (unsigned long long)kShortEntry * (ra.chains / kRecChains + ra.blk_counter[0]);
+}
+
+// Plan-order list of the record entries, a thread per block: packet p's two
+// first blocks (one entry, if the plan's entries are short) before the blocks
+// handed out to it.  pkt_off counts the two as one.
+__global__ void k_block_list(RecordArena ra, const unsigned long long* __restrict__ pairs) {
   if (!records_complete(ra)) return;
-  const uint32_t packets = ra.chains / kRecChains, more = ra.blk_counter[0];
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < packets + more;
-       i += gridDim.x * blockDim.x) {
-    if (i < packets) {
-      const uint32_t b = i * kRecChains;
-      ra.blk_list[ra.pkt_off[i]] = make_uint4(b, i, ra.blk_count[b], ra.blk_count[b + 1]);
-    } else {
-      const uint32_t b = ra.chains + (i - packets);
-      const uint2 own = ra.blk_own[b];
-      ra.blk_list[ra.pkt_off[own.x] + 1u + own.y] = make_uint4(b, own.x, ra.blk_count[b], 0u);
-    }
+  const bool one = short_entries(ra, *pairs);
+  const uint32_t blocks = ra.chains + ra.blk_counter[0];
+  for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < blocks; b += gridDim.x * blockDim.x) {
+    const bool first = b < ra.chains;
+    if (one && first && (b & 1u)) continue;  // listed with the block before it
+    const uint2 own = first ? make_uint2(b / kRecChains, 0u) : ra.blk_own[b];
+    const unsigned long long at = ra.pkt_off[own.x] + (one ? 0u : own.x) +
+                                  (first ? b & 1u : (one ? 1u : kRecChains) + own.y);
+    ra.blk_list[at] = make_uint4(b, own.x, ra.blk_count[b], one && first ? ra.blk_count[b + 1] : 0u);
   }
 }
 
@@ -710,10 +713,34 @@ __device__ __forceinline__ void st_hinted(uint32_t* a, uint32_t v, unsigned long
   asm volatile("st.global.L2::cache_hint.u32 [%0], %1, %2;" ::"l"(a), "r"(v), "l"(policy) : "memory");
 }
 
+// The same for the lanes where `on` is set, as one predicated instruction each
+// and (loads too) in program order: from an `if` around every access the
+// compiler made branches, and moved loads behind stores.
+__device__ __forceinline__ uint32_t ld_hinted_if(bool on, const uint32_t* a, unsigned long long policy) {
+  uint32_t v;
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\tmov.u32 %0, 0;\n\t"
+               "@p ld.global.nc.L2::cache_hint.u32 %0, [%1], %2;\n\t}"
+               : "=&r"(v)
+               : "l"(a), "l"(policy), "r"((uint32_t)on));
+  return v;
+}
+__device__ __forceinline__ void st_hinted_if(bool on, ddm_pair* a, ddm_pair v, unsigned long long policy) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+               "@p st.global.L2::cache_hint.v2.u32 [%0], {%1, %2}, %3;\n\t}" ::"l"(a),
+               "r"(v.upd), "r"(v.sub), "l"(policy), "r"((uint32_t)on)
+               : "memory");
+}
+__device__ __forceinline__ void st_hinted_if(bool on, uint32_t* a, uint32_t v, unsigned long long policy) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t"
+               "@p st.global.L2::cache_hint.u32 [%0], %1, %2;\n\t}" ::"l"(a), "r"(v), "l"(policy),
+               "r"((uint32_t)on)
+               : "memory");
+}
+
 // Write pass from the records of the count pass.  Work unit: one entry (a
-// packet's two first record blocks, or a block of up to 512 records handed
-// out to it), so uneven packets spread over the whole GPU.  A warp loads the
-// block's packet queries (their output offsets) and takes the records 32 at
+// record block of up to 512 records, or a packet's two first blocks where
+// blocks hold few), so uneven packets spread over the whole GPU.  A warp loads
+// the block's packet queries (their output offsets) and takes the records 32 at
 // a time (the next 32 are loaded while these expand), one per lane: each lane
 // works out where its record's pairs go (its query's offset, plus the block
 // header's count of the query's matches before the block, plus the record's
@@ -732,15 +759,13 @@ __device__ __forceinline__ void st_hinted(uint32_t* a, uint32_t v, unsigned long
 // fields exchanged (roles swapped: the tree holds the updates); kOutIds the
 // compressed output, only each pair's subscription id (4 bytes) at the
 // pair's position.
-// Pairs per list entry of the range up to which entries count as short.
-constexpr uint32_t kShortEntry = 256;
 constexpr int kOutPairs = 0, kOutSwapped = 1, kOutIds = 2;
 // Resident CTAs per SM and records expanded per group (their id loads issued
 // before their stores) of the replay kernel, by output form.  Pairs (8-byte
 // stores): two CTAs of eight warps with sixteen records in flight each (128
 // registers, no spill) beat four CTAs with eight (64 registers, spilling):
-// 131.9 against 147.4 ms per step on the clustered d = 3 workload; one CTA,
-// or four records per group, was slower.  Subscription ids (4-byte stores)
+// 131.9 against 147.4 ms per step on the clustered d = 3 workload with an
+// earlier form of the loop; one CTA, or four records per group, was slower.  Subscription ids (4-byte stores)
 // go the other way: four CTAs with eight records take 122.3 ms, three 138.0,
 // two 178.7.
 //
@@ -790,29 +815,24 @@ struct ReplaySmem {
   uint16_t list[kWarps][window];
 };
 
-// Expands the list entries [i0, i1).  SHORT: entries of few records, where
-// the time goes into waiting for one load after the other: the next entry is
-// copied to shared memory (asynchronously, no register waits for it) and the
-// ticket after it taken before the current one is expanded.  With long
-// entries this would cost 2% (warps holding work at the end of the pass).
-// Their records have few hits each: every lane lists its own record's bits,
-// and the pairs are then written 32 at a time (as the ids form does), where
-// a step per record would leave most lanes idle.
-template <bool FILTER_ID, bool WIDE, bool BATCH, int OUT, bool SHORT>
-__device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, BATCH, OUT>& sm, const TreeView& t,
-                                               const QueryView& q, const BatchView& bv,
-                                               const RecordArena& ra, const WriteView& w,
-                                               uint32_t i0, uint32_t i1, uint32_t pb, uint32_t pe,
-                                               uint32_t idb, uint32_t ide,
-                                               unsigned long long base0, unsigned long long need,
-                                               uint32_t* __restrict__ work,
-                                               Status* __restrict__ st) {
+// Expands the entries [i0, i1) of a plan with short ones, where the time goes
+// into waiting for one load after the other: the next entry is copied to shared
+// memory (asynchronously, no register waits for it) and the ticket after it
+// taken before the current one is expanded.  The records have few hits each:
+// every lane lists its own record's bits, and the pairs are then written 32 at
+// a time (as the ids form does), where a step per record would leave most
+// lanes idle.
+template <bool FILTER_ID, bool WIDE, bool BATCH, int OUT>
+__device__ __forceinline__ void replay_short(ReplaySmem<WIDE, BATCH, OUT>& sm, const TreeView& t,
+                                             const QueryView& q, const BatchView& bv,
+                                             const RecordArena& ra, const WriteView& w,
+                                             uint32_t i0, uint32_t i1, uint32_t pb, uint32_t pe,
+                                             uint32_t idb, uint32_t ide, unsigned long long base0,
+                                             unsigned long long need, uint32_t* __restrict__ work,
+                                             Status* __restrict__ st) {
   using Smem = ReplaySmem<WIDE, BATCH, OUT>;
   using Cursor = typename Smem::Cursor;
-  constexpr bool kDense = SHORT || ReplayShape<OUT>::dense;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const uint32_t below = (1u << lane) - 1u;  // lanes below this one
-  const uint32_t lanebit = 1u << lane;
   ddm_pair* __restrict__ pairs = w.pairs;
   uint32_t* __restrict__ ids = w.ids;
   const uint32_t* __restrict__ sid = t.sid;
@@ -845,40 +865,17 @@ __device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, BATCH, OUT>& sm,
       held = tickets ? i0 + warps + atomicAdd(work, 1u) : i1;
     }
   };
-  auto take = [&]() {
-    if (lane == 0) held = tickets ? i0 + warps + atomicAdd(work, 1u) : i1;
-    held = __shfl_sync(0xffffffffu, held, 0);
-  };
-  if (SHORT) fetch();
+  fetch();
   for (;;) {
-    uint4 entry;
-    if (SHORT) {
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      __syncwarp();
-      entry = sm.next[wib];
-      if (entry.x == kNoBlock) break;
-      __syncwarp();
-      fetch();
-    } else {
-      const uint32_t i = held;
-      if (i >= i1) break;
-      if (ra.blk_list) {
-        entry = ra.blk_list[i];
-      } else if (i < packets) {
-        const uint32_t b = i * kRecChains;
-        entry = make_uint4(b, i, ra.blk_count[b], ra.blk_count[b + 1u]);
-      } else {
-        const uint32_t b = ra.chains + (i - packets);
-        entry = make_uint4(b, ra.blk_own[b].x, ra.blk_count[b], 0u);
-      }
-    }
-    // records [0, na) of block blk, then (one entry for two blocks) the rest
-    // from the next block
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+    const uint4 entry = sm.next[wib];
+    if (entry.x == kNoBlock) break;
+    __syncwarp();
+    fetch();
+    // records [0, na) of block blk, then the rest from the next block
     const uint32_t blk = entry.x, p = entry.y, na = entry.z, nrec = entry.z + entry.w;
-    if (nrec == 0u) {
-      if (!SHORT) take();
-      continue;
-    }
+    if (nrec == 0u) continue;
     const uint32_t pos = (p << q.qpp_log2) + lane;
     bool valid = (uint32_t)lane < (1u << q.qpp_log2) && pos >= pb && pos < pe;
     uint32_t Q = 0;
@@ -894,21 +891,14 @@ __device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, BATCH, OUT>& sm,
       sub_base = (uint32_t)bv.sub_off[b];
     }
     const uint32_t vmask = __ballot_sync(0xffffffffu, valid);
-    if (vmask == 0u) {
-      if (!SHORT) take();
-      continue;
-    }
+    if (vmask == 0u) continue;
     const uint32_t* rec = ra.rec + (size_t)blk * kRecWords;
-    // SHORT: the records of both blocks as one sequence; else one block after
-    // the other (a select per load would cost the long entries 3%).
-    uint32_t todo = SHORT ? nrec : na, rest = SHORT ? 0u : nrec - na;
-    for (;;) {
     const uint16_t* rel = reinterpret_cast<const uint16_t*>(rec + 2u * kRecBlock);
     uint32_t nx = 0u, nhb = 0u, nrel = 0u;
     auto load = [&](uint32_t r0) {
       const uint32_t r = r0 + (uint32_t)lane;
-      if (r < todo) {
-        if (SHORT && r >= na) {  // the second of two blocks
+      if (r < nrec) {
+        if (r >= na) {  // the second of two blocks
           const uint32_t* r2 = rec + kRecWords;
           nx = ld_hinted(&r2[r - na], stream);
           nhb = ld_hinted(&r2[kRecBlock + r - na], stream);
@@ -925,7 +915,7 @@ __device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, BATCH, OUT>& sm,
     // before the block
     const uint32_t hdr =
         lane < (int)kRecHdr ? ld_hinted(&rec[2u * kRecBlock + kRecBlock / 2u + lane], stream) : 0u;
-    for (uint32_t r0 = 0; r0 < todo; r0 += 32u) {
+    for (uint32_t r0 = 0; r0 < nrec; r0 += 32u) {
       const uint32_t x = nx, xrel = nrel;
       uint32_t hb = nhb;
       nx = nhb = nrel = 0u;  // lanes past the block's last record hold x = hb = 0
@@ -941,38 +931,27 @@ __device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, BATCH, OUT>& sm,
       constexpr bool kPacked = Smem::packed;
       sm.rec[wib][lane] = make_uint4(x >> 5, hb, Qq, kPacked ? (uint32_t)o : sb);
       if (!kPacked) sm.at[wib][lane] = o;
-      if constexpr (kDense) {
-        // The round's pairs, numbered record by record: an exclusive scan of
-        // the records' hit counts gives each record's first pair; the hit
-        // bits become a list of (record, leaf slot) in that numbering
-        // (lane = leaf slot); then every lane takes one pair of the list at
-        // a time: one id load and one store per 32 pairs.
-        const uint32_t c = __popc(hb);
-        uint32_t incl = c;
+      // The round's pairs, numbered record by record: an exclusive scan of the
+      // records' hit counts gives each record's first pair; the hit bits become
+      // a list of (record, leaf slot) in that numbering; then every lane takes
+      // one pair of the list at a time: one id load and one store per 32 pairs.
+      const uint32_t c = __popc(hb);
+      uint32_t incl = c;
 #pragma unroll
-        for (int dd = 1; dd < 32; dd <<= 1) {
-          const uint32_t v = __shfl_up_sync(0xffffffffu, incl, dd);
-          if (lane >= dd) incl += v;
-        }
-        const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-        sm.pre[wib][lane] = (typename Smem::Pre)(incl - c);
+      for (int dd = 1; dd < 32; dd <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, dd);
+        if (lane >= dd) incl += v;
+      }
+      const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+      sm.pre[wib][lane] = (typename Smem::Pre)(incl - c);
+      __syncwarp();
+      constexpr uint32_t W = Smem::window;
+      for (uint32_t w0 = 0; w0 < total; w0 += W) {  // once, when the window holds a round
+        uint32_t k = incl - c - w0;
+        for (uint32_t h = hb; h; h &= h - 1u, ++k)
+          if (k < W) sm.list[wib][k] = (uint16_t)(((uint32_t)lane << 5) | (uint32_t)(__ffs(h) - 1));
         __syncwarp();
-        constexpr uint32_t W = Smem::window;
-        for (uint32_t w0 = 0; w0 < total; w0 += W) {  // once, when the window holds a round
-          if (SHORT) {
-            uint32_t k = incl - c - w0;
-            for (uint32_t h = hb; h; h &= h - 1u, ++k)
-              if (k < W) sm.list[wib][k] = (uint16_t)(((uint32_t)lane << 5) | (uint32_t)(__ffs(h) - 1));
-          } else {
-#pragma unroll 8
-            for (int u = 0; u < 32; ++u) {
-              const uint32_t h = sm.rec[wib][u].y;
-              if (h & lanebit)
-                sm.list[wib][sm.pre[wib][u] + __popc(h & below)] = (uint16_t)(((uint32_t)u << 5) | (uint32_t)lane);
-            }
-          }
-          __syncwarp();
-          const uint32_t w1 = min(total, w0 + W);
+        const uint32_t w1 = min(total, w0 + W);
 #pragma unroll 2
         for (uint32_t ti = w0 + lane; ti < w1; ti += 32u) {
           const uint32_t ent = sm.list[wib][ti - w0];
@@ -991,47 +970,171 @@ __device__ __forceinline__ void replay_entries(ReplaySmem<WIDE, BATCH, OUT>& sm,
             st_hinted(pairs + (unsigned long long)at, pr, stream);
           }
         }
-          if (W < 1024u) __syncwarp();  // the list is read before the next window
-        }
-        continue;
+        if (W < 1024u) __syncwarp();  // the list is read before the next window
       }
-      __syncwarp();
-      constexpr int G = ReplayShape<OUT>::group;
-      for (int g = 0; g < 32; g += G) {
-        uint4 rr[G];
-        uint32_t sv[G];
-#pragma unroll
-        for (int u = 0; u < G; ++u) {
-          rr[u] = sm.rec[wib][g + u];
-          sv[u] = 0u;
-          if ((rr[u].y & lanebit) && DDM_IN_BOUNDS(rr[u].x * 32u + (uint32_t)lane < t.n, st))
-            sv[u] = ld_hinted(sid + rr[u].x * 32u + (uint32_t)lane, keep);
+    }
+  }
+}
+
+// Expands the entries [i0, i1) of a plan with long ones (single blocks).  A
+// warp's next ticket is taken when it has finished a block: with tickets ahead
+// warps hold work at the end of the pass.  Bound by the latency of the id loads
+// (a group's, by sixteen warps per SM), so what counts is that they are issued
+// together: as predicated instructions, not in branches.  The write pass of
+// 4.41e10 pairs (clustered, d = 3) took 127.7 ms with a branch per record in one
+// function for both forms, 123.9 in a function of its own and a block per entry
+// in place of two, and 119.5 with predicated loads and stores; of the ids alone
+// 112.2 -> 111.7 ms, and 109.4 with two ids per lane and step in flight (four:
+// 111.7).
+template <bool FILTER_ID, bool WIDE, bool BATCH, int OUT>
+__device__ __forceinline__ void replay_long(ReplaySmem<WIDE, BATCH, OUT>& sm, const TreeView& t,
+                                            const QueryView& q, const BatchView& bv,
+                                            const RecordArena& ra, const WriteView& w, uint32_t i0,
+                                            uint32_t i1, uint32_t pb, uint32_t pe, uint32_t idb,
+                                            uint32_t ide, unsigned long long base0,
+                                            unsigned long long need, uint32_t* __restrict__ work,
+                                            Status* __restrict__ st) {
+  using Smem = ReplaySmem<WIDE, BATCH, OUT>;
+  using Cursor = typename Smem::Cursor;
+  constexpr bool kPacked = Smem::packed;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const uint32_t below = (1u << lane) - 1u;  // lanes below this one
+  const uint32_t lanebit = 1u << lane;
+  ddm_pair* __restrict__ pairs = w.pairs;
+  uint32_t* __restrict__ ids = w.ids;
+  const uint32_t* __restrict__ sid = t.sid;
+  const unsigned long long keep = l2_policy_evict_last(), stream = l2_policy_evict_first();
+  const uint32_t warps = gridDim.x * kWarps;
+  uint32_t i = i0 + blockIdx.x * kWarps + wib;
+  while (i < i1) {
+    uint4 entry;
+    if (ra.blk_list)
+      entry = ra.blk_list[i];
+    else
+      entry = make_uint4(i, i < ra.chains ? i / kRecChains : ra.blk_own[i].x, ra.blk_count[i], 0u);
+    const uint32_t blk = entry.x, p = entry.y;
+    const uint32_t pos = (p << q.qpp_log2) + lane;
+    bool valid = (uint32_t)lane < (1u << q.qpp_log2) && pos >= pb && pos < pe;
+    uint32_t Q = 0;
+    if (valid) Q = q.qid[pos];
+    if (FILTER_ID) valid = valid && Q >= idb && Q < ide;
+    Cursor out = 0;
+    if (valid) out = (Cursor)(w.start[w.by_pos ? pos : Q] - base0);
+    uint32_t Qout = Q + w.qbase, sub_base = 0;
+    if (w.qids && valid) Qout = w.qids[Q];
+    if (BATCH && valid) {
+      const uint32_t b = bv.q_inst[pos];
+      Qout = Q - (uint32_t)bv.upd_off[b];
+      sub_base = (uint32_t)bv.sub_off[b];
+    }
+    const uint32_t vmask = __ballot_sync(0xffffffffu, valid);
+    if (vmask != 0u) {
+      const uint32_t nrec = entry.z;
+      const uint32_t* rec = ra.rec + (size_t)blk * kRecWords;
+      const uint16_t* rel = reinterpret_cast<const uint16_t*>(rec + 2u * kRecBlock);
+      uint32_t nx = 0u, nhb = 0u, nrel = 0u;
+      if (lane < nrec) {
+        nx = ld_hinted(&rec[lane], stream);
+        nhb = ld_hinted(&rec[kRecBlock + lane], stream);
+        nrel = ld_hinted(&rel[lane], stream);
+      }
+      // the block header: lane j holds the matches query j of the chain had
+      // before the block
+      const uint32_t hdr =
+          lane < (int)kRecHdr ? ld_hinted(&rec[2u * kRecBlock + kRecBlock / 2u + lane], stream) : 0u;
+      for (uint32_t r0 = 0; r0 < nrec; r0 += 32u) {
+        const uint32_t x = nx, xrel = nrel;
+        uint32_t hb = nhb;
+        nx = nhb = nrel = 0u;  // lanes past the block's last record hold x = hb = 0
+        if (r0 + 32u + lane < nrec) {
+          nx = ld_hinted(&rec[r0 + 32u + lane], stream);
+          nhb = ld_hinted(&rec[kRecBlock + r0 + 32u + lane], stream);
+          nrel = ld_hinted(&rel[r0 + 32u + lane], stream);
         }
+        const int qq = (int)(x & 31u);
+        // the query's matches before this record: header + the record's count
+        const uint32_t bef = __shfl_sync(0xffffffffu, hdr, qq & (int)(kRecHdr - 1)) + xrel;
+        if (!((vmask >> qq) & 1u)) hb = 0u;  // also clears lanes past nrec (x = hb = 0)
+        const Cursor o = __shfl_sync(0xffffffffu, out, qq) + (Cursor)bef;
+        const uint32_t Qq = __shfl_sync(0xffffffffu, Qout, qq);
+        const uint32_t sb = BATCH ? __shfl_sync(0xffffffffu, sub_base, qq) : 0u;
+        __syncwarp();  // the previous round has read s_rec / s_at
+        sm.rec[wib][lane] = make_uint4(x >> 5, hb, Qq, kPacked ? (uint32_t)o : sb);
+        if (!kPacked) sm.at[wib][lane] = o;
+        if constexpr (Smem::dense) {
+          // The round's pairs, numbered record by record: an exclusive scan of
+          // the records' hit counts gives each record's first pair; the hit
+          // bits become a list of (record, leaf slot) in that numbering
+          // (lane = leaf slot); then every lane takes one pair of the list at
+          // a time: one id load and one store per 32 pairs.
+          const uint32_t c = __popc(hb);
+          uint32_t incl = c;
 #pragma unroll
-        for (int u = 0; u < G; ++u) {
-          if (rr[u].y & lanebit) {
+          for (int dd = 1; dd < 32; dd <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, dd);
+            if (lane >= dd) incl += v;
+          }
+          const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+          sm.pre[wib][lane] = (typename Smem::Pre)(incl - c);
+          __syncwarp();
+#pragma unroll 8
+          for (int u = 0; u < 32; ++u) {
+            const uint32_t h = sm.rec[wib][u].y;
+            if (h & lanebit)
+              sm.list[wib][sm.pre[wib][u] + __popc(h & below)] = (uint16_t)(((uint32_t)u << 5) | (uint32_t)lane);
+          }
+          __syncwarp();
+          constexpr uint32_t kEach = 2;  // ids in flight per lane
+          for (uint32_t t0 = 0; t0 < total; t0 += 32u * kEach) {
+            uint32_t sv[kEach], base[kEach];
+            Cursor at[kEach];
+            bool on[kEach];
+#pragma unroll
+            for (uint32_t u = 0; u < kEach; ++u) {
+              const uint32_t ti = t0 + 32u * u + lane;
+              const uint32_t ent = ti < total ? sm.list[wib][ti] : 0u;
+              const uint32_t r = ent >> 5;
+              const uint4 R = sm.rec[wib][r];
+              const uint32_t slot = R.x * 32u + (ent & 31u);
+              at[u] = (kPacked ? (Cursor)R.w : sm.at[wib][r]) + (Cursor)(ti - sm.pre[wib][r]);
+              on[u] = ti < total && DDM_IN_BOUNDS(slot < t.n && (unsigned long long)at[u] < need, st);
+              base[u] = kPacked ? 0u : R.w;
+              sv[u] = ld_hinted_if(on[u], sid + slot, keep);
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < kEach; ++u)
+              st_hinted_if(on[u], ids + (unsigned long long)at[u], sv[u] - base[u], stream);
+          }
+          continue;
+        }
+        __syncwarp();
+        constexpr int G = ReplayShape<OUT>::group;
+        for (int g = 0; g < 32; g += G) {
+          uint4 rr[G];
+          uint32_t sv[G];
+#pragma unroll
+          for (int u = 0; u < G; ++u) {
+            rr[u] = sm.rec[wib][g + u];
+            const uint32_t slot = rr[u].x * 32u + (uint32_t)lane;
+            const bool on = (rr[u].y & lanebit) && DDM_IN_BOUNDS(slot < t.n, st);
+            sv[u] = ld_hinted_if(on, sid + slot, keep);
+          }
+#pragma unroll
+          for (int u = 0; u < G; ++u) {
             const Cursor at = kPacked ? (Cursor)rr[u].w : sm.at[wib][g + u];
             const unsigned long long slot = (unsigned long long)(at + (Cursor)__popc(rr[u].y & below));
-            if (!DDM_IN_BOUNDS(slot < need, st)) continue;
+            const bool on = (rr[u].y & lanebit) && DDM_IN_BOUNDS(slot < need, st);
             const uint32_t sub = sv[u] - (kPacked ? 0u : rr[u].w);
-            if (OUT == kOutIds) {
-              st_hinted(ids + slot, sub, stream);
-            } else {
-              ddm_pair pr;
-              pr.upd = OUT == kOutSwapped ? sub : rr[u].z;
-              pr.sub = OUT == kOutSwapped ? rr[u].z : sub;
-              st_hinted(pairs + slot, pr, stream);
-            }
+            ddm_pair pr;
+            pr.upd = OUT == kOutSwapped ? sub : rr[u].z;
+            pr.sub = OUT == kOutSwapped ? rr[u].z : sub;
+            st_hinted_if(on, pairs + slot, pr, stream);
           }
         }
       }
     }
-    if (rest == 0u) break;
-    rec += kRecWords;
-    todo = rest;
-    rest = 0u;
-    }
-    if (!SHORT) take();
+    if (lane == 0) i = i0 + warps + atomicAdd(work, 1u);
+    i = __shfl_sync(0xffffffffu, i, 0);
   }
 }
 
@@ -1047,6 +1150,8 @@ k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uin
   }
   const unsigned long long base0 = w.start[w.b_idx];
   const unsigned long long need = w.start[w.e_idx] - base0;
+  // Entries go by the whole plan's pairs, as in the list.
+  const bool one = short_entries(ra, w.start[q.m]);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     st->K = need;
     if (need > w.capacity) atomicOr(&st->err, kErrCapacity);
@@ -1057,16 +1162,18 @@ k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uin
   // stay below need <= capacity.
   if (need > w.capacity) return;
   if (!WIDE && need > 0xffffffffull) return;  // host picks WIDE for such ranges
-  // entries of the range; fewer than max_blocks, so 32 bits hold them
-  const uint32_t i0 = ra.blk_list ? (uint32_t)ra.pkt_off[p0] : 0u;
-  const uint32_t i1 = ra.blk_list ? (uint32_t)ra.pkt_off[p1]
-                                  : ra.chains / kRecChains + ra.blk_counter[0];
-  if (need <= (unsigned long long)kShortEntry * (i1 - i0))
-    replay_entries<FILTER_ID, WIDE, BATCH, OUT, true>(sm, t, q, bv, ra, w, i0, i1, pb, pe, idb, ide,
-                                                      base0, need, work, st);
+  // entries of the range; at most max_blocks, so 32 bits hold them
+  uint32_t i0 = 0, i1 = (one ? ra.chains / kRecChains : ra.chains) + ra.blk_counter[0];
+  if (ra.blk_list) {
+    i0 = (uint32_t)ra.pkt_off[p0] + (one ? 0u : p0);
+    i1 = (uint32_t)ra.pkt_off[p1] + (one ? 0u : p1);
+  }
+  if (one)
+    replay_short<FILTER_ID, WIDE, BATCH, OUT>(sm, t, q, bv, ra, w, i0, i1, pb, pe, idb, ide, base0,
+                                              need, work, st);
   else
-    replay_entries<FILTER_ID, WIDE, BATCH, OUT, false>(sm, t, q, bv, ra, w, i0, i1, pb, pe, idb,
-                                                       ide, base0, need, work, st);
+    replay_long<FILTER_ID, WIDE, BATCH, OUT>(sm, t, q, bv, ra, w, i0, i1, pb, pe, idb, ide, base0,
+                                             need, work, st);
 }
 
 template <bool WRITE, bool BATCH>
@@ -1182,10 +1289,11 @@ cudaError_t launch_write(const TreeView& t, const QueryView& q, const BatchView&
   return launch_packets<true>(t, q, bv, flags, nullptr, nullptr, ra, w, work, false, st, sms, s);
 }
 
-cudaError_t launch_block_list(const RecordArena& ra, int sms, cudaStream_t s) {
+cudaError_t launch_block_list(const RecordArena& ra, const unsigned long long* pairs, int sms,
+                              cudaStream_t s) {
   if (ra.max_blocks == 0) return cudaSuccess;
   const uint32_t need = (ra.max_blocks + 255) / 256, cap = (uint32_t)sms * 8u;
-  k_block_list<<<need < cap ? need : cap, 256, 0, s>>>(ra);
+  k_block_list<<<need < cap ? need : cap, 256, 0, s>>>(ra, pairs);
   note_launches(1);
   return cudaGetLastError();
 }
