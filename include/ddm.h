@@ -474,6 +474,16 @@ int ddm_scan_counts_noalloc(const uint32_t *counts, uint32_t m, uint64_t *offset
  * counterpart. */
 int ddm_debug_wait_timeout(ddm_ctx *ctx, uint32_t polls, void *stream);
 
+/* The same for the scan of a plan's match counts, whose tiles wait for the
+ * tiles before them: scans the counts of the current plan (more than 4096
+ * updates, else DDM_ERR_ARG) again without its first tile, with waits of at
+ * most `polls` polls (1..2^22).  Returns DDM_ERR_TIMEOUT; the plan's offsets
+ * are wrong from then on, as after a plan whose wait ran out, and until the
+ * next plan every write of it (and the chunk planning) reports
+ * DDM_ERR_TIMEOUT, or its error bit, and writes nothing.  DDM_ERR_STATE
+ * without a plan.  The paper has no counterpart. */
+int ddm_debug_scan_timeout(ddm_ctx *ctx, uint32_t polls, void *stream);
+
 /* Number of CUDA kernels this library has launched in the calling process
  * since it was loaded (all contexts).  Host-side counter, no GPU access. */
 uint64_t ddm_debug_launch_count(void);

@@ -78,6 +78,7 @@ SIGNATURES = {
     "ddm_set_tiling": (_i, [_vp, _u32, _u32]),
     "ddm_debug_launch_count": (_u64, []),
     "ddm_debug_wait_timeout": (_i, [_vp, _u32, _vp]),
+    "ddm_debug_scan_timeout": (_i, [_vp, _u32, _vp]),
     "ddm_scan_counts_noalloc": (_i, [_vp, _u32, _vp, _vp]),
     "ddm_batch_match": (_i, [_vp, _i, _u32, _vp, _vp, _vp, _u32, _vp, _vp, _vp, _u32, _u32, _vp,
                              _u64, _vp, _pu64, _vp]),
@@ -470,6 +471,12 @@ def ddm_debug_set_alloc_limit(ctx: int, nbytes: int) -> None:
 def ddm_debug_wait_timeout(ctx: int, polls: int, stream=None) -> None:
     """Make a bounded device wait run out (raises DDMError DDM_ERR_TIMEOUT)."""
     _check(lib().ddm_debug_wait_timeout(ctx, polls, _stream(stream)), "ddm_debug_wait_timeout")
+
+
+def ddm_debug_scan_timeout(ctx: int, polls: int, stream=None) -> None:
+    """Make the waits of the plan's scan run out (raises DDMError
+    DDM_ERR_TIMEOUT); the plan's writes then report the same until the next plan."""
+    _check(lib().ddm_debug_scan_timeout(ctx, polls, _stream(stream)), "ddm_debug_scan_timeout")
 
 
 def ddm_debug_launch_count() -> int:

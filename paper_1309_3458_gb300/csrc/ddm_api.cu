@@ -90,7 +90,7 @@ struct ddm_ctx {
   DevBuf leaf_off;              // padded tree of a batch
   // size classes of the tree order (d >= 2)
   DevBuf cls_hist, cls_off;
-  DevBuf probe;                 // word polled by ddm_debug_wait_timeout
+  DevBuf probe;                 // words polled by the ddm_debug_*_timeout calls
   BatchView bv{};               // count 0 = single problem
   // tuning knobs (ddm_set_tuning)
   int str_shift = 0;            // added to the re-sort group exponents
@@ -632,6 +632,14 @@ QueryView query_view(ddm_ctx* c) {
   return q;
 }
 
+// Words before the scans' state in plan_state: the block counter, and whether
+// a wait of the plan's scan ran out (kept until the next plan, since every
+// later call on the plan uses its offsets).
+constexpr size_t kPlanWords = 2;
+uint32_t* plan_failed(const ddm_ctx* c) {
+  return reinterpret_cast<uint32_t*>(static_cast<unsigned long long*>(c->plan_state.p) + 1);
+}
+
 int ensure_queries(ddm_ctx* c, int d, uint32_t m) {
   DDM_TRY(ensure(c, c->qe, sizeof(float2) * (size_t)d * (m ? m : 1)));
   return ensure(c, c->qid, sizeof(uint32_t) * (m ? m : 1));
@@ -732,14 +740,15 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
   }
   // Offsets by update id and, for a plan whose order will be written or read
   // out, by plan position and of the record entries in plan order.  The block
-  // counter (two words) and the scans' state are cleared by one memset.
+  // counter (two words), the plan's failure word (plan_failed) and the scans'
+  // state are cleared by one memset.
   const uint32_t packets = packets_of(c, m);
   const ScanJob jobs[kMaxScanJobs] = {
       {counts, m, offsets, true},
       {counts_pos, m, pos_offsets, false},
       {c->arena.pkt_nblk, packets, c->arena.pkt_off, false}};
   const int njobs = !ordered ? 1 : c->arena.max_blocks ? 3 : 2;
-  const size_t state_words = 1 + scan_state_words(jobs, njobs);
+  const size_t state_words = kPlanWords + scan_state_words(jobs, njobs);
   DDM_TRY(ensure(c, c->plan_state, sizeof(unsigned long long) * state_words));
   if (!ordered)  // what ready_ordered() needs, so that it never allocates
     DDM_TRY(ensure(c, c->order_state,
@@ -760,7 +769,7 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
   }
   const ScanHint hint{c->arena.max_blocks ? c->rec_hint : nullptr, c->arena.blk_counter,
                       c->arena.chains, packets, c->arena.max_blocks};
-  DDM_CUDA(launch_scan_multi(jobs, njobs, state + 1, hint, c->st_dev, s));
+  DDM_CUDA(launch_scan_multi(jobs, njobs, state + kPlanWords, hint, plan_failed(c), c->st_dev, s));
   if (ordered && c->arena.max_blocks)
     DDM_CUDA(launch_block_list(c->arena, pos_offsets + m, c->sms, s));
   c->ordered = ordered;
@@ -802,7 +811,7 @@ int ready_ordered(ddm_ctx* c, cudaStream_t s) {
   DDM_TRY(ensure(c, c->order_state, sizeof(unsigned long long) * words));  // done by the plan
   auto* state = static_cast<unsigned long long*>(c->order_state.p);
   DDM_CUDA(cudaMemsetAsync(state, 0, sizeof(unsigned long long) * words, s));
-  DDM_CUDA(launch_scan_multi(jobs, njobs, state, ScanHint{}, c->st_dev, s));
+  DDM_CUDA(launch_scan_multi(jobs, njobs, state, ScanHint{}, plan_failed(c), c->st_dev, s));
   if (c->arena.max_blocks)
     DDM_CUDA(launch_block_list(c->arena, jobs[0].offsets + c->m, c->sms, s));
   c->ordered = !c->capturing;  // recorded only: it runs with the graph
@@ -839,6 +848,7 @@ int write_async(ddm_ctx* c, uint32_t begin, uint32_t end, ddm_pair* pairs, uint6
     w.e_idx = end;
     w.pairs = pairs;
     w.capacity = capacity;
+    w.failed = plan_failed(c);
     if (c->arena.max_blocks) {
       const bool full = begin == 0 && end == c->m;
       RecordArena ra = c->arena;
@@ -873,6 +883,7 @@ int write_ordered_async(ddm_ctx* c, uint32_t pb, uint32_t pe, ddm_pair* pairs, u
     w.pairs = pairs;
     w.ids = ids;
     w.capacity = capacity;
+    w.failed = plan_failed(c);
     if (c->arena.max_blocks)
       DDM_CUDA(launch_replay(c->tree, q, c->bv, c->arena, w, pb >> c->plan_qpp_log2, packets_of(c, pe), pb, pe, false, 0, 0,
                              c->st_dev->work + 1, zeroed_work(c, 1), c->st_dev, c->sms, s));
@@ -1080,6 +1091,24 @@ int ddm_debug_wait_timeout(ddm_ctx* c, uint32_t polls, void* stream) {
   return status_code(*c->st_host);
 }
 
+int ddm_debug_scan_timeout(ddm_ctx* c, uint32_t polls, void* stream) {
+  if (!c || polls == 0 || polls > (1u << 22)) return DDM_ERR_ARG;
+  if (!c->planned) return DDM_ERR_STATE;
+  const ScanJob job{static_cast<uint32_t*>(c->counts.p), c->m,
+                    static_cast<unsigned long long*>(c->offsets.p), true};
+  if (c->m <= (uint32_t)kScanTile) return DDM_ERR_ARG;
+  DeviceGuard g(c->device);
+  if (!g.ok()) return DDM_ERR_CUDA;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  StreamUse use(c, s);
+  DDM_TRY(ensure(c, c->probe, sizeof(unsigned long long) * scan_state_words(&job, 1)));
+  DDM_TRY(reset_status(c, s));
+  DDM_CUDA(launch_debug_scan(job, static_cast<unsigned long long*>(c->probe.p), polls, plan_failed(c),
+                             c->st_dev, s));
+  DDM_TRY(sync_status(c, s));
+  return status_code(*c->st_host);
+}
+
 uint64_t ddm_debug_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
 
 int ddm_debug_set_alloc_limit(ddm_ctx* c, uint64_t bytes) {
@@ -1149,8 +1178,9 @@ int ddm_chunk_end(ddm_ctx* c, uint32_t begin, uint64_t capacity, uint32_t* upd_e
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   StreamUse use(c, s);
   DDM_CUDA(launch_chunk_end(static_cast<const unsigned long long*>(c->offsets.p), c->m, begin,
-                            capacity, c->st_dev, s));
+                            capacity, plan_failed(c), c->st_dev, s));
   DDM_TRY(sync_status(c, s));
+  if (c->st_host->aux == kPlanFailed) return DDM_ERR_TIMEOUT;
   *upd_end = (uint32_t)c->st_host->aux;
   if (*upd_end == begin && begin < c->m) return DDM_ERR_CAPACITY;
   return DDM_OK;
@@ -1278,8 +1308,9 @@ int ddm_chunk_end_ordered(ddm_ctx* c, uint32_t pos_begin, uint64_t capacity, uin
   StreamUse use(c, s);
   DDM_TRY(ready_ordered(c, s));
   DDM_CUDA(launch_chunk_end(static_cast<const unsigned long long*>(c->pos_offsets.p), c->m,
-                            pos_begin, capacity, c->st_dev, s));
+                            pos_begin, capacity, plan_failed(c), c->st_dev, s));
   DDM_TRY(sync_status(c, s));
+  if (c->st_host->aux == kPlanFailed) return DDM_ERR_TIMEOUT;
   *pos_end = (uint32_t)c->st_host->aux;
   if (*pos_end == pos_begin && pos_begin < c->m) return DDM_ERR_CAPACITY;
   return DDM_OK;

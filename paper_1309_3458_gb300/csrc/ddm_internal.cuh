@@ -103,6 +103,9 @@ struct WriteView {
   ddm_pair* pairs;
   uint32_t* ids;  // when set: only each pair's subscription id is written, here, and pairs is unused
   unsigned long long capacity;
+  // set if a wait of the plan's scan ran out: its offsets are too small, so
+  // that need <= capacity bounds nothing; nothing is written then
+  const uint32_t* failed;
 };
 
 // Batched instances: instance i owns update positions [upd_off[i],
@@ -413,6 +416,8 @@ cudaError_t launch_scan(const uint32_t* counts, uint32_t m, unsigned long long* 
                         unsigned long long* block_sums, Status* st, cudaStream_t s);
 // Up to kMaxScanJobs independent scans of the form above in one launch.
 // `state` holds scan_state_words() words, zeroed by the caller on the stream.
+// A wait that runs out is recorded in st->err and *failed (its offsets are then
+// too small).
 // `hint` (optional) receives the sizing hint of the plan's record arena.
 struct ScanJob {
   const uint32_t* counts;
@@ -430,9 +435,16 @@ struct ScanHint {
 };
 size_t scan_state_words(const ScanJob* jobs, int count);
 cudaError_t launch_scan_multi(const ScanJob* jobs, int count, unsigned long long* state,
-                              const ScanHint& hint, Status* st, cudaStream_t s);
+                              const ScanHint& hint, uint32_t* failed, Status* st, cudaStream_t s);
+// Test hook: the scan of `job` without its first tile, so that the waits of
+// the others, of at most `polls` polls, run out.
+cudaError_t launch_debug_scan(const ScanJob& job, unsigned long long* state, uint32_t polls,
+                              uint32_t* failed, Status* st, cudaStream_t s);
+// st->aux = the largest end, kPlanFailed in its place if *failed is set.
+constexpr unsigned long long kPlanFailed = ~0ull;
 cudaError_t launch_chunk_end(const unsigned long long* offsets, uint32_t m, uint32_t begin,
-                             unsigned long long capacity, Status* st, cudaStream_t s);
+                             unsigned long long capacity, const uint32_t* failed, Status* st,
+                             cudaStream_t s);
 // list = sorted positions i (ascending) with begin <= qid[i] < end; uses
 // flags/offs/sums as scratch.
 cudaError_t launch_select(const uint32_t* qid, uint32_t m, uint32_t begin, uint32_t end,

@@ -206,6 +206,10 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
 
   unsigned long long base0 = 0;
   if (WRITE) {
+    if (*w.failed) {
+      if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&st->err, kErrTimeout);
+      return;
+    }
     if (records_complete(ra)) return;  // the replay kernel writes this range
     base0 = w.start[w.b_idx];
     const unsigned long long need = w.start[w.e_idx] - base0;
@@ -1144,20 +1148,27 @@ k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uin
          uint32_t p1, uint32_t pb, uint32_t pe, uint32_t idb, uint32_t ide,
          uint32_t* __restrict__ work, Status* __restrict__ st) {
   __shared__ ReplaySmem<WIDE, BATCH, OUT> sm;
-  if (!records_complete(ra)) {  // the walking write pass handles this range
-    if (blockIdx.x == 0 && threadIdx.x == 0) st->walk = 1u;
-    return;
-  }
+  // all loads first: a latency each otherwise
+  const uint32_t failed = *w.failed;
+  const bool complete = records_complete(ra);
   const unsigned long long base0 = w.start[w.b_idx];
   const unsigned long long need = w.start[w.e_idx] - base0;
   // Entries go by the whole plan's pairs, as in the list.
   const bool one = short_entries(ra, w.start[q.m]);
+  if (failed) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&st->err, kErrTimeout);
+    return;
+  }
+  if (!complete) {  // the walking write pass handles this range
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->walk = 1u;
+    return;
+  }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     st->K = need;
     if (need > w.capacity) atomicOr(&st->err, kErrCapacity);
   }
-  // Pair positions are bounded by construction: a record's pairs go to its
-  // update's offset plus the matches the count pass had found before it, and
+  // Pair positions are bounded by construction (the scan is whole): a record's
+  // pairs go to its update's offset plus the matches the count pass had found before it, and
   // the update's count is the sum of its records' popcounts, so all writes
   // stay below need <= capacity.
   if (need > w.capacity) return;

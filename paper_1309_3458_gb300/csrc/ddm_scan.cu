@@ -165,7 +165,7 @@ struct ScanJobs {
 constexpr unsigned long long kScanAgg = 1ull << 62;  // the tile's own sum
 constexpr unsigned long long kScanInc = 2ull << 62;  // sum up to and including the tile
 constexpr unsigned long long kScanMask = 3ull << 62;
-constexpr uint32_t kScanSpinLimit = 1u << 22;
+constexpr uint32_t kScanPolls = 1u << 22;
 
 __device__ __forceinline__ unsigned long long ld_relaxed64(const unsigned long long* p) {
   unsigned long long v;
@@ -178,7 +178,8 @@ __device__ __forceinline__ void st_relaxed64(unsigned long long* p, unsigned lon
 
 // Sum of the job's tiles before this one; called by one whole warp.
 __device__ __forceinline__ unsigned long long scan_look_back(const unsigned long long* words,
-                                                             uint32_t tile, Status* st) {
+                                                             uint32_t tile, uint32_t polls,
+                                                             uint32_t* failed, Status* st) {
   const int lane = threadIdx.x & 31;
   unsigned long long sum = 0;
   for (uint32_t end = tile;; end -= 32u) {  // words [end - 32, end), lane 0 the nearest
@@ -186,8 +187,9 @@ __device__ __forceinline__ unsigned long long scan_look_back(const unsigned long
     if ((uint32_t)lane < end) {
       const unsigned long long* p = words + (end - 1u - (uint32_t)lane);
       for (uint32_t spins = 0; !((w = ld_relaxed64(p)) & kScanMask); ++spins) {
-        if (spins >= kScanSpinLimit) {
+        if (spins >= polls) {  // offsets that are too small: no write may use them
           atomicOr(&st->err, kErrTimeout);
+          atomicOr(failed, 1u);
           w = kScanInc;
           break;
         }
@@ -207,7 +209,7 @@ __device__ __forceinline__ unsigned long long scan_look_back(const unsigned long
 
 __global__ void __launch_bounds__(kThreads)
 k_scan_multi(const ScanJobs js, unsigned long long* __restrict__ state, const ScanHint hint,
-             Status* __restrict__ st) {
+             uint32_t polls, uint32_t* __restrict__ failed, Status* __restrict__ st) {
   // one word of padding per thread's 16 items: their strided accesses then
   // fall into different banks (a 16-way conflict took 3 of 8 us per tile)
   __shared__ __align__(8) uint32_t s_c[kScanTile + kThreads];
@@ -246,7 +248,7 @@ k_scan_multi(const ScanJobs js, unsigned long long* __restrict__ state, const Sc
     unsigned long long pre = 0;
     if (tile > 0) {
       if (threadIdx.x == 0) st_relaxed64(words + tile, kScanAgg | tot);
-      pre = scan_look_back(words, tile, st);
+      pre = scan_look_back(words, tile, polls, failed, st);
     }
     if (threadIdx.x == 0) {
       st_relaxed64(words + tile, kScanInc | (pre + tot));
@@ -286,7 +288,12 @@ k_scan_multi(const ScanJobs js, unsigned long long* __restrict__ state, const Sc
 
 // Largest e in [begin, m] with offsets[e] - offsets[begin] <= capacity.
 __global__ void k_chunk_end(const unsigned long long* __restrict__ offsets, uint32_t m, uint32_t begin,
-                            unsigned long long capacity, Status* __restrict__ st) {
+                            unsigned long long capacity, const uint32_t* __restrict__ failed,
+                            Status* __restrict__ st) {
+  if (*failed) {
+    st->aux = kPlanFailed;
+    return;
+  }
   const unsigned long long b0 = offsets[begin];
   uint32_t lo = begin, hi = m;  // invariant: offsets[lo] - b0 <= capacity
   while (lo < hi) {
@@ -358,7 +365,7 @@ size_t scan_state_words(const ScanJob* jobs, int count) {
 }
 
 cudaError_t launch_scan_multi(const ScanJob* jobs, int count, unsigned long long* state,
-                              const ScanHint& hint, Status* st, cudaStream_t s) {
+                              const ScanHint& hint, uint32_t* failed, Status* st, cudaStream_t s) {
   if (count < 1 || count > kMaxScanJobs) return cudaErrorInvalidValue;
   ScanJobs js = {};
   js.count = count;
@@ -366,14 +373,31 @@ cudaError_t launch_scan_multi(const ScanJob* jobs, int count, unsigned long long
     js.job[j] = jobs[j];
     js.tile0[j + 1] = js.tile0[j] + scan_tiles(jobs[j].m);
   }
-  k_scan_multi<<<js.tile0[count], kThreads, 0, s>>>(js, state, hint, st);
+  k_scan_multi<<<js.tile0[count], kThreads, 0, s>>>(js, state, hint, kScanPolls, failed, st);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_debug_scan(const ScanJob& job, unsigned long long* state, uint32_t polls,
+                              uint32_t* failed, Status* st, cudaStream_t s) {
+  const uint32_t tiles = scan_tiles(job.m);
+  if (tiles < 2) return cudaErrorInvalidValue;
+  ScanJobs js = {};
+  js.count = 1;
+  js.job[0] = job;
+  js.tile0[1] = tiles;
+  cudaError_t e = cudaMemsetAsync(state, 0, sizeof(unsigned long long) * scan_state_words(&job, 1), s);
+  if (!e) e = cudaMemsetAsync(state, 1, 1, s);  // ticket 0 is taken, by nobody
+  if (e) return e;
+  k_scan_multi<<<tiles - 1, kThreads, 0, s>>>(js, state, ScanHint{}, polls, failed, st);
   note_launches(1);
   return cudaGetLastError();
 }
 
 cudaError_t launch_chunk_end(const unsigned long long* offsets, uint32_t m, uint32_t begin,
-                             unsigned long long capacity, Status* st, cudaStream_t s) {
-  k_chunk_end<<<1, 1, 0, s>>>(offsets, m, begin, capacity, st);
+                             unsigned long long capacity, const uint32_t* failed, Status* st,
+                             cudaStream_t s) {
+  k_chunk_end<<<1, 1, 0, s>>>(offsets, m, begin, capacity, failed, st);
   note_launches(1);
   return cudaGetLastError();
 }
