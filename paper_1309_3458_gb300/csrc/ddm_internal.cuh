@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include "ddm.h"
+#include "ddm_ranges.h"
 
 namespace ddm {
 
@@ -167,6 +168,14 @@ __host__ __device__ inline uint32_t float_key(float f) {
 // contexts), for launch accounting by callers; defined in ddm_api.cu.
 void note_launches(unsigned count);
 
+// OwnerSearch by one warp.
+__device__ __forceinline__ uint32_t warp_owner(const unsigned long long* __restrict__ prefix,
+                                               uint32_t count, unsigned long long i) {
+  OwnerSearch s(count);
+  while (s.more()) s.take(__ballot_sync(0xffffffffu, s.probe(prefix, threadIdx.x & 31u, i)));
+  return s.lo;
+}
+
 // ---- ddm_layout.cu --------------------------------------------------------
 // Validate a set (lo <= hi, no NaN in every dimension) and (k32 set) emit its
 // sort key: key(lo0), whole (d = 1 tree; st->redo is then set if the lower
@@ -288,9 +297,9 @@ cudaError_t launch_class_plan(const uint32_t* hist, int d, int shift, const Clas
                               cudaStream_t s);
 // Batched sets: group exponents glog2 [d][count] and first chunks cbase
 // [d][count + 1] of every dimension, and (optional) first leaves leaf_off
-// [count + 1] of a padded tree.
-cudaError_t launch_batch_plan(const unsigned long long* off, uint32_t count, int d, int shift,
-                              int tile_log2, int* glog2, unsigned long long* cbase,
+// [count + 1] of a padded tree.  No chunks if `off` descends or passes `total`.
+cudaError_t launch_batch_plan(const unsigned long long* off, uint32_t count, uint32_t total, int d,
+                              int shift, int tile_log2, int* glog2, unsigned long long* cbase,
                               unsigned long long* leaf_off, cudaStream_t s);
 // Stable re-sort of the ids in `vals` by the locality key of lo_k inside each
 // group, in place; with one instance g is its group exponent.  tmp0 and tmp1

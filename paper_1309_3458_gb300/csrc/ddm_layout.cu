@@ -165,7 +165,7 @@ k_validate_class(int d, const float* __restrict__ lo, const float* __restrict__ 
 }
 
 // Instance (batched set, or size class) of every position: the b with
-// off[b] <= i < off[b+1].  A warp fills kFillSpan consecutive positions: one
+// off[b] <= i < off[b+1] (some b for offsets that are no prefix sums).  A warp fills kFillSpan consecutive positions: one
 // search over the offsets (32 places a step), then 32 positions at a time, a
 // lane walking on from the last instance found; so one very large instance is
 // filled by the whole grid, and the pass is bound by its stores (a binary
@@ -177,19 +177,9 @@ k_fill_inst(const unsigned long long* __restrict__ off, uint32_t count, uint32_t
   const uint32_t lane = threadIdx.x & 31u, warps = gridDim.x * (blockDim.x / 32u);
   for (size_t i0 = (size_t)(blockIdx.x * (blockDim.x / 32u) + threadIdx.x / 32u) * kFillSpan;
        i0 < total; i0 += (size_t)warps * kFillSpan) {
-    uint32_t lo = 0, hi = count;  // off[lo] <= i0 < off[hi]
-    while (hi - lo > 1) {
-      const uint32_t step = (hi - lo + 31u) / 32u, at = lo + lane * step;
-      const uint32_t m = __ballot_sync(0xffffffffu, at < hi && off[at] <= i0);
-      lo += (31u - __clz(m)) * step;
-      hi = min(hi, lo + step);
-    }
+    OwnerWalk<const unsigned long long*> owner(off, count, warp_owner(off, count, i0));
     const size_t end = min(i0 + kFillSpan, (size_t)total);
-    unsigned long long next = off[lo + 1];
-    for (size_t i = i0 + lane; i < end; i += 32u) {
-      while (next <= i) next = off[++lo + 1];  // i < total = off[count]
-      inst[i] = lo;
-    }
+    for (size_t i = i0 + lane; i < end; i += 32u) inst[i] = owner.at(i);
   }
 }
 

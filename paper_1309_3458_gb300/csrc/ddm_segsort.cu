@@ -272,26 +272,16 @@ k_segsort(uint32_t* __restrict__ vals, const float* __restrict__ lo_k, uint32_t 
   constexpr uint32_t kTile = THREADS * ITEMS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SegSmem<THREADS, ITEMS>& sm = *reinterpret_cast<SegSmem<THREADS, ITEMS>*>(smem_raw);
-  const uint32_t lane = threadIdx.x & 31u;
   const unsigned long long chunks = off ? cbase[count] : ((unsigned long long)total + kTile - 1) / kTile;
   for (unsigned long long c = blockIdx.x; c < chunks; c += gridDim.x) {
     unsigned long long begin = c * kTile, end = min(begin + kTile, (unsigned long long)total);
     int g = g_one;
     if (off) {
-      // The instance whose chunks include c: each warp searches the prefix,
-      // 32 places a step (cbase[lo] <= c < cbase[hi]).
-      uint32_t lo = 0, hi = count;
-      while (hi - lo > 1) {
-        const uint32_t step = (hi - lo + 31u) / 32u, at = lo + lane * step;
-        const uint32_t m = __ballot_sync(0xffffffffu, at < hi && cbase[at] <= c);
-        const uint32_t l = 31u - __clz(m);  // lane 0 always holds
-        lo += l * step;
-        hi = min(hi, lo + step);
-      }
-      g = glog2[lo];
+      const uint32_t b = warp_owner(cbase, count, c);  // the instance whose chunks include c
+      g = glog2[b];
       const unsigned long long size = max((unsigned long long)kTile, 1ull << g);
-      begin = off[lo] + (c - cbase[lo]) * size;
-      end = min(begin + size, off[lo + 1]);
+      begin = off[b] + (c - cbase[b]) * size;
+      end = min(begin + size, off[b + 1]);
     }
     const uint32_t len = (uint32_t)(end - begin);
     if (len > kTile)
@@ -382,23 +372,33 @@ __device__ __forceinline__ uint32_t scan1024(uint32_t v, uint32_t* s_w, uint32_t
 // Batched sets (one CTA, 4,096 instances a round): the prefix of leaves of a
 // padded tree and, for every dimension k >= 1, each instance's group exponent
 // and the prefix of chunks.  One launch, where a launch per step (counts,
-// scan) put seven on the way of a small batch.
+// scan) put seven on the way of a small batch.  Offsets that descend or pass
+// the set's `total` get no chunks: the re-sorts move ids in place, and chunks
+// of such offsets could overlap or lie outside the set.
 __global__ void __launch_bounds__(1024)
-k_batch_plan(const unsigned long long* __restrict__ off, uint32_t count, int d, int shift,
-             uint32_t tile, int* __restrict__ glog2, unsigned long long* __restrict__ cbase,
+k_batch_plan(const unsigned long long* __restrict__ off, uint32_t count, uint32_t total, int d,
+             int shift, uint32_t tile, int* __restrict__ glog2, unsigned long long* __restrict__ cbase,
              unsigned long long* __restrict__ leaf_off) {
   constexpr int kEach = 4;
   __shared__ uint32_t s_w[32];
   unsigned long long carry[DDM_MAX_DIMS] = {};  // [0]: leaves
+  bool bad = off[count] > total;
   for (uint32_t c0 = 0; c0 < count; c0 += 1024u * kEach) {
     uint32_t n[kEach];
     const uint32_t i0 = c0 + threadIdx.x * kEach;
 #pragma unroll
-    for (int u = 0; u < kEach; ++u) n[u] = i0 + u < count ? (uint32_t)(off[i0 + u + 1] - off[i0 + u]) : 0u;
+    for (int u = 0; u < kEach; ++u) {
+      n[u] = 0u;
+      if (i0 + u < count) {
+        const unsigned long long a = off[i0 + u], b = off[i0 + u + 1];
+        bad |= b < a;
+        n[u] = (uint32_t)(b - a);
+      }
+    }
 #pragma unroll
     for (int k = 0; k < DDM_MAX_DIMS; ++k) {
       if (k >= d || (k == 0 && !leaf_off)) continue;
-      uint32_t v[kEach], sum = 0, total;
+      uint32_t v[kEach], sum = 0, all;
 #pragma unroll
       for (int u = 0; u < kEach; ++u) {
         if (k == 0) {
@@ -410,21 +410,22 @@ k_batch_plan(const unsigned long long* __restrict__ off, uint32_t count, int d, 
         }
         sum += v[u];
       }
-      unsigned long long at = carry[k] + scan1024(sum, s_w, &total);
+      unsigned long long at = carry[k] + scan1024(sum, s_w, &all);
       unsigned long long* out = k == 0 ? leaf_off : cbase + (size_t)k * (count + 1u);
 #pragma unroll
       for (int u = 0; u < kEach; ++u) {
         if (i0 + u < count) out[i0 + u] = at;
         at += v[u];
       }
-      carry[k] += total;
+      carry[k] += all;
     }
   }
+  bad = __syncthreads_or(bad);
   if (threadIdx.x == 0) {
     if (leaf_off) leaf_off[count] = carry[0];
 #pragma unroll
     for (int k = 1; k < DDM_MAX_DIMS; ++k)
-      if (k < d) cbase[(size_t)k * (count + 1u) + count] = carry[k];
+      if (k < d) cbase[(size_t)k * (count + 1u) + count] = bad ? 0ull : carry[k];
   }
 }
 
@@ -512,10 +513,10 @@ cudaError_t ready_group_table() {
   return e;
 }
 
-cudaError_t launch_batch_plan(const unsigned long long* off, uint32_t count, int d, int shift,
-                              int tile_log2, int* glog2, unsigned long long* cbase,
+cudaError_t launch_batch_plan(const unsigned long long* off, uint32_t count, uint32_t total, int d,
+                              int shift, int tile_log2, int* glog2, unsigned long long* cbase,
                               unsigned long long* leaf_off, cudaStream_t s) {
-  k_batch_plan<<<1, 1024, 0, s>>>(off, count, d, shift, 1u << tile_log2, glog2, cbase, leaf_off);
+  k_batch_plan<<<1, 1024, 0, s>>>(off, count, total, d, shift, 1u << tile_log2, glog2, cbase, leaf_off);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -102,16 +102,9 @@ k_gather_build(TreeView t, uint32_t set_n, LeafMap map, const uint32_t* __restri
   if (map.leaf_off && gvalid) {  // warp-uniform
     valid = false;
     if (g < map.leaf_off[map.count]) {
-      // the instance owning leaf g: 32 places a step
-      uint32_t b = 0, hi = map.count;  // leaf_off[b] <= g < leaf_off[hi]
-      while (hi - b > 1) {
-        const uint32_t step = (hi - b + 31u) / 32u, at = b + (uint32_t)lane * step;
-        const uint32_t m = __ballot_sync(0xffffffffu, at < hi && map.leaf_off[at] <= g);
-        b += (31u - __clz(m)) * step;
-        hi = min(hi, b + step);
-      }
+      const uint32_t b = warp_owner(map.leaf_off, map.count, g);  // the instance owning leaf g
       const unsigned long long j = map.off[b] + (g - map.leaf_off[b]) * 32u + lane;
-      valid = j < map.off[b + 1];
+      valid = j < map.off[b + 1] && j < set_n;  // offsets that pass the set: inside it all the same
       from = (uint32_t)j;
     }
   }
