@@ -389,6 +389,7 @@ struct BatchSet {
 int ensure_batch(ddm_ctx* c, OrderBufs& o, int d, uint32_t cnt, uint32_t count) {
   DDM_TRY(ensure_sort(c, o, cnt));
   DDM_TRY(ensure(c, o.bglog2, sizeof(int) * (size_t)d * count));
+  DDM_TRY(ensure(c, o.sums, sizeof(unsigned long long) * batch_plan_words(count, d)));
   return ensure(c, o.bgbase, sizeof(unsigned long long) * (size_t)d * ((size_t)count + 1));
 }
 
@@ -401,7 +402,8 @@ int order_set_batch(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const floa
   auto* gl = static_cast<int*>(o.bglog2.p);
   auto* cb = static_cast<unsigned long long*>(o.bgbase.p);
   if (d > 1 || bs.leaf_off)
-    DDM_CUDA(launch_batch_plan(bs.off, bs.count, cnt, d, c->str_shift, kSegTileLog2, gl, cb, bs.leaf_off, s));
+    DDM_CUDA(launch_batch_plan(bs.off, bs.count, cnt, d, c->str_shift, kSegTileLog2, gl, cb, bs.leaf_off,
+                               static_cast<unsigned long long*>(o.sums.p), s));
   DDM_CUDA(launch_fill_inst(bs.off, bs.count, cnt, bs.inst, c->sms, s));
   const int inst_bits = bits_of(bs.count ? bs.count - 1u : 0u), id_bits = id_bits_of(cnt);
   const bool packed = inst_bits + 24 + id_bits <= 64;

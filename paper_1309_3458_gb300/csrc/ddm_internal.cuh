@@ -298,9 +298,12 @@ cudaError_t launch_class_plan(const uint32_t* hist, int d, int shift, const Clas
 // Batched sets: group exponents glog2 [d][count] and first chunks cbase
 // [d][count + 1] of every dimension, and (optional) first leaves leaf_off
 // [count + 1] of a padded tree.  No chunks if `off` descends or passes `total`.
+// sums: batch_plan_words() words of scratch.
+size_t batch_plan_words(uint32_t count, int d);
 cudaError_t launch_batch_plan(const unsigned long long* off, uint32_t count, uint32_t total, int d,
                               int shift, int tile_log2, int* glog2, unsigned long long* cbase,
-                              unsigned long long* leaf_off, cudaStream_t s);
+                              unsigned long long* leaf_off, unsigned long long* sums,
+                              cudaStream_t s);
 // Stable re-sort of the ids in `vals` by the locality key of lo_k inside each
 // group, in place; with one instance g is its group exponent.  tmp0 and tmp1
 // (`total` words each) are used only by groups larger than a chunk's tile.

@@ -179,6 +179,7 @@ k_fill_inst(const unsigned long long* __restrict__ off, uint32_t count, uint32_t
        i0 < total; i0 += (size_t)warps * kFillSpan) {
     OwnerWalk<const unsigned long long*> owner(off, count, warp_owner(off, count, i0));
     const size_t end = min(i0 + kFillSpan, (size_t)total);
+#pragma unroll 4
     for (size_t i = i0 + lane; i < end; i += 32u) inst[i] = owner.at(i);
   }
 }

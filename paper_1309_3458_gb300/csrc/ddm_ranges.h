@@ -41,15 +41,32 @@ struct OwnerSearch {
   }
 };
 
-// Owners of ascending positions, from instance b (which owns one no later) on.
+// Owners of ascending positions, from instance b (which owns one no later) on:
+// the next few instances one by one, behind a longer run of empty ones a search.
 template <typename Prefix>
 struct OwnerWalk {
   Prefix prefix;
   uint32_t count, b;
-  unsigned long long next;  // first position behind instance b
-  DDM_HD OwnerWalk(Prefix p, uint32_t n, uint32_t from) : prefix(p), count(n), b(from), next(p[from + 1u]) {}
+  unsigned long long next;  // first position behind instance b; none behind the last
+  DDM_HD OwnerWalk(Prefix p, uint32_t n, uint32_t from) : prefix(p), count(n) { enter(from); }
+  DDM_HD void enter(uint32_t to) {
+    b = to;
+    next = to + 1u < count ? prefix[to + 1u] : ~0ull;
+  }
   DDM_HD uint32_t at(unsigned long long i) {
-    while (next <= i && b + 1u < count) next = prefix[++b + 1u];
+    for (int steps = 0; next <= i; ++steps) {
+      if (steps < 8) {
+        enter(b + 1u);
+        continue;
+      }
+      uint32_t lo = b, hi = count;  // prefix[lo] <= i < prefix[hi]
+      while (hi - lo > 1u) {
+        const uint32_t mid = lo + (hi - lo) / 2u;
+        if (prefix[mid] <= i) lo = mid; else hi = mid;
+      }
+      enter(lo);
+      break;
+    }
     return b;
   }
 };

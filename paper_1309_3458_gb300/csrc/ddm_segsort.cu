@@ -369,63 +369,94 @@ __device__ __forceinline__ uint32_t scan1024(uint32_t v, uint32_t* s_w, uint32_t
   return (warp ? pre : 0u) + x - v;
 }
 
-// Batched sets (one CTA, 4,096 instances a round): the prefix of leaves of a
-// padded tree and, for every dimension k >= 1, each instance's group exponent
-// and the prefix of chunks.  One launch, where a launch per step (counts,
-// scan) put seven on the way of a small batch.  Offsets that descend or pass
-// the set's `total` get no chunks: the re-sorts move ids in place, and chunks
-// of such offsets could overlap or lie outside the set.
-__global__ void __launch_bounds__(1024)
+// Sum of one value per thread over 1,024 threads.
+__device__ __forceinline__ unsigned long long sum1024(unsigned long long v, unsigned long long* s_w) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) s_w[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = s_w[lane];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  __syncthreads();
+  return v;
+}
+
+// Batched sets: the prefix of leaves of a padded tree and, for every dimension
+// k >= 1, each instance's group exponent and the prefix of chunks.  A CTA takes
+// kPlanTile instances.  Up to that many are one launch, where a launch per step
+// (counts, scan) put seven on the way of a small batch; more take two, the
+// first for the tiles' sums ([0]: leaves, [k]: chunks, [d]: whether the
+// offsets are unsound), of which each CTA of the second adds up those before it:
+// a match of a million instances, all but one empty, took 1,170 us with one
+// CTA, 211 now.  Offsets that descend or pass the set's `total` get no chunks:
+// the re-sorts move ids in place, and chunks of such offsets could overlap or
+// lie outside the set.
+constexpr uint32_t kPlanEach = 4, kPlanTile = 1024 * kPlanEach;
+enum { kPlanOne, kPlanSums, kPlanRest };  // one tile; the two launches of several
+template <int PHASE>
+__global__ void __launch_bounds__(1024, 1)
 k_batch_plan(const unsigned long long* __restrict__ off, uint32_t count, uint32_t total, int d,
              int shift, uint32_t tile, int* __restrict__ glog2, unsigned long long* __restrict__ cbase,
-             unsigned long long* __restrict__ leaf_off) {
-  constexpr int kEach = 4;
+             unsigned long long* __restrict__ leaf_off, unsigned long long* __restrict__ sums) {
+  __shared__ unsigned long long s_sum[PHASE == kPlanOne ? 1 : 32];
   __shared__ uint32_t s_w[32];
-  unsigned long long carry[DDM_MAX_DIMS] = {};  // [0]: leaves
-  bool bad = off[count] > total;
-  for (uint32_t c0 = 0; c0 < count; c0 += 1024u * kEach) {
-    uint32_t n[kEach];
-    const uint32_t i0 = c0 + threadIdx.x * kEach;
+  const uint32_t tiles = gridDim.x, me = blockIdx.x;
+  const uint32_t i0 = me * kPlanTile + threadIdx.x * kPlanEach;
+  bool bad = false;
+  uint32_t n[kPlanEach];
 #pragma unroll
-    for (int u = 0; u < kEach; ++u) {
-      n[u] = 0u;
-      if (i0 + u < count) {
-        const unsigned long long a = off[i0 + u], b = off[i0 + u + 1];
-        bad |= b < a;
-        n[u] = (uint32_t)(b - a);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < DDM_MAX_DIMS; ++k) {
-      if (k >= d || (k == 0 && !leaf_off)) continue;
-      uint32_t v[kEach], sum = 0, all;
-#pragma unroll
-      for (int u = 0; u < kEach; ++u) {
-        if (k == 0) {
-          v[u] = (n[u] + 31u) / 32u;
-        } else {
-          const int g = used_group(n[u], d, k, shift);
-          if (i0 + u < count) glog2[(size_t)k * count + i0 + u] = g;
-          v[u] = chunks_of(n[u], g, tile);
-        }
-        sum += v[u];
-      }
-      unsigned long long at = carry[k] + scan1024(sum, s_w, &all);
-      unsigned long long* out = k == 0 ? leaf_off : cbase + (size_t)k * (count + 1u);
-#pragma unroll
-      for (int u = 0; u < kEach; ++u) {
-        if (i0 + u < count) out[i0 + u] = at;
-        at += v[u];
-      }
-      carry[k] += all;
+  for (int u = 0; u < (int)kPlanEach; ++u) {
+    n[u] = 0u;
+    if (i0 + u < count) {
+      const unsigned long long a = off[i0 + u], b = off[i0 + u + 1];
+      bad |= b < a || b > total;
+      n[u] = (uint32_t)(b - a);
     }
   }
-  bad = __syncthreads_or(bad);
-  if (threadIdx.x == 0) {
-    if (leaf_off) leaf_off[count] = carry[0];
 #pragma unroll
-    for (int k = 1; k < DDM_MAX_DIMS; ++k)
-      if (k < d) cbase[(size_t)k * (count + 1u) + count] = bad ? 0ull : carry[k];
+  for (int k = 0; k < DDM_MAX_DIMS; ++k) {
+    if (k >= d || (k == 0 && !leaf_off)) continue;
+    uint32_t v[kPlanEach], sum = 0, all;
+#pragma unroll
+    for (int u = 0; u < (int)kPlanEach; ++u) {
+      if (k == 0) {
+        v[u] = (n[u] + 31u) / 32u;
+      } else {
+        const int g = used_group(n[u], d, k, shift);
+        if (PHASE != kPlanSums && i0 + u < count) glog2[(size_t)k * count + i0 + u] = g;
+        v[u] = chunks_of(n[u], g, tile);
+      }
+      sum += v[u];
+    }
+    if (PHASE == kPlanSums) {
+      const unsigned long long mine = sum1024(sum, s_sum);
+      if (threadIdx.x == 0) sums[(size_t)k * tiles + me] = mine;
+      continue;
+    }
+    unsigned long long before = 0;
+    if (PHASE == kPlanRest) {
+      for (uint32_t t = threadIdx.x; t < me; t += 1024u) before += sums[(size_t)k * tiles + t];
+      before = sum1024(before, s_sum);
+    }
+    unsigned long long at = before + scan1024(sum, s_w, &all);
+    unsigned long long* out = k == 0 ? leaf_off : cbase + (size_t)k * (count + 1u);
+#pragma unroll
+    for (int u = 0; u < (int)kPlanEach; ++u) {
+      if (i0 + u < count) out[i0 + u] = at;
+      at += v[u];
+    }
+    if (me + 1u == tiles && threadIdx.x == 0) out[count] = before + all;
+  }
+  if (PHASE == kPlanRest && me + 1u == tiles)
+    for (uint32_t t = threadIdx.x; t < me; t += 1024u) bad |= sums[(size_t)d * tiles + t] != 0ull;
+  bad = __syncthreads_or(bad);
+  if (threadIdx.x != 0) return;
+  if (PHASE == kPlanSums) {
+    sums[(size_t)d * tiles + me] = bad;
+  } else if (bad && me + 1u == tiles) {
+    for (int k = 1; k < d; ++k) cbase[(size_t)k * (count + 1u) + count] = 0ull;
   }
 }
 
@@ -513,11 +544,27 @@ cudaError_t ready_group_table() {
   return e;
 }
 
+size_t batch_plan_words(uint32_t count, int d) {
+  const uint32_t tiles = (count + kPlanTile - 1u) / kPlanTile;
+  return tiles > 1u ? (size_t)tiles * (d + 1) : 0u;
+}
+
 cudaError_t launch_batch_plan(const unsigned long long* off, uint32_t count, uint32_t total, int d,
                               int shift, int tile_log2, int* glog2, unsigned long long* cbase,
-                              unsigned long long* leaf_off, cudaStream_t s) {
-  k_batch_plan<<<1, 1024, 0, s>>>(off, count, total, d, shift, 1u << tile_log2, glog2, cbase, leaf_off);
-  note_launches(1);
+                              unsigned long long* leaf_off, unsigned long long* sums,
+                              cudaStream_t s) {
+  if (count == 0) return cudaSuccess;
+  const uint32_t tiles = (count + kPlanTile - 1u) / kPlanTile, tile = 1u << tile_log2;
+#define DDM_PLAN(PHASE)                                                                           \
+  k_batch_plan<PHASE><<<tiles, 1024, 0, s>>>(off, count, total, d, shift, tile, glog2, cbase, leaf_off, sums)
+  if (tiles == 1u) {
+    DDM_PLAN(kPlanOne);
+  } else {
+    DDM_PLAN(kPlanSums);
+    DDM_PLAN(kPlanRest);
+  }
+#undef DDM_PLAN
+  note_launches(tiles > 1u ? 2u : 1u);
   return cudaGetLastError();
 }
 
