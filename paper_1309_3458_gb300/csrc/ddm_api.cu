@@ -288,8 +288,7 @@ int ensure_sort(ddm_ctx* c, OrderBufs& o, uint32_t cnt) {
 
 // Radix sort of the keys/ids in buffer pair `cur` over `passes` 8-bit
 // digits; `cur` is updated to the buffer pair holding the result.
-int sort_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, int passes, int* cur, cudaStream_t s,
-              const uint32_t* run_if = nullptr) {
+int sort_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, int passes, int* cur, cudaStream_t s) {
   SortScratch sc;
   sc.keys[0] = static_cast<unsigned long long*>(o.keys[*cur].p);
   sc.keys[1] = static_cast<unsigned long long*>(o.keys[*cur ^ 1].p);
@@ -299,7 +298,7 @@ int sort_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, int passes, int* cur, cuda
   sc.lookback = static_cast<uint32_t*>(o.lookback.p);
   sc.counters = static_cast<uint32_t*>(o.counters.p);
   int out = 0;
-  DDM_CUDA(launch_sort64(sc, cnt, passes, &out, run_if, c->st_dev, c->sms, s));
+  DDM_CUDA(launch_sort64(sc, cnt, passes, &out, c->st_dev, c->sms, s));
   *cur ^= out;
   return DDM_OK;
 }
@@ -325,7 +324,7 @@ int id_bits_of(uint32_t cnt) { return std::max(bits_of(cnt - 1u), 1); }
 // Packed sort of a set (launch_sort_packed): the ids end up in vals[0], so
 // *cur becomes 0.  A source's k32 lies in vals[1].
 int packed_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, const uint32_t* hi, bool source, int key_bits,
-                int id_bits, int* cur, cudaStream_t s, bool words_out = false) {
+                int id_bits, int* cur, cudaStream_t s, const float* second = nullptr) {
   SortScratch sc;
   for (int b = 0; b < 2; ++b) {
     sc.keys[b] = static_cast<unsigned long long*>(o.keys[b].p);
@@ -334,9 +333,8 @@ int packed_pass(ddm_ctx* c, OrderBufs& o, uint32_t cnt, const uint32_t* hi, bool
   sc.hist = static_cast<uint32_t*>(o.hist.p);
   sc.lookback = static_cast<uint32_t*>(o.lookback.p);
   sc.counters = static_cast<uint32_t*>(o.counters.p);
-  // the d = 1 tree's words: sorted by both bounds instead if ties abound
-  const SortSource src{source ? sc.vals[1] : nullptr, hi, 24, id_bits, words_out,
-                       words_out ? &c->st_dev->redo : nullptr};
+  const SortSource src{source ? sc.vals[1] : nullptr, hi, 24, id_bits, second != nullptr,
+                       second ? &c->st_dev->both : nullptr, second};
   DDM_CUDA(launch_sort_packed(sc, src, cnt, key_bits, c->st_dev, c->sms, s));
   *cur = 0;
   return DDM_OK;
@@ -527,13 +525,14 @@ int order_set(ddm_ctx* c, OrderBufs& o, int d, const float* lo, const float* hi,
     DDM_CUDA(launch_validate(d, lo, hi, cnt, static_cast<uint32_t*>(o.vals[1].p), tree, aos,
                              c->st_dev, c->sms, s));
     const int id_bits = id_bits_of(cnt);
-    DDM_TRY(packed_pass(c, o, cnt, nullptr, true, tree ? 32 : 24, id_bits, cur, s, tree));
-    if (tree) {  // ties by upper bound; with long runs of ties the sort by both bounds
-      auto* keys = static_cast<unsigned long long*>(o.keys[0].p);
+    DDM_TRY(packed_pass(c, o, cnt, nullptr, true, tree ? 32 : 24, id_bits, cur, s, tree ? hi : nullptr));
+    if (tree) {  // the words are in keys[0]; ties by upper bound
+      auto* words = static_cast<unsigned long long*>(o.keys[0].p);
       auto* vals = static_cast<uint32_t*>(o.vals[0].p);
-      DDM_CUDA(launch_tie_order(keys, cnt, id_bits, hi, vals, &c->st_dev->redo, c->sms, s));
-      DDM_CUDA(launch_tree_keys(lo, hi, cnt, keys, vals, &c->st_dev->redo, c->sms, s));
-      DDM_TRY(sort_pass(c, o, cnt, 8, cur, s, &c->st_dev->redo));  // an even number: vals[0] either way
+      auto* list = static_cast<uint2*>(o.vals[1].p);
+      DDM_CUDA(launch_tie_order(words, cnt, id_bits, hi, vals, list, c->st_dev, c->sms, s));
+      DDM_CUDA(launch_long_ties(words, cnt, id_bits, hi, vals, list,
+                                static_cast<unsigned long long*>(o.keys[1].p), c->st_dev, c->sms, s));
     }
   }
   int glog2[DDM_MAX_DIMS];

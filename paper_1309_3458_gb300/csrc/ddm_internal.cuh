@@ -31,7 +31,10 @@ struct Status {
   unsigned long long aux;  // call-specific (chunk end, ...)
   unsigned long long tests;  // count pass: (query, leaf) tests, 32 subscriptions each
   unsigned int work[2];    // tickets of the packet kernels and of the replay
-  unsigned int redo;       // d = 1 tree: ties too long for the short way
+  // d = 1 tree: sort by both bounds (ties abound), else the runs of equal lower
+  // bounds left to a warp [0] and to a CTA [1] each
+  unsigned int both;
+  unsigned int runs[2];
   unsigned int pad;
 };
 
@@ -178,8 +181,8 @@ __device__ __forceinline__ uint32_t warp_owner(const unsigned long long* __restr
 
 // ---- ddm_layout.cu --------------------------------------------------------
 // Validate a set (lo <= hi, no NaN in every dimension) and (k32 set) emit its
-// sort key: key(lo0), whole (d = 1 tree; st->redo is then set if the lower
-// bounds tie in long runs) or its top 24 bits (a locality order).
+// sort key: key(lo0), whole (d = 1 tree; st->both is then set if one value of
+// the lower bound abounds) or its top 24 bits (a locality order).
 // aos (optional, cnt * d float2): an interleaved copy of the coordinates,
 // aos[i*d + k] = (lo_k, hi_k) of extent i, written while validating, so that
 // the gathers by id read one contiguous record per extent instead of 2d
@@ -187,11 +190,6 @@ __device__ __forceinline__ uint32_t warp_owner(const unsigned long long* __restr
 cudaError_t launch_validate(int d, const float* lo, const float* hi, uint32_t cnt,
                             uint32_t* k32, bool whole_key, float2* aos, Status* st, int sms,
                             cudaStream_t s);
-// Sort keys of the d = 1 tree's order, (key(lo) << 32 | key(hi)), and ids;
-// nothing when *run_if is 0.
-cudaError_t launch_tree_keys(const float* lo, const float* hi, uint32_t cnt,
-                             unsigned long long* keys, uint32_t* vals, const uint32_t* run_if,
-                             int sms, cudaStream_t s);
 // keys[i] = (i >> glog2) << 24 | the top 24 bits of key(lo_k[vals[i]]): re-sort
 // inside groups; with id_bits > 0 the packed word, above the id vals[i].
 cudaError_t launch_rekey(const uint32_t* vals, const float* lo_k, uint32_t cnt, int glog2,
@@ -241,9 +239,8 @@ size_t sort_lookback_words(uint32_t n);
 // Test hook: one warp polls `word` (which nothing sets) with the sort's
 // bounded wait, at most `limit` polls, and records kErrTimeout.
 cudaError_t launch_debug_wait(const uint32_t* word, uint32_t limit, Status* st, cudaStream_t s);
-// With `run_if` the kernels do nothing when *run_if is 0.
-cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf,
-                          const uint32_t* run_if, Status* st, int sms, cudaStream_t s);
+cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf, Status* st, int sms,
+                          cudaStream_t s);
 // The same for keys that fit one 64-bit word together with the id: words key
 // << id_bits | id, sorted by key_bits bits above id_bits; the ids come out in
 // vals[0].  With a source the words are built from it (its arrays may not
@@ -254,13 +251,24 @@ struct SortSource {
   int k32_bits;
   int id_bits;
   bool words_out;       // the sorted words go to keys[0] instead (an even number of passes)
-  const uint32_t* skip_if;  // optional: nothing is done when *skip_if is set
+  // Optional: when *both is set, sorted by (key, key(second)): by the second
+  // key first, then, the words rebuilt from their ids, by the first (a k32 and
+  // 32 key bits each).  The ids come out in vals[0] then.
+  const uint32_t* both;
+  const float* second;  // [n]
 };
-// Order of a d = 1 tree from the words sorted by lower bound: ties put in the
-// order of their upper bound, ids to vals; *redo (zero before) is set if a
-// run of ties is too long for that (nothing is done if it was set).
+// Longest runs of equal lower bounds put in order by the elements themselves, by
+// a warp, and by a CTA on chip (longer ones it sorts in global memory, some 20
+// us per 2,048 elements, so a value that promises more than twice the digits
+// would cost is sorted by both bounds from the start).
+constexpr uint32_t kNearRun = 64, kWarpRun = 128, kCtaRun = 2048;
+// Order of a d = 1 tree from its words: ids to vals, ties of the lower bound in
+// the order of their upper bound (unless st->both: the sort has done that).
+// Runs of more than kNearRun equal lower bounds are listed in `list` (n words, uint2
+// entries: those of a warp from the front, of a CTA from the back) and counted
+// in st->runs, for launch_long_ties, which overwrites words and tmp there.
 cudaError_t launch_tie_order(const unsigned long long* words, uint32_t n, int id_bits,
-                             const float* hi, uint32_t* vals, uint32_t* redo, int sms,
+                             const float* hi, uint32_t* vals, uint2* list, Status* st, int sms,
                              cudaStream_t s);
 cudaError_t launch_sort_packed(SortScratch sc, const SortSource& src, uint32_t n, int key_bits,
                                Status* st, int sms, cudaStream_t s);
@@ -310,6 +318,10 @@ cudaError_t launch_batch_plan(const unsigned long long* off, uint32_t count, uin
 cudaError_t launch_segsort(uint32_t* vals, const float* lo_k, uint32_t total, int g,
                            const SegPlan& plan, int tile_log2, unsigned long long* tmp0,
                            unsigned long long* tmp1, int sms, cudaStream_t s);
+
+cudaError_t launch_long_ties(unsigned long long* words, uint32_t n, int id_bits, const float* hi,
+                             uint32_t* vals, const uint2* list, unsigned long long* tmp,
+                             const Status* st, int sms, cudaStream_t s);
 
 // ---- ddm_tree.cu ----------------------------------------------------------
 void tree_shape(uint32_t n, int* L, uint32_t* cnt, uint32_t* off, uint32_t* total);

@@ -4,8 +4,8 @@
 // paper's segments [low, high], Section III-A); a violation raises
 // kErrExtent.  For the subscription set of a d = 1 tree the same pass emits
 // the lower bound's key; ties are put in the order of their upper bounds
-// after the sort (ddm_sort.cu), or, with long runs of them, the set is sorted
-// by (key(lo0) << 32 | key(hi0)): the interval tree order of Section IV, with
+// after the sort (ddm_sort.cu), or, if one value abounds, the set is sorted
+// by both bounds: the interval tree order of Section IV, with
 // remaining ties in id order.  Every other order (d > 1 trees, the updates) is a locality order:
 // its keys hold the top 24 bits of key(lo) below a class, group or instance.
 //
@@ -32,36 +32,51 @@ constexpr int kThreads = 256;
 constexpr int kLocalityBits = 24;
 constexpr int kLocalityDrop = 32 - kLocalityBits;
 
-// Whether a set's lower bounds tie in long runs (d = 1 tree): one CTA samples
-// kSample of them and counts those whose value another sample had before.
-// Runs of r equal bounds give about kSample^2 / 2 * (r - 1) / cnt repeats (while
-// few samples repeat); from half of what runs of 32 give, and between 4 and a
-// quarter of the samples, *redo is set and the set is sorted by both bounds at
-// once, instead of by the lower bound first and then again (5e5 bounds of 500
-// values: 131 us per build by both bounds alone, 143 with this, 186 without
-// the sample; bounds without such ties 134 -> 115 us).
+// Whether one value of the lower bound abounds in a set (d = 1 tree): one CTA
+// samples kSample of the bounds and counts the most frequent.  From four of a
+// kind, and more than kCtaRun + cnt / 512 of the set by that share, the set is
+// sorted by both bounds; fewer are put in order in place, a run at a time
+// (ddm_sort.cu): a CTA takes 22 us per 2,048 of a run beyond that, four more
+// digits some 20 us and 20 per million.  Builds of
+// 5e5 extents, always by both bounds and now: distinct bounds 139 and 119 us, 12,500
+// values 139 and 130, 500 values 137 and 144, one value 138 and 145, 1% at one
+// value 139 and 149 (195 when such a run had the whole set sorted once more).
 constexpr int kSample = 1024;
-__device__ void sample_ties(const float* __restrict__ lo, uint32_t cnt, uint32_t* redo) {
-  constexpr uint32_t kSlots = 4 * kSample, kEmpty = 0xffffffffu;
-  __shared__ uint32_t s_key[kSlots];
-  __shared__ uint32_t s_repeats;
-  for (uint32_t j = threadIdx.x; j < kSlots; j += kThreads) s_key[j] = kEmpty;
-  if (threadIdx.x == 0) s_repeats = 0u;
+__device__ void sample_ties(const float* __restrict__ lo, uint32_t cnt, Status* __restrict__ st) {
+  constexpr uint32_t kSlots = 2 * kSample, kEmpty = 0xffffffffu;
+  __shared__ uint32_t s_key[kSlots], s_cnt[kSlots];
+  __shared__ uint32_t s_most;
+  for (uint32_t j = threadIdx.x; j < kSlots; j += kThreads) {
+    s_key[j] = kEmpty;
+    s_cnt[j] = 0u;
+  }
+  if (threadIdx.x == 0) s_most = 0u;
+  uint32_t key[kSample / kThreads];
+#pragma unroll
+  for (int u = 0; u < kSample / kThreads; ++u) {
+    const uint32_t j = (uint32_t)u * kThreads + threadIdx.x;
+    key[u] = float_key(__ldg(lo + (uint32_t)((unsigned long long)j * cnt / kSample)));
+  }
   __syncthreads();
-  for (uint32_t j = threadIdx.x; j < (uint32_t)kSample; j += kThreads) {
-    const uint32_t i = (uint32_t)((unsigned long long)j * cnt / kSample);
-    const uint32_t key = float_key(__ldg(lo + i));  // never kEmpty but for NaN
-    uint32_t at = (key * 2654435761u) >> 20;        // 12 bits
+#pragma unroll
+  for (int u = 0; u < kSample / kThreads; ++u) {  // never kEmpty but for NaN
+    uint32_t at = (key[u] * 2654435761u) >> 21;   // 11 bits
     for (uint32_t tries = 0; tries < 16u; ++tries, at = (at + 1u) & (kSlots - 1u)) {
-      const uint32_t was = atomicCAS(&s_key[at], kEmpty, key);
-      if (was == key) atomicAdd(&s_repeats, 1u);
-      if (was == key || was == kEmpty) break;
+      const uint32_t was = atomicCAS(&s_key[at], kEmpty, key[u]);
+      if (was != key[u] && was != kEmpty) continue;
+      atomicAdd(&s_cnt[at], 1u);
+      break;
     }
   }
   __syncthreads();
-  const float runs_of_32 = 0.5f * kSample * kSample * 31.0f / (float)cnt;
-  if (threadIdx.x == 0 && (float)s_repeats >= fminf(fmaxf(4.0f, 0.5f * runs_of_32), 0.25f * kSample))
-    *redo = 1u;
+  uint32_t most = 0;
+  for (uint32_t j = threadIdx.x; j < kSlots; j += kThreads) most = max(most, s_cnt[j]);
+  most = __reduce_max_sync(0xffffffffu, most);
+  if ((threadIdx.x & 31) == 0) atomicMax(&s_most, most);
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  st->both = s_most >= 4u && (unsigned long long)s_most * cnt / kSample > kCtaRun + cnt / 512u;
+  st->runs[0] = st->runs[1] = 0u;
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -72,7 +87,7 @@ k_validate(int d, const float* __restrict__ lo, const float* __restrict__ hi, ui
   uint32_t blocks = gridDim.x;
   if (whole_key) {  // the last CTA looks for ties
     if (blockIdx.x == --blocks) {
-      sample_ties(lo, cnt, &st->redo);
+      sample_ties(lo, cnt, st);
       return;
     }
   }
@@ -88,18 +103,6 @@ k_validate(int d, const float* __restrict__ lo, const float* __restrict__ hi, ui
     if (k32) k32[i] = float_key(__ldg(lo + i)) >> (whole_key ? 0 : kLocalityDrop);
   }
   if (__ballot_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&st->err, kErrExtent);
-}
-
-__global__ void __launch_bounds__(kThreads)
-k_tree_keys(const float* __restrict__ lo, const float* __restrict__ hi, uint32_t cnt,
-            unsigned long long* __restrict__ keys, uint32_t* __restrict__ vals,
-            const uint32_t* __restrict__ run_if) {
-  if (*run_if == 0u) return;
-  const uint32_t stride = gridDim.x * blockDim.x;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += stride) {
-    keys[i] = ((unsigned long long)float_key(__ldg(lo + i)) << 32) | float_key(__ldg(hi + i));
-    vals[i] = i;
-  }
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -312,15 +315,6 @@ cudaError_t launch_rekey_batch(const uint32_t* vals, const float* lo_k, uint32_t
   if (cnt == 0) return cudaSuccess;
   k_rekey_batch<<<grid_for(cnt, sms), kThreads, 0, s>>>(vals, lo_k, cnt, inst, off, glog2, gbase,
                                                         keys, id_bits);
-  note_launches(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_tree_keys(const float* lo, const float* hi, uint32_t cnt,
-                             unsigned long long* keys, uint32_t* vals, const uint32_t* run_if,
-                             int sms, cudaStream_t s) {
-  if (cnt == 0) return cudaSuccess;
-  k_tree_keys<<<grid_for(cnt, sms), kThreads, 0, s>>>(lo, hi, cnt, keys, vals, run_if);
   note_launches(1);
   return cudaGetLastError();
 }

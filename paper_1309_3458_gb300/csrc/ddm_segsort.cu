@@ -128,8 +128,9 @@ __device__ __forceinline__ void rank_digit(Smem& sm,
 // One chunk of at most a tile.  Its words hold the key above the least key of
 // the chunk, in as many bits as the range needs, with the group above that:
 // coordinates of one scale range over some 20 of the 24 bits, so that a
-// chunk of several groups usually takes three digits instead of four.
-template <int THREADS, int ITEMS, typename Smem>
+// chunk of several groups usually takes three digits instead of four.  BITS: of
+// the key; with all 32 the chunk is one group.
+template <int THREADS, int ITEMS, int BITS, typename Smem>
 __device__ __forceinline__ void sort_chunk(Smem& sm, uint32_t* vals, const float* lo_k,
                                            uint32_t len, int g) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -147,7 +148,7 @@ __device__ __forceinline__ void sort_chunk(Smem& sm, uint32_t* vals, const float
   for (int i = 0; i < ITEMS; ++i) {
     const uint32_t at = warp * (ITEMS * 32) + i * 32 + lane;
     if (at < len) {
-      key[i] = float_key(__ldg(lo_k + id[i])) >> (32 - kKeyBits);
+      key[i] = float_key(__ldg(lo_k + id[i])) >> (32 - BITS);
       least = min(least, key[i]);
       most = max(most, key[i]);
     }
@@ -168,8 +169,9 @@ __device__ __forceinline__ void sort_chunk(Smem& sm, uint32_t* vals, const float
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
     const uint32_t at = warp * (ITEMS * 32) + i * 32 + lane;
-    word[i] = at < len ? ((unsigned long long)(((at >> g) << bits) | (key[i] - least)) << 32) | id[i]
-                       : ~0ull;
+    uint32_t high = key[i] - least;
+    if (BITS < 32) high |= (at >> g) << bits;
+    word[i] = at < len ? ((unsigned long long)high << 32) | id[i] : ~0ull;
   }
   for (int p = 0; p < passes; ++p) {
     const int shift = 32 + 8 * p;
@@ -193,17 +195,17 @@ __device__ __forceinline__ void sort_chunk(Smem& sm, uint32_t* vals, const float
 
 // One group larger than a tile (an instance of millions of extents): the same
 // digits, tile by tile through two scratch ranges in global memory.
-template <int THREADS, int ITEMS>
+template <int THREADS, int ITEMS, int BITS>
 __device__ void sort_large_group(SegSmem<THREADS, ITEMS>& sm, uint32_t* vals, const float* lo_k,
                                  uint32_t len, unsigned long long* a, unsigned long long* b) {
   constexpr uint32_t kTile = THREADS * ITEMS;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (uint32_t q = tid; q < len; q += THREADS) {
     const uint32_t id = vals[q];
-    a[q] = ((unsigned long long)(float_key(__ldg(lo_k + id)) >> (32 - kKeyBits)) << 32) | id;
+    a[q] = ((unsigned long long)(float_key(__ldg(lo_k + id)) >> (32 - BITS)) << 32) | id;
   }
   __syncthreads();
-  for (int p = 0; p < kKeyBits / 8; ++p) {
+  for (int p = 0; p < BITS / 8; ++p) {
     const int shift = 32 + 8 * p;
     for (int t = tid; t < kRadix; t += THREADS) sm.base[t] = 0u;
     __syncthreads();
@@ -260,6 +262,21 @@ __device__ void sort_large_group(SegSmem<THREADS, ITEMS>& sm, uint32_t* vals, co
   __syncthreads();
 }
 
+// A chunk or group of `len` positions; a and b as sort_large_group.
+template <int THREADS, int ITEMS, int BITS>
+__device__ __forceinline__ void sort_range(SegSmem<THREADS, ITEMS>& sm, uint32_t* vals, const float* lo_k,
+                                           uint32_t len, int g, unsigned long long* a,
+                                           unsigned long long* b) {
+  if (len > THREADS * ITEMS)
+    sort_large_group<THREADS, ITEMS, BITS>(sm, vals, lo_k, len, a, b);
+  else if (len > THREADS * 2 || (ITEMS == 2 && len > THREADS))
+    sort_chunk<THREADS, ITEMS, BITS>(sm, vals, lo_k, len, g);
+  else if (len > THREADS)
+    sort_chunk<THREADS, 2, BITS>(sm, vals, lo_k, len, g);
+  else if (len > 1)
+    sort_chunk<THREADS, 1, BITS>(sm, vals, lo_k, len, g);
+}
+
 // Re-sort of one set.  With `off` null: one instance of `total` positions and
 // group exponent g_one; else instance i owns positions [off[i], off[i+1]) with
 // exponent glog2[i] (0: left as it is) and chunks [cbase[i], cbase[i+1]).
@@ -284,14 +301,69 @@ k_segsort(uint32_t* __restrict__ vals, const float* __restrict__ lo_k, uint32_t 
       end = min(begin + size, off[b + 1]);
     }
     const uint32_t len = (uint32_t)(end - begin);
-    if (len > kTile)
-      sort_large_group<THREADS, ITEMS>(sm, vals + begin, lo_k, len, tmp0 + begin, tmp1 + begin);
-    else if (len > THREADS * 2 || (ITEMS == 2 && len > THREADS))
-      sort_chunk<THREADS, ITEMS>(sm, vals + begin, lo_k, len, g);
-    else if (len > THREADS)
-      sort_chunk<THREADS, 2>(sm, vals + begin, lo_k, len, g);
-    else if (len > 1)
-      sort_chunk<THREADS, 1>(sm, vals + begin, lo_k, len, g);
+    sort_range<THREADS, ITEMS, kKeyBits>(sm, vals + begin, lo_k, len, g, tmp0 + begin, tmp1 + begin);
+  }
+}
+
+// The runs of equal lower bounds that k_tie_order has listed: ids of each in
+// the order of their upper bound (stably).  A warp counts, for every element of
+// its run, those before it; a CTA sorts its run like a chunk of a re-sort, by
+// all 32 bits.  Small CTAs: while the updates are sorted on another stream,
+// larger ones would wait for a whole SM to fall idle (a match of 2.5e7 + 2.5e7
+// extents 6.10 -> 6.47 ms with CTAs of 1,024 threads).
+constexpr int kTieThreads = 256, kTieItems = 8;
+static_assert(kTieThreads * kTieItems == (int)kCtaRun, "runs of a CTA are sorted on chip");
+
+// A run of at most kWarpRun elements by one warp (a run of 200 took it 40 us).
+__device__ __forceinline__ void warp_run(const unsigned long long* __restrict__ words, uint2 run,
+                                         unsigned long long idm, const float* __restrict__ hi,
+                                         uint32_t* __restrict__ vals) {
+  constexpr int EACH = (int)kWarpRun / 32;
+  const uint32_t lane = threadIdx.x & 31u;
+  uint32_t id[EACH], key[EACH], rank[EACH];
+#pragma unroll
+  for (int c = 0; c < EACH; ++c) {
+    const uint32_t at = c * 32u + lane;
+    id[c] = at < run.y ? (uint32_t)(words[run.x + at] & idm) : 0u;
+    rank[c] = 0u;
+  }
+#pragma unroll
+  for (int c = 0; c < EACH; ++c)
+    key[c] = c * 32u + lane < run.y ? float_key(__ldg(hi + id[c])) : 0xffffffffu;
+#pragma unroll
+  for (int c2 = 0; c2 < EACH; ++c2) {
+    if (c2 * 32u >= run.y) break;  // warp-uniform
+#pragma unroll 4
+    for (uint32_t l = 0; l < 32u; ++l) {
+      const uint32_t k2 = __shfl_sync(0xffffffffu, key[c2], l);
+#pragma unroll
+      for (int c = 0; c < EACH; ++c)
+        rank[c] += (k2 < key[c] || (k2 == key[c] && c2 * 32u + l < c * 32u + lane)) ? 1u : 0u;
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < EACH; ++c)
+    if (c * 32u + lane < run.y) vals[run.x + rank[c]] = id[c];
+}
+
+__global__ void __launch_bounds__(kTieThreads, 4)
+k_long_ties(unsigned long long* __restrict__ words, uint32_t n, int id_bits,
+            const float* __restrict__ hi, uint32_t* __restrict__ vals, const uint2* __restrict__ list,
+            unsigned long long* __restrict__ tmp, const Status* __restrict__ st) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  auto& sm = *reinterpret_cast<SegSmem<kTieThreads, kTieItems>*>(smem_raw);
+  const uint32_t short_runs = st->runs[0], long_runs = st->runs[1];
+  const unsigned long long idm = (1ull << id_bits) - 1ull;
+  for (uint32_t e = blockIdx.x * (kTieThreads / 32) + threadIdx.x / 32u; e < short_runs;
+       e += gridDim.x * (kTieThreads / 32)) {
+    warp_run(words, list[e], idm, hi, vals);
+  }
+  for (uint32_t e = blockIdx.x; e < long_runs; e += gridDim.x) {
+    const uint2 run = list[n / 2u - 1u - e];
+    for (uint32_t q = threadIdx.x; q < run.y; q += kTieThreads)
+      vals[run.x + q] = (uint32_t)(words[run.x + q] & idm);
+    __syncthreads();
+    sort_range<kTieThreads, kTieItems, 32>(sm, vals + run.x, hi, run.y, 31, words + run.x, tmp + run.x);
   }
 }
 
@@ -571,6 +643,18 @@ cudaError_t launch_batch_plan(const unsigned long long* off, uint32_t count, uin
 cudaError_t launch_class_plan(const uint32_t* hist, int d, int shift, const ClassPlan& plan,
                               cudaStream_t s) {
   k_class_plan<<<1, 256, 0, s>>>(hist, d, shift, plan);
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_long_ties(unsigned long long* words, uint32_t n, int id_bits, const float* hi,
+                             uint32_t* vals, const uint2* list, unsigned long long* tmp,
+                             const Status* st, int sms, cudaStream_t s) {
+  if (n <= 1) return cudaSuccess;
+  const size_t smem = sizeof(SegSmem<kTieThreads, kTieItems>);
+  cudaError_t e = cudaFuncSetAttribute(k_long_ties, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e) return e;
+  k_long_ties<<<(uint32_t)sms * 4u, kTieThreads, smem, s>>>(words, n, id_bits, hi, vals, list, tmp, st);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -101,6 +101,15 @@ __device__ __forceinline__ unsigned long long source_word(const SortSource& src,
   return (k << src.id_bits) | i;
 }
 
+// The first words of a sort by both keys, and those rebuilt between the two.
+__device__ __forceinline__ unsigned long long second_word(const SortSource& src, uint32_t i) {
+  return ((unsigned long long)float_key(__ldg(src.second + i)) << src.id_bits) | i;
+}
+__device__ __forceinline__ unsigned long long first_word(const SortSource& src, unsigned long long w) {
+  const uint32_t id = (uint32_t)(w & ((1ull << src.id_bits) - 1ull));
+  return ((unsigned long long)__ldg(src.k32 + id) << src.id_bits) | id;
+}
+
 // Test hook for the bounded waits: poll a word nothing sets.
 __global__ void k_debug_wait(const uint32_t* __restrict__ word, uint32_t limit,
                              Status* __restrict__ st) {
@@ -111,9 +120,7 @@ __global__ void k_debug_wait(const uint32_t* __restrict__ word, uint32_t limit,
 
 // All eight digit histograms in one read of the keys.
 __global__ void __launch_bounds__(kThreads)
-k_histogram(const unsigned long long* __restrict__ keys, uint32_t n, uint32_t* __restrict__ hist,
-            const uint32_t* __restrict__ run_if) {
-  if (run_if && *run_if == 0u) return;
+k_histogram(const unsigned long long* __restrict__ keys, uint32_t n, uint32_t* __restrict__ hist) {
   __shared__ uint32_t h[kPasses * kRadix];
   for (int t = threadIdx.x; t < kPasses * kRadix; t += kThreads) h[t] = 0;
   __syncthreads();
@@ -164,9 +171,7 @@ __global__ void __launch_bounds__(kThreads, 3)
 k_onesweep(const unsigned long long* __restrict__ in_keys, const uint32_t* __restrict__ in_vals,
            unsigned long long* __restrict__ out_keys, uint32_t* __restrict__ out_vals, uint32_t n,
            int shift, const uint32_t* __restrict__ digit_base, uint32_t* __restrict__ lookback,
-           uint32_t* __restrict__ counter, const uint32_t* __restrict__ run_if,
-           Status* __restrict__ st) {
-  if (run_if && *run_if == 0u) return;
+           uint32_t* __restrict__ counter, Status* __restrict__ st) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   OnesweepSmem& sm = *reinterpret_cast<OnesweepSmem*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -283,8 +288,10 @@ k_onesweep(const unsigned long long* __restrict__ in_keys, const uint32_t* __res
 __global__ void __launch_bounds__(kThreads)
 k_histogram_packed(const unsigned long long* __restrict__ words, SortSource src, uint32_t n,
                    int passes, uint32_t* __restrict__ hist) {
-  if (src.skip_if && *src.skip_if) return;
   __shared__ uint32_t h[kPasses * kRadix];
+  const bool both = src.both && *src.both;
+  const int half = passes;  // the first key's digits, behind them the second's
+  if (both) passes = 2 * half;
   for (int t = threadIdx.x; t < passes * kRadix; t += kThreads) h[t] = 0;
   __syncthreads();
   const uint32_t stride = gridDim.x * kThreads;
@@ -301,13 +308,18 @@ k_histogram_packed(const unsigned long long* __restrict__ words, SortSource src,
       const size_t first = i0 + (size_t)u * stride;
       const bool whole = first + 32u <= n;  // warp-uniform
       if (!whole && first + lane >= n) continue;
-      for (int p = 0; p < passes; ++p) {
+      for (int p = 0; p < half; ++p) {
         const uint32_t d = (uint32_t)(k[u] >> (p * kRadixBits)) & (kRadix - 1);
         if (whole && __all_sync(0xffffffffu, d == __shfl_sync(0xffffffffu, d, 0))) {
           if (lane == 0) atomicAdd(&h[p * kRadix + d], 32u);
         } else {
           atomicAdd(&h[p * kRadix + d], 1u);
         }
+      }
+      if (both) {
+        const unsigned long long k2 = second_word(src, (uint32_t)(first + lane)) >> src.id_bits;
+        for (int p = half; p < passes; ++p)
+          atomicAdd(&h[p * kRadix + ((uint32_t)(k2 >> ((p - half) * kRadixBits)) & (kRadix - 1))], 1u);
       }
     }
   }
@@ -319,8 +331,10 @@ k_histogram_packed(const unsigned long long* __restrict__ words, SortSource src,
 // The onesweep pass on packed words: 512 threads with eight words each, so
 // that three CTAs fit an SM in 40 registers (the pass on keys and ids needs 80
 // and spills), half the words per thread to wait for and to rank in turn, one
-// scattered stream instead of two.  FIRST: the words come from the source;
-// LAST: only the ids go out.
+// scattered stream instead of two.  FROM: where the words come from (kFromFirst:
+// the source, or, between the two halves of a sort by both keys, rebuilt; the
+// passes of kFromSecond's half, `second_half`, do nothing otherwise); LAST:
+// only the ids go out (as from the `final` pass of a sort by both keys).
 constexpr int kPackThreads = 512;
 constexpr int kPackWarps = kPackThreads / 32;
 constexpr int kPackItems = kSortTile / kPackThreads;  // 8
@@ -334,14 +348,17 @@ struct PackedSmem {
   unsigned long long words[kSortTile];
 };
 
-template <bool FIRST, bool LAST>
+enum { kFromWords, kFromFirst, kFromSecond };
+template <int FROM, bool LAST>
 __global__ void __launch_bounds__(kPackThreads, 3)
 k_onesweep_packed(const unsigned long long* __restrict__ in, SortSource src,
                   unsigned long long* __restrict__ out, uint32_t* __restrict__ out_ids, uint32_t n,
                   int shift, const uint32_t* __restrict__ digit_base,
                   uint32_t* __restrict__ lookback, uint32_t* __restrict__ counter,
-                  Status* __restrict__ st) {
-  if (src.skip_if && *src.skip_if) return;
+                  bool second_half, bool final, Status* __restrict__ st) {
+  const bool both = (second_half || final || FROM == kFromFirst) && src.both && *src.both;
+  if (second_half && !both) return;
+  const bool ids = final && both;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   PackedSmem& sm = *reinterpret_cast<PackedSmem*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -357,7 +374,14 @@ k_onesweep_packed(const unsigned long long* __restrict__ in, SortSource src,
 #pragma unroll
   for (int i = 0; i < kPackItems; ++i) {
     const uint32_t local = warp * (kPackItems * 32) + i * 32 + lane;
-    word[i] = local >= valid ? ~0ull : FIRST ? source_word(src, base + local) : in[base + local];
+    if (local >= valid)
+      word[i] = ~0ull;
+    else if (FROM == kFromSecond)
+      word[i] = second_word(src, base + local);
+    else if (FROM == kFromFirst)
+      word[i] = both ? first_word(src, in[base + local]) : source_word(src, base + local);
+    else
+      word[i] = in[base + local];
   }
 #pragma unroll
   for (int i = 0; i < kPackItems; ++i) {
@@ -426,7 +450,7 @@ k_onesweep_packed(const unsigned long long* __restrict__ in, SortSource src,
     const unsigned long long k = sm.words[q];
     const uint32_t g = sm.gbase[(uint32_t)(k >> shift) & (kRadix - 1)] + q;
     if (!DDM_IN_BOUNDS(g < n, st)) continue;
-    if (LAST)
+    if (LAST || ids)
       out_ids[g] = (uint32_t)(k & ((1ull << src.id_bits) - 1ull));
     else
       out[g] = k;
@@ -578,9 +602,11 @@ template <int ITEMS, bool PACKED>
 __global__ void __launch_bounds__(kSmallThreads, ITEMS <= 8 ? 2 : 1)
 k_sort_grid(unsigned long long* __restrict__ keys0, uint32_t* __restrict__ vals0,
             unsigned long long* __restrict__ keys1, uint32_t* __restrict__ vals1, uint32_t n,
-            int passes, SortSource src, const uint32_t* __restrict__ run_if,
-            uint32_t* __restrict__ table, uint32_t* __restrict__ bar, Status* __restrict__ st) {
-  if ((run_if && *run_if == 0u) || (src.skip_if && *src.skip_if)) return;  // every CTA alike
+            int passes, SortSource src, uint32_t* __restrict__ table, uint32_t* __restrict__ bar,
+            Status* __restrict__ st) {
+  const bool both = PACKED && src.both && *src.both;  // every CTA alike
+  const int half = passes;  // a sort by both keys: twice, the second key first
+  if (both) passes = 2 * half;
   constexpr uint32_t kTile = kSmallThreads * ITEMS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   GridSortSmem<ITEMS, PACKED>& sm = *reinterpret_cast<GridSortSmem<ITEMS, PACKED>*>(smem_raw);
@@ -599,20 +625,30 @@ k_sort_grid(unsigned long long* __restrict__ keys0, uint32_t* __restrict__ vals0
     uint32_t* ov = (p & 1) ? vals0 : vals1;
     (void)iv;
     (void)ov;
-    // written by other CTAs of this launch: read through L2, not L1
+    auto at = [&](int i) { return (uint32_t)(warp * (ITEMS * 32) + i * 32 + lane); };
+    if (PACKED && p == 0 && src.k32) {
+      if (both) {
 #pragma unroll
-    for (int i = 0; i < ITEMS; ++i) {
-      const uint32_t local = warp * (ITEMS * 32) + i * 32 + lane;
-      if constexpr (PACKED) {
-        key[i] = local >= valid          ? ~0ull
-                 : p == 0 && src.k32     ? source_word(src, (uint32_t)base + local)
-                                         : __ldcg(ik + base + local);
+        for (int i = 0; i < ITEMS; ++i)
+          key[i] = at(i) < valid ? second_word(src, (uint32_t)base + at(i)) : ~0ull;
       } else {
-        key[i] = local < valid ? __ldcg(ik + base + local) : ~0ull;
-        val[i] = local < valid ? __ldcg(iv + base + local) : 0u;
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i)
+          key[i] = at(i) < valid ? source_word(src, (uint32_t)base + at(i)) : ~0ull;
+      }
+    } else {  // written by other CTAs of this launch: read through L2, not L1
+#pragma unroll
+      for (int i = 0; i < ITEMS; ++i) {
+        key[i] = at(i) < valid ? __ldcg(ik + base + at(i)) : ~0ull;
+        if constexpr (!PACKED) val[i] = at(i) < valid ? __ldcg(iv + base + at(i)) : 0u;
+      }
+      if (both && p == half) {
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i)
+          if (at(i) < valid) key[i] = first_word(src, key[i]);
       }
     }
-    const int shift = p * kRadixBits + (PACKED ? src.id_bits : 0);
+    const int shift = (PACKED && p >= half ? p - half : p) * kRadixBits + (PACKED ? src.id_bits : 0);
     const uint32_t count = rank_tile<ITEMS>(sm.r, key, rank, shift);
     uint32_t* gsum = table + kGridRowWords + (size_t)(p & 1) * kGridGroups * kRadix;
     if (tid < kRadix) {  // this tile's counts: its row (two 16-bit digits per word), its group's sums
@@ -667,7 +703,7 @@ k_sort_grid(unsigned long long* __restrict__ keys0, uint32_t* __restrict__ vals0
       const uint32_t g = sm.gbase[(uint32_t)(k >> shift) & (kRadix - 1)] + q;
       if (!DDM_IN_BOUNDS(g < n, st)) continue;
       if constexpr (PACKED) {
-        if (p + 1 < passes || src.words_out)
+        if (p + 1 < passes || (src.words_out && !both))
           ok[g] = k;
         else
           vals0[g] = (uint32_t)(k & ((1ull << src.id_bits) - 1ull));
@@ -729,8 +765,10 @@ template <int ITEMS, bool PACKED>
 __global__ void __launch_bounds__(kSmallThreads, 1)
 k_sort_cluster(const unsigned long long* __restrict__ in_k, const uint32_t* __restrict__ in_v,
                unsigned long long* __restrict__ out_k, uint32_t* __restrict__ out_v, uint32_t n,
-               int passes, SortSource src, const uint32_t* __restrict__ run_if) {
-  if ((run_if && *run_if == 0u) || (src.skip_if && *src.skip_if)) return;  // every CTA alike
+               int passes, SortSource src) {
+  const bool both = PACKED && src.both && *src.both;  // every CTA alike
+  const int half = passes;
+  if (both) passes = 2 * half;
   constexpr uint32_t kTile = kSmallThreads * ITEMS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ClusterSortSmem<ITEMS, PACKED>& sm = *reinterpret_cast<ClusterSortSmem<ITEMS, PACKED>*>(smem_raw);
@@ -744,14 +782,17 @@ k_sort_cluster(const unsigned long long* __restrict__ in_k, const uint32_t* __re
   for (int i = 0; i < ITEMS; ++i) {
     const uint32_t local = warp * (ITEMS * 32) + i * 32 + lane;
     if constexpr (PACKED) {
-      key[i] = local >= valid ? ~0ull : src.k32 ? source_word(src, base + local) : in_k[base + local];
+      key[i] = local >= valid ? ~0ull
+               : both         ? second_word(src, base + local)
+               : src.k32      ? source_word(src, base + local)
+                              : in_k[base + local];
     } else {
       key[i] = local < valid ? in_k[base + local] : ~0ull;
       val[i] = local < valid ? in_v[base + local] : 0u;
     }
   }
   for (int p = 0; p < passes; ++p) {
-    const int shift = p * kRadixBits + (PACKED ? src.id_bits : 0);
+    const int shift = (PACKED && p >= half ? p - half : p) * kRadixBits + (PACKED ? src.id_bits : 0);
     const uint32_t count = rank_tile<ITEMS>(sm.r, key, rank, shift);
     if (tid < kRadix)
       for (uint32_t j = 0; j < ctas; ++j) st_remote(remote_smem(&sm.table[me][tid], j), count);
@@ -795,7 +836,7 @@ k_sort_cluster(const unsigned long long* __restrict__ in_k, const uint32_t* __re
       if (!DDM_IN_BOUNDS(g < n, nullptr)) continue;
       if (last) {
         if constexpr (PACKED) {
-          if (src.words_out)
+          if (src.words_out && !both)
             out_k[g] = k;
           else
             out_v[g] = (uint32_t)(k & ((1ull << src.id_bits) - 1ull));
@@ -815,6 +856,7 @@ k_sort_cluster(const unsigned long long* __restrict__ in_k, const uint32_t* __re
     for (int i = 0; i < ITEMS; ++i) {
       const uint32_t local = warp * (ITEMS * 32) + i * 32 + lane;
       key[i] = local < valid ? sm.tile_k[local] : ~0ull;
+      if (PACKED && both && p + 1 == half && local < valid) key[i] = first_word(src, key[i]);
       if constexpr (!PACKED) val[i] = local < valid ? sm.tile_v[local] : 0u;
     }
   }
@@ -822,49 +864,98 @@ k_sort_cluster(const unsigned long long* __restrict__ in_k, const uint32_t* __re
 
 // The d = 1 tree's order is by lower bound, upper bound, id.  The upper bound
 // matters only among equal lower bounds, so the set is sorted by the lower
-// bound alone (four digits instead of eight), and the thread at the start of
-// each run of equal keys puts the run in the order of the upper bounds
-// (stably: ids ascend already).  Runs longer than kMaxRun ask for the full
-// sort (*redo), which waits behind this in launches that do nothing otherwise.
-constexpr uint32_t kMaxRun = 32;
+// bound alone (four digits instead of eight) unless one value abounds.  Then
+// every element counts those of its run (equal keys, next to it) that come
+// before it, by upper bound and, ids ascending already, by position: a CTA
+// stages a tile's keys and kNearRun on either side, and the upper bounds of
+// those with an equal neighbour.  Bound by reading the words and writing the
+// ids where few tie.  Longer runs are listed for a warp or a CTA each
+// (k_long_ties).  The build of 2e7 extents in runs of 40: 2.58 ms by both
+// bounds, 1.68 so; without ties 2.60 and 1.55.
+constexpr uint32_t kTieTile = 1024, kTieSpan = kTieTile + 2 * kNearRun;
 __global__ void __launch_bounds__(256)
 k_tie_order(const unsigned long long* __restrict__ words, uint32_t n, int id_bits,
-            const float* __restrict__ hi, uint32_t* __restrict__ vals, uint32_t* __restrict__ redo) {
-  if (*reinterpret_cast<volatile uint32_t*>(redo)) return;
+            const float* __restrict__ hi, uint32_t* __restrict__ vals, uint2* __restrict__ list,
+            Status* __restrict__ st) {
+  if (st->both != 0u) return;  // sorted by both bounds: the ids are there
+  __shared__ uint32_t s_lo[kTieSpan], s_hi[kTieSpan];
+  __shared__ uint32_t s_head[kTieSpan / 32];  // bit j: a run starts at j (or the set ends)
   const unsigned long long idm = (1ull << id_bits) - 1ull;
-  for (uint32_t i = blockIdx.x * 256u + threadIdx.x; i < n; i += gridDim.x * 256u) {
-    const unsigned long long w = words[i], k = w >> id_bits;
-    if (i > 0 && (words[i - 1] >> id_bits) == k) continue;  // inside a run
-    if (i + 1 == n || (words[i + 1] >> id_bits) != k) {
-      vals[i] = (uint32_t)(w & idm);
-      continue;
-    }
-    uint32_t len = 1, last = float_key(__ldg(hi + (uint32_t)(w & idm)));
-    bool ordered = true;
-    for (; i + len < n; ++len) {
-      const unsigned long long v = words[i + len];
-      if ((v >> id_bits) != k) break;
-      if (len == kMaxRun) {
-        *redo = 1u;
-        return;  // the full sort overwrites vals
+  constexpr int kEach = (kTieSpan + 255) / 256;
+  for (uint32_t t0 = blockIdx.x * kTieTile; t0 < n; t0 += gridDim.x * kTieTile) {
+    // index j of the span is position t0 + j - kNearRun; [first, last) exist
+    const uint32_t first = t0 ? 0u : kNearRun, last = min(kTieSpan, n - t0 + kNearRun);
+    uint32_t id[kEach];
+    __syncthreads();  // the previous tile has been read
+#pragma unroll
+    for (int u = 0; u < kEach; ++u) {
+      const uint32_t j = (uint32_t)u * 256u + threadIdx.x;
+      id[u] = 0u;
+      if (j >= first && j < last) {
+        const unsigned long long w = words[t0 + j - kNearRun];
+        s_lo[j] = (uint32_t)(w >> id_bits);
+        id[u] = (uint32_t)(w & idm);
       }
-      const uint32_t u = float_key(__ldg(hi + (uint32_t)(v & idm)));
-      ordered = ordered && last <= u;
-      last = u;
     }
-    if (ordered) {
-      for (uint32_t j = 0; j < len; ++j) vals[i + j] = (uint32_t)(words[i + j] & idm);
-      continue;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kEach; ++u) {
+      const uint32_t j = (uint32_t)u * 256u + threadIdx.x;
+      if (j >= kTieSpan) break;  // whole warps
+      const uint32_t heads =
+          __ballot_sync(0xffffffffu, j <= first || j >= last || s_lo[j] != s_lo[j - 1u]);
+      if ((threadIdx.x & 31u) == 0u) s_head[j / 32u] = heads;
     }
-    unsigned long long run[kMaxRun];  // (upper bound, id), insertion sort
-    for (uint32_t j = 0; j < len; ++j) {
-      const uint32_t id = (uint32_t)(words[i + j] & idm);
-      const unsigned long long x = ((unsigned long long)float_key(__ldg(hi + id)) << 32) | id;
-      uint32_t at = j;
-      for (; at > 0 && run[at - 1] > x; --at) run[at] = run[at - 1];
-      run[at] = x;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kEach; ++u) {
+      const uint32_t j = (uint32_t)u * 256u + threadIdx.x;
+      if (j < first || j >= last) continue;
+      const uint32_t next = j + 1u;
+      const bool alone = (s_head[j / 32u] >> (j & 31u) & 1u) &&
+                         (next == kTieSpan || (s_head[next / 32u] >> (next & 31u) & 1u));
+      if (!alone) s_hi[j] = float_key(__ldg(hi + id[u]));
     }
-    for (uint32_t j = 0; j < len; ++j) vals[i + j] = (uint32_t)run[j];
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kEach; ++u) {
+      const uint32_t j = (uint32_t)u * 256u + threadIdx.x;
+      if (j < kNearRun || j >= min(last, kNearRun + kTieTile)) continue;  // not of this tile
+      // its run [a, b), as far as two words of heads on either side tell
+      const uint32_t wi = j / 32u, upto = 0xffffffffu >> (31u - (j & 31u));
+      const uint32_t h0 = s_head[wi] & upto, h1 = s_head[wi - 1u], h2 = s_head[wi - 2u];
+      const uint32_t n0 = s_head[wi] & ~upto, n1 = s_head[wi + 1u], n2 = s_head[wi + 2u];
+      const uint32_t base = wi * 32u, none = 2u * kTieSpan;
+      const uint32_t a = h0 ? base + 31u - __clz(h0) : h1 ? base - 1u - __clz(h1) : h2 ? base - 33u - __clz(h2) : none;
+      const uint32_t b = n0 ? base + __ffs(n0) - 1u : n1 ? base + 31u + __ffs(n1) : n2 ? base + 63u + __ffs(n2) : none;
+      if (a != none && b != none && b - a <= kNearRun) {
+        uint32_t at = t0 + a - kNearRun;
+        if (b - a > 1u) {
+          const uint32_t h = s_hi[j];
+#pragma unroll 4
+          for (uint32_t i = a; i < b; ++i) at += (s_hi[i] < h || (s_hi[i] == h && i < j)) ? 1u : 0u;
+        }
+        vals[at] = id[u];
+      } else if (a == j) {
+        const uint32_t i = t0 + j - kNearRun;
+        const unsigned long long key = words[i] >> id_bits;
+        // its end: equal at i + lo, not at i + up (or behind the set)
+        uint32_t lo = kNearRun, up = 2u * kNearRun;
+        while (up < n - i && (words[i + up] >> id_bits) == key) {
+          lo = up;
+          up *= 2u;
+        }
+        up = min(up, n - i);
+        while (up - lo > 1u) {
+          const uint32_t mid = lo + (up - lo) / 2u;
+          if ((words[i + mid] >> id_bits) == key) lo = mid; else up = mid;
+        }
+        if (up <= kWarpRun)
+          list[atomicAdd(&st->runs[0], 1u)] = make_uint2(i, up);
+        else
+          list[n / 2u - 1u - atomicAdd(&st->runs[1], 1u)] = make_uint2(i, up);
+      }
+    }
   }
 }
 
@@ -916,7 +1007,7 @@ int cluster_sort_ctas() {
 // true then (or an error), else nothing is enqueued.
 template <int ITEMS, bool PACKED>
 cudaError_t try_sort_cluster(SortScratch sc, const SortSource& src, uint32_t n, int passes,
-                             const uint32_t* run_if, cudaStream_t s, bool* done) {
+                             cudaStream_t s, bool* done) {
   *done = false;
   constexpr uint32_t kTile = kSmallThreads * ITEMS;
   const uint32_t ctas = (n + kTile - 1) / kTile;
@@ -935,7 +1026,7 @@ cudaError_t try_sort_cluster(SortScratch sc, const SortSource& src, uint32_t n, 
   cfg.numAttrs = 1;
   const int out = PACKED ? 0 : passes & 1;
   cudaError_t e = cudaLaunchKernelEx(&cfg, k_sort_cluster<ITEMS, PACKED>, sc.keys[0], sc.vals[0],
-                                     sc.keys[out], sc.vals[out], n, passes, src, run_if);
+                                     sc.keys[out], sc.vals[out], n, passes, src);
   if (e == cudaSuccess) {
     note_launches(1);
     *done = true;
@@ -972,7 +1063,7 @@ int grid_sort_tiles(int sms) {
 // *done = true then (or an error), else nothing is enqueued.
 template <int ITEMS, bool PACKED>
 cudaError_t try_sort_grid(SortScratch sc, const SortSource& src, uint32_t n, int passes,
-                          const uint32_t* run_if, Status* st, int sms, cudaStream_t s, bool* done) {
+                          Status* st, int sms, cudaStream_t s, bool* done) {
   *done = false;
   constexpr uint32_t kTile = kSmallThreads * ITEMS;
   const uint32_t tiles = (n + kTile - 1) / kTile;
@@ -992,7 +1083,7 @@ cudaError_t try_sort_grid(SortScratch sc, const SortSource& src, uint32_t n, int
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   e = cudaLaunchKernelEx(&cfg, k_sort_grid<ITEMS, PACKED>, sc.keys[0], sc.vals[0], sc.keys[1], sc.vals[1],
-                         n, passes, src, run_if, sc.lookback, sums + kGridSumWords, st);
+                         n, passes, src, sc.lookback, sums + kGridSumWords, st);
   if (e == cudaErrorCooperativeLaunchTooLarge) {  // fewer SMs available than counted
     cudaGetLastError();
     return cudaSuccess;
@@ -1023,7 +1114,7 @@ namespace {
 // The one-launch forms, smallest first: *done = false if none fits.
 template <bool PACKED>
 cudaError_t sort_in_one(SortScratch sc, const SortSource& src, uint32_t n, int passes,
-                        const uint32_t* run_if, Status* st, int sms, cudaStream_t s, bool* done) {
+                        Status* st, int sms, cudaStream_t s, bool* done) {
   // Up to 16 tiles of 2,048 keys: one cluster, keys kept on chip; else one
   // cooperative launch when every tile can be resident at once, with the
   // smallest tile that allows it.  Measured (8 passes, one GB300): 5,000
@@ -1033,10 +1124,10 @@ cudaError_t sort_in_one(SortScratch sc, const SortSource& src, uint32_t n, int p
   // with the same attributes): 256 batched instances in a graph took 187 us
   // with the multi-launch form recorded instead, 149 with these.
   cudaError_t e;
-  if ((e = try_sort_cluster<4, PACKED>(sc, src, n, passes, run_if, s, done)) || *done) return e;
-  if ((e = try_sort_grid<4, PACKED>(sc, src, n, passes, run_if, st, sms, s, done)) || *done) return e;
-  if ((e = try_sort_grid<8, PACKED>(sc, src, n, passes, run_if, st, sms, s, done)) || *done) return e;
-  return try_sort_grid<16, PACKED>(sc, src, n, passes, run_if, st, sms, s, done);
+  if ((e = try_sort_cluster<4, PACKED>(sc, src, n, passes, s, done)) || *done) return e;
+  if ((e = try_sort_grid<4, PACKED>(sc, src, n, passes, st, sms, s, done)) || *done) return e;
+  if ((e = try_sort_grid<8, PACKED>(sc, src, n, passes, st, sms, s, done)) || *done) return e;
+  return try_sort_grid<16, PACKED>(sc, src, n, passes, st, sms, s, done);
 }
 
 cudaError_t clear_onesweep(SortScratch sc, uint32_t tiles, int passes, cudaStream_t s) {
@@ -1046,28 +1137,32 @@ cudaError_t clear_onesweep(SortScratch sc, uint32_t tiles, int passes, cudaStrea
   return cudaMemsetAsync(sc.lookback, 0, sizeof(uint32_t) * (size_t)passes * tiles * kRadix, s);
 }
 
-template <bool FIRST, bool LAST>
-cudaError_t onesweep_packed_pass(SortScratch sc, const SortSource& src, uint32_t n, int p,
-                                 Status* st, cudaStream_t s) {
+// Pass p; in the second half (the second key's passes, run first) its counts
+// follow the first key's.
+template <int FROM, bool LAST>
+cudaError_t onesweep_packed_pass(SortScratch sc, const SortSource& src, uint32_t n, int p, int passes,
+                                 bool second_half, Status* st, cudaStream_t s) {
   const uint32_t tiles = (n + kSortTile - 1) / kSortTile;
   const size_t smem = sizeof(PackedSmem);
-  cudaError_t e = cudaFuncSetAttribute(k_onesweep_packed<FIRST, LAST>,
+  cudaError_t e = cudaFuncSetAttribute(k_onesweep_packed<FROM, LAST>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e) return e;
-  k_onesweep_packed<FIRST, LAST><<<tiles, kPackThreads, smem, s>>>(
+  const int at = second_half ? passes + p : p;
+  k_onesweep_packed<FROM, LAST><<<tiles, kPackThreads, smem, s>>>(
       sc.keys[p & 1], src, sc.keys[(p & 1) ^ 1], sc.vals[0], n, src.id_bits + p * kRadixBits,
-      sc.hist + p * kRadix, sc.lookback + (size_t)p * tiles * kRadix, sc.counters + p, st);
+      sc.hist + at * kRadix, sc.lookback + (size_t)at * tiles * kRadix, sc.counters + at, second_half,
+      !second_half && p + 1 == passes, st);
   return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_tie_order(const unsigned long long* words, uint32_t n, int id_bits,
-                             const float* hi, uint32_t* vals, uint32_t* redo, int sms,
+                             const float* hi, uint32_t* vals, uint2* list, Status* st, int sms,
                              cudaStream_t s) {
   if (n == 0) return cudaSuccess;
-  const uint32_t need = (n + 255) / 256, cap = (uint32_t)sms * 64u;
-  k_tie_order<<<need < cap ? need : cap, 256, 0, s>>>(words, n, id_bits, hi, vals, redo);
+  const uint32_t need = (n + kTieTile - 1) / kTieTile, cap = (uint32_t)sms * 16u;
+  k_tie_order<<<need < cap ? need : cap, 256, 0, s>>>(words, n, id_bits, hi, vals, list, st);
   note_launches(1);
   return cudaGetLastError();
 }
@@ -1076,34 +1171,42 @@ cudaError_t launch_sort_packed(SortScratch sc, const SortSource& src, uint32_t n
                                Status* st, int sms, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   const int passes = std::max((key_bits + kRadixBits - 1) / kRadixBits, 1);
+  const int halves = src.both ? 2 : 1;
   cudaError_t e;
   bool done = false;
-  if ((e = sort_in_one<true>(sc, src, n, passes, nullptr, st, sms, s, &done)) || done) return e;
+  if ((e = sort_in_one<true>(sc, src, n, passes, st, sms, s, &done)) || done) return e;
   const uint32_t tiles = (n + kSortTile - 1) / kSortTile;
-  if ((e = clear_onesweep(sc, tiles, passes, s))) return e;
+  if ((e = clear_onesweep(sc, tiles, halves * passes, s))) return e;
   const uint32_t hb = std::min((n + kThreads * 16 - 1) / (kThreads * 16), (uint32_t)sms * 8u);
   k_histogram_packed<<<hb, kThreads, 0, s>>>(sc.keys[0], src, n, passes, sc.hist);
-  k_hist_scan<<<passes, kRadix, 0, s>>>(sc.hist);
+  k_hist_scan<<<halves * passes, kRadix, 0, s>>>(sc.hist);
+  if (src.both) {  // an even number of passes: the words return to keys[0]
+    for (int p = 0; p < passes; ++p) {
+      e = p == 0 ? onesweep_packed_pass<kFromSecond, false>(sc, src, n, p, passes, true, st, s)
+                 : onesweep_packed_pass<kFromWords, false>(sc, src, n, p, passes, true, st, s);
+      if (e) return e;
+    }
+  }
   for (int p = 0; p < passes; ++p) {
     const bool first = p == 0 && src.k32, last = p + 1 == passes && !src.words_out;
-    e = first ? (last ? onesweep_packed_pass<true, true>(sc, src, n, p, st, s)
-                      : onesweep_packed_pass<true, false>(sc, src, n, p, st, s))
-              : (last ? onesweep_packed_pass<false, true>(sc, src, n, p, st, s)
-                      : onesweep_packed_pass<false, false>(sc, src, n, p, st, s));
+    e = first ? (last ? onesweep_packed_pass<kFromFirst, true>(sc, src, n, p, passes, false, st, s)
+                      : onesweep_packed_pass<kFromFirst, false>(sc, src, n, p, passes, false, st, s))
+              : (last ? onesweep_packed_pass<kFromWords, true>(sc, src, n, p, passes, false, st, s)
+                      : onesweep_packed_pass<kFromWords, false>(sc, src, n, p, passes, false, st, s));
     if (e) return e;
   }
-  note_launches(2u + (unsigned)passes);
+  note_launches(2u + (unsigned)(halves * passes));
   return cudaSuccess;
 }
 
-cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf,
-                          const uint32_t* run_if, Status* st, int sms, cudaStream_t s) {
+cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf, Status* st, int sms,
+                          cudaStream_t s) {
   *out_buf = 0;
   if (n <= 1 || passes <= 0) return cudaSuccess;
   if (passes > kPasses) passes = kPasses;
   cudaError_t e;
   bool done = false;
-  if ((e = sort_in_one<false>(sc, SortSource{}, n, passes, run_if, st, sms, s, &done)) || done) {
+  if ((e = sort_in_one<false>(sc, SortSource{}, n, passes, st, sms, s, &done)) || done) {
     *out_buf = passes & 1;
     return e;
   }
@@ -1111,7 +1214,7 @@ cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf,
   if ((e = clear_onesweep(sc, tiles, passes, s))) return e;
   uint32_t hb = (n + kThreads * 16 - 1) / (kThreads * 16);
   if (hb > (uint32_t)sms * 4u) hb = (uint32_t)sms * 4u;
-  k_histogram<<<hb, kThreads, 0, s>>>(sc.keys[0], n, sc.hist, run_if);
+  k_histogram<<<hb, kThreads, 0, s>>>(sc.keys[0], n, sc.hist);
   k_hist_scan<<<kPasses, kRadix, 0, s>>>(sc.hist);
   const size_t smem = sizeof(OnesweepSmem);
   if ((e = cudaFuncSetAttribute(k_onesweep, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1123,7 +1226,7 @@ cudaError_t launch_sort64(SortScratch sc, uint32_t n, int passes, int* out_buf,
                                              sc.vals[src ^ 1], n, p * kRadixBits,
                                              sc.hist + p * kRadix,
                                              sc.lookback + (size_t)p * tiles * kRadix,
-                                             sc.counters + p, run_if, st);
+                                             sc.counters + p, st);
   }
   note_launches(2u + (unsigned)passes);
   *out_buf = passes & 1;
