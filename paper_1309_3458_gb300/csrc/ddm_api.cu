@@ -65,7 +65,9 @@ struct ddm_ctx {
 
   // Ordering workspace: [0] serves both sets in turn; [1] the updates of a
   // one-shot call, ordered on `side` while the tree is built.
+  // Between calls and after the join [1] is given back when room runs out.
   OrderBufs ob[2];
+  bool side_busy = false;
   cudaStream_t side = nullptr;
   cudaEvent_t fork = nullptr, joined = nullptr;
   // tree
@@ -173,6 +175,7 @@ class StreamUse {
   ~StreamUse() {
     c_->work_zeroed[0] = c_->work_zeroed[1] = false;
     c_->walk_pending = false;
+    c_->side_busy = false;
     if (!capturing_ && cudaEventRecord(c_->done, s_) == cudaSuccess) {
       c_->done_pending = true;
       c_->last = s_;
@@ -194,9 +197,24 @@ bool zeroed_work(ddm_ctx* c, int i) {
   return z;
 }
 
-int ensure(ddm_ctx* c, DevBuf& b, size_t bytes) {
-  if (bytes <= b.cap) return DDM_OK;
-  if (c->capturing) return DDM_ERR_NOMEM;  // a graph cannot own the workspace
+void release_now(ddm_ctx* c, DevBuf& b) {
+  if (b.p) {
+    cudaFreeAsync(b.p, c->cur);
+    c->allocated -= b.cap;
+  }
+  b.p = nullptr;
+  b.cap = 0;
+}
+
+// Gives the side stream's workspace back; false if there is none.
+bool release_side(ddm_ctx* c) {
+  const uint64_t before = c->allocated;
+  for (DevBuf* b : c->ob[1].all) release_now(c, *b);
+  release_now(c, c->ob[1].sums);
+  return c->allocated != before;
+}
+
+int grow(ddm_ctx* c, DevBuf& b, size_t bytes) {
   size_t want = bytes + bytes / 4;  // headroom against regrowth
   if (b.p) {
     cudaFreeAsync(b.p, c->cur);  // after the work already enqueued on this stream
@@ -216,6 +234,15 @@ int ensure(ddm_ctx* c, DevBuf& b, size_t bytes) {
   b.cap = want;
   c->allocated += want;
   return DDM_OK;
+}
+
+int ensure(ddm_ctx* c, DevBuf& b, size_t bytes) {
+  if (bytes <= b.cap) return DDM_OK;
+  if (c->capturing) return DDM_ERR_NOMEM;  // a graph cannot own the workspace
+  int rc = grow(c, b, bytes);
+  // What a call needs goes before what only runs it faster.
+  if (rc == DDM_ERR_NOMEM && !c->side_busy && release_side(c)) rc = grow(c, b, bytes);
+  return rc;
 }
 
 // Interleaved copy of a set's coordinates for the gathers by id; NULL (the
@@ -895,15 +922,6 @@ int write_ordered_async(ddm_ctx* c, uint32_t pb, uint32_t pe, ddm_pair* pairs, u
   return DDM_OK;
 }
 
-void release_now(ddm_ctx* c, DevBuf& b) {
-  if (b.p) {
-    cudaFreeAsync(b.p, c->cur);
-    c->allocated -= b.cap;
-  }
-  b.p = nullptr;
-  b.cap = 0;
-}
-
 // Build and plan of a one-shot call: the updates are ordered on the context's
 // side stream while the tree is built -- both are chains of short launches
 // that leave most of the chip idle.  The side stream starts after the work
@@ -924,6 +942,7 @@ int build_and_plan(ddm_ctx* c, int d, const float* slo, const float* shi, uint32
     return plan_async(c, ulo, uhi, m, flags, record, false, s, bs_u, sorted);
   };
   if (m > 0 && n > 0) {
+    c->side_busy = true;
     int rc = bs_u ? ensure_batch(c, o, d, m, bs_u->count) : ensure_sort(c, o, m);
     if (rc == DDM_OK) rc = ensure_queries(c, d, m);
     if (rc == DDM_OK) {
@@ -935,14 +954,13 @@ int build_and_plan(ddm_ctx* c, int d, const float* slo, const float* shi, uint32
         rc = order_updates(c, o, d, ulo, uhi, m, bs_u, aos, c->side);
         DDM_CUDA(cudaEventRecord(c->joined, c->side));  // also after an error: joined before returning
         DDM_CUDA(cudaStreamWaitEvent(s, c->joined, 0));
+        c->side_busy = false;
         if (rc == DDM_OK) rc = sequel(true);
       }
     }
+    c->side_busy = false;
     if (rc != DDM_ERR_NOMEM) return rc;
-    if (!c->capturing) {  // a recorded call neither allocates nor frees
-      for (DevBuf* b : o.all) release_now(c, *b);
-      release_now(c, o.sums);
-    }
+    if (!c->capturing) release_side(c);  // a recorded call neither allocates nor frees
   }
   DDM_TRY(build_async(c, d, slo, shi, n, s, bs_s));
   return sequel(false);
