@@ -778,10 +778,9 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
   const int njobs = !ordered ? 1 : c->arena.max_blocks ? 3 : 2;
   const size_t state_words = kPlanWords + scan_state_words(jobs, njobs);
   DDM_TRY(ensure(c, c->plan_state, sizeof(unsigned long long) * state_words));
-  if (!ordered)  // what ready_ordered() needs, so that it never allocates
-    DDM_TRY(ensure(c, c->order_state,
-                   sizeof(unsigned long long) *
-                       scan_state_words(jobs + 1, c->arena.max_blocks ? 2 : 1)));
+  // what ready_ordered() needs, so that it never allocates
+  DDM_TRY(ensure(c, c->order_state,
+                 sizeof(unsigned long long) * scan_state_words(jobs + 1, c->arena.max_blocks ? 2 : 1)));
   auto* state = static_cast<unsigned long long*>(c->plan_state.p);
   DDM_CUDA(cudaMemsetAsync(state, 0, sizeof(unsigned long long) * state_words, s));
   if (c->arena.max_blocks) c->arena.blk_counter = reinterpret_cast<uint32_t*>(state);
@@ -826,23 +825,25 @@ int walk_or_hold(ddm_ctx* c, const QueryView& q, const WriteView& w, bool synced
 }
 
 // The plan order's offsets and record entries, for a staged call after a
-// one-shot call's plan (a plan made for staged calls has them).
+// one-shot call's plan (a plan made for staged calls has them).  Under capture
+// (ddm_plan_order alone) the offsets are always recorded, from the counts that
+// every plan leaves: the graph may run again after a plan of the other kind.
 int ready_ordered(ddm_ctx* c, cudaStream_t s) {
-  if (c->ordered) return DDM_OK;
+  if (c->ordered && !c->capturing) return DDM_OK;
   const uint32_t packets = packets_of(c, c->m);
   const ScanJob jobs[2] = {
       {static_cast<uint32_t*>(c->counts_pos.p), c->m,
        static_cast<unsigned long long*>(c->pos_offsets.p), false},
       {c->arena.pkt_nblk, packets, c->arena.pkt_off, false}};
-  const int njobs = c->arena.max_blocks ? 2 : 1;
+  const bool list = c->arena.max_blocks && !c->capturing;
+  const int njobs = list ? 2 : 1;
   const size_t words = scan_state_words(jobs, njobs);
   DDM_TRY(ensure(c, c->order_state, sizeof(unsigned long long) * words));  // done by the plan
   auto* state = static_cast<unsigned long long*>(c->order_state.p);
   DDM_CUDA(cudaMemsetAsync(state, 0, sizeof(unsigned long long) * words, s));
   DDM_CUDA(launch_scan_multi(jobs, njobs, state, ScanHint{}, plan_failed(c), c->st_dev, s));
-  if (c->arena.max_blocks)
-    DDM_CUDA(launch_block_list(c->arena, jobs[0].offsets + c->m, c->sms, s));
-  c->ordered = !c->capturing;  // recorded only: it runs with the graph
+  if (list) DDM_CUDA(launch_block_list(c->arena, jobs[0].offsets + c->m, c->sms, s));
+  if (!c->capturing) c->ordered = true;
   return DDM_OK;
 }
 
