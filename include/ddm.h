@@ -379,7 +379,10 @@ int ddm_tree_export(ddm_ctx *ctx, uint32_t *order, float *node_lo, float *node_h
 /* Record budget of the write pass.  While counting, ddm_plan (and the
  * one-shot calls) can keep a compact record of every (update, leaf) test
  * that found pairs -- 10 bytes per record plus 64 bytes per block of 512
- * records, about one record per 12 pairs on clustered d = 3 extents --
+ * records, about one record per 12 pairs on clustered d = 3 extents, but at
+ * least two blocks (10,432 bytes with what is kept beside them) per packet of
+ * queries where the budget reaches for that: 326 bytes per update at 32
+ * queries per packet, 2,608 at the 4 of a plan of few updates --
  * so that the write pass expands the records instead of walking the tree a
  * second time.  The records live in a context arena of at most `bytes`
  * (default: a quarter of the device's memory); the arena is sized from what

@@ -749,6 +749,8 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
     }
     const uint64_t cap_blocks = c->replay_budget / per_block;
     if (want > cap_blocks) want = cap_blocks;
+    // no room for a first block of every chain: all from the counter
+    const bool firsts = want >= (uint64_t)packets * kRecChains;
     if (want > 0xfffffff0ull) want = 0xfffffff0ull;
     if (want > 0 && ensure(c, c->rec, (size_t)want * kRecWords * sizeof(uint32_t)) == DDM_OK &&
         ensure(c, c->blk_own, (size_t)want * sizeof(uint2)) == DDM_OK &&
@@ -762,7 +764,7 @@ int plan_async(ddm_ctx* c, const float* ulo, const float* uhi, uint32_t m, uint3
       c->arena.blk_list = static_cast<uint4*>(c->blk_list.p);
       c->arena.pkt_nblk = static_cast<uint32_t*>(c->pkt_nblk.p);
       c->arena.pkt_off = static_cast<unsigned long long*>(c->pkt_off.p);
-      c->arena.chains = packets * kRecChains;
+      c->arena.chains = firsts ? packets * kRecChains : 0u;
       c->arena.max_blocks = (uint32_t)want;
     }
   }

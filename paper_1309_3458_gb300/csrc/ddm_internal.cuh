@@ -352,7 +352,9 @@ cudaError_t launch_export_nodes(const TreeView& t, float* node_lo, float* node_h
 //
 // The first block of each chain belongs to it from the start (its header is
 // zero); only the blocks after it are taken from a counter, so that the
-// packets of a sparse problem make no atomic.  Every block is an entry of the
+// packets of a sparse problem make no atomic.  (If the record budget does not
+// reach for that, every block is taken from the counter: a plan whose hits lie
+// in few packets can still be recorded.)  Every block is an entry of the
 // write pass, but for the two first blocks of a packet, which are one if the
 // plan has few pairs per entry.
 // A write laid out by update id takes the blocks as they are (the chains'
@@ -387,7 +389,7 @@ struct RecordArena {
   uint32_t* blk_counter;   // [0] blocks handed out beyond the chains' first (may
                            // exceed the arena), [1] such blocks the whole pass
                            // needed
-  uint32_t chains;         // chains of the plan's packets
+  uint32_t chains;         // chains of the plan's packets, 0: no first blocks of their own
   uint32_t max_blocks;     // 0: no recording
 };
 // Pairs per entry of a plan up to which its entries count as short: the write

@@ -296,8 +296,10 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
     // packet stops writing but keeps counting the blocks it would need.
     const bool recording = !WRITE && ra.max_blocks > 0;
     bool rec_write = recording && ra.chains <= ra.max_blocks;
-    uint32_t cur0 = p * 2u, cur1 = p * 2u + 1u, fill0 = 0, fill1 = 0;
-    uint32_t nblk = 0;  // blocks after the chains' first
+    // without first blocks of their own the chains start with none, and full
+    uint32_t cur0 = ra.chains ? p * 2u : kNoBlock, cur1 = ra.chains ? p * 2u + 1u : kNoBlock;
+    uint32_t fill0 = ra.chains ? 0u : kRecBlock, fill1 = fill0;
+    uint32_t nblk = 0;  // blocks handed out to the packet
     uint32_t blk_cnt = 0;  // this query's matches before its chain's current block
     // Test the 32 level-1 nodes (leaves) from g1 on against the packet box,
     // then run the packet's queries over each surviving leaf.
@@ -550,7 +552,7 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
                   b += ra.chains;
                   if (lane == 0) {
                     ra.blk_own[b] = make_uint2(p, nblk);
-                    ra.blk_count[cb] = fl;
+                    if (cb != kNoBlock) ra.blk_count[cb] = fl;
                   }
                   // header: the chain's queries' matches before this leaf
                   if ((uint32_t)(lane >> 4) == (uint32_t)ch) {
@@ -653,10 +655,11 @@ k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
       if (rec_write) {
         // the first blocks' headers: no query had matches before them
         const uint32_t ch = (uint32_t)lane >> 4;
-        ra.rec[((size_t)p * 2u + ch) * kRecWords + 2u * kRecBlock + kRecBlock / 2u + (lane & 15)] = 0u;
-        if (lane < 2) ra.blk_count[lane ? cur1 : cur0] = lane ? fill1 : fill0;
+        if (ra.chains)
+          ra.rec[((size_t)p * 2u + ch) * kRecWords + 2u * kRecBlock + kRecBlock / 2u + (lane & 15)] = 0u;
+        if (lane < 2 && (lane ? cur1 : cur0) != kNoBlock) ra.blk_count[lane ? cur1 : cur0] = lane ? fill1 : fill0;
       }
-      if (lane == 0) ra.pkt_nblk[p] = rec_write ? 1u + nblk : 0u;
+      if (lane == 0) ra.pkt_nblk[p] = rec_write ? (ra.chains ? 1u : 0u) + nblk : 0u;
     }
   }
   if (!WRITE && st && lane == 0 && ntests) atomicAdd(&st->tests, (unsigned long long)ntests);
@@ -677,8 +680,9 @@ __global__ void k_block_list(RecordArena ra, const unsigned long long* __restric
     const bool first = b < ra.chains;
     if (one && first && (b & 1u)) continue;  // listed with the block before it
     const uint2 own = first ? make_uint2(b / kRecChains, 0u) : ra.blk_own[b];
-    const unsigned long long at = ra.pkt_off[own.x] + (one ? 0u : own.x) +
-                                  (first ? b & 1u : (one ? 1u : kRecChains) + own.y);
+    const uint32_t firsts = !ra.chains ? 0u : one ? 1u : kRecChains;  // entries before them
+    const unsigned long long at = ra.pkt_off[own.x] + (firsts > 1u ? own.x : 0u) +
+                                  (first ? b & 1u : firsts + own.y);
     ra.blk_list[at] = make_uint4(b, own.x, ra.blk_count[b], one && first ? ra.blk_count[b + 1] : 0u);
   }
 }
@@ -1176,8 +1180,9 @@ k_replay(TreeView t, QueryView q, BatchView bv, RecordArena ra, WriteView w, uin
   // entries of the range; at most max_blocks, so 32 bits hold them
   uint32_t i0 = 0, i1 = (one ? ra.chains / kRecChains : ra.chains) + ra.blk_counter[0];
   if (ra.blk_list) {
-    i0 = (uint32_t)ra.pkt_off[p0] + (one ? 0u : p0);
-    i1 = (uint32_t)ra.pkt_off[p1] + (one ? 0u : p1);
+    const bool two = ra.chains && !one;  // pkt_off counts the first blocks as one
+    i0 = (uint32_t)ra.pkt_off[p0] + (two ? p0 : 0u);
+    i1 = (uint32_t)ra.pkt_off[p1] + (two ? p1 : 0u);
   }
   if (one)
     replay_short<FILTER_ID, WIDE, BATCH, OUT>(sm, t, q, bv, ra, w, i0, i1, pb, pe, idb, ide, base0,
