@@ -202,6 +202,20 @@ def poisson_schedule(rate: float, duration: float, federates: int, size_lo: int,
     return out
 
 
+RECORD_BLOCK = 5184 + 28  # a block of 512 records with its header and list entries
+
+
+def first_record_bytes(size: int, sms: int) -> int:
+    """Bytes of the record blocks that the packets of a plan of `size` updates
+    own from the start: packets of 32 queries, or of 16, 8 or 4 until there are
+    16 of them per SM, with two blocks each; an eighth of a block per packet
+    and a quarter of headroom beside."""
+    q = 32
+    while q > 4 and -(-size // q) < 16 * sms:
+        q //= 2
+    return int(-(-size // q) * 2.125 * RECORD_BLOCK * 1.25)
+
+
 class Server:
     """Continuous batching of match requests under a device-memory budget.
 
@@ -223,6 +237,8 @@ class Server:
     a launch hold ids within the launch, and request r's slice is shifted by
     its base id ``r.base`` (done when ``keep_pairs`` copies them out)."""
 
+    sms = 152  # of a GB300; the constructor asks the device
+
     def __init__(self, regions: ResidentRegions, l: float, slots: int = 4,
                  budget_bytes: Optional[int] = None, pair_capacity: int = 1 << 25,
                  max_batch_updates: int = 1 << 24, max_batch_requests: int = 1024,
@@ -230,6 +246,7 @@ class Server:
         import torch
         self.regions = regions
         self.l = l
+        self.sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
         self.keep_pairs = keep_pairs
         free, _ = torch.cuda.mem_get_info()
         self.budget = budget_bytes if budget_bytes is not None else int(free * 0.5)
@@ -268,10 +285,12 @@ class Server:
 
     def estimate(self, r: Request) -> int:
         """Device bytes a request occupies while it runs: its share of a
-        plan's workspace (sort, sorted copy, counts, offsets, records) and of
-        the pair buffer."""
+        plan's workspace (sort, sorted copy, counts, offsets), the records of
+        its hits, or the blocks that its packets own without any, and its share
+        of the pair buffer."""
         r.est_pairs = self.expected_pairs(r)
-        return int(r.size * (72 + 16 * self.regions.d) + 16 * r.est_pairs)
+        return int(r.size * (72 + 16 * self.regions.d) + 16 * r.est_pairs
+                   + first_record_bytes(r.size, self.sms))
 
     def _launch(self, slot, batch: List[Request]):
         import torch
