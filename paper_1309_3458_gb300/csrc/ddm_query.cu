@@ -61,12 +61,15 @@ constexpr uint32_t kCompareSwapMin = 24;
 
 // The d = 1 count pass fits six in 40 registers and, waiting for memory most of
 // the time, gains by them: 1.71 ms with four at 2.5e7 + 2.5e7 extents, 1.52
-// with five, 1.46 with six.  For d > 3 the bounds of more dimensions want more
-// registers: the pass of 33,333 queries (d = 5) took 1.17 ms with four CTAs,
-// 1.02 with three, 1.09 with two (2.75 with a run-time dimension count).
-template <int D, bool WRITE>
+// with five, 1.46 with six.  Batched it spills with six (68 bytes): a match of
+// four instances of 2e6 + 2e6 1,816 us with four, 1,775 with five, 1,793 with
+// six, of 4,096 of 1,000 + 1,000 952, 940 and 951.  For d > 3 the bounds of more
+// dimensions want more registers: the pass of 33,333 queries (d = 5) took 1.17
+// ms with four CTAs, 1.02 with three, 1.09 with two (2.75 with a run-time
+// dimension count).
+template <int D, bool WRITE, bool BATCH>
 constexpr int packet_ctas() {
-  return WRITE ? DDM_PACKET_MIN_BLOCKS : D == 1 ? 6 : D > 3 ? 3 : DDM_PACKET_MIN_BLOCKS;
+  return WRITE ? DDM_PACKET_MIN_BLOCKS : D == 1 ? (BATCH ? 5 : 6) : D > 3 ? 3 : DDM_PACKET_MIN_BLOCKS;
 }
 template <bool OPEN>
 __device__ __forceinline__ bool le(float a, float b) {
@@ -181,7 +184,7 @@ DDM_SEG_OR(lt)
 // BATCH: every query matches only its instance's subscription positions, and
 // pairs carry instance-local ids.
 template <int D, bool OPEN, bool WRITE, bool BATCH>
-__global__ void __launch_bounds__(kThreads, packet_ctas<D, WRITE>())
+__global__ void __launch_bounds__(kThreads, packet_ctas<D, WRITE, BATCH>())
 k_packets(TreeView t, QueryView q, BatchView bv, uint32_t* __restrict__ counts,
           uint32_t* __restrict__ counts_pos, RecordArena ra, WriteView w,
           uint32_t* __restrict__ work, Status* __restrict__ st) {
@@ -1240,7 +1243,7 @@ cudaError_t launch_packets(const TreeView& t, const QueryView& q, const BatchVie
   qv.take_log2 = packets / (blocks * kWarps) >= 32u ? 2u : 0u;
   // With every warp resident at once each takes one packet, without tickets
   // (and without the counter to clear).
-  if (blocks <= (uint32_t)sms * packet_ctas<0, WRITE>() && packets <= blocks * kWarps) {
+  if (blocks <= (uint32_t)sms * packet_ctas<0, WRITE, false>() && packets <= blocks * kWarps) {
     work = nullptr;
   } else if (!zeroed) {
     cudaError_t e = cudaMemsetAsync(work, 0, sizeof(uint32_t), s);
