@@ -285,14 +285,15 @@ k_onesweep(const unsigned long long* __restrict__ in_keys, const uint32_t* __res
 // The digits of a warp's elements are often all equal (high digits, instance
 // numbers): then one lane adds them at once, where 32 atomics on one word
 // would take 32 turns.
+// TWO: the second key's digits too (behind the first's) if the sort is by both.
+template <bool TWO>
 __global__ void __launch_bounds__(kThreads)
 k_histogram_packed(const unsigned long long* __restrict__ words, SortSource src, uint32_t n,
                    int passes, uint32_t* __restrict__ hist) {
   __shared__ uint32_t h[kPasses * kRadix];
-  const bool both = src.both && *src.both;
-  const int half = passes;  // the first key's digits, behind them the second's
-  if (both) passes = 2 * half;
-  for (int t = threadIdx.x; t < passes * kRadix; t += kThreads) h[t] = 0;
+  const bool both = TWO && *src.both;
+  const int total = both ? 2 * passes : passes;
+  for (int t = threadIdx.x; t < total * kRadix; t += kThreads) h[t] = 0;
   __syncthreads();
   const uint32_t stride = gridDim.x * kThreads;
   const int lane = threadIdx.x & 31;
@@ -308,7 +309,7 @@ k_histogram_packed(const unsigned long long* __restrict__ words, SortSource src,
       const size_t first = i0 + (size_t)u * stride;
       const bool whole = first + 32u <= n;  // warp-uniform
       if (!whole && first + lane >= n) continue;
-      for (int p = 0; p < half; ++p) {
+      for (int p = 0; p < passes; ++p) {
         const uint32_t d = (uint32_t)(k[u] >> (p * kRadixBits)) & (kRadix - 1);
         if (whole && __all_sync(0xffffffffu, d == __shfl_sync(0xffffffffu, d, 0))) {
           if (lane == 0) atomicAdd(&h[p * kRadix + d], 32u);
@@ -316,15 +317,17 @@ k_histogram_packed(const unsigned long long* __restrict__ words, SortSource src,
           atomicAdd(&h[p * kRadix + d], 1u);
         }
       }
-      if (both) {
-        const unsigned long long k2 = second_word(src, (uint32_t)(first + lane)) >> src.id_bits;
-        for (int p = half; p < passes; ++p)
-          atomicAdd(&h[p * kRadix + ((uint32_t)(k2 >> ((p - half) * kRadixBits)) & (kRadix - 1))], 1u);
-      }
+    }
+  }
+  if (TWO && both) {
+    for (size_t i = blockIdx.x * kThreads + threadIdx.x; i < n; i += stride) {
+      const uint32_t k = float_key(__ldg(src.second + i));
+      for (int p = 0; p < passes; ++p)
+        atomicAdd(&h[(passes + p) * kRadix + ((k >> (p * kRadixBits)) & (kRadix - 1))], 1u);
     }
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < passes * kRadix; t += kThreads)
+  for (int t = threadIdx.x; t < total * kRadix; t += kThreads)
     if (h[t]) atomicAdd(&hist[t], h[t]);
 }
 
@@ -1178,7 +1181,10 @@ cudaError_t launch_sort_packed(SortScratch sc, const SortSource& src, uint32_t n
   const uint32_t tiles = (n + kSortTile - 1) / kSortTile;
   if ((e = clear_onesweep(sc, tiles, halves * passes, s))) return e;
   const uint32_t hb = std::min((n + kThreads * 16 - 1) / (kThreads * 16), (uint32_t)sms * 8u);
-  k_histogram_packed<<<hb, kThreads, 0, s>>>(sc.keys[0], src, n, passes, sc.hist);
+  if (src.both)
+    k_histogram_packed<true><<<hb, kThreads, 0, s>>>(sc.keys[0], src, n, passes, sc.hist);
+  else
+    k_histogram_packed<false><<<hb, kThreads, 0, s>>>(sc.keys[0], src, n, passes, sc.hist);
   k_hist_scan<<<halves * passes, kRadix, 0, s>>>(sc.hist);
   if (src.both) {  // an even number of passes: the words return to keys[0]
     for (int p = 0; p < passes; ++p) {
