@@ -394,8 +394,11 @@ struct RecordArena {
 };
 // Pairs per entry of a plan up to which its entries count as short: the write
 // pass then takes a packet's two first blocks as one entry and expands by
-// listing pairs instead of record by record.
-constexpr uint32_t kShortEntry = 256;
+// listing pairs instead of record by record.  Writes of 5e5 + 5e5 extents, short
+// and long form: d = 1, 65 pairs per entry 54 / 66 us, 129: 65 / 66, 257: 78 /
+// 66, 384: 90 / 68; d = 2, 64: 53 / 66, 128: 65 / 66, 256: 77 / 71; d = 3 (3e5 +
+// 3e5), 130: 53 / 54, 262: 64 / 66, 526: 80 / 69.
+constexpr uint32_t kShortEntry = 160;
 // The records of the last count pass are complete (the write pass may
 // replay them) iff recording was on and the arena did not run out.
 __device__ __forceinline__ bool records_complete(const RecordArena& ra) {

@@ -134,8 +134,8 @@ k_gather(int d, const uint32_t* __restrict__ vals, const float* __restrict__ lo,
 
 // Validation plus the first sort key of the tree order for d >= 2: the size
 // class of the extent -- the binary exponent of its largest side (the float
-// exponent field) -- then the dimension-0 lower bound and, in the low 24
-// bits, the top of the upper bound.  Sorting by class first keeps extents of
+// exponent field) -- above the top 24 bits of the dimension-0 lower bound's
+// key.  Sorting by class first keeps extents of
 // similar size together, so that one long extent does not widen the boxes
 // of a leaf of short ones; the order is a heuristic (node bounds come from
 // the coordinates whatever the order).  hist[class] counts the extents.

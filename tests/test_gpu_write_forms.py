@@ -1,11 +1,11 @@
 """The two forms of the write pass from records (GPU).
 
-Whether a plan's record entries count as short (at most 256 pairs each on
-average: a packet's two first blocks are then one entry) is decided by the whole
-plan, and every range of it follows.  Plans on both sides of the limit that mix
-updates meeting almost everything with updates meeting almost nothing, so that
-ranges of the plan order are far denser or sparser than the plan: pairs in plan
-order, the compressed output and pairs by update id equal the walking write pass.
+Whether a plan's record entries count as short (few pairs each on average: a
+packet's two first blocks are then one entry) is decided by the whole plan, and
+every range of it follows.  Plans on both sides of the limit that mix updates
+meeting almost everything with updates meeting almost nothing, so that ranges of
+the plan order are far denser or sparser than the plan: pairs in plan order, the
+compressed output and pairs by update id equal the walking write pass.
 """
 import numpy as np
 import pytest
