@@ -65,9 +65,10 @@ struct ddm_ctx {
 
   // Ordering workspace: [0] serves both sets in turn; [1] the updates of a
   // one-shot call, ordered on `side` while the tree is built.
-  // Between calls and after the join [1] is given back when room runs out.
+  // Between calls and after the join [1] is given back when room runs out,
+  // unless a recorded call uses it.
   OrderBufs ob[2];
-  bool side_busy = false;
+  bool side_busy = false, side_recorded = false;
   cudaStream_t side = nullptr;
   cudaEvent_t fork = nullptr, joined = nullptr;
   // tree
@@ -206,8 +207,9 @@ void release_now(ddm_ctx* c, DevBuf& b) {
   b.cap = 0;
 }
 
-// Gives the side stream's workspace back; false if there is none.
+// Gives the side stream's workspace back; false if there is none to give.
 bool release_side(ddm_ctx* c) {
+  if (c->side_recorded) return false;
   const uint64_t before = c->allocated;
   for (DevBuf* b : c->ob[1].all) release_now(c, *b);
   release_now(c, c->ob[1].sums);
@@ -953,6 +955,7 @@ int build_and_plan(ddm_ctx* c, int d, const float* slo, const float* shi, uint32
       DDM_CUDA(cudaEventRecord(c->fork, s));
       rc = build_async(c, d, slo, shi, n, s, bs_s);
       if (rc == DDM_OK) {
+        c->side_recorded |= c->capturing;
         DDM_CUDA(cudaStreamWaitEvent(c->side, c->fork, 0));
         rc = order_updates(c, o, d, ulo, uhi, m, bs_u, aos, c->side);
         DDM_CUDA(cudaEventRecord(c->joined, c->side));  // also after an error: joined before returning
