@@ -79,13 +79,14 @@ __device__ void sample_ties(const float* __restrict__ lo, uint32_t cnt, Status* 
   st->runs[0] = st->runs[1] = 0u;
 }
 
+// TREE: the d = 1 tree's keys (whole), else a locality order's.
+template <bool TREE>
 __global__ void __launch_bounds__(kThreads)
 k_validate(int d, const float* __restrict__ lo, const float* __restrict__ hi, uint32_t cnt,
-           uint32_t* __restrict__ k32, bool whole_key, float2* __restrict__ aos,
-           Status* __restrict__ st) {
+           uint32_t* __restrict__ k32, float2* __restrict__ aos, Status* __restrict__ st) {
   bool bad = false;
   uint32_t blocks = gridDim.x;
-  if (whole_key) {  // the last CTA looks for ties
+  if constexpr (TREE) {  // the last CTA looks for ties
     if (blockIdx.x == --blocks) {
       sample_ties(lo, cnt, st);
       return;
@@ -100,7 +101,7 @@ k_validate(int d, const float* __restrict__ lo, const float* __restrict__ hi, ui
       bad |= !(a <= b);  // false for NaN as well as for lo > hi
       if (aos) aos[(size_t)i * d + k] = make_float2(a, b);
     }
-    if (k32) k32[i] = float_key(__ldg(lo + i)) >> (whole_key ? 0 : kLocalityDrop);
+    if (k32) k32[i] = float_key(__ldg(lo + i)) >> (TREE ? 0 : kLocalityDrop);
   }
   if (__ballot_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&st->err, kErrExtent);
 }
@@ -323,7 +324,10 @@ cudaError_t launch_validate(int d, const float* lo, const float* hi, uint32_t cn
                             uint32_t* k32, bool whole_key, float2* aos, Status* st, int sms,
                             cudaStream_t s) {
   if (cnt == 0) return cudaSuccess;
-  k_validate<<<grid_for(cnt, sms) + (whole_key ? 1u : 0u), kThreads, 0, s>>>(d, lo, hi, cnt, k32, whole_key, aos, st);
+  if (whole_key)
+    k_validate<true><<<grid_for(cnt, sms) + 1u, kThreads, 0, s>>>(d, lo, hi, cnt, k32, aos, st);
+  else
+    k_validate<false><<<grid_for(cnt, sms), kThreads, 0, s>>>(d, lo, hi, cnt, k32, aos, st);
   note_launches(1);
   return cudaGetLastError();
 }

@@ -781,17 +781,20 @@ k_sort_cluster(const unsigned long long* __restrict__ in_k, const uint32_t* __re
   const uint32_t valid = min(kTile, n - base);
   unsigned long long key[ITEMS];
   uint32_t val[PACKED ? 1 : ITEMS], rank[ITEMS];
+  auto at = [&](int i) { return (uint32_t)(warp * (ITEMS * 32) + i * 32 + lane); };
+  if (PACKED && src.k32) {
+    if (both) {
 #pragma unroll
-  for (int i = 0; i < ITEMS; ++i) {
-    const uint32_t local = warp * (ITEMS * 32) + i * 32 + lane;
-    if constexpr (PACKED) {
-      key[i] = local >= valid ? ~0ull
-               : both         ? second_word(src, base + local)
-               : src.k32      ? source_word(src, base + local)
-                              : in_k[base + local];
+      for (int i = 0; i < ITEMS; ++i) key[i] = at(i) < valid ? second_word(src, base + at(i)) : ~0ull;
     } else {
-      key[i] = local < valid ? in_k[base + local] : ~0ull;
-      val[i] = local < valid ? in_v[base + local] : 0u;
+#pragma unroll
+      for (int i = 0; i < ITEMS; ++i) key[i] = at(i) < valid ? source_word(src, base + at(i)) : ~0ull;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+      key[i] = at(i) < valid ? in_k[base + at(i)] : ~0ull;
+      if constexpr (!PACKED) val[i] = at(i) < valid ? in_v[base + at(i)] : 0u;
     }
   }
   for (int p = 0; p < passes; ++p) {
@@ -859,8 +862,12 @@ k_sort_cluster(const unsigned long long* __restrict__ in_k, const uint32_t* __re
     for (int i = 0; i < ITEMS; ++i) {
       const uint32_t local = warp * (ITEMS * 32) + i * 32 + lane;
       key[i] = local < valid ? sm.tile_k[local] : ~0ull;
-      if (PACKED && both && p + 1 == half && local < valid) key[i] = first_word(src, key[i]);
       if constexpr (!PACKED) val[i] = local < valid ? sm.tile_v[local] : 0u;
+    }
+    if (both && p + 1 == half) {
+#pragma unroll
+      for (int i = 0; i < ITEMS; ++i)
+        if (at(i) < valid) key[i] = first_word(src, key[i]);
     }
   }
 }
